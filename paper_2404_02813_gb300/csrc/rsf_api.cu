@@ -178,7 +178,7 @@ rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, cons
         unsigned long long tot[4] = {0, 0, 0, 0};
         for (int i = 0; i < nb; ++i) {
             unsigned cnt[4];
-            rsf::tiled_cta_counts(gs.bricks[i], cnt);
+            rsf::tiled_cta_counts(gs.bricks[i], gs.force, gs.taps.R, cnt);
             for (int k = 0; k < 4; ++k) {
                 starts[s0 + (size_t)k * (nb + 1) + i] = (int)tot[k];
                 tot[k] += cnt[k];
@@ -522,12 +522,14 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         b.dt = dt;
         b.zc = c->opt_zchunk;
         b.xyp = rsf::kDefaultXYPlanes;
-        if (b.zc <= 0) {  // enough z chunks for about 16 CTAs per SM
+        b.zs = b.zc;
+        if (b.zc <= 0) {
             int sms = 0;
             RSF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
             const long long nxy = (long long)((nx + 31) / 32) * ((ny + 7) / 8);
             const long long chunks = std::max<long long>(1, (16LL * sms + nxy - 1) / nxy);
             b.zc = (int)std::max<long long>(16, (nz + chunks - 1) / chunks);
+            b.zs = rsf::tiled_update_planes({b}, force, taps.R, b.zc, sms);
         }
         b.dump = dump;  // only rsf_step_stages asks for stages, and it runs one iteration
         std::vector<GroupSpec> specs(1);

@@ -71,8 +71,13 @@ std::string group_key(const GroupSpec &g) {
     return buf;
 }
 
-void set_zc(GroupSpec &g, int zc) {
-    for (rsf::BrickDev &b : g.bricks) b.zc = zc;
+// sms > 0: a chunk may be split over several CTAs; 0: one CTA per chunk.
+void set_zc(GroupSpec &g, int zc, int sms) {
+    const int zs = sms > 0 ? rsf::tiled_update_planes(g.bricks, g.force, g.taps.R, zc, sms) : zc;
+    for (rsf::BrickDev &b : g.bricks) {
+        b.zc = zc;
+        b.zs = zs;
+    }
 }
 
 // One iteration of every group at `parity`.
@@ -89,8 +94,8 @@ void set_xyp(GroupSpec &g, int xyp) {
 }
 
 // The tuned choices on a group whose bricks are in largest-first order.
-void apply_tuned(GroupSpec &g, const TunedGroup &t) {
-    set_zc(g, t.zc);
+void apply_tuned(GroupSpec &g, const TunedGroup &t, int sms) {
+    set_zc(g, t.zc, sms);
     set_xyp(g, t.xyp);
     if (t.order) std::reverse(g.bricks.begin(), g.bricks.end());
 }
@@ -121,7 +126,7 @@ rsf_status autotune(rsf_ctx *c, GroupSpec &g, int sms) {
     const std::string key = group_key(g);
     auto hit = c->tuned.find(key);
     if (hit != c->tuned.end()) {
-        apply_tuned(g, hit->second);
+        apply_tuned(g, hit->second, sms);
         return RSF_OK;
     }
     int maxnz = 16;
@@ -133,7 +138,7 @@ rsf_status autotune(rsf_ctx *c, GroupSpec &g, int sms) {
     rsf_status st = RSF_OK;
     auto trial = [&](const TunedGroup &t, float *ms) {
         GroupSpec h = base;
-        apply_tuned(h, t);
+        apply_tuned(h, t, sms);
         return time_iteration(c, h, e0, e1, ms);
     };
     TunedGroup best;
@@ -172,7 +177,7 @@ rsf_status autotune(rsf_ctx *c, GroupSpec &g, int sms) {
     cudaEventDestroy(e1);
     if (st) return st;
     c->tuned[key] = best;
-    apply_tuned(g, best);
+    apply_tuned(g, best, sms);
     return RSF_OK;
 }
 
@@ -263,7 +268,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         d.nu = b.nu;
         d.mu = b.mu;
         d.dt = b.dt;
-        d.zc = 16;
+        d.zc = d.zs = 16;
         d.xyp = rsf::kDefaultXYPlanes;
         rsf::Fields f;
         f.d = rsf::Dims{d.nx, d.ny, d.nz, (long long)b.nx * b.ny, n};
@@ -322,11 +327,11 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         for (GroupSpec &g : specs) {
             RSF_CUDA(rsf::tiled_prepare(storage, g.taps.R, force));
             if (c->opt_zchunk > 0) {
-                set_zc(g, c->opt_zchunk);
+                set_zc(g, c->opt_zchunk, 0);
             } else if (c->opt_autotune && t == 0 && !tuned_once) {
                 if ((st = autotune(c, g, sms))) return st;
             } else {
-                set_zc(g, default_zc(g.bricks, sms));
+                set_zc(g, default_zc(g.bricks, sms), sms);
             }
         }
         tuned_once = true;

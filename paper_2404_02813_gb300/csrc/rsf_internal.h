@@ -103,7 +103,8 @@ struct BrickDev {
                             // Eq. (15) form: the fits (f1, f2))
     float *ki;              // pitched K*I~ (the centred image convolved), FP32, set once per solve
     float eps, lambda1, lambda2, nu, mu, dt;
-    int zc;                 // z chunk of the update kernel
+    int zc;                 // z chunk of the update kernel (the normals' rounding follows it)
+    int zs;                 // planes per CTA of the update kernel: a z chunk is split into parts of zs
     int xyp;                // z planes per CTA of the x/y kernels (<= 0: kDefaultXYPlanes)
     int flip;               // this brick's buffer parity is the launch parity xor flip
     float *dump;            // optional 5 * n stage fields (f1, f2, g, kappa, L)
@@ -155,7 +156,10 @@ cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, 
 constexpr int tiled_xy_in_pitch(int R) { return ((32 + 2 * R + 15) / 16) * 16 + 2; }
 cudaError_t tiled_prepare(int storage, int R, int force);
 cudaError_t tiled_iterate(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
-void tiled_cta_counts(const BrickDev &b, unsigned counts[4]);
+// CTAs of the four kernels for one brick of a group of the given form and radius.
+void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]);
+// Planes per CTA of the update kernel (at most zc) for bricks launched together with z chunk zc.
+int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, int zc, int sms);
 size_t tiled_stage_bytes(int storage, long long np);
 // Views of one brick's intermediate fields in a block of tiled_stage_bytes(storage, np)
 // bytes, for Li's form (force 0) or the Eq. (15) form (u2 then holds two pairs per

@@ -262,7 +262,7 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
     d.nu = q.nu;
     d.mu = q.mu;
     d.dt = q.dt;
-    d.zc = 16;
+    d.zc = d.zs = 16;
     d.xyp = rsf::kDefaultXYPlanes;
     d.flip = (int)(s->lanes[r->lane].tick & 1);  // its iteration k runs at its lane's tick (admission + k)
     // centring constants (the profiles are set below, exactly as rsf_evolve computes them)
@@ -347,7 +347,11 @@ bool rebuild_groups(Server *s, Lane &L) {
             maxnz = std::max(maxnz, b.nz);
         }
         const int zc = (int)std::min<long long>(maxnz, std::max<long long>(16, work / std::max(1LL, 16LL * s->sms)));
-        for (rsf::BrickDev &b : g.bricks) b.zc = zc;
+        const int zs = rsf::tiled_update_planes(g.bricks, g.force, g.taps.R, zc, s->sms);
+        for (rsf::BrickDev &b : g.bricks) {
+            b.zc = zc;
+            b.zs = zs;
+        }
     }
     // the copy comes from pageable memory and waits for the compute stream; the
     // loop already bounds how far it runs ahead, so this costs one short sync

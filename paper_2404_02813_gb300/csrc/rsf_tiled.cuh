@@ -22,9 +22,10 @@
 //              b = l1 f1^2 - l2 f2^2 (stored FP32, FP16 or BF16).
 //   rsf_tb_xy  the x/y kernel on (a, b); its output stays FP32 (the data term
 //              below is a difference of terms much larger than itself).
-//   rsf_tb_z   a z march over a 32x8 column tile: a register ring of (a, b)
-//              planes, a phi ring and a unit-normal ring in shared memory
-//              (each normal computed once per tile position, not per use);
+//   rsf_tb_z   a z march over a 32 x 14 column tile (12 or 10 rows at larger
+//              radii), two columns per thread: (a, b) and phi rings in shared
+//              memory filled by cp.async, the unit normal computed once per
+//              column and plane;
 //              g = s^2 [ (l1 - l2) K1 I~^2 - 2 I~ K*a + K*b ]  (Eqs. 11-12),
 //              kappa and the Laplacian (Eqs. 3-4), the update of Eqs. (1),
 //              (13), (14), and q of the new phi for the next rsf_ta_xy.
@@ -40,6 +41,7 @@
 
 #include <cstdint>
 #include <type_traits>
+#include <utility>
 
 #include "rsf_internal.h"
 
@@ -50,12 +52,10 @@ constexpr int kXYT = 32;          // x/y kernel: output tile edge (x and y)
 constexpr int kXYThreads = 256;   // 8 warps
 // z-planes per CTA of the x/y kernel: BrickDev::xyp (tuned per brick group), kDefaultXYPlanes by default
 __host__ __device__ __forceinline__ int xy_planes(const BrickDev &B) { return B.xyp > 0 ? B.xyp : kDefaultXYPlanes; }
-constexpr int kZX = 32, kZY = 8;  // z march: columns per CTA
-constexpr int kZThreads = kZX * kZY;
+constexpr int kZX = 32;           // z march: columns (x) per CTA
 constexpr int kAZT = 64;          // x-z slab: output planes per CTA
 constexpr int kAZThreads = 256;
 constexpr int kAZO = kAZT / (kAZThreads / 32);
-constexpr int kPFB = 2;           // (a, b) planes loaded ahead in the z march
 
 __device__ __forceinline__ float2 f2fma(float2 a, float2 b, float2 c) { return __ffma2_rn(a, b, c); }
 
@@ -1240,398 +1240,536 @@ __device__ __forceinline__ float2 heaviside_q_fast2(float2 u, float eps) {
     return make_float2(copysignf(ax >= eps ? at.x : lo.x, u.x), copysignf(ay >= eps ? at.y : lo.y, u.y));
 }
 
-// z march over a 32x8 column tile of one brick, z chunk [z0, z0 + zc), two
-// output planes per step.  Planes are numbered relative to the chunk start
-// (r = z - z0); ring slots are r mod ring size, so with the step loop unrolled
-// over 2 SPB planes every slot index is a compile-time constant.
+// z march over a column tile of one brick: 32 columns x tbz_rows(R) rows, z chunk
+// [z0, z0 + zc), two output planes per step.  Planes are numbered relative to the
+// chunk start (r = z - z0).
 //
-// Step k, outputs zo = z0 + 2k and zo + 1: bring in the planes later steps
-// need (below); barrier; unit normals of planes zo+3, zo+4; outputs zo, zo+1,
-// which read phi zo-1 .. zo+2 and the normals of zo-1 .. zo+2 (earlier steps).
-// Rings: phi 16 planes, normals 8, (a, b) in registers M = 16 or 32 (2R+2
-// planes in use plus those of the next step).  Finite differences use the
-// logical planes, which hold reflect-101 copies outside the brick; the unit
-// normal is itself padded by reflect-101, so the normal of plane -1 is that of
-// plane 1 and the normal of plane nz that of plane nz-2 (the prologue and the
-// step loop copy them).
+// What bounds it: instruction issue first (an earlier form, one column per thread with
+// the three normal components of the whole tile in shared memory, issued 204 thread
+// instructions per voxel and ran at 0.42 of the HBM rate), the shared-memory pipe next.
+// So a thread owns two adjacent columns (x, x + 1): loads, stores and shared-memory
+// accesses are 8 or 16 bytes, the pair is one packed f32x2 operand, and what only its
+// own columns need stays in registers: phi along z, the z component of the unit
+// normal, the in-plane part of the Laplacian (formed from the neighbours the gradient
+// has loaded anyway) and of the curvature.  Shared memory passes to the neighbours only
+// phi, n_x and n_y.  A warp covers two rows of 16 pairs; one more warp marches the
+// rows above and below the tile (for their n_y), the columns left and right of it (for
+// their n_x) and loads phi's halo.
 //
-// Two schedules by radius (measured per radius):
-//   R <= 6: three CTAs per SM at 80 registers.  Step k loads the (a, b) planes
-//     of the next step (zo+R+2, zo+R+3) into the register ring, stores phi
-//     planes zo+4, zo+5 (loaded one step earlier) into the phi ring and loads
-//     zo+6, zo+7, and loads the image and p_z of planes zo+2, zo+3.
-//   R >= 8 (a 32-plane register ring): two CTAs per SM at up to 128
-//     registers, so the loads run two steps ahead to cover the HBM latency at
-//     16 warps per SM.  Step k copies (cp.async) phi planes zo+8, zo+9 straight
-//     into the phi ring and this thread's (a, b) of planes zo+R+6, zo+R+7 into
-//     an 8-plane staging ring, waits for the copies of two steps ago, moves
-//     (a, b) planes zo+R+2, zo+R+3 from the staging ring into the register
-//     ring, and loads the image and p_z of planes zo+4, zo+5.  Offsets within a
-//     field are 32-bit (bricks of fewer than 2^32 pitched voxels).
+// Step k, outputs r0 = 2k and r0 + 1:
+//   unit normals of planes r0 + 1, r0 + 2 from phi planes r0 .. r0 + 3; n_x and n_y into
+//   one of two buffers; wait for the copies issued two steps ago; barrier; issue phi
+//   planes r0 + 9, r0 + 10 (cp.async) into the ring slots of r0 + 1, r0 + 2; the
+//   neighbours' n_x, n_y; outputs.
+// The step k = -1 only brings the march up (normals of planes -1 and 0).
+// Every second step convolves (a, b) along z for four planes at once: the thread's own
+// 2R + 4 planes are in a shared-memory ring that no other thread reads (16 bytes per
+// plane: both columns' pair; cp.async, no barrier), so each 16-byte read serves four
+// planes and no radius needs its planes in registers.  The four planes it frees are
+// refilled at once, two steps before their use.  The ring's slots are compile-time
+// constants in M / 4 copies of the convolution alone (a uniform branch picks the copy);
+// the rest of a step is one piece of code.
+//
+// Tile rows: two CTAs' rings fit an SM's shared memory; 14 rows make eight warps, two on
+// each of the SM's quarters, at 128 registers (nine warps are held to 96, and spilled).
+//
+// Finite differences use reflect-101 for phi (the copies read the mirrored voxel) and
+// for the normal (the reads of n_x, n_y at the first and last column or row take the
+// neighbour on the other side, n_z likewise along z).
+//
+// 512^3, uint16, per launch: radius 6 1.034 -> 0.726 ms, 448 x 512 x 320 radius 10 0.663 -> 0.467 ms;
+// 500^3 uint8, Eq. (15) form 0.906 -> 0.575 ms; 64^3 uint8 21.7 -> 9.1 us (its chunks split).
+// At radius 6 it issues 117 thread instructions per voxel and reaches 0.60 of the HBM rate.
 template <int R>
-constexpr bool tbz_deep() { return R > 6; }
-template <int R>
-constexpr int tbz_ring() { return 2 * R + 4 <= 4 ? 4 : (2 * R + 4 <= 8 ? 8 : (2 * R + 4 <= 16 ? 16 : 32)); }
+constexpr int tbz_rows() { return R <= 8 ? 14 : (R <= 10 ? 12 : 10); }
 
-constexpr int kZPhiRing = 16, kZNrmRing = 8, kZAbRing = 8;
-constexpr int kZPW = kZX + 4, kZPH = kZY + 4;  // phi tile, halo 2
-constexpr int kZNW = kZX + 2, kZNH = kZY + 2;  // normal tile, halo 1
 template <int R>
-constexpr size_t tbz_smem() {
-    return sizeof(float) * (kZPhiRing * kZPH * kZPW + kZNrmRing * 3 * kZNH * kZNW) +
-           (tbz_deep<R>() ? sizeof(float2) * kZAbRing * kZThreads : 0);
+struct TBZ {
+    static constexpr int TY = tbz_rows<R>();
+    static constexpr int NWC = TY / 2;                  // warps with outputs
+    static constexpr int THREADS = (NWC + 1) * 32;
+    static constexpr int M = (2 * R + 4 + 3) / 4 * 4;   // (a, b) planes in the ring
+    static constexpr int PW = kZX + 4, PH = TY + 4;     // phi plane, halo 2: tile column c at c + 2
+    static constexpr int PPL = PW * PH, NPHI = 8;
+    static constexpr int NXP = kZX + 4, NYP = kZX, NH = TY + 2;  // n_x, n_y planes: rows -1 .. TY
+    static constexpr int NPL = NH * (NXP + NYP);
+    static constexpr int ABPL = NWC * 32;               // float4 per (a, b) plane
+    static constexpr size_t bytes = sizeof(float4) * M * ABPL + sizeof(float) * (NPHI * PPL + 4 * NPL);
+    static_assert(2 * TY <= 32, "one lane per column-halo site");
+};
+// f(0), f(1), ... with compile-time arguments
+template <int... D, class F>
+__device__ __forceinline__ void unroll(std::integer_sequence<int, D...>, const F &f) {
+    (f(std::integral_constant<int, D>{}), ...);
 }
 
-__device__ __forceinline__ void cp_async_wait2() { asm volatile("cp.async.wait_group 2;\n" ::: "memory"); }
 __device__ __forceinline__ void cp_async_wait0() { asm volatile("cp.async.wait_group 0;\n" ::: "memory"); }
+__device__ __forceinline__ float sqrt_approx_ftz(float x) {
+    float y;
+    asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+__device__ __forceinline__ float2 ld2(const float *p) { return *reinterpret_cast<const float2 *>(p); }
+// Read-only loads that stay where they are written (a plain load may be moved down to its
+// use behind the barrier, where its latency shows), kept as loaded until that use: unpacking
+// two 8- or 16-bit values beside the load would wait for it there.
+__device__ __forceinline__ float ldg_now(const float *p) {
+    float v;
+    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+template <class ImgT> struct ImgPair;  // two columns' image values: both at once (even nx) or one by one
+template <> struct ImgPair<float> {
+    float a, b;
+    __device__ __forceinline__ void load2(const float *p) {
+        asm volatile("ld.global.nc.v2.f32 {%0, %1}, [%2];" : "=f"(a), "=f"(b) : "l"(p));
+    }
+    __device__ __forceinline__ void load_a(const float *p) { a = ldg_now(p); }
+    __device__ __forceinline__ void load_b(const float *p) { b = ldg_now(p); }
+    template <bool VEC> __device__ __forceinline__ float2 get() const { return make_float2(a, b); }
+};
+template <> struct ImgPair<uint8_t> {
+    uint32_t a, b;
+    __device__ __forceinline__ void load2(const uint8_t *p) {
+        asm volatile("ld.global.nc.u16 %0, [%1];" : "=r"(a) : "l"(p));
+    }
+    __device__ __forceinline__ void load_a(const uint8_t *p) {
+        asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(a) : "l"(p));
+    }
+    __device__ __forceinline__ void load_b(const uint8_t *p) {
+        asm volatile("ld.global.nc.u8 %0, [%1];" : "=r"(b) : "l"(p));
+    }
+    template <bool VEC> __device__ __forceinline__ float2 get() const {
+        return VEC ? make_float2((float)(a & 255u), (float)(a >> 8)) : make_float2((float)a, (float)b);
+    }
+};
+template <> struct ImgPair<uint16_t> {
+    uint32_t a, b;
+    __device__ __forceinline__ void load2(const uint16_t *p) {
+        asm volatile("ld.global.nc.u32 %0, [%1];" : "=r"(a) : "l"(p));
+    }
+    __device__ __forceinline__ void load_a(const uint16_t *p) {
+        asm volatile("ld.global.nc.u16 %0, [%1];" : "=r"(a) : "l"(p));
+    }
+    __device__ __forceinline__ void load_b(const uint16_t *p) {
+        asm volatile("ld.global.nc.u16 %0, [%1];" : "=r"(b) : "l"(p));
+    }
+    template <bool VEC> __device__ __forceinline__ float2 get() const {
+        return VEC ? make_float2((float)(a & 0xffffu), (float)(a >> 16)) : make_float2((float)a, (float)b);
+    }
+};
 
+// Unit normal of two columns from their differences; the central differences' factor
+// 1/2 cancels: d / (|d| + 2e-10) = (d/2) / (|d/2| + 1e-10).  (Where |d|^2 is denormal,
+// 2e-10 + |d| rounds to 2e-10 whether or not the square root flushes it.)  `first_x`
+// takes the sum of squares as z + (x + [y]) instead of z + (y + [x]), [.] rounded alone.
+__device__ __forceinline__ void unit_normal2(float2 gx, float2 gy, float2 gz, bool first_x, float2 &nx, float2 &ny,
+                                             float2 &nz) {
+    float2 ss = __ffma2_rn(gy, gy, f2mul(gx, gx));
+    if (first_x) ss = __ffma2_rn(gx, gx, f2mul(gy, gy));
+    ss = __ffma2_rn(gz, gz, ss);
+    const float2 r = f2add(make_float2(sqrt_approx_ftz(ss.x), sqrt_approx_ftz(ss.y)), f2v(2e-10f));
+    const float2 inv = make_float2(rcp_approx(r.x), rcp_approx(r.y));
+    nx = f2mul(gx, inv);
+    ny = f2mul(gy, inv);
+    nz = f2mul(gz, inv);
+}
+
+// VEC: nx even and the image base aligned for two values, so that a thread's two
+// columns are both inside or both outside the brick and are read and written together.
 // DUMP: also write g, kappa and L of every output to B.dump (rsf_step_stages); a
 // separate instantiation keeps the iteration's kernel free of it.
-template <int R, class ImgT, bool DUMP = false>
-__global__ void __launch_bounds__(kZThreads, tbz_deep<R>() ? 2 : 3) k_tb_z(GroupArgs G, TapPairs t) {
-    constexpr bool DEEP = tbz_deep<R>();
-    constexpr bool PHI_ASYNC = DEEP;  // phi planes copied into the ring two steps ahead (cp.async)
-    using Off = typename std::conditional<DEEP, unsigned, long long>::type;  // offsets within a field
-    constexpr int NIV = DEEP ? 4 : 2;  // image and p_z registers: planes zo .. zo + NIV - 1
+template <int R, class ImgT, bool VEC, bool DUMP>
+__device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B, int bi, const TapPairs &t) {
+    using Z = TBZ<R>;
+    constexpr int TY = Z::TY, M = Z::M, PW = Z::PW, PPL = Z::PPL, NXP = Z::NXP, NYP = Z::NYP, NPL = Z::NPL;
     constexpr int T = 2 * R + 1;
-    constexpr int M = tbz_ring<R>();
-    constexpr int SPB = (M < kZPhiRing ? kZPhiRing : M) / 2;  // steps per unrolled body: 2 SPB planes, a multiple
-                                                              // of every ring size and of NIV
-    constexpr int PW = kZPW, PH = kZPH, NW = kZNW, NH = kZNH;
-    constexpr int PPL = PH * PW, NPL = 3 * NH * NW;
-    constexpr int NPE = (PH * PW + kZThreads - 1) / kZThreads;
-    constexpr int NNE = (NH * NW + kZThreads - 1) / kZThreads;
-    extern __shared__ float zsm[];
-    float *const sphi = zsm;                                                 // [kZPhiRing][PH * PW]
-    float *const snrm = zsm + kZPhiRing * PPL;                               // [kZNrmRing][3][NH * NW]
-    float2 *const sab = reinterpret_cast<float2 *>(snrm + kZNrmRing * NPL);  // DEEP: [kZAbRing][kZThreads]
+    using Img2 = ImgPair<ImgT>;
+    extern __shared__ __align__(16) float zsm[];
+    float4 *const sab = reinterpret_cast<float4 *>(zsm);  // [M][ABPL]
+    float *const sphi = zsm + 4 * M * Z::ABPL;            // [NPHI][PPL]
+    float *const snx = sphi + Z::NPHI * PPL;              // [2 buffers][2 planes]{n_x [NH][NXP], n_y [NH][NYP]}
 
-    const int bi = find_brick(G.starts, G.nb, blockIdx.x);
-    const BrickDev B = G.bricks[bi];
     const int local = blockIdx.x - __ldg(G.starts + bi);
-    const int nbx = (B.nx + kZX - 1) / kZX, nby = (B.ny + kZY - 1) / kZY;
-    const int bx = local % nbx, rr = local / nbx;
     const int nx = B.nx, ny = B.ny, nz = B.nz;
-    const Off plane = (Off)nx * (Off)ny;
-
-    const int tx = threadIdx.x & (kZX - 1), ty = threadIdx.x / kZX;
-    const int x0 = bx * kZX, y0 = (rr % nby) * kZY;
-    const int x = x0 + tx, y = y0 + ty;
-    const bool active = x < nx && y < ny;
-    const int z0 = (rr / nby) * B.zc;
-    const int z1 = min(z0 + B.zc, nz);
-    const int nout = z1 - z0;
-    const int nplanes = nout + 2 * R;  // (a, b) planes of the chunk, r = -R .. nout + R - 1
-    const long long col = (long long)min(y, ny - 1) * nx + min(x, nx - 1);
-    // this thread's column: in its pointers (R <= 6) or in its 32-bit offsets, from warp-uniform
-    // field bases (R >= 8)
-    const long long colp = DEEP ? 0 : col;
-    const Off colo = DEEP ? (Off)col : (Off)0;
-    const int px = B.px;
-    const Off pplane = (Off)px * (Off)ny;
+    const int nbx = (nx + kZX - 1) / kZX, nby = (ny + TY - 1) / TY;
+    const int bx = local % nbx, rr = local / nbx;
+    const int x0 = bx * kZX, y0 = (rr % nby) * TY;
+    const int zpart = rr / nby, parts = (B.zc + B.zs - 1) / B.zs;
+    const int zch = zpart / parts * B.zc;                    // the z chunk of this CTA's planes
+    const int z0 = zch + zpart % parts * B.zs;
+    const int nout = min(min(z0 + B.zs, zch + B.zc), nz) - z0;
+    if (nout <= 0) return;
+    const unsigned plane = (unsigned)nx * (unsigned)ny;      // offsets within a field are 32-bit
     const int par = G.parity ^ B.flip;
     const float *phi = par ? B.phi[1] : B.phi[0];
 
-    int poff[NPE], noff[NNE];
-#pragma unroll
-    for (int e = 0; e < NPE; ++e) {
-        const int i = min((int)threadIdx.x + e * kZThreads, PH * PW - 1);
-        const int ly = i / PW, lx = i - ly * PW;
-        const int gx = refl101(clampi(x0 + lx - 2, -2, nx + 1), nx);
-        const int gy = refl101(clampi(y0 + ly - 2, -2, ny + 1), ny);
-        poff[e] = gy * nx + gx;
-    }
-#pragma unroll
-    for (int e = 0; e < NNE; ++e) {
-        const int i = min((int)threadIdx.x + e * kZThreads, NH * NW - 1);
-        const int ly = i / NW, lx = i - ly * NW;
-        const int qx = refl101(clampi(x0 + lx - 1, -1, nx), nx);
-        const int qy = refl101(clampi(y0 + ly - 1, -1, ny), ny);
-        noff[e] = clampi(qy - y0 + 2, 1, PH - 2) * PW + clampi(qx - x0 + 2, 1, PW - 2);
-    }
-    auto phi_at = [&](int r) { return sphi + ((r + kZPhiRing) & (kZPhiRing - 1)) * PPL; };
-    auto nrm_at = [&](int r) { return snrm + ((r + kZNrmRing) & (kZNrmRing - 1)) * NPL; };
-    auto ab_at = [&](int s) { return sab + (s & (kZAbRing - 1)) * kZThreads; };
-    // phi plane z (logical, -2 .. nz+1 hold reflect-101 copies; planes past nz+1, never read, are
-    // clamped): into registers and then the ring (R <= 6), or copied into the ring (R >= 8)
-    auto phi_plane = [&](int z) { return phi + (Off)refl101(clampi(z, -2, nz + 1), nz) * plane; };
-    auto fetch_phi = [&](int z, float *v) {
-        const float *src = phi_plane(z);
-#pragma unroll
-        for (int e = 0; e < NPE; ++e) v[e] = __ldg(src + poff[e]);
-    };
-    auto store_phi = [&](float *dst, const float *v) {
-#pragma unroll
-        for (int e = 0; e < NPE; ++e)
-            if ((int)threadIdx.x + e * kZThreads < PH * PW) dst[threadIdx.x + e * kZThreads] = v[e];
-    };
-    auto issue_phi = [&](int z, float *dst) {
-        const Off zb = (Off)refl101(clampi(z, -2, nz + 1), nz) * plane;
-#pragma unroll
-        for (int e = 0; e < NPE; ++e)
-            if ((int)threadIdx.x + e * kZThreads < PH * PW)
-                cp_async4(dst + threadIdx.x + e * kZThreads, phi + (zb + (Off)poff[e]), true);
-    };
-    // (a, b) plane s of the chunk (z = z0 - R + s) at this thread's column; zero outside the
-    // brick and past the chunk: a load (R <= 6) or a copy into a staging slot (R >= 8)
-    const long long cab = (long long)min(y, ny - 1) * px + min(x, nx - 1);
-    const float2 *src = B.abxy + (DEEP ? 0 : cab);
-    const Off cabo = DEEP ? (Off)cab : (Off)0;
-    auto ab_ok = [&](int s) { return active && s < nplanes && (unsigned)(z0 - R + s) < (unsigned)nz; };
-    auto load_ab = [&](int s) -> float2 {
-        return ab_ok(s) ? __ldg(src + (cabo + (Off)(z0 - R + s) * pplane)) : make_float2(0.f, 0.f);
-    };
-    auto issue_ab = [&](int s, float2 *slot) {
-        const bool ok = ab_ok(s);
-        cp_async8(slot + threadIdx.x, src + (ok ? cabo + (Off)(z0 - R + s) * pplane : (Off)0), ok);
-    };
-    // unit normals of one plane from phi planes pm, pc, pp of the ring; the
-    // central differences' factor 1/2 cancels: d / (|d| + 2e-10) = (d/2) / (|d/2| + 1e-10)
-    auto normals = [&](const float *pm, const float *pc, const float *pp, float *dst) {
-#pragma unroll
-        for (int e = 0; e < NNE; ++e) {
-            const int i = threadIdx.x + e * kZThreads;
-            if (i < NH * NW) {
-                const int o = noff[e];
-                const float gx = pc[o + 1] - pc[o - 1];
-                const float gy = pc[o + PW] - pc[o - PW];
-                const float gz = pp[o] - pm[o];
-                const float inv = rcp_approx(sqrt_approx(gx * gx + gy * gy + gz * gz) + 2e-10f);
-                dst[i] = gx * inv;
-                dst[NH * NW + i] = gy * inv;
-                dst[2 * NH * NW + i] = gz * inv;
-            }
+    // this thread's pair of columns: rows 2 warp, 2 warp + 1 of the tile, or (halo warp) rows -1, TY
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool comp = warp < Z::NWC;
+    const int hl = lane >> 4, c = 2 * (lane & 15);
+    const int row = comp ? 2 * warp + hl : (hl ? TY : -1);
+    const int x = x0 + c, y = y0 + row;
+    const bool act0 = comp && x < nx && y < ny, act1 = comp && x + 1 < nx && y < ny;
+    const auto refl_y = [&](int v) { return refl101(clampi(v, -2, ny + 1), ny); };
+    const auto refl_x = [&](int v) { return refl101(clampi(v, -2, nx + 1), nx); };
+    // offsets within a plane of the values copied for a pair: two adjacent ones (VEC: a pair
+    // right of the last column is read from nx - 2, whose first value is the mirror of nx)
+    struct PairOff { unsigned a, b; };
+    const auto pair_off = [&](int yy) -> PairOff {
+        const unsigned base = (unsigned)refl_y(yy) * (unsigned)nx;
+        if constexpr (VEC) {
+            const int xs = x < nx ? x : nx - 2;
+            return PairOff{base + xs, base + xs + 1};
+        } else {
+            return PairOff{base + refl_x(x), base + refl_x(x + 1)};
         }
     };
-    // unit normals of two consecutive planes c, c + 1 from phi planes c - 1 .. c + 2, with
-    // packed arithmetic (per lane the operations of normals(), bit for bit)
-    auto normals2 = [&](const float *pm, const float *pc, const float *pp, const float *pq, float *dc, float *dp) {
-#pragma unroll
-        for (int e = 0; e < NNE; ++e) {
-            const int i = threadIdx.x + e * kZThreads;
-            if (i < NH * NW) {
-                const int o = noff[e];
-                const float2 gx = f2sub(make_float2(pc[o + 1], pp[o + 1]), make_float2(pc[o - 1], pp[o - 1]));
-                const float2 gy = f2sub(make_float2(pc[o + PW], pp[o + PW]), make_float2(pc[o - PW], pp[o - PW]));
-                const float2 gz = f2sub(make_float2(pp[o], pq[o]), make_float2(pm[o], pc[o]));
-                const float2 ss = __ffma2_rn(gz, gz, __ffma2_rn(gy, gy, f2mul(gx, gx)));
-                const float2 r = f2add(make_float2(sqrt_approx(ss.x), sqrt_approx(ss.y)), f2v(2e-10f));
-                const float2 inv = make_float2(rcp_approx(r.x), rcp_approx(r.y));
-                const float2 nx2 = f2mul(gx, inv), ny2 = f2mul(gy, inv), nz2 = f2mul(gz, inv);
-                dc[i] = nx2.x;
-                dc[NH * NW + i] = ny2.x;
-                dc[2 * NH * NW + i] = nz2.x;
-                dp[i] = nx2.y;
-                dp[NH * NW + i] = ny2.y;
-                dp[2 * NH * NW + i] = nz2.y;
-            }
+    const auto copy_pair = [&](float *dst, unsigned zoff, const PairOff &o) {
+        if constexpr (VEC) {
+            cp_async8(dst, phi + (zoff + o.a), true);
+        } else {
+            cp_async4(dst, phi + (zoff + o.a), true);
+            cp_async4(dst + 1, phi + (zoff + o.b), true);
         }
     };
-    auto copy_normals = [&](const float *from, float *dst) {
-#pragma unroll
-        for (int e = 0; e < NNE; ++e) {
-            const int i = threadIdx.x + e * kZThreads;
-            if (i < NH * NW) {
-                dst[i] = from[i];
-                dst[NH * NW + i] = from[NH * NW + i];
-                dst[2 * NH * NW + i] = from[2 * NH * NW + i];
+    const PairOff own = pair_off(y);
+    const int si = (row + 2) * PW + c + 2;  // own pair in a phi plane
+    // halo warp: the rows -2 and TY + 1; one column site per lane (column -1 or 32) with
+    // the column beyond it (-2 or 33); the four corners beside the rows -1 and TY
+    const int row2 = hl ? TY + 1 : -2;
+    const PairOff far_row = pair_off(y0 + row2);
+    const int si2 = (row2 + 2) * PW + c + 2;
+    const bool site = !comp && lane < 2 * TY;
+    const int side = lane >= TY ? 1 : 0, srow = min(lane - side * TY, TY - 1);
+    const int ss = (srow + 2) * PW + (side ? kZX + 2 : 1);       // the site in a phi plane
+    const int sf = ss + (side ? 1 : -1);                         // the column beyond it
+    const unsigned so = (unsigned)refl_y(y0 + srow) * (unsigned)nx;
+    const unsigned site_off = so + refl_x(side ? x0 + kZX : x0 - 1), far_off = so + refl_x(side ? x0 + kZX + 1 : x0 - 2);
+    const int crow = (lane & 2) ? TY : -1, ccol = (lane & 1) ? kZX : -1;
+    const int sc = (crow + 2) * PW + ccol + 2;
+    const unsigned corner_off = (unsigned)refl_y(y0 + crow) * (unsigned)nx + refl_x(x0 + ccol);
+
+    // the phi plane at offset zoff of the field into a ring slot
+    const auto copy_phi = [&](float *dst, unsigned zoff) {
+        copy_pair(dst + si, zoff, own);
+        if (!comp) {
+            copy_pair(dst + si2, zoff, far_row);
+            if (site) {
+                cp_async4(dst + ss, phi + (zoff + site_off), true);
+                cp_async4(dst + sf, phi + (zoff + far_off), true);
             }
+            if (lane < 4) cp_async4(dst + sc, phi + (zoff + corner_off), true);
+        }
+    };
+    // phi plane r (relative) into its ring slot (r - 1) mod 8; planes outside the brick are
+    // the mirrored ones, planes past nout + 1 are never read
+    const auto issue_phi = [&](int r) {
+        if (r <= nout + 1)
+            copy_phi(sphi + ((r + 7) & 7) * PPL, (unsigned)refl101(clampi(z0 + r, -2, nz + 1), nz) * plane);
+    };
+    // (a, b) planes r .. r + 3 of this thread's columns into its ring slots from `slot`; zero
+    // outside the brick (the convolution's padding) and past the chunk.  IN: all inside
+    const unsigned px = (unsigned)B.px, pplane = px * (unsigned)ny;
+    const float2 *const abxy = B.abxy;
+    const unsigned ab0 = (unsigned)min(y, ny - 1) * px + (unsigned)min(x, (int)px - 2);
+    float4 *const myab = sab + threadIdx.x;
+    const auto issue_ab = [&](auto in, int r, int slot) {
+        constexpr bool IN = decltype(in)::value;
+        if (!comp) return;
+        unsigned off = ab0 + (unsigned)(z0 + r) * pplane;
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+            const bool ok = act0 && (IN || ((unsigned)(z0 + r + j) < (unsigned)nz && r + j < nout + R));
+            cp_async16(myab + (slot + j) * Z::ABPL, abxy + (IN || ok ? off : ab0), ok);
+            off += pplane;
         }
     };
 
     // K*1 = p_x p_y p_z; with R = 0 (the Eq. (15) form, sigma_2 = 0) the data terms
     // take no convolution and K*1 is 1
-    const float pxy = R == 0 ? 1.f : (active ? __ldg(B.prof + x) * __ldg(B.prof + nx + y) : 0.f);
+    float2 pxy = make_float2(0.f, 0.f);
+    if (R == 0) {
+        pxy = f2v(1.f);
+    } else if (comp && y < ny) {
+        const float py = __ldg(B.prof + nx + y);
+        if (act0) pxy.x = __ldg(B.prof + x) * py;
+        if (act1) pxy.y = __ldg(B.prof + x + 1) * py;
+    }
     const float *profz = B.prof + nx + ny + z0;
     const float l1 = B.lambda1, l2 = B.lambda2, s2 = B.cs[2];
     // the data term's constants folded: s^2 (l1 - l2) p_x p_y (times p_z per plane), -2 s^2, and
     // for the Eq. (15) form s^2 l1, s^2 l2
-    const float cK = s2 * (l1 - l2) * pxy, m2s2 = -2.f * s2, s2l1 = s2 * l1, s2l2 = s2 * l2;
+    const float2 cK = f2mul(f2v(s2 * (l1 - l2)), pxy);
+    const float m2s2 = -2.f * s2, s2l1 = s2 * l1, s2l2 = s2 * l2;
     const float inv_s = B.cs[1], nms = -B.cs[0] * B.cs[1];
     const float eps = B.eps, eps2 = eps * eps;
     const float nu = B.nu, dt_mu = B.dt * B.mu, dt_eps_pi = B.dt * (eps * INV_PI);
-    const ImgT *img = reinterpret_cast<const ImgT *>(B.img) + colp;
-    float *phi_out = (par ? B.phi[0] : B.phi[1]) + colp;
-    float *q_out = (par ? B.q[0] : B.q[1]) + colp;
     float *const dump = DUMP ? B.dump : nullptr;
     const long long n = (long long)plane * nz;
-    // the centred image and p_z at output plane r (unused values past the chunk: 0 and 1)
-    auto img_at = [&](int r) -> float {
-        return (active && r < nout) ? centred(img, (long long)(colo + (Off)(z0 + r) * plane), inv_s, nms) : 0.f;
-    };
-    auto pz_at = [&](int r) -> float { return (R == 0 || r >= nout) ? 1.f : __ldg(profz + r); };
-
-    // prologue: phi planes z0-2 .. z0+3 (R <= 6; z0+4, z0+5 in registers) or z0-2 .. z0+7 and
-    // (a, b) planes s = 2R+2 .. 2R+5 (R >= 8, copies); the register ring's planes s = 0 .. 2R+1
-    // and the image of planes z0 .. z0+NIV-1
-    float pva[NPE], pvb[NPE];
-    if constexpr (PHI_ASYNC) {
-#pragma unroll 1
-        for (int r = -2; r <= 7; ++r) issue_phi(z0 + r, phi_at(r));
-    }
-    if constexpr (DEEP) {
-#pragma unroll
-        for (int j = 2 * R + 2; j < 2 * R + 6; ++j) issue_ab(j, ab_at(j));
-    }
-    if constexpr (PHI_ASYNC || DEEP) {
-        cp_async_commit();
-    } else {
-#pragma unroll 1
-        for (int r = -2; r <= 3; ++r) {
-            fetch_phi(z0 + r, pva);
-            store_phi(phi_at(r), pva);
+    const ImgT *const img = reinterpret_cast<const ImgT *>(B.img);
+    float *const phi_out = par ? B.phi[0] : B.phi[1];
+    float *const q_out = par ? B.q[0] : B.q[1];
+    const unsigned out0 = (unsigned)z0 * plane + (unsigned)min(y, ny - 1) * (unsigned)nx + (unsigned)min(x, nx - 1);
+    // the image of output plane r at this thread's columns (not read past the chunk)
+    const auto img_at = [&](auto in, int r, unsigned off) -> Img2 {
+        Img2 v{};
+        if (decltype(in)::value || r < nout) {
+            if constexpr (VEC) {
+                if (act0) v.load2(img + off);
+            } else {
+                if (act0) v.load_a(img + off);
+                if (act1) v.load_b(img + off + 1);
+            }
         }
-    }
-    float2 ring[M];
-#pragma unroll
-    for (int s = 0; s < 2 * R + 2; ++s) ring[s] = load_ab(s);
-    float iv[NIV], kz[NIV];
-#pragma unroll
-    for (int j = 0; j < NIV; ++j) {
-        iv[j] = img_at(j);
-        kz[j] = pz_at(j);
-    }
-    if constexpr (PHI_ASYNC || DEEP) cp_async_wait0();
-    __syncthreads();
-#pragma unroll 1
-    for (int r = -1; r <= 2; ++r) {
-        const int q = refl101(clampi(z0 + r, -1, nz), nz) - z0;  // physical plane, relative
-        normals(phi_at(q - 1), phi_at(q), phi_at(q + 1), nrm_at(r));
-    }
-    if constexpr (!PHI_ASYNC) {
-        fetch_phi(z0 + 4, pva);
-        fetch_phi(z0 + 5, pvb);
-    }
+        return v;
+    };
+    const auto pz_at = [&](auto in, int r) -> float {
+        return (R == 0 || (!decltype(in)::value && r >= nout)) ? 1.f : ldg_now(profz + r);
+    };
 
-    Off zoff = colo + (Off)z0 * plane;            // offset of the step's first output plane
-    Off aoff = (Off)(z0 + R + 2) * pplane;        // offset of the next step's first (a, b) plane (R <= 6)
-    for (int base = 0; 2 * base < nout; base += SPB) {
+    // reads of the neighbours' n_x, n_y: the mirrored one at the brick's faces
+    const int nxi = (row + 1) * NXP + c + 2, nyi = (row + 1) * NYP + c;
+    const int nxl = x == 0 ? nxi + 1 : nxi - 1;               // left of the first column
+    const int nxr = x + 1 == nx - 1 ? nxi : nxi + 2;          // right of the second
+    const bool lone = x == nx - 1;                            // the second column lies outside
+    const int nyu = y == 0 ? nyi + NYP : nyi - NYP, nyd = y == ny - 1 ? nyi - NYP : nyi + NYP;
+    const int sni = (srow + 1) * NXP + (side ? kZX + 2 : 1);  // the column site's n_x
+
+    // prologue: phi planes -2 .. 5; (a, b) planes -R .. M - R - 1
+    using Edge = std::integral_constant<bool, false>;
+    using Inner = std::integral_constant<bool, true>;
+#pragma unroll 1
+    for (int r = -2; r <= 5; ++r) issue_phi(r);
+    cp_async_commit();
+#pragma unroll 1
+    for (int j = 0; j < M; j += 4) issue_ab(Edge{}, j - R, j);
+    cp_async_commit();
+    cp_async_wait1();
+    __syncthreads();
+
+    float2 phm = f2v(0.f), ph0 = ld2(sphi + 5 * PPL + si), ph1 = ld2(sphi + 6 * PPL + si);
+    float st0 = sphi[5 * PPL + ss], st1 = sphi[6 * PPL + ss];  // the column site's phi planes r0, r0 + 1
+    float2 lxy0 = f2v(0.f), kxy0 = f2v(0.f), nzm = f2v(0.f), nz0 = f2v(0.f);
+    float2 acc[4][2];         // (K*a, K*b) of four planes and both columns,
+    Img2 raw[4];              // their image values
+    float pzq[4];             // and p_z
+    unsigned out = out0;      // offset of the step's first output plane at this thread's columns
+
+    // taps k = -R .. R in order, as each plane of the ring is read once
+    const auto convolve = [&](auto dc) {
+        constexpr int SLOT = 4 * decltype(dc)::value;
 #pragma unroll
-        for (int kk = 0; kk < SPB; ++kk) {
-            const int k = base + kk;
-            const int r0 = 2 * k;  // relative output plane
-            if (r0 < nout) {
-                const int zo = z0 + r0;
-                // the next step's (a, b) planes s = r0 + 2R + 2, + 3 (z = zo + R + 2, + 3) and phi
-                if constexpr (PHI_ASYNC) {
-                    issue_phi(zo + 8, phi_at(2 * kk + 8));
-                    issue_phi(zo + 9, phi_at(2 * kk + 9));
-                }
-                if constexpr (DEEP) {
-                    issue_ab(r0 + 2 * R + 6, ab_at(2 * kk + 2 * R + 6));
-                    issue_ab(r0 + 2 * R + 7, ab_at(2 * kk + 2 * R + 7));
-                }
-                if constexpr (PHI_ASYNC || DEEP) {
-                    cp_async_commit();
-                    cp_async_wait2();  // this thread's copies of two steps ago have landed
-                }
-                if constexpr (DEEP) {
-                    ring[(2 * kk + 2 * R + 2) % M] = ab_at(2 * kk + 2 * R + 2)[threadIdx.x];
-                    ring[(2 * kk + 2 * R + 3) % M] = ab_at(2 * kk + 2 * R + 3)[threadIdx.x];
-                } else {
-                    const bool in2 = active && r0 + 2 < nout && zo + R + 2 < nz;
-                    const bool in3 = active && r0 + 3 < nout && zo + R + 3 < nz;
-                    ring[(2 * kk + 2 * R + 2) % M] = in2 ? __ldg(src + aoff) : make_float2(0.f, 0.f);
-                    ring[(2 * kk + 2 * R + 3) % M] = in3 ? __ldg(src + aoff + pplane) : make_float2(0.f, 0.f);
-                    aoff += 2 * pplane;
-                }
-                if constexpr (!PHI_ASYNC) {
-                    store_phi(phi_at(2 * kk + 4), pva);
-                    store_phi(phi_at(2 * kk + 5), pvb);
-                    fetch_phi(zo + 6, pva);
-                    fetch_phi(zo + 7, pvb);
-                }
-                const float im0 = iv[(2 * kk) % NIV], im1 = iv[(2 * kk + 1) % NIV];
-                const float pz0 = kz[(2 * kk) % NIV], pz1 = kz[(2 * kk + 1) % NIV];
-                iv[(2 * kk) % NIV] = img_at(r0 + NIV);
-                iv[(2 * kk + 1) % NIV] = img_at(r0 + NIV + 1);
-                kz[(2 * kk) % NIV] = pz_at(r0 + NIV);
-                kz[(2 * kk + 1) % NIV] = pz_at(r0 + NIV + 1);
-                __syncthreads();
-                if (zo + 4 < nz) {
-                    normals2(phi_at(2 * kk + 2), phi_at(2 * kk + 3), phi_at(2 * kk + 4), phi_at(2 * kk + 5),
-                             nrm_at(2 * kk + 3), nrm_at(2 * kk + 4));
-                } else {
+        for (int p = 0; p < 4; ++p) acc[p][0] = acc[p][1] = f2v(0.f);
 #pragma unroll
-                    for (int c = 3; c <= 4; ++c) {
-                        if (zo + c < nz)
-                            normals(phi_at(2 * kk + c - 1), phi_at(2 * kk + c), phi_at(2 * kk + c + 1),
-                                    nrm_at(2 * kk + c));
-                        else if (zo + c == nz)
-                            copy_normals(nrm_at(2 * kk + c - 2), nrm_at(2 * kk + c));
-                    }
-                }
-                if (active) {
-                    // outputs zo and zo + 1 together: lane c of every float2 below is plane zo + c
-                    float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
+        for (int j = 0; j < 2 * R + 4; ++j) {
+            const float4 v = myab[(SLOT + j) % M * Z::ABPL];
 #pragma unroll
-                    for (int kt = 0; kt < T; ++kt) {
-                        a0 = f2fma(t.g[kt], ring[(2 * kk + kt) % M], a0);
-                        a1 = f2fma(t.g[kt], ring[(2 * kk + 1 + kt) % M], a1);
-                    }
-                    const float2 im = make_float2(im0, im1);
+            for (int p = 0; p < 4; ++p)
+                if (j - p >= 0 && j - p < T) {
+                    acc[p][0] = f2fma(t.g[j - p], make_float2(v.x, v.y), acc[p][0]);
+                    acc[p][1] = f2fma(t.g[j - p], make_float2(v.z, v.w), acc[p][1]);
+                }
+        }
+    };
+    // Which planes take the other association of the normal's sum of squares: the first four
+    // of a z chunk (offsets -1 .. 2) and the brick's last plane at an odd offset.  Results
+    // stay bit for bit what they were when these planes had code of their own, so that a
+    // suspended run resumes to the same phi.
+    const auto first_x = [&](int r) {
+        const int o = z0 + r - zch;
+        return o <= 2 || (z0 + r == nz - 1 && (o & 1));
+    };
+
+    // one step; OUT: -1 none, 0 / 1 outputs from acc planes 2 OUT, 2 OUT + 1; IN: the planes it
+    // reads and brings in lie inside the chunk (no mirroring, no checks)
+    const auto step = [&](const int k, auto out_c, auto in_c) {
+        constexpr int OUT = decltype(out_c)::value;
+        constexpr bool IN = decltype(in_c)::value;
+        const int r0 = 2 * k;
+        float *const pA = sphi + 2 * (k & 3) * PPL, *const pB = pA + PPL;  // planes r0 + 1, r0 + 2 (later r0 + 9, r0 + 10)
+        const float *const pC = sphi + 2 * ((k + 1) & 3) * PPL;            // plane r0 + 3
+        float *const nA = snx + (OUT == 0 ? 0 : 2) * NPL, *const nB = nA + NPL;
+        if constexpr (OUT == 0) {  // used after the barrier
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {
+                raw[s] = img_at(in_c, r0 + s, out + s * plane);
+                pzq[s] = pz_at(in_c, r0 + s);
+            }
+        }
+        const float2 ph2 = ld2(pB + si), ph3 = ld2(pC + si);
+        float2 nx1, ny1, nz1, nx2, ny2, nz2, lxy1, lxy2;
+        {
+            const float2 xp = make_float2(ph1.y, pA[si + 2]), xm = make_float2(pA[si - 1], ph1.x);
+            const float2 yp = ld2(pA + si + PW), ym = ld2(pA + si - PW);
+            unit_normal2(f2sub(xp, xm), f2sub(yp, ym), f2sub(ph2, ph0), !IN && first_x(r0 + 1), nx1, ny1, nz1);
+            const float2 m2 = f2mul(f2v(-2.f), ph1);
+            lxy1 = f2add(f2add(f2add(xp, xm), m2), f2add(f2add(yp, ym), m2));
+        }
+        {
+            const float2 xp = make_float2(ph2.y, pB[si + 2]), xm = make_float2(pB[si - 1], ph2.x);
+            const float2 yp = ld2(pB + si + PW), ym = ld2(pB + si - PW);
+            unit_normal2(f2sub(xp, xm), f2sub(yp, ym), f2sub(ph3, ph1), !IN && first_x(r0 + 2), nx2, ny2, nz2);
+            const float2 m2 = f2mul(f2v(-2.f), ph2);
+            lxy2 = f2add(f2add(f2add(xp, xm), m2), f2add(f2add(yp, ym), m2));
+        }
+        *reinterpret_cast<float2 *>(nA + nxi) = nx1;
+        *reinterpret_cast<float2 *>(nA + Z::NH * NXP + nyi) = ny1;
+        *reinterpret_cast<float2 *>(nB + nxi) = nx2;
+        *reinterpret_cast<float2 *>(nB + Z::NH * NXP + nyi) = ny2;
+        if (!comp) {  // the column sites: planes r0 + 1 and r0 + 2 as the two packed lanes
+            const float st2 = pB[ss], st3 = pC[ss];
+            if (site) {
+                const float2 gx = f2sub(make_float2(pA[ss + 1], pB[ss + 1]), make_float2(pA[ss - 1], pB[ss - 1]));
+                const float2 gy = f2sub(make_float2(pA[ss + PW], pB[ss + PW]), make_float2(pA[ss - PW], pB[ss - PW]));
+                const float2 gz = f2sub(make_float2(st2, st3), make_float2(st0, st1));
+                float2 a, b, d;
+                unit_normal2(gx, gy, gz, !IN && first_x(r0 + 1), a, b, d);
+                nA[sni] = a.x;
+                if (!IN) unit_normal2(gx, gy, gz, first_x(r0 + 2), a, b, d);
+                nB[sni] = a.y;
+            }
+            st0 = st2;
+            st1 = st3;
+        }
+        cp_async_wait1();  // the copies issued two steps ago have landed
+        __syncthreads();   // for every thread; the normals are complete, phi planes r0 + 1, r0 + 2 free
+        if constexpr (IN) {
+            const unsigned zoff = (unsigned)(z0 + r0 + 9) * plane;
+            copy_phi(pA, zoff);
+            copy_phi(pB, zoff + plane);
+        } else {
+            if constexpr (OUT < 0) issue_phi(6);  // into the slot of plane -2
+            issue_phi(r0 + 9);
+            issue_phi(r0 + 10);
+        }
+        if (comp) {
+            float2 kxy1, kxy2;
+            {
+                const float2 l = make_float2(nA[nxl], nx1.x);
+                float2 p = make_float2(nx1.y, nA[nxr]);
+                if (!VEC && lone) p.x = l.x;
+                kxy1 = f2add(f2sub(p, l), f2sub(ld2(nA + Z::NH * NXP + nyd), ld2(nA + Z::NH * NXP + nyu)));
+            }
+            {
+                const float2 l = make_float2(nB[nxl], nx2.x);
+                float2 p = make_float2(nx2.y, nB[nxr]);
+                if (!VEC && lone) p.x = l.x;
+                kxy2 = f2add(f2sub(p, l), f2sub(ld2(nB + Z::NH * NXP + nyd), ld2(nB + Z::NH * NXP + nyu)));
+            }
+            if constexpr (OUT == 0) {  // K*a, K*b of planes r0 .. r0 + 3
+                const int d = (k >> 1) % (M / 4);  // the ring slot of plane r0 - R is 4 d
+                unroll(std::make_integer_sequence<int, M / 4>{}, [&](auto dc) {
+                    if (d == dc.value) convolve(dc);
+                });
+                issue_ab(in_c, r0 - R + M, 4 * d);
+            }
+            if constexpr (OUT >= 0) {
+                // the normal beyond the brick's first and last plane is the mirrored one
+                const float2 nzb = !IN && z0 + r0 == 0 ? nz1 : nzm;
+                const float2 nza = !IN && z0 + r0 == nz - 1 ? nzm : nz1;
+                const float2 nzc = !IN && z0 + r0 + 1 == nz - 1 ? nz0 : nz2;
+                const float2 kap[2] = {f2mul(f2add(kxy0, f2sub(nza, nzb)), f2v(0.5f)),
+                                       f2mul(f2add(kxy1, f2sub(nzc, nz0)), f2v(0.5f))};
+                const float2 ph[2] = {ph0, ph1};
+                const float2 lap[2] = {f2add(lxy0, f2add(f2add(ph1, phm), f2mul(f2v(-2.f), ph0))),
+                                       f2add(lxy1, f2add(f2add(ph2, ph0), f2mul(f2v(-2.f), ph1)))};
+                const unsigned o0 = out, o1 = out + plane;
+                out = o1 + plane;
+#pragma unroll
+                for (int s = 0; s < 2; ++s) {
+                    if (!IN && s == 1 && r0 + 1 >= nout) break;
+                    const float2 a0 = acc[2 * OUT + s][0], a1 = acc[2 * OUT + s][1];
+                    const float2 im = f2fma(raw[2 * OUT + s].template get<VEC>(), f2v(inv_s), f2v(nms));
                     float2 g;
-                    if constexpr (R == 0) {  // Eq. (15), sigma_2 = 0: the ring holds (f1, f2)
+                    if constexpr (R == 0) {  // Eq. (15), sigma_2 = 0: (a, b) are the fits (f1, f2)
                         const float2 d1 = f2sub(im, make_float2(a0.x, a1.x)), d2 = f2sub(im, make_float2(a0.y, a1.y));
-                        g = __ffma2_rn(f2v(s2l1), f2mul(d1, d1), f2mul(f2v(-s2l2), f2mul(d2, d2)));
+                        g = f2fma(f2v(s2l1), f2mul(d1, d1), f2mul(f2v(-s2l2), f2mul(d2, d2)));
                     } else {  // Li's data terms from K*a, K*b: s^2 [(l1 - l2) K1 I~^2 - 2 I~ K*a + K*b]
-                        const float2 t1 = f2mul(f2mul(f2v(cK), make_float2(pz0, pz1)), f2mul(im, im));
-                        const float2 t2 = __ffma2_rn(f2mul(f2v(m2s2), im), make_float2(a0.x, a1.x), t1);
-                        g = __ffma2_rn(f2v(s2), make_float2(a0.y, a1.y), t2);
+                        const float2 t1 = f2mul(f2mul(cK, f2v(pzq[2 * OUT + s])), f2mul(im, im));
+                        const float2 t2 = f2fma(f2mul(f2v(m2s2), im), make_float2(a0.x, a1.x), t1);
+                        g = f2fma(f2v(s2), make_float2(a0.y, a1.y), t2);
                     }
-                    const int pc0 = (ty + 2) * PW + tx + 2;
-                    const float *pm = phi_at(2 * kk - 1), *p0 = phi_at(2 * kk), *p1 = phi_at(2 * kk + 1),
-                                *pp = phi_at(2 * kk + 2);
-                    const float2 ph = make_float2(p0[pc0], p1[pc0]);
-                    const float2 m2ph = f2mul(f2v(-2.f), ph);
-                    const float2 lap =
-                        f2add(f2add(f2add(f2add(make_float2(p0[pc0 + 1], p1[pc0 + 1]), make_float2(p0[pc0 - 1], p1[pc0 - 1])), m2ph),
-                                    f2add(f2add(make_float2(p0[pc0 + PW], p1[pc0 + PW]), make_float2(p0[pc0 - PW], p1[pc0 - PW])), m2ph)),
-                              f2add(f2add(make_float2(p1[pc0], pp[pc0]), make_float2(pm[pc0], p0[pc0])), m2ph));
-                    const int nc0 = (ty + 1) * NW + tx + 1;
-                    const float *nm = nrm_at(2 * kk - 1), *n0 = nrm_at(2 * kk), *n1 = nrm_at(2 * kk + 1),
-                                *np1 = nrm_at(2 * kk + 2);
-                    constexpr int NZ = 2 * NH * NW;
-                    const float2 kap = f2mul(
-                        f2add(f2add(f2sub(make_float2(n0[nc0 + 1], n1[nc0 + 1]), make_float2(n0[nc0 - 1], n1[nc0 - 1])),
-                                    f2sub(make_float2(n0[NH * NW + nc0 + NW], n1[NH * NW + nc0 + NW]),
-                                          make_float2(n0[NH * NW + nc0 - NW], n1[NH * NW + nc0 - NW]))),
-                              f2sub(make_float2(n1[NZ + nc0], np1[NZ + nc0]), make_float2(nm[NZ + nc0], n0[NZ + nc0]))),
-                        f2v(0.5f));
-                    const float2 den = __ffma2_rn(ph, ph, f2v(eps2));
+                    const float2 den = f2fma(ph[s], ph[s], f2v(eps2));
                     // dt delta (Eq. 14), then phi + dt mu (L - kappa) + dt delta (nu kappa - g) (Eqs. 1, 13)
                     const float2 dtdel = f2mul(f2v(dt_eps_pi), make_float2(rcp_approx(den.x), rcp_approx(den.y)));
-                    const float2 pn = __ffma2_rn(f2v(dt_mu), f2sub(lap, kap),
-                                                 __ffma2_rn(dtdel, __ffma2_rn(f2v(nu), kap, make_float2(-g.x, -g.y)), ph));
+                    const float2 pn =
+                        f2fma(f2v(dt_mu), f2sub(lap[s], kap[s]),
+                              f2fma(dtdel, f2fma(f2v(nu), kap[s], make_float2(-g.x, -g.y)), ph[s]));
                     const float2 qn = heaviside_q_fast2(pn, eps);
-                    phi_out[zoff] = pn.x;
-                    q_out[zoff] = qn.x;
-                    if (r0 + 1 < nout) {
-                        phi_out[zoff + plane] = pn.y;
-                        q_out[zoff + plane] = qn.y;
+                    const unsigned o = s ? o1 : o0;
+                    if constexpr (VEC) {
+                        if (act0) {
+                            *reinterpret_cast<float2 *>(phi_out + o) = pn;
+                            *reinterpret_cast<float2 *>(q_out + o) = qn;
+                        }
+                    } else {
+                        if (act0) {
+                            phi_out[o] = pn.x;
+                            q_out[o] = qn.x;
+                        }
+                        if (act1) {
+                            phi_out[o + 1] = pn.y;
+                            q_out[o + 1] = qn.y;
+                        }
                     }
                     if constexpr (DUMP) {
-                        const long long q0 = colp + (long long)zoff, q1 = q0 + (long long)plane;
-                        dump[2 * n + q0] = g.x;
-                        dump[3 * n + q0] = kap.x;
-                        dump[4 * n + q0] = lap.x;
-                        if (r0 + 1 < nout) {
-                            dump[2 * n + q1] = g.y;
-                            dump[3 * n + q1] = kap.y;
-                            dump[4 * n + q1] = lap.y;
+                        float *const d = dump + o;
+                        if (act0) {
+                            d[2 * n] = g.x;
+                            d[3 * n] = kap[s].x;
+                            d[4 * n] = lap[s].x;
+                        }
+                        if (act1) {
+                            d[2 * n + 1] = g.y;
+                            d[3 * n + 1] = kap[s].y;
+                            d[4 * n + 1] = lap[s].y;
                         }
                     }
                 }
-                zoff += 2 * plane;
             }
+            kxy0 = kxy2;
+        }
+        cp_async_commit();
+        phm = ph1;
+        ph0 = ph2;
+        ph1 = ph3;
+        lxy0 = lxy2;
+        nzm = nz1;
+        nz0 = nz2;
+    };
+    using Out0 = std::integral_constant<int, 0>;
+    using Out1 = std::integral_constant<int, 1>;
+    step(-1, std::integral_constant<int, -1>{}, Edge{});
+    // two steps at a time; both inner when neither the first planes nor the last the second
+    // step brings in (phi r0 + 12, (a, b) r0 - R + M + 3) are near the chunk's ends
+    constexpr int AHEAD = M - R + 3 > 12 ? M - R + 3 : 12;
+#pragma unroll 1
+    for (int k = 0; 2 * k < nout; k += 2) {
+        if (k > 0 && 2 * k + AHEAD < nout) {
+            step(k, Out0{}, Inner{});
+            step(k + 1, Out1{}, Inner{});
+        } else {
+            step(k, Out0{}, Edge{});
+            if (2 * k + 2 < nout) step(k + 1, Out1{}, Edge{});
         }
     }
-    if constexpr (PHI_ASYNC || DEEP) cp_async_wait0();  // no copy into this CTA's shared memory outlives it
+    cp_async_wait0();  // no copy into this CTA's shared memory outlives it
+}
+
+template <int R, class ImgT, bool DUMP = false>
+__global__ void __launch_bounds__(TBZ<R>::THREADS, 2) k_tb_z(GroupArgs G, TapPairs t) {
+    const int bi = find_brick(G.starts, G.nb, blockIdx.x);
+    const BrickDev &B = G.bricks[bi];
+    if (B.nx % 2 == 0 && reinterpret_cast<uintptr_t>(B.img) % (2 * sizeof(ImgT)) == 0)
+        tb_z_march<R, ImgT, true, DUMP>(G, B, bi, t);
+    else
+        tb_z_march<R, ImgT, false, DUMP>(G, B, bi, t);
 }
 
 // ------------------------------------------------------------ launchers
 
-// The update kernel (storage independent; defined in rsf_tiled_f32.cu).
+// The update kernel (storage independent; dispatched in rsf_tiled_f32.cu).
 cudaError_t launch_tb_z(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
 cudaError_t prepare_tb_z(int R);
 

@@ -1,7 +1,8 @@
 // rsf_tiled_f32.cu -- instantiates the tiled iteration with FP32 storage (see
-// rsf_tiled.cuh), the storage-independent update kernel, the q set-up kernel
-// and the host-side launch dispatch.
+// rsf_tiled.cuh), the q set-up kernel and the host-side launch dispatch.
 #include <cudaTypedefs.h>  // PFN_cuTensorMapEncodeTiled
+
+#include <cmath>
 
 #include "rsf_tiled.cuh"
 
@@ -9,76 +10,31 @@ namespace rsf {
 namespace tiled {
 
 namespace {
-template <int R, class ImgT>
-cudaError_t launch_bz_r(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s) {
-    GroupArgs G{g.bricks, g.starts[3], g.nb, parity, g.err, g.fault_tx};
-    ProfScope ps(prof, KID_TB_Z);
-    Taps t = g.taps;
-    if (R == 0) {  // the Eq. (15) form: one unit tap, no convolution of (a, b)
-        t.R = 0;
-        t.g[0] = 1.f;
-    }
-    if (g.dump)
-        k_tb_z<R, ImgT, true><<<g.ncta[3], kZThreads, tbz_smem<R>(), s>>>(G, tap_pairs(t));
-    else
-        k_tb_z<R, ImgT><<<g.ncta[3], kZThreads, tbz_smem<R>(), s>>>(G, tap_pairs(t));
-    return cudaGetLastError();
-}
-template <int R, bool DUMP>
-cudaError_t prepare_bz_d() {
-    cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_tb_z<R, uint8_t, DUMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tbz_smem<R>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_tb_z<R, uint16_t, DUMP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tbz_smem<R>())) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_tb_z<R, float, DUMP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tbz_smem<R>());
-}
-template <int R>
-cudaError_t prepare_bz_i() {
-    const cudaError_t e = prepare_bz_d<R, false>();
-    return e != cudaSuccess ? e : prepare_bz_d<R, true>();
-}
-template <int R>
-cudaError_t launch_bz_i(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s) {
-    switch (g.imgtype) {
-        case 0: return launch_bz_r<R, uint8_t>(g, parity, prof, s);
-        case 1: return launch_bz_r<R, uint16_t>(g, parity, prof, s);
-        default: return launch_bz_r<R, float>(g, parity, prof, s);
-    }
-}
 __global__ void k_q_init(const float *__restrict__ phi, float *__restrict__ q, long long n, float eps) {
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
         q[i] = heaviside_q_fast(__ldg(phi + i), eps);
 }
 }  // namespace
 
+// the update kernel per image type (rsf_tiled_update_*.cu)
+cudaError_t prepare_update_u8(int R);
+cudaError_t prepare_update_u16(int R);
+cudaError_t prepare_update_img32(int R);
+cudaError_t launch_update_u8(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+cudaError_t launch_update_u16(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+cudaError_t launch_update_img32(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+
 cudaError_t prepare_tb_z(int R) {
-    switch (R) {
-        case 0: return prepare_bz_i<0>();
-        case 2: return prepare_bz_i<2>();
-        case 3: return prepare_bz_i<3>();
-        case 4: return prepare_bz_i<4>();
-        case 5: return prepare_bz_i<5>();
-        case 6: return prepare_bz_i<6>();
-        case 8: return prepare_bz_i<8>();
-        case 10: return prepare_bz_i<10>();
-        case 12: return prepare_bz_i<12>();
-        default: return cudaErrorInvalidValue;
-    }
+    cudaError_t e = prepare_update_u8(R);
+    if (e == cudaSuccess) e = prepare_update_u16(R);
+    return e != cudaSuccess ? e : prepare_update_img32(R);
 }
 
 cudaError_t launch_tb_z(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s) {
-    switch (g.force ? 0 : g.taps.R) {
-        case 0: return launch_bz_i<0>(g, parity, prof, s);
-        case 2: return launch_bz_i<2>(g, parity, prof, s);
-        case 3: return launch_bz_i<3>(g, parity, prof, s);
-        case 4: return launch_bz_i<4>(g, parity, prof, s);
-        case 5: return launch_bz_i<5>(g, parity, prof, s);
-        case 6: return launch_bz_i<6>(g, parity, prof, s);
-        case 8: return launch_bz_i<8>(g, parity, prof, s);
-        case 10: return launch_bz_i<10>(g, parity, prof, s);
-        case 12: return launch_bz_i<12>(g, parity, prof, s);
-        default: return cudaErrorInvalidValue;
+    switch (g.imgtype) {
+        case 0: return launch_update_u8(g, parity, prof, s);
+        case 1: return launch_update_u16(g, parity, prof, s);
+        default: return launch_update_img32(g, parity, prof, s);
     }
 }
 
@@ -229,14 +185,68 @@ cudaError_t tiled_iterate(const TiledGroup &g, int parity, Profiler *prof, cudaS
     }
 }
 
-void tiled_cta_counts(const BrickDev &b, unsigned counts[4]) {
+namespace {
+// Tile rows and (a, b) ring planes of the update kernel for radius R (0: the Eq. (15) form).
+struct UpdateTile { int rows, planes; };
+template <int R>
+UpdateTile update_tile_r() { return UpdateTile{tiled::TBZ<R>::TY, tiled::TBZ<R>::M}; }
+UpdateTile update_tile(int R) {
+    switch (R) {
+        case 0: return update_tile_r<0>();
+        case 2: return update_tile_r<2>();
+        case 3: return update_tile_r<3>();
+        case 4: return update_tile_r<4>();
+        case 5: return update_tile_r<5>();
+        case 6: return update_tile_r<6>();
+        case 8: return update_tile_r<8>();
+        case 10: return update_tile_r<10>();
+        default: return update_tile_r<12>();
+    }
+}
+}  // namespace
+
+void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]) {
     const unsigned ntx = (b.nx + tiled::kXYT - 1) / tiled::kXYT, nty = (b.ny + tiled::kXYT - 1) / tiled::kXYT;
     const unsigned nzp = (b.nz + tiled::xy_planes(b) - 1) / tiled::xy_planes(b);
+    const int rows = update_tile(force ? 0 : R).rows;
     counts[0] = ntx * nty * nzp;
     counts[1] = (unsigned)((b.nz + tiled::kAZT - 1) / tiled::kAZT) * ((b.nx + 31) / 32) * b.ny;
     counts[2] = counts[0];
-    counts[3] = (unsigned)((b.nx + tiled::kZX - 1) / tiled::kZX) * ((b.ny + tiled::kZY - 1) / tiled::kZY) *
-                ((b.nz + b.zc - 1) / b.zc);
+    counts[3] = (unsigned)((b.nx + tiled::kZX - 1) / tiled::kZX) * ((b.ny + rows - 1) / rows) *
+                ((b.nz + b.zc - 1) / b.zc) * ((b.zc + b.zs - 1) / b.zs);
+}
+
+// A CTA of the update kernel costs its zs output planes plus about 4 + 0.4 M plane times to
+// fill its rings (M (a, b) planes at 8 of the 22 bytes a voxel moves, and the latency of the
+// first copies).  Two CTAs share an SM.  Few CTAs run in whole waves; many even out but for
+// about half a CTA at the end.
+int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, int zc, int sms) {
+    const UpdateTile tile = update_tile(force ? 0 : R);
+    const double fill = 4.0 + 0.4 * tile.planes, slots = 2.0 * sms;
+    int best = zc, last = 0;
+    double best_cost = 0.0;
+    for (int parts = 1; parts <= zc; ++parts) {
+        int zs = (zc + parts - 1) / parts;
+        if (parts > 1) zs = (zs + 3) / 4 * 4;
+        if (zs == last) {
+            if (zs <= 4) break;
+            continue;
+        }
+        last = zs;
+        double ctas = 0.0;
+        for (const BrickDev &b : bricks) {
+            const int chunks = b.nz / zc, rest = b.nz % zc;
+            ctas += (double)((b.nx + tiled::kZX - 1) / tiled::kZX) * ((b.ny + tile.rows - 1) / tile.rows) *
+                    (chunks * ((zc + zs - 1) / zs) + (rest + zs - 1) / zs);
+        }
+        const double waves = ctas / slots;
+        const double cost = (waves < 4.0 ? std::ceil(waves) : waves + 0.5) * (zs + fill);
+        if (parts == 1 || cost < best_cost) {
+            best_cost = cost;
+            best = zs;
+        }
+    }
+    return best;
 }
 
 // Per pitched voxel, Li's form: (H I~, H) 8 bytes, (a, b) 2 elements of the
@@ -271,7 +281,7 @@ cudaError_t ki_init_r(const BrickDev &b, const Taps &taps, cudaStream_t s) {
     static_assert(tiled::XYLayout<R, 1>::bytes <= 48 * 1024, "k_ki_xy needs no shared-memory opt-in");
     const tiled::TapPairs tp = tiled::tap_pairs(taps);
     unsigned counts[4];
-    tiled_cta_counts(b, counts);
+    tiled_cta_counts(b, 0, R, counts);
     tiled::k_ki_xy<R, ImgT><<<counts[0], tiled::kXYThreads, tiled::XYLayout<R, 1>::bytes, s>>>(b, tp);
     tiled::k_ki_z<R><<<counts[1], tiled::kAZThreads, 0, s>>>(b, tp);
     return cudaGetLastError();

@@ -245,9 +245,10 @@ rsf_status rsf_step_stages(rsf_ctx *ctx, const void *volume, rsf_dtype vt, int64
  *                   else the six-pass iteration; RSF_PATH_PASSES: always the
  *                   six-pass iteration; RSF_PATH_TILED: the tiled iteration
  *                   (other radii then fail with RSF_E_INVAL).
- *   RSF_OPT_ZCHUNK  z planes per CTA of the z-marching kernel; 0 (default)
- *                   picks enough chunks for about 16 CTAs per SM; else >= 8.
- *                   Results do not depend on it.
+ *   RSF_OPT_ZCHUNK  z chunk of the z-marching kernel: the planes of one CTA; 0
+ *                   (default) picks it from the volume's size and may split
+ *                   it over several CTAs; else >= 8.  Results do not depend
+ *                   on it beyond the FP32 rounding of the unit normal.
  *   RSF_OPT_STORAGE rsf_storage of the tiled path's stored fits'
  *                   combinations a, b; RSF_STORE_F32 (default), RSF_STORE_BF16
  *                   or RSF_STORE_F16.  Accumulation is FP32 throughout; phi,
@@ -258,9 +259,9 @@ rsf_status rsf_step_stages(rsf_ctx *ctx, const void *volume, rsf_dtype vt, int64
  *                   16-bit storage needs the tiled path.
  *   RSF_OPT_AUTOTUNE 1: rsf_evolve_batch picks each brick group's launch
  *                   shape by timing discarded first iterations, one knob after
- *                   the other: z planes per CTA of the x/y kernels (16, 8, 32),
- *                   the update kernel's z chunk (a size heuristic, 32, 64, 128,
- *                   256) and the brick-to-CTA order (largest or smallest bricks
+ *                   the other: z planes per CTA of the x/y kernels (16, 8, 32,
+ *                   fewer in groups too small to fill the GPU with that), the
+ *                   update kernel's z chunk (a size heuristic, 32, 64, 128, 256) and the brick-to-CTA order (largest or smallest bricks
  *                   first); the choice is remembered in the context per group
  *                   (radius, image type, storage, form, brick count, size
  *                   class) and listed by rsf_autotune_report.  0 (default):

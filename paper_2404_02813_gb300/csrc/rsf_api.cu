@@ -172,7 +172,6 @@ rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, cons
         for (const rsf::BrickDev &b : gs.bricks) g.dump |= b.dump != nullptr;
         g.err = c->d_err;
         g.fault_tx = c->opt_fault_wait ? 16u : 0u;
-        g.xy_tma = 1;
         const size_t s0 = starts.size();
         starts.resize(s0 + 4 * (size_t)(nb + 1));
         unsigned long long tot[4] = {0, 0, 0, 0};
@@ -194,7 +193,6 @@ rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, cons
             const cudaError_t e = rsf::tiled_encode_maps(b, gs.force, gs.storage, gs.imgtype, gs.taps.R);
             if (e != cudaSuccess) return fail(RSF_E_CUDA, "TMA descriptor of a %dx%dx%d brick: %s", b.nx, b.ny, b.nz,
                                               cudaGetErrorString(e));
-            g.xy_tma &= b.xy_tma;
             all.push_back(b);
         }
         out->push_back(g);
@@ -210,7 +208,8 @@ static void free_fields(rsf_ctx *c) {
     size_t fb = sizeof(float) * (size_t)c->cap_n;
     dev_free(c, c->f.I, fb);
     for (float *&p : c->f.phi) { dev_free(c, p, fb); p = nullptr; }
-    for (float *&p : c->f.q) { dev_free(c, p, fb); p = nullptr; }
+    dev_free(c, c->f.q, 2 * fb);
+    c->f.q = nullptr;
     dev_free(c, c->f.t[0], sizeof(float) * 8 * (size_t)c->cap_np);
     for (float *&p : c->f.t) p = nullptr;
     c->f.I = nullptr;
@@ -236,8 +235,7 @@ rsf_status ensure_fields(rsf_ctx *c, int nx, int ny, int nz) {
         if ((st = dev_alloc(c, (void **)&c->f.I, fb))) return st;
         for (float *&p : c->f.phi)
             if ((st = dev_alloc(c, (void **)&p, fb))) return st;
-        for (float *&p : c->f.q)
-            if ((st = dev_alloc(c, (void **)&p, fb))) return st;
+        if ((st = dev_alloc(c, (void **)&c->f.q, 2 * fb))) return st;
         if ((st = dev_alloc(c, (void **)&c->f.t[0], sizeof(float) * 8 * (size_t)np))) return st;
         for (int i = 1; i < 8; ++i) c->f.t[i] = c->f.t[0] + (size_t)i * np;
         c->cap_n = d.n;
@@ -457,7 +455,7 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     if (st) return st;
     rsf::Fields &f = c->f;
     const long long n = f.d.n;
-    bool ready = f.I && f.prof && f.cs && f.partials && f.phi[0] && f.phi[1] && f.q[0] && f.q[1];
+    bool ready = f.I && f.prof && f.cs && f.partials && f.phi[0] && f.phi[1] && f.q;
     for (float *p : f.t) ready = ready && p;
     if (!ready) return fail(RSF_E_CUDA, "internal error: working fields are not allocated");
     float *dump = nullptr;
@@ -495,7 +493,8 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     RSF_CUDA(rsf::setup_image(vol, (int)vt, taps, f, c->stream, !tiled));
     if (c->opt_poison) {  // NaN bytes in everything the iteration must write before it reads
         RSF_CUDA(cudaMemsetAsync(f.t[0], 0xFF, sizeof(float) * 8 * (size_t)c->cap_np, c->stream));
-        for (float *p : {f.phi[1], f.q[0], f.q[1]}) RSF_CUDA(cudaMemsetAsync(p, 0xFF, sizeof(float) * n, c->stream));
+        RSF_CUDA(cudaMemsetAsync(f.phi[1], 0xFF, sizeof(float) * n, c->stream));
+        RSF_CUDA(cudaMemsetAsync(f.q, 0xFF, 2 * sizeof(float) * n, c->stream));
     }
     RSF_CUDA(xfer(f.phi[0], phi0, sizeof(float) * n, c->stream));
     int cur = 0;
@@ -505,15 +504,12 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         b.nx = (int)nx;
         b.ny = (int)ny;
         b.nz = (int)nz;
-        b.px = f.px;
         b.img = vol;
         b.cs = f.cs;
         b.prof = f.prof;
         b.phi[0] = f.phi[0];
         b.phi[1] = f.phi[1];
-        b.q[0] = f.q[0];
-        b.q[1] = f.q[1];
-        rsf::tiled_stage_views(storage, force, f.t[0], (long long)f.px * ny * nz, &b.u2, &b.ab, &b.abxy, &b.ki);
+        rsf::tiled_place_fields(b, storage, force, (int)vt, f.t[0], sizeof(float) * 8 * (size_t)f.px * ny * nz, f.q, nullptr);
         b.eps = eps;
         b.lambda1 = lambda1;
         b.lambda2 = lambda2;
@@ -521,11 +517,11 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         b.mu = mu;
         b.dt = dt;
         b.zc = c->opt_zchunk;
-        b.xyp = rsf::kDefaultXYPlanes;
         b.zs = b.zc;
+        int sms = 0;
+        RSF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
+        b.xyp = rsf::tiled_xy_planes({b}, force, taps.R, sms);
         if (b.zc <= 0) {
-            int sms = 0;
-            RSF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
             const long long nxy = (long long)((nx + 31) / 32) * ((ny + 7) / 8);
             const long long chunks = std::max<long long>(1, (16LL * sms + nxy - 1) / nxy);
             b.zc = (int)std::max<long long>(16, (nz + chunks - 1) / chunks);
@@ -542,8 +538,8 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         if ((st = upload_groups(c, c->desc, c->stream, specs, &groups))) return st;
         const rsf::TiledGroup &g = groups[0];
         if (iters > 0) {
-            RSF_CUDA(rsf::tiled_q_init(f.phi[0], f.q[0], n, eps, c->stream));
-            RSF_CUDA(rsf::tiled_ki_init(b, (int)vt, taps, c->stream));
+            RSF_CUDA(rsf::tiled_start(b, (int)vt, c->stream));
+            RSF_CUDA(rsf::tiled_ki_init(b, (int)vt, taps, c->d_err, c->stream));
         }
         for (int it = 0; it < iters; ++it) {
             cudaError_t e = rsf::tiled_iterate(g, it & 1, &c->prof, c->stream);

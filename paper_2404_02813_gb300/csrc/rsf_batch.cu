@@ -41,14 +41,15 @@ struct BrickState {
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Device bytes one brick needs in the pool.
-size_t brick_bytes(const rsf_brick &b, int storage, bool stage_image) {
+size_t brick_bytes(const rsf_brick &b, int storage, int force, bool stage_image) {
     const long long n = (long long)b.nx * b.ny * b.nz;
     const long long np = (long long)rsf::tiled_pitch((int)b.nx) * b.ny * b.nz;
-    size_t s = 4 * align256(sizeof(float) * n);                          // phi[2], q[2]
+    size_t s = 4 * align256(sizeof(float) * n);                          // phi[2], q block
     s += align256(sizeof(float) * (b.nx + b.ny + b.nz)) + align256(64);  // profiles, centring constants
     s += align256(rsf::tiled_stage_bytes(storage, np));
     if (stage_image) s += align256(dtype_size(b.vt) * n);
-    return s;
+    return s + align256(rsf::tiled_extra_bytes(stage_image ? nullptr : b.volume, (int)b.nx, (int)b.ny, (int)b.nz,
+                                               (int)b.vt, storage, force));
 }
 
 int default_zc(const std::vector<rsf::BrickDev> &g, int sms) {
@@ -89,14 +90,19 @@ rsf_status launch_all(rsf_ctx *c, const std::vector<rsf::TiledGroup> &groups, in
     return RSF_OK;
 }
 
-void set_xyp(GroupSpec &g, int xyp) {
-    for (rsf::BrickDev &b : g.bricks) b.xyp = xyp;
+// At most xyp planes per x/y CTA, fewer where the group is too small to fill the GPU with that
+// (16 is the most the size heuristic takes; 32 goes beyond it).
+constexpr int kXYPlanes = 16;
+void set_xyp(GroupSpec &g, int xyp, int sms) {
+    const int fit = rsf::tiled_xy_planes(g.bricks, g.force, g.taps.R, sms);
+    const int planes = fit == kXYPlanes ? xyp : std::min(xyp, fit);
+    for (rsf::BrickDev &b : g.bricks) b.xyp = planes;
 }
 
 // The tuned choices on a group whose bricks are in largest-first order.
 void apply_tuned(GroupSpec &g, const TunedGroup &t, int sms) {
     set_zc(g, t.zc, sms);
-    set_xyp(g, t.xyp);
+    set_xyp(g, t.xyp, sms);
     if (t.order) std::reverse(g.bricks.begin(), g.bricks.end());
 }
 
@@ -120,8 +126,9 @@ rsf_status time_iteration(rsf_ctx *c, const GroupSpec &g, cudaEvent_t e0, cudaEv
 // Pick the group's launch choices by timing iterations, one knob after the other from
 // the defaults: z planes per x/y CTA {16, 8, 32}, then the update kernel's z chunk
 // {size heuristic, 32, 64, 128, 256}, then the brick order (largest or smallest
-// first).  The iterations are discarded (the real first iteration rewrites their
-// outputs); the choice is cached in the context per group key.
+// first).  The iterations are discarded: the real first iteration rewrites their
+// outputs, and q, which they rewrite for phi[1], is made again from phi[0].  The choice
+// is cached in the context per group key.
 rsf_status autotune(rsf_ctx *c, GroupSpec &g, int sms) {
     const std::string key = group_key(g);
     auto hit = c->tuned.find(key);
@@ -143,7 +150,7 @@ rsf_status autotune(rsf_ctx *c, GroupSpec &g, int sms) {
     };
     TunedGroup best;
     best.zc = default_zc(g.bricks, sms);
-    best.xyp = rsf::kDefaultXYPlanes;
+    best.xyp = kXYPlanes;
     float ms = 0.f;
     if (!(st = trial(best, &ms))) {
         best.ms = best.ms_default = ms;
@@ -176,6 +183,7 @@ rsf_status autotune(rsf_ctx *c, GroupSpec &g, int sms) {
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (st) return st;
+    for (const rsf::BrickDev &b : g.bricks) RSF_CUDA(rsf::tiled_start(b, g.imgtype, c->stream));
     c->tuned[key] = best;
     apply_tuned(g, best, sms);
     return RSF_OK;
@@ -208,7 +216,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
     size_t total = 0;
     for (int i = 0; i < nb; ++i) {
         stage_img[i] = !on_device(bricks[i].volume);
-        total += brick_bytes(bricks[i], storage, stage_img[i]);
+        total += brick_bytes(bricks[i], storage, force, stage_img[i]);
     }
     if (total > c->pool_cap) {
         dev_free(c, c->pool, c->pool_cap);
@@ -235,7 +243,6 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         const rsf_brick &b = bricks[i];
         BrickState &s = bs[i];
         const long long n = (long long)b.nx * b.ny * b.nz;
-        const int px = rsf::tiled_pitch((int)b.nx);
         s.index = i;
         s.iters = b.iters;
         s.vt = b.vt;
@@ -246,15 +253,14 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         d.nx = (int)b.nx;
         d.ny = (int)b.ny;
         d.nz = (int)b.nz;
-        d.px = px;
         for (int k = 0; k < 2; ++k) d.phi[k] = reinterpret_cast<float *>(take(sizeof(float) * n));
-        for (int k = 0; k < 2; ++k) d.q[k] = reinterpret_cast<float *>(take(sizeof(float) * n));
+        void *q = take(2 * align256(sizeof(float) * n));
         float *prof = reinterpret_cast<float *>(take(sizeof(float) * (b.nx + b.ny + b.nz)));
         float *cs = reinterpret_cast<float *>(take(64));
         d.prof = prof;
         d.cs = cs;
-        const long long np = (long long)px * b.ny * b.nz;
-        rsf::tiled_stage_views(storage, force, take(rsf::tiled_stage_bytes(storage, np)), np, &d.u2, &d.ab, &d.abxy, &d.ki);
+        const size_t stage_bytes = rsf::tiled_stage_bytes(storage, (long long)rsf::tiled_pitch(d.nx) * b.ny * b.nz);
+        void *stage = take(stage_bytes);
         if (stage_img[i]) {
             void *img = take(dtype_size(b.vt) * n);
             RSF_CUDA(xfer(img, b.volume, dtype_size(b.vt) * n, c->stream));
@@ -262,6 +268,8 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         } else {
             d.img = b.volume;
         }
+        rsf::tiled_place_fields(d, storage, force, (int)b.vt, stage, stage_bytes, q,
+                                take(rsf::tiled_extra_bytes(d.img, d.nx, d.ny, d.nz, (int)b.vt, storage, force)));
         d.eps = b.eps;
         d.lambda1 = b.lambda1;
         d.lambda2 = b.lambda2;
@@ -269,7 +277,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         d.mu = b.mu;
         d.dt = b.dt;
         d.zc = d.zs = 16;
-        d.xyp = rsf::kDefaultXYPlanes;
+        d.xyp = 1;
         rsf::Fields f;
         f.d = rsf::Dims{d.nx, d.ny, d.nz, (long long)b.nx * b.ny, n};
         f.partials = c->f.partials;
@@ -277,13 +285,14 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         f.prof = prof;
         RSF_CUDA(rsf::setup_image(d.img, (int)b.vt, make_taps(b.sigma), f, c->stream, false));
         if (c->opt_poison) {  // NaN bytes in everything the iteration must write before it reads
-            RSF_CUDA(cudaMemsetAsync(d.u2, 0xFF, rsf::tiled_stage_bytes(storage, np), c->stream));
-            for (float *q : {d.phi[1], d.q[0], d.q[1]}) RSF_CUDA(cudaMemsetAsync(q, 0xFF, sizeof(float) * n, c->stream));
+            RSF_CUDA(cudaMemsetAsync(stage, 0xFF, stage_bytes, c->stream));
+            RSF_CUDA(cudaMemsetAsync(q, 0xFF, 2 * sizeof(float) * n, c->stream));
+            RSF_CUDA(cudaMemsetAsync(d.phi[1], 0xFF, sizeof(float) * n, c->stream));
         }
         RSF_CUDA(xfer(d.phi[0], b.phi0, sizeof(float) * n, c->stream));
         if (b.iters > 0) {
-            RSF_CUDA(rsf::tiled_q_init(d.phi[0], d.q[0], n, b.eps, c->stream));
-            RSF_CUDA(rsf::tiled_ki_init(d, (int)b.vt, make_taps(b.sigma), c->stream));
+            RSF_CUDA(rsf::tiled_start(d, (int)b.vt, c->stream));
+            RSF_CUDA(rsf::tiled_ki_init(d, (int)b.vt, make_taps(b.sigma), c->d_err, c->stream));
         }
     }
 
@@ -326,6 +335,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         }
         for (GroupSpec &g : specs) {
             RSF_CUDA(rsf::tiled_prepare(storage, g.taps.R, force));
+            set_xyp(g, kXYPlanes, sms);
             if (c->opt_zchunk > 0) {
                 set_zc(g, c->opt_zchunk, 0);
             } else if (c->opt_autotune && t == 0 && !tuned_once) {

@@ -62,10 +62,9 @@ struct Fields {
     float *cs = nullptr;      // [0] m, [1] 1/s, [2] s^2, [3] s   (centring constants)
     float *partials = nullptr;// reduction scratch, 3 * kStatBlocks floats
     float *phi[2] = {nullptr, nullptr};
-    float *q[2] = {nullptr, nullptr};   // tiled path: +-atan(eps/|phi|)/pi of phi[i]
+    float *q = nullptr;       // tiled path: 2 n floats, +-atan(eps/|phi|)/pi of the current phi, pitched
     float *t[8] = {};         // stage buffers: one block of 8 * capacity floats, t[i] = t[0] + i * capacity,
-                              // capacity >= px * ny * nz (the tiled path's pitched fields use the block
-                              // as u (float4), ab and abxy (float2) at offsets 0, 4 np, 6 np)
+                              // capacity >= px * ny * nz (the tiled path's fields: tiled_place_fields)
     int px = 0;               // x pitch of the tiled path's intermediate fields (multiple of 32)
 };
 
@@ -93,30 +92,32 @@ void set_last_error(const char *msg);
 struct BrickDev {
     int nx, ny, nz, px;     // dimensions; x pitch of the intermediate fields
     const void *img;        // image, nx*ny*nz values of the group's image type
+    const void *img_t;      // the image as the TMA boxes read it: img, or a copy with 16-byte rows
+    int ip;                 // row pitch of img_t (values)
+    int qp;                 // row pitch of q (nx rounded up to 4)
     const float *cs;        // centring constants [m, 1/s, s^2, s]
     const float *prof;      // K*1 profiles p_x[nx], p_y[ny], p_z[nz]
-    float *phi[2], *q[2];   // ping-pong level set and its q = +-atan(eps/|phi|)/pi
+    float *phi[2];          // ping-pong level set
+    float *q;               // q = +-atan(eps/|phi|)/pi of the current phi: read by group A's x/y kernel,
+                            // rewritten by the update at the end of the iteration
     float2 *u2;             // pitched x/y-convolved (H I~, H), FP32 (Eq. (15) form: one float4 per voxel,
                             // ((H I~, H), ((1-H) I~, 1-H)))
     void *ab;               // pitched (a, b), storage type
-    float2 *abxy;           // pitched x/y-convolved (a, b), FP32 (also the set-up's scratch for ki;
-                            // Eq. (15) form: the fits (f1, f2))
+    float2 *abxy;           // pitched x/y-convolved (a, b), FP32 (also the set-up's scratch for ki); the memory
+                            // of u2, which is read before this is written (Eq. (15) form: the fits (f1, f2),
+                            // memory of their own)
     float *ki;              // pitched K*I~ (the centred image convolved), FP32, set once per solve
     float eps, lambda1, lambda2, nu, mu, dt;
     int zc;                 // z chunk of the update kernel (the normals' rounding follows it)
     int zs;                 // planes per CTA of the update kernel: a z chunk is split into parts of zs
-    int xyp;                // z planes per CTA of the x/y kernels (<= 0: kDefaultXYPlanes)
+    int xyp;                // z planes per CTA of the x/y kernels
     int flip;               // this brick's buffer parity is the launch parity xor flip
     float *dump;            // optional 5 * n stage fields (f1, f2, g, kappa, L)
     // TMA descriptors (tiled_encode_maps).  Group A's z pass: u2 as FP32 [nz][ny][c nx]
     // (row pitch c px; c = 2, or 4 in the Eq. (15) form) in boxes of 32 c floats x 1 row x
-    // (64 + 2R) planes, and ki as FP32 [nz][ny][nx] in boxes of 32 x 1 x 64.  Group B's x/y
-    // kernel (Li's form, FP32 storage, even R): ab as FP32 [nz][ny][2 nx] in boxes of one
-    // input tile, 2 tiled_xy_in_pitch(R) floats x (32 + 2R) rows x 1 plane.  Group A's x/y
-    // kernel (Li's form, even R, xy_tma): q[0], q[1] as FP32 [nz][ny][nx] and the image in
-    // its type, in boxes of one staged plane (16-byte aligned column origin, 32 + 2R rows)
-    CUtensorMap tm_u, tm_k, tm_ab, tm_q[2], tm_img;
-    int xy_tma;             // 1: tm_q and tm_img are encoded (rows a multiple of 16 bytes, aligned bases)
+    // (64 + 2R) planes, and ki as FP32 [nz][ny][nx] in boxes of 32 x 1 x 64.  The x/y kernels:
+    // one staged plane of a tile (XYField in rsf_tiled.cuh) of q, the image and (Li's form) ab.
+    CUtensorMap tm_u, tm_k, tm_ab, tm_q, tm_img;
 };
 
 // A set of bricks launched together: same radius, image type and storage.
@@ -132,14 +133,11 @@ struct TiledGroup {
     int dump;               // 1: some brick has a stage dump (its update kernel writes g, kappa, L)
     int *err;               // device-visible error word of the kernels' bounded waits (nonzero: expired)
     unsigned fault_tx;      // bytes the TMA barriers expect beyond their copies (0; > 0 in a fault test)
-    int xy_tma;             // 1: every brick has xy_tma set; group A's x/y kernel takes its inputs by TMA
 };
 
 // Device error word values (TiledGroup::err).
 constexpr int kErrWaitExpired = 1;  // a bounded wait for a TMA copy ran out (1 s)
 constexpr int kErrSmemAlign = 2;    // a TMA destination in shared memory was not 128-byte aligned
-
-constexpr int kDefaultXYPlanes = 16;
 
 // Tiled four-kernel path (rsf_tiled*.cu) for the radii it is instantiated for.
 bool tiled_supports(int R);
@@ -147,30 +145,32 @@ bool tiled_supports(int R);
 // bricks of fewer than 2^32 pitched voxels.
 bool tiled_fits(long long nx, long long ny, long long nz);
 int tiled_pitch(int nx);
-// Encodes b's tensor maps from its dimensions, pitch and field views for its
-// group's form (force), storage and radius R: b.tm_u, b.tm_k (Li's form) and
-// b.tm_ab (Li's form, FP32 storage, even R); the others zeroed.
+// Encodes b's tensor maps from its dimensions, pitches and field views for its
+// group's form (force), storage, image type and radius R; those not used are zeroed.
 cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, int R);
-// Row pitch (float2) of the x/y kernels' input tile for radius R: 32 + 2R
-// rounded up to a multiple of 16, plus 2.
-constexpr int tiled_xy_in_pitch(int R) { return ((32 + 2 * R + 15) / 16) * 16 + 2; }
 cudaError_t tiled_prepare(int storage, int R, int force);
 cudaError_t tiled_iterate(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
 // CTAs of the four kernels for one brick of a group of the given form and radius.
 void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]);
+// Planes per CTA of the x/y kernels for bricks launched together (results do not depend on it).
+int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int sms);
 // Planes per CTA of the update kernel (at most zc) for bricks launched together with z chunk zc.
 int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, int zc, int sms);
+// A brick's working memory beside its phi buffers: a stage block of
+// tiled_stage_bytes(storage, px ny nz) bytes, a q block of 8 nx ny nz bytes, and
+// tiled_extra_bytes (0 unless both are too small for a copied image).
 size_t tiled_stage_bytes(int storage, long long np);
-// Views of one brick's intermediate fields in a block of tiled_stage_bytes(storage, np)
-// bytes, for Li's form (force 0) or the Eq. (15) form (u2 then holds two pairs per
-// voxel, abxy the fits (f1, f2); ab and ki are null).
-void tiled_stage_views(int storage, int force, void *base, long long np, float2 **u2, void **ab, float2 **abxy,
-                       float **ki);
-// q = +-atan(eps/|phi|)/pi (sign of phi) before the first tiled iteration.
-cudaError_t tiled_q_init(const float *phi, float *q, long long n, float eps, cudaStream_t s);
-// b.ki = K*I~ before the first tiled iteration (b.img, b.cs set; uses b.abxy as scratch);
-// nothing when b.ki is null (the Eq. (15) form).
-cudaError_t tiled_ki_init(const BrickDev &b, int imgtype, const Taps &taps, cudaStream_t s);
+size_t tiled_extra_bytes(const void *img, int nx, int ny, int nz, int imgtype, int storage, int force);
+// Sets b's pitches and field pointers from its dimensions and image (b.nx, ny, nz, img) in
+// those three blocks (256-byte aligned; stage may be larger than the minimum).
+void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q,
+                        void *extra);
+// Before the first iteration: the image copied to b.img_t where its rows are not 16-byte
+// aligned, and q = +-atan(eps/|phi|)/pi (sign of phi) of b.phi[0].
+cudaError_t tiled_start(const BrickDev &b, int imgtype, cudaStream_t s);
+// b.ki = K*I~ before the first tiled iteration (after tiled_start; b.cs set; uses b.abxy as
+// scratch); nothing when b.ki is null (the Eq. (15) form).  err: the error word of its waits.
+cudaError_t tiled_ki_init(const BrickDev &b, int imgtype, const Taps &taps, int *err, cudaStream_t s);
 
 // One iteration of the separable pass path: phi_in -> phi_out.
 // `stages`, when not null, receives RSF_NSTAGES fields (f1, f2, g, kappa, L).

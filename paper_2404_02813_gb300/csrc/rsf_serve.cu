@@ -170,13 +170,14 @@ void CUDART_CB done_cb(void *p) {
 
 // Device bytes of one served brick: phi and q pairs, profiles, centring
 // constants, the pitched intermediate fields and (host images) a device copy.
-size_t footprint(const rsf_request &r, bool stage_image) {
+size_t footprint(const rsf_request &r, int force, bool stage_image) {
     const long long n = (long long)r.nx * r.ny * r.nz;
     const long long np = (long long)rsf::tiled_pitch((int)r.nx) * r.ny * r.nz;
     size_t b = 4 * align256(sizeof(float) * n) + align256(sizeof(float) * (r.nx + r.ny + r.nz)) + align256(64);
     b += align256(rsf::tiled_stage_bytes((int)r.storage, np));
     if (stage_image) b += align256(dtype_size(r.vt) * n);
-    return b;
+    return b + align256(rsf::tiled_extra_bytes(stage_image ? nullptr : r.volume, (int)r.nx, (int)r.ny, (int)r.nz, (int)r.vt,
+                                               (int)r.storage, force));
 }
 
 // Finish a request that never became active (or failed in set-up).
@@ -197,7 +198,7 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
         return false;
     }
     const bool stage_img = !on_device(q.volume);
-    r->bytes = footprint(q, stage_img);
+    r->bytes = footprint(q, r->force, stage_img);
     {
         std::lock_guard<std::mutex> lk(c->alloc_mu);
         c->used += r->bytes;
@@ -222,7 +223,6 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
         return fail_admit(RSF_E_NOMEM);
     }
     const long long n = (long long)q.nx * q.ny * q.nz;
-    const int px = rsf::tiled_pitch((int)q.nx);
     r->n = n;
     r->lane = lane_of(n);
     r->taps = make_taps(q.sigma);
@@ -239,15 +239,14 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
     d.nx = (int)q.nx;
     d.ny = (int)q.ny;
     d.nz = (int)q.nz;
-    d.px = px;
     for (int k = 0; k < 2; ++k) d.phi[k] = reinterpret_cast<float *>(take(sizeof(float) * n));
-    for (int k = 0; k < 2; ++k) d.q[k] = reinterpret_cast<float *>(take(sizeof(float) * n));
+    void *qb = take(2 * align256(sizeof(float) * n));
     float *prof = reinterpret_cast<float *>(take(sizeof(float) * (q.nx + q.ny + q.nz)));
     float *cs = reinterpret_cast<float *>(take(64));
     d.prof = prof;
     d.cs = cs;
-    const long long np = (long long)px * q.ny * q.nz;
-    rsf::tiled_stage_views(r->storage, r->force, take(rsf::tiled_stage_bytes(r->storage, np)), np, &d.u2, &d.ab, &d.abxy, &d.ki);
+    const size_t stage_bytes = rsf::tiled_stage_bytes(r->storage, (long long)rsf::tiled_pitch(d.nx) * q.ny * q.nz);
+    void *stage = take(stage_bytes);
     if (stage_img) {
         void *img = take(dtype_size(q.vt) * n);
         if (xfer(img, q.volume, dtype_size(q.vt) * n, s->s_setup) != cudaSuccess)
@@ -256,6 +255,8 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
     } else {
         d.img = q.volume;
     }
+    rsf::tiled_place_fields(d, r->storage, r->force, (int)q.vt, stage, stage_bytes, qb,
+                            take(rsf::tiled_extra_bytes(d.img, d.nx, d.ny, d.nz, (int)q.vt, r->storage, r->force)));
     d.eps = q.eps;
     d.lambda1 = q.lambda1;
     d.lambda2 = q.lambda2;
@@ -263,7 +264,7 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
     d.mu = q.mu;
     d.dt = q.dt;
     d.zc = d.zs = 16;
-    d.xyp = rsf::kDefaultXYPlanes;
+    d.xyp = 1;
     d.flip = (int)(s->lanes[r->lane].tick & 1);  // its iteration k runs at its lane's tick (admission + k)
     // centring constants (the profiles are set below, exactly as rsf_evolve computes them)
     rsf::Fields f;
@@ -281,16 +282,16 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
         k_put<<<(ch.count + 255) / 256, 256, 0, s->s_setup>>>(ch, prof);
     }
     if (s->poison) {  // NaN bytes in everything the iteration must write before it reads
-        if (cudaMemsetAsync(d.u2, 0xFF, rsf::tiled_stage_bytes(r->storage, np), s->s_setup) != cudaSuccess)
+        if (cudaMemsetAsync(stage, 0xFF, stage_bytes, s->s_setup) != cudaSuccess ||
+            cudaMemsetAsync(qb, 0xFF, 2 * sizeof(float) * n, s->s_setup) != cudaSuccess ||
+            cudaMemsetAsync(d.phi[1], 0xFF, sizeof(float) * n, s->s_setup) != cudaSuccess)
             return fail_admit(RSF_E_CUDA);
-        for (float *p : {d.phi[1], d.q[0], d.q[1]})
-            if (cudaMemsetAsync(p, 0xFF, sizeof(float) * n, s->s_setup) != cudaSuccess) return fail_admit(RSF_E_CUDA);
     }
     if (xfer(d.phi[0], q.phi0, sizeof(float) * n, s->s_setup) != cudaSuccess)
         return fail_admit(RSF_E_CUDA);
-    if (q.iters > 0 && rsf::tiled_q_init(d.phi[0], d.q[0], n, q.eps, s->s_setup) != cudaSuccess)
+    if (q.iters > 0 && rsf::tiled_start(d, (int)q.vt, s->s_setup) != cudaSuccess)
         return fail_admit(RSF_E_CUDA);
-    if (q.iters > 0 && rsf::tiled_ki_init(d, (int)q.vt, r->taps, s->s_setup) != cudaSuccess)
+    if (q.iters > 0 && rsf::tiled_ki_init(d, (int)q.vt, r->taps, s->ctx->d_err, s->s_setup) != cudaSuccess)
         return fail_admit(RSF_E_CUDA);
     if (rsf::tiled_prepare(r->storage, r->taps.R, r->force) != cudaSuccess) return fail_admit(RSF_E_CUDA);
     if (cudaEventCreateWithFlags(&r->ready, cudaEventDisableTiming) != cudaSuccess) return fail_admit(RSF_E_CUDA);
@@ -347,10 +348,12 @@ bool rebuild_groups(Server *s, Lane &L) {
             maxnz = std::max(maxnz, b.nz);
         }
         const int zc = (int)std::min<long long>(maxnz, std::max<long long>(16, work / std::max(1LL, 16LL * s->sms)));
+        const int xyp = rsf::tiled_xy_planes(g.bricks, g.force, g.taps.R, s->sms);
         const int zs = rsf::tiled_update_planes(g.bricks, g.force, g.taps.R, zc, s->sms);
         for (rsf::BrickDev &b : g.bricks) {
             b.zc = zc;
             b.zs = zs;
+            b.xyp = xyp;
         }
     }
     // the copy comes from pageable memory and waits for the compute stream; the
@@ -459,7 +462,7 @@ void loop(Server *s) {
                     lk.lock();
                     continue;
                 }
-                const size_t need = footprint(r->req, !on_device(r->req.volume));
+                const size_t need = footprint(r->req, r->force, !on_device(r->req.volume));
                 uint64_t used, budget;
                 {
                     std::lock_guard<std::mutex> al(c->alloc_mu);
@@ -599,7 +602,7 @@ extern "C" rsf_status rsf_submit(rsf_ctx *c, const rsf_request *req, uint64_t *t
                            2 * (int64_t)req->halo >= req->nz))
         return fail(RSF_E_INVAL, "halo %d leaves no core in a %lld x %lld x %lld brick", (int)req->halo,
                     (long long)req->nx, (long long)req->ny, (long long)req->nz);
-    const size_t need = footprint(*req, !on_device(req->volume));
+    const size_t need = footprint(*req, c->opt_force, !on_device(req->volume));
     if (need > c->budget)
         return fail(RSF_E_NOMEM, "request needs %zu bytes of device memory; the budget is %llu", need,
                     (unsigned long long)c->budget);

@@ -7,11 +7,10 @@
 // paper's volume-level parallelism, Sec. 4.1).  A CTA finds its brick by a
 // binary search over the per-kernel CTA offsets of the group.
 //
-//   rsf_ta_xy  per z-plane, a 32x32 output tile plus an R halo in shared
-//              memory: forms H I~ and H (Eqs. 6, 8-10) from the image
-//              (centred on load; four columns per load where alignment
-//              allows) and q = +-atan(eps/|phi|)/pi, convolves the pair along
-//              x then y (packed f32x2 FMAs) and stores it (FP32).
+//   rsf_ta_xy  per z-plane and 32-column tile, q = +-atan(eps/|phi|)/pi and the
+//              image by TMA; forms H I~ and H (Eqs. 6, 8-10; the image centred)
+//              as it reads them, convolves the pair along x then y (packed f32x2
+//              FMAs) and stores it (FP32).
 //   rsf_ta_z   x-z slabs (32 columns x 64 output planes) staged in shared
 //              memory by cp.async, two slabs in flight; z convolution over a
 //              register window; the local fits f1 = K*(H I~)/K*H and
@@ -50,8 +49,6 @@ namespace tiled {
 
 constexpr int kXYT = 32;          // x/y kernel: output tile edge (x and y)
 constexpr int kXYThreads = 256;   // 8 warps
-// z-planes per CTA of the x/y kernel: BrickDev::xyp (tuned per brick group), kDefaultXYPlanes by default
-__host__ __device__ __forceinline__ int xy_planes(const BrickDev &B) { return B.xyp > 0 ? B.xyp : kDefaultXYPlanes; }
 constexpr int kZX = 32;           // z march: columns (x) per CTA
 constexpr int kAZT = 64;          // x-z slab: output planes per CTA
 constexpr int kAZThreads = 256;
@@ -117,13 +114,6 @@ template <> struct Store<__nv_bfloat16> {
     __device__ __forceinline__ static V2 pack2(float2 v) { return p(v.x, v.y); }
     __device__ __forceinline__ static float2 unpack2(V2 v) { return u(v); }
 };
-
-// Image value, centred and scaled on load: (I - m) / s = I * (1/s) + (-m/s),
-// one rounding (1/s is a power of two), the same value the centring kernel stores.
-template <class T>
-__device__ __forceinline__ float centred(const T *img, long long p, float inv_s, float nms) {
-    return fmaf((float)__ldg(img + p), inv_s, nms);
-}
 
 // ------------------------------------------------------------ brick table
 
@@ -224,648 +214,380 @@ __device__ __forceinline__ void report_error(int *err, int code) {
 
 // ---------------------------------------------------------------- x / y
 
-// A producer of the x/y kernel's input pairs: plane(off) gives the plane at
-// element offset `off`, fetch(plane, o) the raw values at offset o within it,
-// apply() the NP float2 pairs (zero outside the brick).
-template <class ImgT>
-struct ProH {  // (H I~, H) from q and the centred image
-    const float *q;
-    const ImgT *img;
+// The x/y kernels: per z-plane and tile of 32 columns x XYG::TH rows, the x then the y
+// convolution (zero padding) of one or two FP32 pairs per voxel.
+//
+// What bounds them: the shared-memory pipe (an earlier form, with 32 x 32 tiles, a pass
+// that wrote the products into a tile of their own and four outputs per thread in both
+// phases, moved 1.02 wavefronts per voxel at radius 6 and kept that pipe 85 % busy).  So
+//  - the TMA box of a plane (q and image, or (a, b)) is the x phase's own input: the
+//    products H I~, H are formed in registers as the window is read;
+//  - a warp's x phase is one item of 8 rows x 32 columns, eight outputs per lane, so that
+//    a window of 8 + 2R inputs serves eight outputs; rows of all items are at most 64,
+//    one item per warp;
+//  - the y phase gives each lane TH / 8 rows of one column.
+// Reads and writes are 16 bytes wherever the row pitch allows; an 8-lane phase covers
+// 8 rows, whose pitch is an odd number of 16-byte units: no bank conflicts.
+// A staging buffer is refilled as soon as the x phase has read it.  (H I~, H): one buffer,
+// four CTAs per SM (two buffers: the same time; three CTAs: 4 % slower).  (a, b), whose
+// boxes are larger and whose phases shorter: two buffers, three CTAs per SM (0.342 against
+// 0.370 ms at 512^3 with one buffer and four CTAs).
+//
+// Per launch, before and now: 512^3 uint16 radius 6, (H I~, H) 0.541 -> 0.463 ms (issue and
+// FMA pipe 60 and 50 % busy), (a, b) 0.393 -> 0.342 ms (0.92 of the HBM rate); 512 x 448 x
+// 320 radius 10 0.519 -> 0.400 and 0.327 -> 0.282 ms; both pairs, 500^3 uint8 radius 10,
+// 1.741 -> 1.12 ms (FMA pipe 65 %: 105 packed FMAs per voxel); (a, b) in BF16, 768^3, 1.764
+// -> 1.083 ms; 64^3 uint8 21.6 -> 8.1 and 15.7 -> 6.3 us (fewer planes per CTA).
+template <int R>
+struct XYG {
+    static constexpr int TH = R <= 8 ? 48 : 40;  // output rows
+    static constexpr int H = TH + 2 * R;         // staged rows: at most 64 (one item of 8 rows per warp)
+    static constexpr int YT = TH / (kXYThreads / 32);
+    static constexpr int NI = 8 + 2 * R;         // inputs of an x-phase window
+    static constexpr int T = 2 * R + 1;
+    static_assert(H <= 64 && TH % 8 == 0, "x/y tile rows");
+};
+constexpr int round_up(int v, int m) { return (v + m - 1) / m * m; }
+// the smallest multiple of `unit` >= need that is an odd number of units
+constexpr int odd_pitch(int need, int unit) { return (round_up(need, unit) / unit) % 2 ? round_up(need, unit) : round_up(need, unit) + unit; }
+// Staging geometry of one field with E values per 16 bytes, read by windows of V values
+// (V values are 8 or 16 bytes): the box starts RA >= R columns left of the tile (16-byte
+// aligned), a window's first aligned read at column xo + B, its first input O values in.
+template <int R, int E, int V>
+struct XYField {
+    static constexpr int RA = round_up(R, E);
+    static constexpr int O = (RA - R) % V, B = RA - R - O;
+    static constexpr int N = (O + XYG<R>::NI + V - 1) / V;  // reads per window
+    static constexpr int need = 24 + B + N * V > 32 + RA + R ? 24 + B + N * V : 32 + RA + R;
+    static constexpr int W = odd_pitch(need, E);            // box width and row pitch (values)
+    static_assert(W <= 256, "box width");
+};
+
+template <class T> struct ImgVec;  // eight bytes of uint8, sixteen of the others
+template <> struct ImgVec<uint8_t> {
+    static constexpr int V = 8;
+    uint2 w;
+    __device__ __forceinline__ void load(const uint8_t *p) { w = *reinterpret_cast<const uint2 *>(p); }
+    __device__ __forceinline__ float get(int i) const { return (float)(((i < 4 ? w.x : w.y) >> (8 * (i & 3))) & 255u); }
+};
+template <> struct ImgVec<uint16_t> {
+    static constexpr int V = 8;
+    uint4 w;
+    __device__ __forceinline__ void load(const uint16_t *p) { w = *reinterpret_cast<const uint4 *>(p); }
+    __device__ __forceinline__ float get(int i) const {
+        const uint32_t u = i < 2 ? w.x : (i < 4 ? w.y : (i < 6 ? w.z : w.w));
+        return (float)((u >> (16 * (i & 1))) & 0xffffu);
+    }
+};
+template <> struct ImgVec<float> {
+    static constexpr int V = 4;
+    float4 w;
+    __device__ __forceinline__ void load(const float *p) { w = *reinterpret_cast<const float4 *>(p); }
+    __device__ __forceinline__ float get(int i) const { return i == 0 ? w.x : (i == 1 ? w.y : (i == 2 ? w.z : w.w)); }
+};
+
+// A source of the x phase: CTAs per SM and staging buffers its kernel is built for, geometry of
+// its staging buffer, issue() of one plane's boxes
+// (one thread), fix() of what the copies' zero fill gets wrong outside the brick (all
+// threads; FIX: it is needed), and window(): f(j, pairs) for the NI inputs of a window.
+template <int R, class ImgT, int NP_>
+struct SrcH {  // NP = 1: (H I~, H); NP = 2: also ((1-H) I~, 1-H), the other side of Eq. (10)
+    static constexpr int NP = NP_, CTAS = NP == 1 ? 4 : 3, NS = 1;
+    static constexpr bool FIX = true;
+    using G = XYG<R>;
+    using FQ = XYField<R, 4, 4>;
+    using FI = XYField<R, 16 / (int)sizeof(ImgT), ImgVec<ImgT>::V>;
+    static constexpr int QB = FQ::W * G::H * 4, IB = FI::W * G::H * (int)sizeof(ImgT);
+    static constexpr int IOFF = round_up(QB, 128), BYTES = IOFF + round_up(IB, 128);
+    const CUtensorMap *mq, *mi;
     float inv_s, nms;
-    struct Raw { float q, im; };
-    struct Plane { const float *q; const ImgT *img; };
-    __device__ __forceinline__ Plane plane(long long off) const { return Plane{q + off, img + off}; }
-    __device__ __forceinline__ Raw fetch(const Plane &pl, int o) const {
-        return Raw{__ldg(pl.q + o), fmaf((float)__ldg(pl.img + o), inv_s, nms)};
+    __device__ __forceinline__ void fence() const {
+        fence_tensormap(mq);
+        fence_tensormap(mi);
     }
-    __device__ __forceinline__ Raw zero() const { return Raw{0.f, 0.f}; }
-    __device__ __forceinline__ void apply(const Raw &r, bool inside, float2 *v) const {
-        const float h = h_of_q(r.q);
-        v[0] = inside ? make_float2(h * r.im, h) : make_float2(0.f, 0.f);
+    __device__ __forceinline__ void issue(unsigned char *st, int x0, int y0, int z, uint64_t *bar, unsigned more) const {
+        mbar_arrive_expect_tx(bar, (unsigned)(QB + IB) + more);
+        tma_load_3d(st, mq, x0 - FQ::RA, y0 - R, z, bar);
+        tma_load_3d(st + IOFF, mi, x0 - FI::RA, y0 - R, z, bar);
+    }
+    // q = 1 outside the brick: h_of_q(1) = 0, so both products vanish there (q itself is at
+    // most 1/2 in magnitude; zero-filled q would read as H = 1)
+    __device__ __forceinline__ void fix(unsigned char *st, int x0, int y0, int nx, int ny) const {
+        float *q = reinterpret_cast<float *>(st);
+        const int lane = threadIdx.x & 31;
+        for (int row = threadIdx.x >> 5; row < G::H; row += kXYThreads / 32) {
+            const bool out = (unsigned)(y0 - R + row) >= (unsigned)ny;
+            for (int c = lane; c < FQ::W; c += 32)
+                if (out || (unsigned)(x0 - FQ::RA + c) >= (unsigned)nx) q[row * FQ::W + c] = 1.f;
+        }
+    }
+    template <class F>
+    __device__ __forceinline__ void window(const unsigned char *st, int row, int xo, const F &f) const {
+        const float *q = reinterpret_cast<const float *>(st) + row * FQ::W + xo + FQ::B;
+        const ImgT *im = reinterpret_cast<const ImgT *>(st + IOFF) + row * FI::W + xo + FI::B;
+        float4 q4 = make_float4(0.f, 0.f, 0.f, 0.f);
+        ImgVec<ImgT> iv;
+#pragma unroll
+        for (int j = 0; j < G::NI; ++j) {
+            const int jq = j + FQ::O, ji = j + FI::O;
+            if (j == 0 || jq % 4 == 0) q4 = *reinterpret_cast<const float4 *>(q + jq / 4 * 4);
+            if (j == 0 || ji % ImgVec<ImgT>::V == 0) iv.load(im + ji / ImgVec<ImgT>::V * ImgVec<ImgT>::V);
+            const float qj = jq % 4 == 0 ? q4.x : (jq % 4 == 1 ? q4.y : (jq % 4 == 2 ? q4.z : q4.w));
+            const float v = fmaf(iv.get(ji % ImgVec<ImgT>::V), inv_s, nms);
+            const float h = h_of_q(qj);
+            float2 p[NP];
+            p[0] = make_float2(__fmul_rn(h, v), h);
+            if constexpr (NP == 2) {
+                const float hc = qj < 0.75f ? hc_of_q(qj) : 0.f;
+                p[1] = make_float2(__fmul_rn(hc, v), hc);
+            }
+            f(j, p);
+        }
     }
 };
 
-template <class ImgT>
-struct ProH2 : ProH<ImgT> {  // (H I~, H) and ((1-H) I~, 1-H): both sides of Eq. (10) for the Eq. (15) form
-    using typename ProH<ImgT>::Raw;
-    __device__ __forceinline__ void apply(const Raw &r, bool inside, float2 *v) const {
-        const float h = h_of_q(r.q), hc = hc_of_q(r.q);
-        v[0] = inside ? make_float2(h * r.im, h) : make_float2(0.f, 0.f);
-        v[1] = inside ? make_float2(hc * r.im, hc) : make_float2(0.f, 0.f);
-    }
-};
-
-template <class ImgT>
-struct ProI {  // (I~, 0): the centred image alone, for K*I~
-    const ImgT *img;
+template <int R, class ImgT>
+struct SrcI {  // (I~, 0): the centred image alone, for K*I~
+    static constexpr int NP = 1, CTAS = 4, NS = 1;
+    static constexpr bool FIX = false;
+    using G = XYG<R>;
+    using FI = XYField<R, 16 / (int)sizeof(ImgT), ImgVec<ImgT>::V>;
+    static constexpr int IB = FI::W * G::H * (int)sizeof(ImgT), BYTES = round_up(IB, 128);
+    const CUtensorMap *mi;
     float inv_s, nms;
-    using Raw = float;
-    struct Plane { const ImgT *img; };
-    __device__ __forceinline__ Plane plane(long long off) const { return Plane{img + off}; }
-    __device__ __forceinline__ Raw fetch(const Plane &pl, int o) const {
-        return fmaf((float)__ldg(pl.img + o), inv_s, nms);
+    int x0, y0, nx, ny;
+    __device__ __forceinline__ void fence() const { fence_tensormap(mi); }
+    __device__ __forceinline__ void issue(unsigned char *st, int, int, int z, uint64_t *bar, unsigned more) const {
+        mbar_arrive_expect_tx(bar, (unsigned)IB + more);
+        tma_load_3d(st, mi, x0 - FI::RA, y0 - R, z, bar);
     }
-    __device__ __forceinline__ Raw zero() const { return 0.f; }
-    __device__ __forceinline__ void apply(const Raw &r, bool inside, float2 *v) const {
-        v[0] = make_float2(inside ? r : 0.f, 0.f);
-    }
-};
-
-template <class S>
-struct ProAB {  // (a, b) as stored by rsf_ta_z (pitched)
-    const typename Store<S>::V2 *ab;
-    using Raw = typename Store<S>::V2;
-    struct Plane { const typename Store<S>::V2 *ab; };
-    __device__ __forceinline__ Plane plane(long long off) const { return Plane{ab + off}; }
-    __device__ __forceinline__ Raw fetch(const Plane &pl, int o) const { return __ldg(pl.ab + o); }
-    __device__ __forceinline__ Raw zero() const { return Raw{}; }
-    __device__ __forceinline__ void apply(const Raw &r, bool inside, float2 *v) const {
-        v[0] = inside ? Store<S>::unpack2(r) : make_float2(0.f, 0.f);
-    }
-};
-
-// Shared-memory layout of the x/y kernel (float2 units): the input tile of NP
-// pairs and the x-convolved rows of XCP pairs (NP, or 1 when the pairs pass
-// through the x and y convolutions one after the other).
-template <int R, int NP, int XCP = NP>
-struct XYLayout {
-    static constexpr int W = kXYT + 2 * R;              // loaded width
-    static constexpr int H = kXYT + 2 * R;              // loaded rows
-    // row pitch = 2 (mod 16) float2: rows start 16-byte aligned, and the x pass's
-    // 16-byte window reads (an 8-lane phase covers 2 rows x 4 column groups 8 floats
-    // apart, or 4 rows x 2 groups 16 floats apart) hit distinct banks
-    static constexpr int P = tiled_xy_in_pitch(R);
-    static_assert(P == ((W + 15) / 16) * 16 + 2, "input tile pitch");
-    static constexpr int IN = NP * H * P;               // input tile
-    // x-convolved rows, room for a row pitch of up to 34 (XYCfg)
-    static constexpr int XC = XCP * H * (kXYT + 2);
-    static constexpr size_t bytes = sizeof(float2) * (IN + XC);
-};
-
-// Resident CTAs per SM the x/y kernels are compiled for: 3 (4 for rsf_ta_xy at
-// radius <= 6) measured faster than 2 at radii 8-12 in spite of a few spilled words.
-
-// Loads the x/y kernel's input tile of one plane entry by entry (any row
-// pitch): entry e of this thread has its offset within the plane (-1 outside
-// the brick) and its shared-memory index; entries e < NFULL always lie inside
-// the tile.  fetch(z) issues the global loads of plane z into registers,
-// store(in) writes the NP pairs into the tile.
-template <int R, int NP, class Pro>
-struct ScalarLoader {
-    using L = XYLayout<R, NP>;
-    using Raw = typename Pro::Raw;
-    static constexpr int NE = (L::H * L::W + kXYThreads - 1) / kXYThreads;
-    static constexpr int NFULL = L::H * L::W / kXYThreads;
-    static_assert(NE <= 32, "too many tile entries per thread");
-    const Pro &pro;
-    long long iplane;
-    int eoff[NE], esm[NE];
-    Raw raw[NE];
-    __device__ __forceinline__ ScalarLoader(const Pro &p, int nx, int ny, int ipx, int x0, int y0)
-        : pro(p), iplane((long long)ipx * ny) {
+    __device__ __forceinline__ void fix(unsigned char *, int, int, int, int) const {}
+    template <class F>
+    __device__ __forceinline__ void window(const unsigned char *st, int row, int xo, const F &f) const {
+        const ImgT *im = reinterpret_cast<const ImgT *>(st) + row * FI::W + xo + FI::B;
+        const bool in_y = (unsigned)(y0 - R + row) < (unsigned)ny;
+        const int gx = x0 - R + xo;
+        ImgVec<ImgT> iv;
 #pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            const int i = threadIdx.x + e * kXYThreads;
-            const int ii = min(i, L::H * L::W - 1);
-            const int ly = ii / L::W, lx = ii - ly * L::W;
-            const int gx = x0 + lx - R, gy = y0 + ly - R;
-            const bool in_vol = i < L::H * L::W && gx >= 0 && gx < nx && gy >= 0 && gy < ny;
-            eoff[e] = in_vol ? gy * ipx + gx : -1;
-            esm[e] = i < L::H * L::W ? ly * L::P + lx : -1;
+        for (int j = 0; j < G::NI; ++j) {
+            const int ji = j + FI::O;
+            if (j == 0 || ji % ImgVec<ImgT>::V == 0) iv.load(im + ji / ImgVec<ImgT>::V * ImgVec<ImgT>::V);
+            const bool in = in_y && (unsigned)(gx + j) < (unsigned)nx;
+            const float2 p[1] = {make_float2(in ? fmaf(iv.get(ji % ImgVec<ImgT>::V), inv_s, nms) : 0.f, 0.f)};
+            f(j, p);
         }
     }
-    __device__ __forceinline__ void fetch(int z) {
-        const auto pl = pro.plane((long long)z * iplane);
-#pragma unroll
-        for (int e = 0; e < NE; ++e) raw[e] = eoff[e] >= 0 ? pro.fetch(pl, eoff[e]) : pro.zero();
+};
+
+// (a, b) as stored by rsf_ta_z: FP32 pairs, or 16-bit pairs widened as the window is read
+template <int R, class S>
+struct SrcAB {
+    static constexpr int NP = 1, CTAS = 3, NS = 2;
+    static constexpr bool FIX = false;  // the zero fill is the convolution's padding
+    using G = XYG<R>;
+    using V2 = typename Store<S>::V2;
+    static constexpr int E = 16 / (int)sizeof(V2);  // pairs per 16 bytes
+    using FA = XYField<R, E, E>;
+    static constexpr int AB = FA::W * G::H * (int)sizeof(V2), BYTES = round_up(AB, 128);
+    const CUtensorMap *ma;
+    __device__ __forceinline__ void fence() const { fence_tensormap(ma); }
+    __device__ __forceinline__ void issue(unsigned char *st, int x0, int y0, int z, uint64_t *bar, unsigned more) const {
+        mbar_arrive_expect_tx(bar, (unsigned)AB + more);
+        tma_load_3d(st, ma, (x0 - FA::RA) * (int)(sizeof(V2) / 4), y0 - R, z, bar);
     }
-    __device__ __forceinline__ void store(float2 *in) const {
+    __device__ __forceinline__ void fix(unsigned char *, int, int, int, int) const {}
+    template <class F>
+    __device__ __forceinline__ void window(const unsigned char *st, int row, int xo, const F &f) const {
+        const V2 *a = reinterpret_cast<const V2 *>(st) + row * FA::W + xo + FA::B;
+        float2 v[E];
 #pragma unroll
-        for (int e = 0; e < NE; ++e) {
-            if (e < NFULL || esm[e] >= 0) {
-                float2 v[NP];
-                pro.apply(raw[e], eoff[e] >= 0, v);
+        for (int j = 0; j < G::NI; ++j) {
+            const int ja = j + FA::O;
+            if (j == 0 || ja % E == 0) {
+                const uint4 w = *reinterpret_cast<const uint4 *>(a + ja / E * E);
+                const V2 *u = reinterpret_cast<const V2 *>(&w);
 #pragma unroll
-                for (int p = 0; p < NP; ++p) in[p * L::H * L::P + esm[e]] = v[p];
+                for (int e = 0; e < E; ++e) v[e] = Store<S>::unpack2(u[e]);
             }
+            const float2 p[1] = {v[ja % E]};
+            f(j, p);
         }
     }
 };
 
-// The same tile of (H I~, H) loaded four columns at a time: one 16-byte load
-// of q and one load of four image values per group, window columns
-// [x0 - RA, x0 + 32 + RA) with RA = R rounded up to a multiple of 4.  Needs an
-// even R <= 8 (used for R <= 6) and a row pitch (= nx) that is a multiple of 4, so that a group
-// lies wholly inside or wholly outside the brick and its pairs of columns are
-// 16-byte aligned in the tile (two 16-byte shared stores per group).
-template <class T> struct Vec4;
-template <> struct Vec4<uint8_t> { using V = uchar4; };
-template <> struct Vec4<uint16_t> { using V = ushort4; };
-template <> struct Vec4<float> { using V = float4; };
-
-template <int R, class ImgT, int NP = 1>
-struct VecLoaderH {  // NP = 1: (H I~, H); NP = 2: also ((1-H) I~, 1-H) (the Eq. (15) form)
-    using L = XYLayout<R, NP>;
-    static_assert(R % 2 == 0 && R <= 8, "even radius <= 8");
-    static constexpr int RA = (R + 3) / 4 * 4;
-    static constexpr int NG = (32 + 2 * RA) / 4;                       // groups per row
-    static constexpr int NV = (L::H * NG + kXYThreads - 1) / kXYThreads;  // groups per thread
-    using V = typename Vec4<ImgT>::V;
-    const float *q;
-    const ImgT *img;
-    float inv_s, nms;
-    long long iplane;
-    int goff[NV];  // group offset in the plane (-1: outside the brick)
-    int sm0[NV];   // tile index of the group's first column (may lie left of the tile)
-    int lx0[NV];   // tile column of the group's first column; kNone: no group for this thread
-    static constexpr int kNone = -1 << 20;
-    float4 rq[NV];
-    V ri[NV];
-    __device__ __forceinline__ VecLoaderH(const float *q_, const ImgT *img_, float inv_s_, float nms_, int nx, int ny,
-                                          int x0, int y0)
-        : q(q_), img(img_), inv_s(inv_s_), nms(nms_), iplane((long long)nx * ny) {
-#pragma unroll
-        for (int e = 0; e < NV; ++e) {
-            const int i = threadIdx.x + e * kXYThreads;
-            const int ii = min(i, L::H * NG - 1);
-            const int row = ii / NG, g = ii - row * NG;
-            const int gy = y0 + row - R, gx = x0 - RA + 4 * g;
-            const bool in_vol = i < L::H * NG && gx >= 0 && gx < nx && gy >= 0 && gy < ny;
-            goff[e] = in_vol ? gy * nx + gx : -1;
-            sm0[e] = row * L::P + 4 * g - RA + R;
-            lx0[e] = i < L::H * NG ? 4 * g - RA + R : kNone;
-        }
-    }
-    __device__ __forceinline__ void fetch(int z) {
-        const float *qp = q + (long long)z * iplane;
-        const ImgT *ip = img + (long long)z * iplane;
-#pragma unroll
-        for (int e = 0; e < NV; ++e) {
-            if (goff[e] >= 0) {
-                rq[e] = __ldg(reinterpret_cast<const float4 *>(qp + goff[e]));
-                ri[e] = __ldg(reinterpret_cast<const V *>(ip + goff[e]));
-            } else {
-                rq[e] = make_float4(0.f, 0.f, 0.f, 0.f);
-                ri[e] = V{};
-            }
-        }
-    }
-    // two adjacent columns (q, image value) of each input pair into the tile at index c
-    __device__ __forceinline__ void put(float2 *in, int c, float qa, float ia, float qb, float ib, bool inside) const {
-        const float ha = h_of_q(qa), hb = h_of_q(qb);
-        const float xa = fmaf(ia, inv_s, nms), xb = fmaf(ib, inv_s, nms);
-        *reinterpret_cast<float4 *>(in + c) =
-            inside ? make_float4(ha * xa, ha, hb * xb, hb) : make_float4(0.f, 0.f, 0.f, 0.f);
-        if constexpr (NP == 2) {
-            const float ca = hc_of_q(qa), cb = hc_of_q(qb);
-            *reinterpret_cast<float4 *>(in + L::H * L::P + c) =
-                inside ? make_float4(ca * xa, ca, cb * xb, cb) : make_float4(0.f, 0.f, 0.f, 0.f);
-        }
-    }
-    __device__ __forceinline__ void store(float2 *in) const {
-#pragma unroll
-        for (int e = 0; e < NV; ++e) {
-            const int c0 = sm0[e], lx = lx0[e];
-            const bool inside = goff[e] >= 0;
-            if (lx >= 0 && lx + 1 < L::W) put(in, c0, rq[e].x, (float)ri[e].x, rq[e].y, (float)ri[e].y, inside);
-            if (lx != kNone && lx + 2 >= 0 && lx + 3 < L::W)
-                put(in, c0 + 2, rq[e].z, (float)ri[e].z, rq[e].w, (float)ri[e].w, inside);
-        }
-    }
-};
-
-// The x/y kernel body for one CTA of one brick: planes [za, za + np) of
-// tile (x0, y0).  The global loads of plane z+1 are issued right after the
-// first barrier of plane z and land in registers while the convolutions run.
-// `Out` writes the NP pairs (pitch out.px).
-// Two pairs pass through the x and y convolutions one after the other (one
-// pair of x-convolved rows in shared memory) where that lets three CTAs share
-// an SM: radius >= 10.
-template <int R, int NP>
-constexpr bool xy_seq() { return NP == 2 && R >= 10; }
-template <int R, int NP>
-constexpr size_t xy_smem() { return XYLayout<R, NP, xy_seq<R, NP>() ? 1 : NP>::bytes; }
-
-// x phase of the x/y kernel: XT outputs per thread and the row pitch XS of the
-// x-convolved rows.  XT = 8: items of 8 rows x 32 columns, each 8-lane phase of
-// a 16-byte window read covering 4 rows x 2 column groups, stores of two outputs
-// (16 bytes) at pitch 34, so that both fall on distinct banks (37 % fewer
-// shared-load wavefronts than XT = 4 at radius 6).  XT = 4 in the single-pair
-// (H I~, H) kernel, whose loader keeps more registers live (XT = 8 measured no
-// faster there): items of 8 rows x 16 columns, 64-bit stores at pitch 33 (rows
-// r..r+3 of a half-warp, four columns apart, on 32 distinct banks; a pitch of 32
-// puts 8 rows on one bank set), pitch 32 at radius >= 10 (measured 8 % faster:
-// its schedule under the 80-register cap differs).
-template <int R, int NP, bool HLOAD>
-struct XYCfg {
-    static constexpr bool H1 = HLOAD && NP == 1;
-    static constexpr int XT = H1 ? 4 : 8;
-    static constexpr int XS = XT == 8 ? kXYT + 2 : (R >= 10 ? kXYT : kXYT + 1);
-};
-
-// x then y convolution of plane z of the input tile `in` (NP pairs, row pitch
-// L::P) through the x-convolved rows `xc`, written by `out`; ends with a barrier
-// (both tiles are free again).
-template <int R, int NP, class Cfg, class Out>
-__device__ __forceinline__ void xy_plane(const float2 *in, float2 *xc, const Out &out, int z, int nx, int ny,
-                                         int x0, int y0, const TapPairs &t) {
-    constexpr bool SEQ = xy_seq<R, NP>();
-    constexpr int NPX = SEQ ? 1 : NP;        // pairs per x/y round
-    using L = XYLayout<R, NP, NPX>;
-    constexpr int T = 2 * R + 1;
-    constexpr int XT = Cfg::XT, XS = Cfg::XS, YT = 4;  // outputs per thread in the x and y phases; pitch
-    static_assert((XT == 4 && XS <= kXYT + 1) || (XT == 8 && XS == kXYT + 2), "x phase layout");
-    constexpr int NRB = (L::H + 7) / 8;      // 8-row blocks of the x phase
-    constexpr int NCB = kXYT / (4 * XT);     // column blocks of an item row
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-    for (int ps = 0; ps < NP / NPX; ++ps) {  // rounds of NPX pairs (one round unless SEQ)
-    {
-        const int h = lane >> 4;
-        const int r = XT == 8 ? (lane >> 1) & 3 : (lane >> 2) & 3;
-        const int g = XT == 8 ? (lane & 1) | ((lane >> 2) & 2) : lane & 3;
-        // items (8 rows x 4 XT columns of one pair) dealt to the warps round-robin; at radius
-        // <= 6 and for two pairs a warp's items warp + 8 i run in a compile-time number of
-        // rounds (measured faster there; slower at radius 8 with one pair)
-        constexpr int NITEMS = NPX * NRB * NCB, NW8 = kXYThreads / 32;
-        constexpr bool STATIC = R <= 6 || NP == 2;
-        constexpr int NROUNDS = STATIC ? (NITEMS + NW8 - 1) / NW8 : 1;
-#pragma unroll
-        for (int i = 0; i < NROUNDS; ++i)
-        for (int item = warp + NW8 * i; item < NITEMS; item += STATIC ? NITEMS : NW8) {
-            const int pl = item / (NRB * NCB);  // pair within the round
-            const int p = SEQ ? ps : pl;         // pair of the input tile
-            const int rem = item - pl * NRB * NCB;
-            const int row = (rem / NCB) * 8 + h * 4 + r;
-            const int xo = (rem % NCB) * 16 + g * XT;
-            if (row < L::H) {
-                const float4 *src = reinterpret_cast<const float4 *>(in + (p * L::H + row) * L::P + xo);
-                // streamed: each loaded pair feeds the outputs it contributes to
-                // (output o takes taps k = 0..T-1 in order, as a window would)
-                float2 acc[XT];
-#pragma unroll
-                for (int o = 0; o < XT; ++o) acc[o] = make_float2(0.f, 0.f);
-#pragma unroll
-                for (int j2 = 0; j2 < (XT + 2 * R) / 2; ++j2) {
-                    const float4 q = src[j2];
-#pragma unroll
-                    for (int h2 = 0; h2 < 2; ++h2) {
-                        const int j = 2 * j2 + h2;
-                        const float2 v = h2 ? make_float2(q.z, q.w) : make_float2(q.x, q.y);
-#pragma unroll
-                        for (int o = 0; o < XT; ++o)
-                            if (j - o >= 0 && j - o < T) acc[o] = f2fma(t.g[j - o], v, acc[o]);
-                    }
-                }
-                float2 *dst = xc + (pl * L::H + row) * XS + xo;
-                if constexpr (XT == 8) {
-#pragma unroll
-                    for (int o = 0; o < XT; o += 2)
-                        *reinterpret_cast<float4 *>(dst + o) =
-                            make_float4(acc[o].x, acc[o].y, acc[o + 1].x, acc[o + 1].y);
-                } else {
-#pragma unroll
-                    for (int o = 0; o < XT; ++o) dst[o] = acc[o];
-                }
-            }
-        }
-    }
-    __syncthreads();
-    {
-        const int gx = x0 + lane;
-        float2 res[NPX][YT];
-#pragma unroll
-        for (int p = 0; p < NPX; ++p) {
-#pragma unroll
-            for (int o = 0; o < YT; ++o) res[p][o] = make_float2(0.f, 0.f);
-#pragma unroll
-            for (int j = 0; j < YT + 2 * R; ++j) {
-                const float2 v = xc[(p * L::H + warp * YT + j) * XS + lane];
-#pragma unroll
-                for (int o = 0; o < YT; ++o)
-                    if (j - o >= 0 && j - o < T) res[p][o] = f2fma(t.g[j - o], v, res[p][o]);
-            }
-        }
-        if (gx < nx) {
-            const int gy0 = y0 + warp * YT;
-            const auto op = out.plane(z);
-#pragma unroll
-            for (int o = 0; o < YT; ++o) {
-                if (gy0 + o < ny) {
-                    if constexpr (SEQ)
-                        out.half(op, (gy0 + o) * out.px + gx, ps, res[0][o]);
-                    else
-                        out(op, (gy0 + o) * out.px + gx, res[0][o], res[NPX - 1][o]);
-                }
-            }
-        }
-    }
-    __syncthreads();  // the next round or plane reuses the tiles
-    }
-}
-
-template <int R, int NP, class Cfg, class Loader, class Out>
-__device__ __forceinline__ void xy_tile(Loader &ld, const Out &out, int nx, int ny, int nz, int x0, int y0, int za,
-                                        int np, const TapPairs &t, float2 *sm) {
-    using L = XYLayout<R, NP, xy_seq<R, NP>() ? 1 : NP>;
-    float2 *in = sm;
-    float2 *xc = sm + L::IN;
-    const int zb_end = min(za + np, nz);
-    ld.fetch(za);
-    for (int z = za; z < zb_end; ++z) {
-        ld.store(in);
-        __syncthreads();
-        if (z + 1 < zb_end) ld.fetch(z + 1);
-        xy_plane<R, NP, Cfg>(in, xc, out, z, nx, ny, x0, y0, t);
-    }
-}
-
-// Writers of the x/y kernel's outputs: plane(z) gives plane z, operator()
-// stores at offset y * px + x within it.
-struct OutF2 {  // one x/y-convolved pair, FP32, pitched
+// Where the x/y-convolved pairs go: pitched, FP32, NP pairs interleaved per voxel.
+struct OutXY {
     float2 *u;
     int px;
     long long pplane;
-    __device__ __forceinline__ float2 *plane(int z) const { return u + (long long)z * pplane; }
-    __device__ __forceinline__ void operator()(float2 *pl, int o, float2 a, float2) const { pl[o] = a; }
 };
 
-struct OutF4 {  // two x/y-convolved pairs interleaved per voxel (16 bytes), FP32, pitched
-    float4 *u;
-    int px;
-    long long pplane;
-    __device__ __forceinline__ float4 *plane(int z) const { return u + (long long)z * pplane; }
-    __device__ __forceinline__ void operator()(float4 *pl, int o, float2 a, float2 b) const {
-        pl[o] = make_float4(a.x, a.y, b.x, b.y);
-    }
-    // pair p alone (the pairs convolved one after the other): its half of the voxel's 16 bytes
-    __device__ __forceinline__ void half(float4 *pl, int o, int p, float2 v) const {
-        reinterpret_cast<float2 *>(pl + o)[p] = v;
-    }
+// Shared memory: NS staging buffers, the x-convolved rows, an mbarrier per buffer.  Row pitch
+// of the x-convolved rows: 34 float2 (17 units of 16 bytes) or 33 float4.
+template <int R, class Src>
+struct XYSmem {
+    static constexpr int XS = Src::NP == 1 ? 34 : 33;
+    static constexpr int XC = Src::NP * (int)sizeof(float2) * XYG<R>::H * XS;
+    static constexpr int NS = Src::NS;
+    static constexpr size_t bytes = NS * Src::BYTES + XC + NS * sizeof(uint64_t);
 };
 
-// CTA -> (brick, tile) for the x/y kernels: tiles (tx, ty, tz) of 32 x 32 x xy_planes(B).
-struct XYTile {
-    int b, x0, y0, za;
-};
-__device__ __forceinline__ XYTile xy_tile_of(const GroupArgs &G, const BrickDev &B, int b) {
-    const int local = blockIdx.x - __ldg(G.starts + b);
-    const int ntx = (B.nx + kXYT - 1) / kXYT, nty = (B.ny + kXYT - 1) / kXYT;
-    const int tx = local % ntx, r = local / ntx;
-    return XYTile{b, tx * kXYT, (r % nty) * kXYT, (r / nty) * xy_planes(B)};
-}
-
-// NP = 1: (H I~, H) into B.u2 (Li's form); NP = 2: both sides of Eq. (10),
-// ((H I~, H), ((1-H) I~, 1-H)) interleaved per voxel into B.u2 read as float4
-// (the Eq. (15) form, which convolves the complement directly).
-template <int R, class ImgT, int NP = 1>
-__global__ void __launch_bounds__(kXYThreads, NP == 1 ? (R <= 6 ? 4 : 3) : (R <= 8 || xy_seq<R, NP>() ? 3 : 2))
-    k_ta_xy(GroupArgs G, TapPairs t) {
-    extern __shared__ float2 sm[];
-    const int b = find_brick(G.starts, G.nb, blockIdx.x);
-    const BrickDev B = G.bricks[b];
-    const XYTile tl = xy_tile_of(G, B, b);
-    const float inv_s = B.cs[1], nms = -B.cs[0] * B.cs[1];
-    const float *q = (G.parity ^ B.flip) ? B.q[1] : B.q[0];
-    const ImgT *img = reinterpret_cast<const ImgT *>(B.img);
-    using Out = typename std::conditional<NP == 1, OutF2, OutF4>::type;
-    using OutV = typename std::conditional<NP == 1, float2, float4>::type;
-    const Out out{reinterpret_cast<OutV *>(B.u2), B.px, (long long)B.px * B.ny};
-    if constexpr (R % 2 == 0 && R <= 6) {
-        // four columns per load where the row pitch and both base addresses allow it (uniform per CTA);
-        // at radius 8 the second code path cost more registers than the loads saved (measured)
-        if (B.nx % 4 == 0 && reinterpret_cast<uintptr_t>(q) % 16 == 0 &&
-            reinterpret_cast<uintptr_t>(img) % (4 * sizeof(ImgT)) == 0) {
-            VecLoaderH<R, ImgT, NP> ld(q, img, inv_s, nms, B.nx, B.ny, tl.x0, tl.y0);
-            xy_tile<R, NP, XYCfg<R, NP, true>>(ld, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, xy_planes(B), t, sm);
-            return;
-        }
-    }
-    using Pro = typename std::conditional<NP == 1, ProH<ImgT>, ProH2<ImgT>>::type;
-    Pro pro{};
-    pro.q = q;
-    pro.img = img;
-    pro.inv_s = inv_s;
-    pro.nms = nms;
-    ScalarLoader<R, NP, Pro> ld(pro, B.nx, B.ny, B.nx, tl.x0, tl.y0);
-    xy_tile<R, NP, XYCfg<R, NP, true>>(ld, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, xy_planes(B), t, sm);
-}
-
-// Group A's x/y kernel of Li's form with its inputs copied by TMA (even radius;
-// used for a brick group whose bricks all have q and image rows of a multiple of
-// 16 bytes and aligned bases): per plane one box of q and one of the image land
-// in a staging buffer, each starting at the 16-byte aligned column at or left of
-// x0 - R; a transform pass writes (H I~, H) of the tile from it, two columns per
-// step, zero outside the brick (the copies' zero fill would give H = 1 there),
-// with the arithmetic of the register loaders; the next plane's boxes are then in
-// flight while the tile is convolved.
-template <int R, class ImgT>
-struct XYStageH {
-    static_assert(R % 2 == 0, "even radius: the staged columns' offsets are even");
-    static constexpr int H = kXYT + 2 * R, W = kXYT + 2 * R;
-    static constexpr int RQ = (R + 3) / 4 * 4;                              // q: 4 floats per 16 bytes
-    static constexpr int AI = 16 / (int)sizeof(ImgT);                       // image values per 16 bytes
-    static constexpr int RI = (R + AI - 1) / AI * AI;
-    static constexpr int WQ = kXYT + 2 * RQ, WI = kXYT + 2 * RI;            // box widths (elements)
-    static constexpr int QB = WQ * H * 4, IB = WI * H * (int)sizeof(ImgT);  // box bytes
-    static constexpr int IOFF = (QB + 127) / 128 * 128;                     // image box offset (bytes)
-    static constexpr int BYTES = IOFF + (IB + 127) / 128 * 128;             // staging bytes
-    using L = XYLayout<R, 1>;
-    static constexpr size_t smem = BYTES + sizeof(float2) * (L::IN + L::XC) + sizeof(uint64_t);
-};
-template <class T> struct Pair2;
-template <> struct Pair2<uint8_t> { using V = uchar2; };
-template <> struct Pair2<uint16_t> { using V = ushort2; };
-template <> struct Pair2<float> { using V = float2; };
-
-template <int R, class ImgT>
-__global__ void __launch_bounds__(kXYThreads, R <= 6 ? 4 : 3) k_ta_xy_tma(GroupArgs G, TapPairs t) {
-    using S = XYStageH<R, ImgT>;
-    using L = XYLayout<R, 1>;
-    extern __shared__ __align__(128) unsigned char xsm[];
-    const float *sq = reinterpret_cast<const float *>(xsm);
-    const ImgT *simg = reinterpret_cast<const ImgT *>(xsm + S::IOFF);
-    float2 *tile = reinterpret_cast<float2 *>(xsm + S::BYTES);
-    float2 *xc = tile + L::IN;
-    uint64_t *bar = reinterpret_cast<uint64_t *>(xc + L::XC);
-    const int b = find_brick(G.starts, G.nb, blockIdx.x);
-    const BrickDev &B = G.bricks[b];
-    const XYTile tl = xy_tile_of(G, B, b);
-    const int nx = B.nx, ny = B.ny, nz = B.nz, x0 = tl.x0, y0 = tl.y0, za = tl.za;
-    const float inv_s = B.cs[1], nms = -B.cs[0] * B.cs[1];
-    const CUtensorMap *mq = (G.parity ^ B.flip) ? &B.tm_q[1] : &B.tm_q[0];
-    const CUtensorMap *mi = &B.tm_img;
-    const OutF2 out{B.u2, B.px, (long long)B.px * ny};
-    const int zb_end = min(za + xy_planes(B), nz);
-    if (smem_addr(xsm) % 128u != 0u) {
-        report_error(G.err, kErrSmemAlign);
-        return;
-    }
-    if (threadIdx.x == 0) {
-        mbar_init(bar, 1);
-        mbar_init_fence();
-    }
-    __syncthreads();
-    const auto issue = [&](int z) {
-        mbar_arrive_expect_tx(bar, (unsigned)(S::QB + S::IB) + G.fault_tx);
-        tma_load_3d(xsm, mq, x0 - S::RQ, y0 - R, z, bar);
-        tma_load_3d(xsm + S::IOFF, mi, x0 - S::RI, y0 - R, z, bar);
-    };
-    bool pending = false;
-    if (za < zb_end) {
-        if (threadIdx.x == 0) {
-            fence_tensormap(mq);
-            fence_tensormap(mi);
-            issue(za);
-        }
-        pending = true;
-    }
-    unsigned phase = 0u;
-    bool ok = true;
-    for (int z = za; z < zb_end; ++z) {
-        if (!mbar_wait(bar, phase)) {
-            ok = false;
-            break;
-        }
-        phase ^= 1u;
-        pending = false;
-        constexpr int NPAIRS = S::H * S::W / 2, W2 = S::W / 2;
-#pragma unroll
-        for (int k = 0; k < (NPAIRS + kXYThreads - 1) / kXYThreads; ++k) {
-            const int i = threadIdx.x + k * kXYThreads;
-            if (i < NPAIRS) {
-                const int row = i / W2, col = 2 * (i - row * W2);
-                const float2 qv = *reinterpret_cast<const float2 *>(sq + row * S::WQ + col + (S::RQ - R));
-                const typename Pair2<ImgT>::V iv =
-                    *reinterpret_cast<const typename Pair2<ImgT>::V *>(simg + row * S::WI + col + (S::RI - R));
-                const int gx = x0 - R + col, gy = y0 - R + row;
-                const bool iny = (unsigned)gy < (unsigned)ny;
-                const bool in0 = iny && (unsigned)gx < (unsigned)nx, in1 = iny && (unsigned)(gx + 1) < (unsigned)nx;
-                const float h0 = h_of_q(qv.x), h1 = h_of_q(qv.y);
-                const float v0 = fmaf((float)iv.x, inv_s, nms), v1 = fmaf((float)iv.y, inv_s, nms);
-                *reinterpret_cast<float4 *>(tile + row * L::P + col) =
-                    make_float4(in0 ? h0 * v0 : 0.f, in0 ? h0 : 0.f, in1 ? h1 * v1 : 0.f, in1 ? h1 : 0.f);
-            }
-        }
-        __syncthreads();  // the staging buffer is consumed, the tile complete
-        if (z + 1 < zb_end) {
-            if (threadIdx.x == 0) {
-                fence_proxy_async_smem();
-                issue(z + 1);
-            }
-            pending = true;
-        }
-        xy_plane<R, 1, XYCfg<R, 1, true>>(tile, xc, out, z, nx, ny, x0, y0, t);
-    }
-    if (!ok) {
-        report_error(G.err, kErrWaitExpired);
-        if (pending) mbar_wait_until(bar, phase, globaltimer_ns() + kWaitNs);
-        return;
-    }
-    if (threadIdx.x == 0) mbar_inval(bar);
-}
-
-// Group B's x/y kernel takes its FP32 (a, b) tile from TMA at even radius: the box's
-// x origin, 2 (x0 - R) floats, is then 16-byte aligned.
-constexpr bool tbxy_tma(int R) { return R % 2 == 0; }
-
-// The single-pair x/y kernel body with the input tile copied by TMA: one box per
-// plane, H rows x P pairs of an FP32 pair field from (x0 - R, y0 - R) -- zeros
-// outside the brick, exactly the convolutions' padding, and the tile's own row
-// pitch, so the x phase reads it as it is.  Two tile stages: plane z + 1 is in
-// flight while plane z is convolved.  Shared memory: the stages (each rounded up
-// to 128 bytes), the x-convolved rows, two mbarriers.  Waits are bounded as in
-// the z pass (expiry reported in the group's error word).
-template <int R>
-struct XYTma {
-    using L = XYLayout<R, 1>;
-    static constexpr int STAGE = (L::IN + 15) / 16 * 16;  // float2 units, a multiple of 128 bytes
-    static constexpr size_t bytes = sizeof(float2) * (2 * STAGE + L::XC) + 2 * sizeof(uint64_t);
-};
-
-template <int R, class Cfg, class Out>
-__device__ __forceinline__ void xy_tile_tma(const GroupArgs &G, const CUtensorMap *map, const Out &out, int nx, int ny,
-                                            int nz, int x0, int y0, int za, int np, const TapPairs &t, float2 *sm) {
-    using L = XYLayout<R, 1>;
-    constexpr int STAGE = XYTma<R>::STAGE;
-    constexpr unsigned BOX = sizeof(float2) * L::IN;  // bytes of one plane's box
-    float2 *xc = sm + 2 * STAGE;
-    uint64_t *bars = reinterpret_cast<uint64_t *>(xc + L::XC);
+// Planes [za, za + np) of tile (x0, y0).  Waits are bounded (expiry reported in the group's
+// error word).
+template <int R, class Src>
+__device__ __forceinline__ void xy_tile(const GroupArgs &G, const Src &src, const OutXY &out, int nx, int ny, int nz,
+                                        int x0, int y0, int za, int np, const TapPairs &t, unsigned char *sm) {
+    using X = XYG<R>;
+    constexpr int NP = Src::NP, T = X::T, YT = X::YT;
+    constexpr int XS = XYSmem<R, Src>::XS, NS = XYSmem<R, Src>::NS;
+    float2 *xc = reinterpret_cast<float2 *>(sm + NS * Src::BYTES);
+    uint64_t *bar = reinterpret_cast<uint64_t *>(sm + NS * Src::BYTES + XYSmem<R, Src>::XC);
     if (smem_addr(sm) % 128u != 0u) {
         report_error(G.err, kErrSmemAlign);
         return;
     }
     const int zb_end = min(za + np, nz);
+    if (za >= zb_end) return;
     if (threadIdx.x == 0) {
-        mbar_init(bars, 1);
-        mbar_init(bars + 1, 1);
+        for (int i = 0; i < NS; ++i) mbar_init(bar + i, 1);
         mbar_init_fence();
     }
     __syncthreads();
-    const auto issue = [&](int z, int st) {
-        mbar_arrive_expect_tx(bars + st, BOX + G.fault_tx);
-        tma_load_3d(sm + st * STAGE, map, 2 * (x0 - R), y0 - R, z, bars + st);
-    };
-    unsigned phase = 0u, pending = 0u;  // bit s: parity of stage s's next phase; stage s awaits its copy
-    if (za < zb_end) {
-        if (threadIdx.x == 0) {
-            fence_tensormap(map);
-            issue(za, 0);
-        }
-        pending = 1u;
-    }
-    bool ok = true;
-    for (int z = za; z < zb_end; ++z) {
-        const int st = (z - za) & 1;
-        if (z + 1 < zb_end) {  // the other stage was last read by plane z - 1's x phase, before a barrier
-            if (threadIdx.x == 0) {
-                fence_proxy_async_smem();
-                issue(z + 1, st ^ 1);
-            }
-            pending |= 1u << (st ^ 1);
-        }
-        if (!mbar_wait(bars + st, (phase >> st) & 1u)) {
-            ok = false;
-            break;
-        }
-        phase ^= 1u << st;
-        pending &= ~(1u << st);
-        xy_plane<R, 1, Cfg>(sm + st * STAGE, xc, out, z, nx, ny, x0, y0, t);
-    }
-    if (!ok) {
-        report_error(G.err, kErrWaitExpired);
-        const unsigned long long deadline = globaltimer_ns() + kWaitNs;
-        for (int b = 0; b < 2; ++b)
-            if ((pending >> b) & 1u) mbar_wait_until(bars + b, (phase >> b) & 1u, deadline);
-        return;
-    }
     if (threadIdx.x == 0) {
-        mbar_inval(bars);
-        mbar_inval(bars + 1);
+        src.fence();
+        for (int i = 0; i < NS && za + i < zb_end; ++i) src.issue(sm + i * Src::BYTES, x0, y0, za + i, bar + i, G.fault_tx);
     }
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int row = warp * 8 + (lane & 7), xo = (lane >> 3) * 8;  // x phase: eight outputs of one row
+    const int rows = min(X::TH, ny - y0);                        // output rows inside the brick
+    const bool xrow = row < rows + 2 * R;
+    const bool fix = Src::FIX && (x0 < R || y0 < R || x0 + 32 + R > nx || y0 + X::TH + R > ny);
+    const int yr = warp * YT;                                    // y phase: YT rows of one column
+    const bool yrow = yr < rows, col = x0 + lane < nx;
+    float2 *o = out.u + ((long long)za * out.pplane + (long long)(y0 + yr) * out.px + x0 + lane) * NP;
+    for (int z = za; z < zb_end; ++z) {
+        const int i = (z - za) % NS;
+        const unsigned phase = (unsigned)((z - za) / NS) & 1u;
+        unsigned char *const st = sm + i * Src::BYTES;
+        if (!mbar_wait(bar + i, phase)) {  // then the same time again for the copies to land
+            report_error(G.err, kErrWaitExpired);
+            const unsigned long long deadline = globaltimer_ns() + kWaitNs;
+            mbar_wait_until(bar + i, phase, deadline);
+            if (NS == 2 && z + 1 < zb_end) mbar_wait_until(bar + (i ^ 1), (unsigned)((z + 1 - za) / NS) & 1u, deadline);
+            return;
+        }
+        if (fix) {
+            src.fix(st, x0, y0, nx, ny);
+            __syncthreads();
+        }
+        if (xrow) {
+            float2 acc[NP][8];
+#pragma unroll
+            for (int p = 0; p < NP; ++p)
+#pragma unroll
+                for (int i = 0; i < 8; ++i) acc[p][i] = make_float2(0.f, 0.f);
+            // each input feeds the outputs it contributes to: output i takes taps 0 .. T-1 in order
+            src.window(st, row, xo, [&](int j, const float2 *v) {
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    if (j - i >= 0 && j - i < T)
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) acc[p][i] = f2fma(t.g[j - i], v[p], acc[p][i]);
+            });
+            if constexpr (NP == 1) {
+                float4 *dst = reinterpret_cast<float4 *>(xc + row * XS + xo);
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    dst[i] = make_float4(acc[0][2 * i].x, acc[0][2 * i].y, acc[0][2 * i + 1].x, acc[0][2 * i + 1].y);
+            } else {
+                float4 *dst = reinterpret_cast<float4 *>(xc) + row * XS + xo;
+#pragma unroll
+                for (int i = 0; i < 8; ++i)
+                    dst[i] = make_float4(acc[0][i].x, acc[0][i].y, acc[NP - 1][i].x, acc[NP - 1][i].y);
+            }
+        }
+        __syncthreads();  // the staging buffer is read, the rows complete
+        if (threadIdx.x == 0 && z + NS < zb_end) {
+            fence_proxy_async_smem();
+            src.issue(st, x0, y0, z + NS, bar + i, G.fault_tx);
+        }
+        if (yrow) {
+            float2 res[YT][NP];
+#pragma unroll
+            for (int i = 0; i < YT; ++i)
+#pragma unroll
+                for (int p = 0; p < NP; ++p) res[i][p] = make_float2(0.f, 0.f);
+#pragma unroll
+            for (int j = 0; j < YT + 2 * R; ++j) {
+                float2 v[NP];
+                if constexpr (NP == 1) {
+                    v[0] = xc[(yr + j) * XS + lane];
+                } else {
+                    const float4 w = reinterpret_cast<const float4 *>(xc)[(yr + j) * XS + lane];
+                    v[0] = make_float2(w.x, w.y);
+                    v[NP - 1] = make_float2(w.z, w.w);
+                }
+#pragma unroll
+                for (int i = 0; i < YT; ++i)
+                    if (j - i >= 0 && j - i < T)
+#pragma unroll
+                        for (int p = 0; p < NP; ++p) res[i][p] = f2fma(t.g[j - i], v[p], res[i][p]);
+            }
+            if (col) {
+#pragma unroll
+                for (int i = 0; i < YT; ++i) {
+                    if (yr + i < rows) {
+                        float2 *d = o + (long long)(i * out.px) * NP;
+                        if constexpr (NP == 1)
+                            *d = res[i][0];
+                        else
+                            *reinterpret_cast<float4 *>(d) =
+                                make_float4(res[i][0].x, res[i][0].y, res[i][NP - 1].x, res[i][NP - 1].y);
+                    }
+                }
+            }
+        }
+        o += out.pplane * NP;
+        __syncthreads();  // the next plane's x phase rewrites the rows
+    }
+    if (threadIdx.x == 0)
+        for (int i = 0; i < NS; ++i) mbar_inval(bar + i);
 }
 
-// Dynamic shared memory of group B's x/y kernel for storage S.
-template <int R, class S>
-constexpr size_t tbxy_smem() {
-    return std::is_same<S, float>::value && tbxy_tma(R) ? XYTma<R>::bytes : XYLayout<R, 1>::bytes;
+// CTA -> (brick, tile) for the x/y kernels: tiles (tx, ty, tz) of 32 x TH x B.xyp.
+struct XYTile {
+    int x0, y0, za;
+};
+template <int R>
+__device__ __forceinline__ XYTile xy_tile_of(int local, const BrickDev &B) {
+    const int ntx = (B.nx + kXYT - 1) / kXYT, nty = (B.ny + XYG<R>::TH - 1) / XYG<R>::TH;
+    const int tx = local % ntx, r = local / ntx;
+    return XYTile{tx * kXYT, (r % nty) * XYG<R>::TH, (r / nty) * B.xyp};
 }
 
-template <int R, class S>
-__global__ void __launch_bounds__(kXYThreads, 3) k_tb_xy(GroupArgs G, TapPairs t) {
-    extern __shared__ __align__(128) float2 sm[];
+// Group A's x/y kernel: (H I~, H) into B.u2 (Li's form, NP = 1), or both sides of Eq. (10),
+// ((H I~, H), ((1-H) I~, 1-H)) interleaved per voxel (the Eq. (15) form, NP = 2).
+template <int R, class ImgT, int NP>
+__global__ void __launch_bounds__(kXYThreads, (SrcH<R, ImgT, NP>::CTAS)) k_ta_xy(GroupArgs G, TapPairs t) {
+    extern __shared__ __align__(128) unsigned char xsm[];
     const int b = find_brick(G.starts, G.nb, blockIdx.x);
-    const BrickDev B = G.bricks[b];
-    const XYTile tl = xy_tile_of(G, B, b);
-    OutF2 out{B.abxy, B.px, (long long)B.px * B.ny};
-    if constexpr (std::is_same<S, float>::value && tbxy_tma(R)) {
-        xy_tile_tma<R, XYCfg<R, 1, false>>(G, &G.bricks[b].tm_ab, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za,
-                                           xy_planes(B), t, sm);
-    } else {
-        ProAB<S> pro{reinterpret_cast<const typename Store<S>::V2 *>(B.ab)};
-        ScalarLoader<R, 1, ProAB<S>> ld(pro, B.nx, B.ny, B.px, tl.x0, tl.y0);
-        xy_tile<R, 1, XYCfg<R, 1, false>>(ld, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, xy_planes(B), t, sm);
-    }
+    const BrickDev &B = G.bricks[b];
+    const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
+    const SrcH<R, ImgT, NP> src{&B.tm_q, &B.tm_img, B.cs[1], -B.cs[0] * B.cs[1]};
+    const OutXY out{B.u2, B.px, (long long)B.px * B.ny};
+    xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
+}
+
+// Group B's x/y kernel: (a, b) into B.abxy.
+template <int R, class S>
+__global__ void __launch_bounds__(kXYThreads, (SrcAB<R, S>::CTAS)) k_tb_xy(GroupArgs G, TapPairs t) {
+    extern __shared__ __align__(128) unsigned char xsm[];
+    const int b = find_brick(G.starts, G.nb, blockIdx.x);
+    const BrickDev &B = G.bricks[b];
+    const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
+    const SrcAB<R, S> src{&B.tm_ab};
+    const OutXY out{B.abxy, B.px, (long long)B.px * B.ny};
+    xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
 }
 
 // ------------------------------------------------------------------ A: z
@@ -1156,14 +878,14 @@ __global__ void __launch_bounds__(kAZThreads, 2) k_ta_z4(GroupArgs G, TapPairs t
 // then a z convolution of its first component into b.ki.  Launched per brick
 // (the descriptor by value), on the x/y kernel's tiles and the slabs of group A.
 template <int R, class ImgT>
-__global__ void __launch_bounds__(kXYThreads) k_ki_xy(BrickDev B, TapPairs t) {
-    extern __shared__ float2 sm[];
-    const int ntx = (B.nx + kXYT - 1) / kXYT, nty = (B.ny + kXYT - 1) / kXYT;
-    const int tx = blockIdx.x % ntx, r = blockIdx.x / ntx;
-    ProI<ImgT> pro{reinterpret_cast<const ImgT *>(B.img), B.cs[1], -B.cs[0] * B.cs[1]};
-    OutF2 out{B.abxy, B.px, (long long)B.px * B.ny};
-    ScalarLoader<R, 1, ProI<ImgT>> ld(pro, B.nx, B.ny, B.nx, tx * kXYT, (r % nty) * kXYT);
-    xy_tile<R, 1, XYCfg<R, 1, false>>(ld, out, B.nx, B.ny, B.nz, tx * kXYT, (r % nty) * kXYT, (r / nty) * xy_planes(B), xy_planes(B), t, sm);
+__global__ void __launch_bounds__(kXYThreads, 4) k_ki_xy(const __grid_constant__ BrickDev B, int *err, TapPairs t) {
+    extern __shared__ __align__(128) unsigned char xsm[];
+    const XYTile tl = xy_tile_of<R>(blockIdx.x, B);
+    const SrcI<R, ImgT> src{&B.tm_img, B.cs[1], -B.cs[0] * B.cs[1], tl.x0, tl.y0, B.nx, B.ny};
+    const OutXY out{B.abxy, B.px, (long long)B.px * B.ny};
+    GroupArgs G{};
+    G.err = err;
+    xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
 }
 
 template <int R>
@@ -1509,7 +1231,8 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
     const long long n = (long long)plane * nz;
     const ImgT *const img = reinterpret_cast<const ImgT *>(B.img);
     float *const phi_out = par ? B.phi[0] : B.phi[1];
-    float *const q_out = par ? B.q[0] : B.q[1];
+    float *const q_out = B.q;
+    const unsigned qplane = (unsigned)B.qp * (unsigned)ny;  // q rows have a pitch of their own
     const unsigned out0 = (unsigned)z0 * plane + (unsigned)min(y, ny - 1) * (unsigned)nx + (unsigned)min(x, nx - 1);
     // the image of output plane r at this thread's columns (not read past the chunk)
     const auto img_at = [&](auto in, int r, unsigned off) -> Img2 {
@@ -1554,7 +1277,8 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
     float2 acc[4][2];         // (K*a, K*b) of four planes and both columns,
     Img2 raw[4];              // their image values
     float pzq[4];             // and p_z
-    unsigned out = out0;      // offset of the step's first output plane at this thread's columns
+    unsigned out = out0;      // offset of the step's first output plane at this thread's columns,
+    unsigned qout = (unsigned)z0 * qplane + (unsigned)min(y, ny - 1) * (unsigned)B.qp + (unsigned)min(x, nx - 1);  // and in q
 
     // taps k = -R .. R in order, as each plane of the ring is read once
     const auto convolve = [&](auto dc) {
@@ -1675,7 +1399,9 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
                 const float2 lap[2] = {f2add(lxy0, f2add(f2add(ph1, phm), f2mul(f2v(-2.f), ph0))),
                                        f2add(lxy1, f2add(f2add(ph2, ph0), f2mul(f2v(-2.f), ph1)))};
                 const unsigned o0 = out, o1 = out + plane;
+                const unsigned q0 = qout, q1 = qout + qplane;
                 out = o1 + plane;
+                qout = q1 + qplane;
 #pragma unroll
                 for (int s = 0; s < 2; ++s) {
                     if (!IN && s == 1 && r0 + 1 >= nout) break;
@@ -1697,20 +1423,20 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
                         f2fma(f2v(dt_mu), f2sub(lap[s], kap[s]),
                               f2fma(dtdel, f2fma(f2v(nu), kap[s], make_float2(-g.x, -g.y)), ph[s]));
                     const float2 qn = heaviside_q_fast2(pn, eps);
-                    const unsigned o = s ? o1 : o0;
+                    const unsigned o = s ? o1 : o0, oq = s ? q1 : q0;
                     if constexpr (VEC) {
                         if (act0) {
                             *reinterpret_cast<float2 *>(phi_out + o) = pn;
-                            *reinterpret_cast<float2 *>(q_out + o) = qn;
+                            *reinterpret_cast<float2 *>(q_out + oq) = qn;
                         }
                     } else {
                         if (act0) {
                             phi_out[o] = pn.x;
-                            q_out[o] = qn.x;
+                            q_out[oq] = qn.x;
                         }
                         if (act1) {
                             phi_out[o + 1] = pn.y;
-                            q_out[o + 1] = qn.y;
+                            q_out[oq + 1] = qn.y;
                         }
                     }
                     if constexpr (DUMP) {
@@ -1780,23 +1506,35 @@ int &az_persist() {
     return n;
 }
 
+template <int R, class ImgT, int NP>
+constexpr size_t taxy_smem() { return XYSmem<R, SrcH<R, ImgT, NP>>::bytes; }
+template <int R, class S>
+constexpr size_t tbxy_smem() { return XYSmem<R, SrcAB<R, S>>::bytes; }
+
+// Dynamic shared memory of group A's x/y kernel for each image type.
+template <int R, int NP>
+cudaError_t prepare_ta_xy() {
+    cudaError_t e;
+    if ((e = cudaFuncSetAttribute(k_ta_xy<R, uint8_t, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)taxy_smem<R, uint8_t, NP>())) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_ta_xy<R, uint16_t, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                  (int)taxy_smem<R, uint16_t, NP>())) != cudaSuccess) return e;
+    return cudaFuncSetAttribute(k_ta_xy<R, float, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                (int)taxy_smem<R, float, NP>());
+}
+template <int R, int NP>
+void launch_ta_xy(const TiledGroup &g, const GroupArgs &G, const TapPairs &tp, cudaStream_t s) {
+    switch (g.imgtype) {
+        case 0: k_ta_xy<R, uint8_t, NP><<<g.ncta[0], kXYThreads, taxy_smem<R, uint8_t, NP>(), s>>>(G, tp); break;
+        case 1: k_ta_xy<R, uint16_t, NP><<<g.ncta[0], kXYThreads, taxy_smem<R, uint16_t, NP>(), s>>>(G, tp); break;
+        default: k_ta_xy<R, float, NP><<<g.ncta[0], kXYThreads, taxy_smem<R, float, NP>(), s>>>(G, tp);
+    }
+}
+
 template <int R, class S>
 cudaError_t prepare_storage() {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_ta_xy<R, uint8_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)XYLayout<R, 1>::bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_ta_xy<R, uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)XYLayout<R, 1>::bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_ta_xy<R, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)XYLayout<R, 1>::bytes)) != cudaSuccess) return e;
-    if constexpr (R % 2 == 0) {
-        if ((e = cudaFuncSetAttribute(k_ta_xy_tma<R, uint8_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)XYStageH<R, uint8_t>::smem)) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(k_ta_xy_tma<R, uint16_t>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)XYStageH<R, uint16_t>::smem)) != cudaSuccess) return e;
-        if ((e = cudaFuncSetAttribute(k_ta_xy_tma<R, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                      (int)XYStageH<R, float>::smem)) != cudaSuccess) return e;
-    }
+    if ((e = prepare_ta_xy<R, 1>()) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_ta_z<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)az_smem<R>())) !=
         cudaSuccess) return e;
     {
@@ -1818,25 +1556,7 @@ cudaError_t launch_storage(const TiledGroup &g, int parity, Profiler *prof, cuda
     {
         ProfScope ps(prof, KID_TA_XY);
         G.starts = g.starts[0];
-        constexpr size_t sm = XYLayout<R, 1>::bytes;
-        bool staged = false;  // inputs by TMA (every brick's rows allow the copies)
-        if constexpr (R % 2 == 0) {
-            if (g.xy_tma) {
-                staged = true;
-                switch (g.imgtype) {
-                    case 0: k_ta_xy_tma<R, uint8_t><<<g.ncta[0], kXYThreads, XYStageH<R, uint8_t>::smem, s>>>(G, tp); break;
-                    case 1: k_ta_xy_tma<R, uint16_t><<<g.ncta[0], kXYThreads, XYStageH<R, uint16_t>::smem, s>>>(G, tp); break;
-                    default: k_ta_xy_tma<R, float><<<g.ncta[0], kXYThreads, XYStageH<R, float>::smem, s>>>(G, tp);
-                }
-            }
-        }
-        if (!staged) {
-            switch (g.imgtype) {
-                case 0: k_ta_xy<R, uint8_t><<<g.ncta[0], kXYThreads, sm, s>>>(G, tp); break;
-                case 1: k_ta_xy<R, uint16_t><<<g.ncta[0], kXYThreads, sm, s>>>(G, tp); break;
-                default: k_ta_xy<R, float><<<g.ncta[0], kXYThreads, sm, s>>>(G, tp);
-            }
-        }
+        launch_ta_xy<R, 1>(g, G, tp, s);
     }
     {
         ProfScope ps(prof, KID_TA_Z);

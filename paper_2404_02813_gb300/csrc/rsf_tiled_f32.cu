@@ -10,9 +10,26 @@ namespace rsf {
 namespace tiled {
 
 namespace {
-__global__ void k_q_init(const float *__restrict__ phi, float *__restrict__ q, long long n, float eps) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x)
-        q[i] = heaviside_q_fast(__ldg(phi + i), eps);
+// q of phi; rows of nx values at a pitch of qp (one row of n values when they are dense)
+__global__ void k_q_init(const float *__restrict__ phi, float *__restrict__ q, long long rows, long long nx,
+                         long long qp, float eps) {
+    if (rows == 1) {
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nx; i += (long long)gridDim.x * blockDim.x)
+            q[i] = heaviside_q_fast(__ldg(phi + i), eps);
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
+         r += ((long long)gridDim.x * blockDim.x) >> 5)
+        for (int x = lane; x < nx; x += 32) q[r * qp + x] = heaviside_q_fast(__ldg(phi + r * nx + x), eps);
+}
+// rows of nx values copied to a pitch of ip
+template <class T>
+__global__ void k_pitch_rows(const T *__restrict__ src, T *__restrict__ dst, long long rows, int nx, int ip) {
+    const int lane = threadIdx.x & 31;
+    for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
+         r += ((long long)gridDim.x * blockDim.x) >> 5)
+        for (int x = lane; x < nx; x += 32) dst[r * ip + x] = src[r * nx + x];
 }
 }  // namespace
 
@@ -103,55 +120,62 @@ cudaError_t encode_map(CUtensorMap *m, const void *base, int c, const BrickDev &
     return encode_typed(m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, base, c, b.px, b, bx, by, bz);
 }
 
-// Group A's x/y staging maps (q[0], q[1], the image) of an even-radius brick when
-// its unpitched rows allow them; b.xy_tma says whether they were made.
-template <class ImgT>
-cudaError_t encode_xy_stage(BrickDev &b, CUtensorMapDataType type, int R) {
-    b.xy_tma = 0;
+// Box widths (values) and rows of the x/y kernels' staged planes.
+struct XYBoxes { int rows, q, img, ab32, ab16; };
+template <int R>
+XYBoxes xy_boxes_r(int imgtype) {
+    using namespace tiled;
+    const int img = imgtype == 0 ? SrcH<R, uint8_t, 1>::FI::W : (imgtype == 1 ? SrcH<R, uint16_t, 1>::FI::W : SrcH<R, float, 1>::FI::W);
+    return XYBoxes{XYG<R>::H, SrcH<R, float, 1>::FQ::W, img, SrcAB<R, float>::FA::W, SrcAB<R, __half>::FA::W};
+}
+XYBoxes xy_boxes(int R, int imgtype) {
     switch (R) {
-        case 2: case 4: case 6: case 8: case 10: case 12: break;
-        default: return cudaSuccess;
+        case 2: return xy_boxes_r<2>(imgtype);
+        case 3: return xy_boxes_r<3>(imgtype);
+        case 4: return xy_boxes_r<4>(imgtype);
+        case 5: return xy_boxes_r<5>(imgtype);
+        case 6: return xy_boxes_r<6>(imgtype);
+        case 8: return xy_boxes_r<8>(imgtype);
+        case 10: return xy_boxes_r<10>(imgtype);
+        default: return xy_boxes_r<12>(imgtype);
     }
-    // the same box geometry as the kernel's staging (XYStageH)
-    const int H = 32 + 2 * R, RQ = (R + 3) / 4 * 4, AI = 16 / (int)sizeof(ImgT), RI = (R + AI - 1) / AI * AI;
-    const int WQ = 32 + 2 * RQ, WI = 32 + 2 * RI;
-    const unsigned long long qrow = 4ull * b.nx, irow = (unsigned long long)sizeof(ImgT) * b.nx;
-    if (!map_ok(b.q[0], qrow, WQ, H, 1, 4) || !map_ok(b.q[1], qrow, WQ, H, 1, 4) ||
-        !map_ok(b.img, irow, WI, H, 1, (int)sizeof(ImgT)))
-        return cudaSuccess;  // not eligible: the register loaders serve this brick's group
-    cudaError_t e = encode_typed(&b.tm_q[0], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, b.q[0], 1, b.nx, b, WQ, H, 1);
-    if (e == cudaSuccess) e = encode_typed(&b.tm_q[1], CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, b.q[1], 1, b.nx, b, WQ, H, 1);
-    if (e == cudaSuccess)
-        e = encode_typed(&b.tm_img, type, (int)sizeof(ImgT), b.img, 1, b.nx, b, WI, H, 1);
-    if (e == cudaSuccess) b.xy_tma = 1;
-    return e;
 }
 }  // namespace
 
 cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, int R) {
-    const int rows = tiled::kAZT + 2 * R;
-    b.tm_k = CUtensorMap{};
-    b.tm_ab = CUtensorMap{};
-    b.tm_q[0] = b.tm_q[1] = b.tm_img = CUtensorMap{};
-    b.xy_tma = 0;
-    if (force == 1)  // the Eq. (15) form: four fields per voxel, no K*I~, no group B
-        return encode_map(&b.tm_u, b.u2, 4, b, 128, 1, rows);
-    cudaError_t e = encode_map(&b.tm_u, b.u2, 2, b, 64, 1, rows);
-    if (e == cudaSuccess) e = encode_map(&b.tm_k, b.ki, 1, b, 32, 1, tiled::kAZT);
-    if (e == cudaSuccess && storage == 0 && tiled::tbxy_tma(R))
-        e = encode_map(&b.tm_ab, b.ab, 2, b, 2 * tiled_xy_in_pitch(R), 32 + 2 * R, 1);
-    if (e == cudaSuccess) {
-        switch (imgtype) {
-            case 0: e = encode_xy_stage<uint8_t>(b, CU_TENSOR_MAP_DATA_TYPE_UINT8, R); break;
-            case 1: e = encode_xy_stage<uint16_t>(b, CU_TENSOR_MAP_DATA_TYPE_UINT16, R); break;
-            default: e = encode_xy_stage<float>(b, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, R);
-        }
+    const int zrows = tiled::kAZT + 2 * R;
+    const XYBoxes box = xy_boxes(R, imgtype);
+    b.tm_k = b.tm_ab = CUtensorMap{};
+    cudaError_t e = encode_typed(&b.tm_q, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, b.q, 1, b.qp, b, box.q, box.rows, 1);
+    if (e != cudaSuccess) return e;
+    switch (imgtype) {
+        case 0: e = encode_typed(&b.tm_img, CU_TENSOR_MAP_DATA_TYPE_UINT8, 1, b.img_t, 1, b.ip, b, box.img, box.rows, 1); break;
+        case 1: e = encode_typed(&b.tm_img, CU_TENSOR_MAP_DATA_TYPE_UINT16, 2, b.img_t, 1, b.ip, b, box.img, box.rows, 1); break;
+        default: e = encode_typed(&b.tm_img, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, b.img_t, 1, b.ip, b, box.img, box.rows, 1);
     }
-    return e;
+    if (e != cudaSuccess) return e;
+    if (force == 1)  // the Eq. (15) form: four fields per voxel, no K*I~, no group B
+        return encode_map(&b.tm_u, b.u2, 4, b, 128, 1, zrows);
+    e = encode_map(&b.tm_u, b.u2, 2, b, 64, 1, zrows);
+    if (e == cudaSuccess) e = encode_map(&b.tm_k, b.ki, 1, b, 32, 1, tiled::kAZT);
+    if (e != cudaSuccess) return e;
+    if (storage == 0) return encode_map(&b.tm_ab, b.ab, 2, b, 2 * box.ab32, box.rows, 1);
+    // a 16-bit pair is one 32-bit value of the map
+    return encode_typed(&b.tm_ab, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, b.ab, 1, b.px, b, box.ab16, box.rows, 1);
 }
 
-cudaError_t tiled_q_init(const float *phi, float *q, long long n, float eps, cudaStream_t s) {
-    tiled::k_q_init<<<1216, 256, 0, s>>>(phi, q, n, eps);
+cudaError_t tiled_start(const BrickDev &b, int imgtype, cudaStream_t s) {
+    const long long rows = (long long)b.ny * b.nz;
+    if (b.img_t != b.img) {
+        void *d = const_cast<void *>(b.img_t);
+        switch (imgtype) {
+            case 0: tiled::k_pitch_rows<<<1216, 256, 0, s>>>((const uint8_t *)b.img, (uint8_t *)d, rows, b.nx, b.ip); break;
+            case 1: tiled::k_pitch_rows<<<1216, 256, 0, s>>>((const uint16_t *)b.img, (uint16_t *)d, rows, b.nx, b.ip); break;
+            default: tiled::k_pitch_rows<<<1216, 256, 0, s>>>((const float *)b.img, (float *)d, rows, b.nx, b.ip);
+        }
+    }
+    const bool dense = b.qp == b.nx;
+    tiled::k_q_init<<<1216, 256, 0, s>>>(b.phi[0], b.q, dense ? 1 : rows, dense ? rows * b.nx : b.nx, b.qp, b.eps);
     return cudaGetLastError();
 }
 
@@ -206,14 +230,38 @@ UpdateTile update_tile(int R) {
 }  // namespace
 
 void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]) {
-    const unsigned ntx = (b.nx + tiled::kXYT - 1) / tiled::kXYT, nty = (b.ny + tiled::kXYT - 1) / tiled::kXYT;
-    const unsigned nzp = (b.nz + tiled::xy_planes(b) - 1) / tiled::xy_planes(b);
+    const unsigned th = R <= 8 ? tiled::XYG<8>::TH : tiled::XYG<12>::TH;
+    const unsigned ntx = (b.nx + tiled::kXYT - 1) / tiled::kXYT, nty = (b.ny + th - 1) / th;
+    const unsigned nzp = (b.nz + b.xyp - 1) / b.xyp;
     const int rows = update_tile(force ? 0 : R).rows;
     counts[0] = ntx * nty * nzp;
     counts[1] = (unsigned)((b.nz + tiled::kAZT - 1) / tiled::kAZT) * ((b.nx + 31) / 32) * b.ny;
     counts[2] = counts[0];
     counts[3] = (unsigned)((b.nx + tiled::kZX - 1) / tiled::kZX) * ((b.ny + rows - 1) / rows) *
                 ((b.nz + b.zc - 1) / b.zc) * ((b.zc + b.zs - 1) / b.zs);
+}
+
+// A CTA of the x/y kernels costs its planes plus about one plane time (set-up and the first
+// copies; 64^3: 1 plane per CTA 8.1 us, 16 planes 37 us; 512^3: 16 planes 0.463 ms, 32 planes
+// 0.480 ms, so 16 is the most); three or four share an SM.  Few CTAs run in whole waves; many even out but for
+// about half a CTA at the end.
+int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int sms) {
+    const int th = R <= 8 ? tiled::XYG<8>::TH : tiled::XYG<12>::TH;
+    const double slots = (force ? 3.0 : 4.0) * sms;
+    int best = 1;
+    double best_cost = 0.0;
+    for (int p : {1, 2, 3, 4, 6, 8, 12, 16}) {
+        double ctas = 0.0;
+        for (const BrickDev &b : bricks)
+            ctas += (double)((b.nx + tiled::kXYT - 1) / tiled::kXYT) * ((b.ny + th - 1) / th) * ((b.nz + p - 1) / p);
+        const double waves = ctas / slots;
+        const double cost = (waves < 4.0 ? std::ceil(waves) : waves + 0.5) * (p + 1.0);
+        if (p == 1 || cost < best_cost) {
+            best_cost = cost;
+            best = p;
+        }
+    }
+    return best;
 }
 
 // A CTA of the update kernel costs its zs output planes plus about 4 + 0.4 M plane times to
@@ -249,64 +297,100 @@ int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, i
     return best;
 }
 
-// Per pitched voxel, Li's form: (H I~, H) 8 bytes, (a, b) 2 elements of the
-// storage type, x/y-convolved (a, b) 8 bytes, K*I~ 4 bytes (24 or 28 bytes; np
-// is even: every view is 8-byte aligned).  The Eq. (15) form: the two
-// x/y-convolved pairs 16 bytes, the fits (f1, f2) 8 bytes (24 bytes, within
-// the count for every storage type; no (a, b), no K*I~).
-size_t tiled_stage_bytes(int storage, long long np) {
-    const size_t e = storage == 0 ? 4 : 2;
-    return (8 + 2 * e + 8 + 4) * (size_t)np;
+// Per pitched voxel, Li's form: (H I~, H) and, after it in the same memory, the x/y-convolved
+// (a, b): 8 bytes; (a, b) 2 elements of the storage type; K*I~ 4 bytes; 8 bytes left.  The
+// Eq. (15) form: the two x/y-convolved pairs 16 bytes, the fits (f1, f2) 8 bytes; 4 bytes left
+// with FP32 storage, none with 16-bit.  What is left, or what q leaves of its block, holds the
+// copied image of a brick whose rows are not 16-byte aligned (at most 4 bytes per pitched voxel).
+size_t tiled_stage_bytes(int storage, long long np) { return (size_t)(storage == 0 ? 28 : 24) * (size_t)np; }
+
+namespace {
+int image_size(int imgtype) { return imgtype == 0 ? 1 : (imgtype == 1 ? 2 : 4); }
+int image_pitch(int nx, int imgtype) {
+    const int per = 16 / image_size(imgtype);
+    return (nx + per - 1) / per * per;
+}
+bool copied_image(const void *img, int nx, int imgtype) {
+    return image_pitch(nx, imgtype) != nx || reinterpret_cast<uintptr_t>(img) % 16 != 0;
+}
+size_t field_bytes(int storage, int force, long long np) { return (size_t)(force ? 24 : (storage == 0 ? 20 : 16)) * np; }
+int q_pitch(int nx) { return (nx + 3) / 4 * 4; }
+}  // namespace
+
+size_t tiled_extra_bytes(const void *img, int nx, int ny, int nz, int imgtype, int storage, int force) {
+    if (!copied_image(img, nx, imgtype)) return 0;
+    const long long rows = (long long)ny * nz, np = tiled_pitch(nx) * rows;
+    const size_t need = (size_t)image_size(imgtype) * image_pitch(nx, imgtype) * rows;
+    if (field_bytes(storage, force, np) + need <= tiled_stage_bytes(storage, np)) return 0;
+    return 4ull * q_pitch(nx) * rows + need <= 8ull * nx * rows ? 0 : need;
 }
 
-void tiled_stage_views(int storage, int force, void *base, long long np, float2 **u2, void **ab, float2 **abxy,
-                       float **ki) {
-    char *p = static_cast<char *>(base);
-    *u2 = reinterpret_cast<float2 *>(p);
+void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q,
+                        void *extra) {
+    const long long rows = (long long)b.ny * b.nz;
+    b.px = tiled_pitch(b.nx);
+    const long long np = b.px * rows;
+    char *p = static_cast<char *>(stage);
+    b.u2 = reinterpret_cast<float2 *>(p);
     if (force) {
-        *ab = nullptr;
-        *abxy = reinterpret_cast<float2 *>(p + 16 * np);
-        *ki = nullptr;
-        return;
+        b.ab = nullptr;
+        b.abxy = reinterpret_cast<float2 *>(p + 16 * np);
+        b.ki = nullptr;
+    } else {
+        b.abxy = b.u2;
+        b.ab = p + 8 * np;
+        b.ki = reinterpret_cast<float *>(p + (storage == 0 ? 16 : 12) * np);
     }
-    const size_t e = storage == 0 ? 4 : 2;
-    *ab = p + 8 * np;
-    *abxy = reinterpret_cast<float2 *>(p + (8 + 2 * e) * np);
-    *ki = reinterpret_cast<float *>(p + (16 + 2 * e) * np);
+    b.q = static_cast<float *>(q);
+    b.qp = q_pitch(b.nx);
+    b.img_t = b.img;
+    b.ip = b.nx;
+    if (copied_image(b.img, b.nx, imgtype)) {
+        b.ip = image_pitch(b.nx, imgtype);
+        const size_t need = (size_t)image_size(imgtype) * b.ip * rows, used = field_bytes(storage, force, np);
+        const size_t qb = 4ull * b.qp * rows;  // a multiple of 16
+        b.img_t = used + need <= stage_bytes ? p + used
+                                             : (qb + need <= 8ull * b.nx * rows ? static_cast<char *>(q) + qb
+                                                                                : static_cast<char *>(extra));
+    }
 }
 
 namespace {
 template <int R, class ImgT>
-cudaError_t ki_init_r(const BrickDev &b, const Taps &taps, cudaStream_t s) {
-    static_assert(tiled::XYLayout<R, 1>::bytes <= 48 * 1024, "k_ki_xy needs no shared-memory opt-in");
+cudaError_t ki_init_r(const BrickDev &b, const Taps &taps, int *err, cudaStream_t s) {
+    constexpr size_t sm = tiled::XYSmem<R, tiled::SrcI<R, ImgT>>::bytes;
+    static_assert(sm <= 48 * 1024, "k_ki_xy needs no shared-memory opt-in");
     const tiled::TapPairs tp = tiled::tap_pairs(taps);
     unsigned counts[4];
     tiled_cta_counts(b, 0, R, counts);
-    tiled::k_ki_xy<R, ImgT><<<counts[0], tiled::kXYThreads, tiled::XYLayout<R, 1>::bytes, s>>>(b, tp);
+    tiled::k_ki_xy<R, ImgT><<<counts[0], tiled::kXYThreads, sm, s>>>(b, err, tp);
     tiled::k_ki_z<R><<<counts[1], tiled::kAZThreads, 0, s>>>(b, tp);
     return cudaGetLastError();
 }
 template <int R>
-cudaError_t ki_init_i(const BrickDev &b, int imgtype, const Taps &taps, cudaStream_t s) {
+cudaError_t ki_init_i(const BrickDev &b, int imgtype, const Taps &taps, int *err, cudaStream_t s) {
     switch (imgtype) {
-        case 0: return ki_init_r<R, uint8_t>(b, taps, s);
-        case 1: return ki_init_r<R, uint16_t>(b, taps, s);
-        default: return ki_init_r<R, float>(b, taps, s);
+        case 0: return ki_init_r<R, uint8_t>(b, taps, err, s);
+        case 1: return ki_init_r<R, uint16_t>(b, taps, err, s);
+        default: return ki_init_r<R, float>(b, taps, err, s);
     }
 }
 }  // namespace
 
-cudaError_t tiled_ki_init(const BrickDev &b, int imgtype, const Taps &taps, cudaStream_t s) {
-    if (!b.ki) return cudaSuccess;  // the Eq. (15) form convolves the complement directly
+cudaError_t tiled_ki_init(const BrickDev &brick, int imgtype, const Taps &taps, int *err, cudaStream_t s) {
+    if (!brick.ki) return cudaSuccess;  // the Eq. (15) form convolves the complement directly
+    BrickDev b = brick;
+    const cudaError_t e = tiled_encode_maps(b, 0, 0, imgtype, taps.R);
+    if (e != cudaSuccess) return e;
     switch (taps.R) {
-        case 2: return ki_init_i<2>(b, imgtype, taps, s);
-        case 3: return ki_init_i<3>(b, imgtype, taps, s);
-        case 4: return ki_init_i<4>(b, imgtype, taps, s);
-        case 5: return ki_init_i<5>(b, imgtype, taps, s);
-        case 6: return ki_init_i<6>(b, imgtype, taps, s);
-        case 8: return ki_init_i<8>(b, imgtype, taps, s);
-        case 10: return ki_init_i<10>(b, imgtype, taps, s);
-        case 12: return ki_init_i<12>(b, imgtype, taps, s);
+        case 2: return ki_init_i<2>(b, imgtype, taps, err, s);
+        case 3: return ki_init_i<3>(b, imgtype, taps, err, s);
+        case 4: return ki_init_i<4>(b, imgtype, taps, err, s);
+        case 5: return ki_init_i<5>(b, imgtype, taps, err, s);
+        case 6: return ki_init_i<6>(b, imgtype, taps, err, s);
+        case 8: return ki_init_i<8>(b, imgtype, taps, err, s);
+        case 10: return ki_init_i<10>(b, imgtype, taps, err, s);
+        case 12: return ki_init_i<12>(b, imgtype, taps, err, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -489,8 +489,10 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     if (force != RSF_FORCE_LI && !tiled)
         return fail(RSF_E_INVAL, "the Eq. (15) force form needs the tiled path (radius %d, path option %d)", taps.R,
                     c->opt_path);
-    // the tiled path reads the image in its own type and centres it on load
-    RSF_CUDA(rsf::setup_image(vol, (int)vt, taps, f, c->stream, !tiled));
+    // the exact arithmetic of the separable passes, in the tiled schedule where that takes the volume
+    const bool exact = !tiled && rsf::exact_supports(taps.R) && rsf::tiled_fits(nx, ny, nz);
+    // the tiled schedule centres the image itself, on load or into its own field
+    RSF_CUDA(rsf::setup_image(vol, (int)vt, taps, f, c->stream, !tiled && !exact));
     if (c->opt_poison) {  // NaN bytes in everything the iteration must write before it reads
         RSF_CUDA(cudaMemsetAsync(f.t[0], 0xFF, sizeof(float) * 8 * (size_t)c->cap_np, c->stream));
         RSF_CUDA(cudaMemsetAsync(f.phi[1], 0xFF, sizeof(float) * n, c->stream));
@@ -498,8 +500,9 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     }
     RSF_CUDA(xfer(f.phi[0], phi0, sizeof(float) * n, c->stream));
     int cur = 0;
-    if (tiled) {
-        RSF_CUDA(rsf::tiled_prepare(storage, taps.R, force));
+    if (tiled || exact) {
+        const int form = exact ? rsf::kForceExact : force;
+        RSF_CUDA(rsf::tiled_prepare(storage, taps.R, form));
         rsf::BrickDev b{};
         b.nx = (int)nx;
         b.ny = (int)ny;
@@ -509,7 +512,10 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         b.prof = f.prof;
         b.phi[0] = f.phi[0];
         b.phi[1] = f.phi[1];
-        rsf::tiled_place_fields(b, storage, force, (int)vt, f.t[0], sizeof(float) * 8 * (size_t)f.px * ny * nz, f.q, nullptr);
+        if (exact)
+            rsf::exact_place_fields(b, f.t[0], f.q);
+        else
+            rsf::tiled_place_fields(b, storage, force, (int)vt, f.t[0], sizeof(float) * 8 * (size_t)f.px * ny * nz, f.q, nullptr);
         b.eps = eps;
         b.lambda1 = lambda1;
         b.lambda2 = lambda2;
@@ -520,25 +526,28 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         b.zs = b.zc;
         int sms = 0;
         RSF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
-        b.xyp = rsf::tiled_xy_planes({b}, force, taps.R, sms);
+        b.xyp = rsf::tiled_xy_planes({b}, form, taps.R, sms);
         if (b.zc <= 0) {
             const long long nxy = (long long)((nx + 31) / 32) * ((ny + 7) / 8);
             const long long chunks = std::max<long long>(1, (16LL * sms + nxy - 1) / nxy);
             b.zc = (int)std::max<long long>(16, (nz + chunks - 1) / chunks);
-            b.zs = rsf::tiled_update_planes({b}, force, taps.R, b.zc, sms);
+            b.zs = rsf::tiled_update_planes({b}, form, taps.R, b.zc, sms);
         }
         b.dump = dump;  // only rsf_step_stages asks for stages, and it runs one iteration
         std::vector<GroupSpec> specs(1);
         specs[0].storage = storage;
-        specs[0].force = force;
-        specs[0].imgtype = (int)vt;
+        specs[0].force = form;
+        specs[0].imgtype = exact ? (int)RSF_F32 : (int)vt;
         specs[0].taps = taps;
         specs[0].bricks.push_back(b);
         std::vector<rsf::TiledGroup> groups;
         if ((st = upload_groups(c, c->desc, c->stream, specs, &groups))) return st;
         const rsf::TiledGroup &g = groups[0];
         if (iters > 0) {
-            RSF_CUDA(rsf::tiled_start(b, (int)vt, c->stream));
+            if (exact)
+                RSF_CUDA(rsf::exact_start(b, vol, (int)vt, c->stream));
+            else
+                RSF_CUDA(rsf::tiled_start(b, (int)vt, c->stream));
             RSF_CUDA(rsf::tiled_ki_init(b, (int)vt, taps, c->d_err, c->stream));
         }
         for (int it = 0; it < iters; ++it) {

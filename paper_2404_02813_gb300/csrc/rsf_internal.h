@@ -123,7 +123,8 @@ struct BrickDev {
 // A set of bricks launched together: same radius, image type and storage.
 struct TiledGroup {
     int storage;            // 0 FP32, 1 BF16, 2 FP16 (rsf_storage)
-    int force;              // 0 Li's data terms (group B convolutions), 1 Eq. (15) with sigma_2 = 0
+    int force;              // 0 Li's data terms (group B convolutions), 1 Eq. (15) with sigma_2 = 0,
+                            // kForceExact Li's in the exact arithmetic
     int imgtype;            // 0 uint8, 1 uint16, 2 float
     Taps taps;
     const BrickDev *bricks; // device array of nb descriptors
@@ -134,6 +135,8 @@ struct TiledGroup {
     int *err;               // device-visible error word of the kernels' bounded waits (nonzero: expired)
     unsigned fault_tx;      // bytes the TMA barriers expect beyond their copies (0; > 0 in a fault test)
 };
+
+constexpr int kForceExact = 2;
 
 // Device error word values (TiledGroup::err).
 constexpr int kErrWaitExpired = 1;  // a bounded wait for a TMA copy ran out (1 s)
@@ -168,6 +171,15 @@ void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *
 // Before the first iteration: the image copied to b.img_t where its rows are not 16-byte
 // aligned, and q = +-atan(eps/|phi|)/pi (sign of phi) of b.phi[0].
 cudaError_t tiled_start(const BrickDev &b, int imgtype, cudaStream_t s);
+// The exact arithmetic (rsf_exact.cuh): radii 1 to 16.  Fields in a stage block of
+// exact_stage_bytes and a q block of exact_q_bytes (at most the 8 nx ny nz above); before the
+// first iteration the centred image (b.img, FP32, pitched; from the caller's vol and b.cs)
+// and q.
+bool exact_supports(int R);
+size_t exact_stage_bytes(int nx, int ny, int nz);
+size_t exact_q_bytes(int nx, int ny, int nz);
+void exact_place_fields(BrickDev &b, void *stage, float *q);
+cudaError_t exact_start(const BrickDev &b, const void *vol, int vt, cudaStream_t s);
 // b.ki = K*I~ before the first tiled iteration (after tiled_start; b.cs set; uses b.abxy as
 // scratch); nothing when b.ki is null (the Eq. (15) form).  err: the error word of its waits.
 cudaError_t tiled_ki_init(const BrickDev &b, int imgtype, const Taps &taps, int *err, cudaStream_t s);

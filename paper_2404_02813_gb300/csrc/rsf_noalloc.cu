@@ -19,7 +19,9 @@
 #include <cuda_runtime.h>
 
 #include <cmath>
+#include <cstddef>
 #include <cstdio>
+#include <cstring>
 #include <mutex>
 
 #include "rsf.h"
@@ -30,14 +32,19 @@ namespace {
 
 constexpr long long kMaxVoxels = 1LL << 18;              // 262,144 voxels (for example 64^3)
 constexpr long long kMaxProfile = kMaxVoxels / 16 + 8;   // nx+ny+nz when every side is >= 4
-constexpr long long kOffI = 0;                           // centred image
-constexpr long long kOffPhi = kOffI + kMaxVoxels;        // one phi buffer (phi_out is the other)
-constexpr long long kOffT = kOffPhi + kMaxVoxels;        // eight stage buffers
+constexpr long long kOffPhi = 0;                         // one phi buffer (phi_out is the other)
+constexpr long long kOffI = kOffPhi + kMaxVoxels;        // centred image
+constexpr long long kOffT = kOffI + kMaxVoxels;          // eight stage buffers
 constexpr long long kOffProf = kOffT + 8 * kMaxVoxels;   // K*1 profiles
 constexpr long long kOffCs = kOffProf + ((kMaxProfile + 63) / 64) * 64;
 constexpr long long kOffPart = kOffCs + 64;              // reduction partials
 constexpr long long kScratchFloats = kOffPart + 3 * rsf::kStatBlocks;
 constexpr int kMaxDevices = 64;
+// The tiled kernels' fields take the same memory from kOffI on: launch descriptor (with the
+// CTA offsets after it), q and stage blocks, where the x pitch (a multiple of 32) leaves room
+// for them: always when nx is a multiple of 32, or below about 0.8 of the voxel limit at nx >= 33.
+constexpr size_t kDescBytes = (sizeof(rsf::BrickDev) + 64 + 255) / 256 * 256;
+constexpr size_t kFieldBytes = sizeof(float) * 9 * (size_t)kMaxVoxels;
 
 }  // namespace
 
@@ -101,6 +108,53 @@ __global__ void k_noalloc_put(ParamChunk c, float *__restrict__ dst) {
         dst[c.offset + i] = c.v[i];
 }
 
+
+void put_floats(const float *v, int n, float *dst, cudaStream_t s) {
+    for (int o = 0; o < n; o += kParamChunk) {
+        ParamChunk c;
+        c.offset = o;
+        c.count = n - o < kParamChunk ? n - o : kParamChunk;
+        memcpy(c.v, v + o, sizeof(float) * c.count);
+        k_noalloc_put<<<(c.count + 255) / 256, 256, 0, s>>>(c, dst);
+    }
+}
+
+// The iterations in the tiled schedule (rsf_exact.cuh), all fields in `mem`; phi[0] holds phi0.
+cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Taps &taps, int iters, char *mem, int dev,
+                         cudaStream_t s) {
+    char *const q = mem + kDescBytes;
+    rsf::exact_place_fields(b, q + (rsf::exact_q_bytes(b.nx, b.ny, b.nz) + 255) / 256 * 256, reinterpret_cast<float *>(q));
+    int sms = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    if ((e = rsf::tiled_prepare(0, taps.R, rsf::kForceExact)) != cudaSuccess) return e;
+    b.xyp = rsf::tiled_xy_planes({b}, rsf::kForceExact, taps.R, sms);
+    b.zc = b.nz;
+    b.zs = rsf::tiled_update_planes({b}, rsf::kForceExact, taps.R, b.zc, sms);
+    if ((e = rsf::tiled_encode_maps(b, rsf::kForceExact, 0, 2, taps.R)) != cudaSuccess) return e;
+    rsf::TiledGroup g{};
+    g.force = rsf::kForceExact;
+    g.imgtype = 2;
+    g.taps = taps;
+    g.nb = 1;
+    rsf::tiled_cta_counts(b, g.force, taps.R, g.ncta);
+    struct {
+        rsf::BrickDev b;
+        int starts[8];
+    } d{};
+    d.b = b;
+    for (int k = 0; k < 4; ++k) d.starts[2 * k + 1] = (int)g.ncta[k];
+    static_assert(sizeof(d) <= kDescBytes && sizeof(d) % sizeof(float) == 0, "descriptor");
+    const rsf::BrickDev *db = reinterpret_cast<const rsf::BrickDev *>(mem);
+    g.bricks = db;
+    for (int k = 0; k < 4; ++k) g.starts[k] = reinterpret_cast<const int *>(mem + offsetof(decltype(d), starts)) + 2 * k;
+    put_floats(reinterpret_cast<const float *>(&d), (int)(sizeof(d) / sizeof(float)), reinterpret_cast<float *>(mem), s);
+    if ((e = rsf::exact_start(b, vol, vt, s)) != cudaSuccess) return e;
+    for (int it = 0; it < iters; ++it)
+        if ((e = rsf::tiled_iterate(g, it & 1, nullptr, s)) != cudaSuccess) return e;
+    return cudaGetLastError();
+}
+
 }  // namespace
 
 extern "C" rsf_status rsf_evolve_noalloc(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int64_t nz,
@@ -150,31 +204,48 @@ extern "C" rsf_status rsf_evolve_noalloc(const void *volume, rsf_dtype vt, int64
         else e = cudaSuccess;
         return e == cudaSuccess ? RSF_OK : err(RSF_E_CUDA, cudaGetErrorString(e));
     }
-    if ((e = rsf::centre_image(volume, (int)vt, f, s)) != cudaSuccess) return err(RSF_E_CUDA, cudaGetErrorString(e));
+    const bool tiled = rsf::exact_supports(R) &&
+                       kDescBytes + (rsf::exact_q_bytes((int)nx, (int)ny, (int)nz) + 255) / 256 * 256 +
+                               rsf::exact_stage_bytes((int)nx, (int)ny, (int)nz) <= kFieldBytes;
+    e = tiled ? rsf::image_stats(volume, (int)vt, f, s) : rsf::centre_image(volume, (int)vt, f, s);
+    if (e != cudaSuccess) return err(RSF_E_CUDA, cudaGetErrorString(e));
     // zero-padding profiles (K*1 = p_x p_y p_z), by the same host routine as rsf_evolve's;
     // nx + ny + nz <= kMaxProfile within the voxel limit
     float prof[kMaxProfile];
-    const int np = (int)(nx + ny + nz);
     rsf::zero_padding_profiles(taps, (int)nx, (int)ny, (int)nz, prof);
-    for (int o = 0; o < np; o += kParamChunk) {
-        ParamChunk c;
-        c.offset = o;
-        c.count = np - o < kParamChunk ? np - o : kParamChunk;
-        for (int i = 0; i < c.count; ++i) c.v[i] = prof[o + i];
-        k_noalloc_put<<<(c.count + 255) / 256, 256, 0, s>>>(c, f.prof);
-    }
+    put_floats(prof, (int)(nx + ny + nz), f.prof, s);
     // phi0 is copied first so that phi_out may alias it; the iterations then
     // alternate between the static buffer and phi_out
     if ((e = cudaMemcpyAsync(scratch_phi, phi0, sizeof(float) * n, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)
         return err(RSF_E_CUDA, cudaGetErrorString(e));
     const float *in = scratch_phi;
-    float *out = phi_out;
-    for (int it = 0; it < iters; ++it) {
-        if ((e = rsf::iterate_passes(taps, co, f, in, out, nullptr, nullptr, s)) != cudaSuccess)
+    if (tiled) {
+        rsf::BrickDev b{};
+        b.nx = (int)nx;
+        b.ny = (int)ny;
+        b.nz = (int)nz;
+        b.cs = f.cs;
+        b.prof = f.prof;
+        b.phi[0] = scratch_phi;
+        b.phi[1] = phi_out;
+        b.eps = eps;
+        b.lambda1 = lambda1;
+        b.lambda2 = lambda2;
+        b.nu = nu;
+        b.mu = mu;
+        b.dt = dt;
+        if ((e = evolve_tiled(b, volume, (int)vt, taps, iters, reinterpret_cast<char *>(base + kOffI), dev, s)) != cudaSuccess)
             return err(RSF_E_CUDA, cudaGetErrorString(e));
-        float *nxt = (out == phi_out) ? scratch_phi : phi_out;
-        in = out;
-        out = nxt;
+        in = iters % 2 ? phi_out : scratch_phi;
+    } else {
+        float *out = phi_out;
+        for (int it = 0; it < iters; ++it) {
+            if ((e = rsf::iterate_passes(taps, co, f, in, out, nullptr, nullptr, s)) != cudaSuccess)
+                return err(RSF_E_CUDA, cudaGetErrorString(e));
+            float *nxt = (out == phi_out) ? scratch_phi : phi_out;
+            in = out;
+            out = nxt;
+        }
     }
     if (in != phi_out) {
         if ((e = cudaMemcpyAsync(phi_out, in, sizeof(float) * n, cudaMemcpyDeviceToDevice, s)) != cudaSuccess)

@@ -240,7 +240,7 @@ __device__ __forceinline__ void report_error(int *err, int code) {
 // -> 1.083 ms; 64^3 uint8 21.6 -> 8.1 and 15.7 -> 6.3 us (fewer planes per CTA).
 template <int R>
 struct XYG {
-    static constexpr int TH = R <= 8 ? 48 : 40;  // output rows
+    static constexpr int TH = R <= 8 ? 48 : (R <= 12 ? 40 : 32);  // output rows
     static constexpr int H = TH + 2 * R;         // staged rows: at most 64 (one item of 8 rows per warp)
     static constexpr int YT = TH / (kXYThreads / 32);
     static constexpr int NI = 8 + 2 * R;         // inputs of an x-phase window
@@ -290,7 +290,8 @@ template <> struct ImgVec<float> {
 // its staging buffer, issue() of one plane's boxes
 // (one thread), fix() of what the copies' zero fill gets wrong outside the brick (all
 // threads; FIX: it is needed), and window(): f(j, pairs) for the NI inputs of a window.
-template <int R, class ImgT, int NP_>
+// EX: q from the exact arithmetic, whose zero keeps its sign (q = -0: H = 0)
+template <int R, class ImgT, int NP_, bool EX>
 struct SrcH {  // NP = 1: (H I~, H); NP = 2: also ((1-H) I~, 1-H), the other side of Eq. (10)
     static constexpr int NP = NP_, CTAS = NP == 1 ? 4 : 3, NS = 1;
     static constexpr bool FIX = true;
@@ -334,11 +335,12 @@ struct SrcH {  // NP = 1: (H I~, H); NP = 2: also ((1-H) I~, 1-H), the other sid
             if (j == 0 || ji % ImgVec<ImgT>::V == 0) iv.load(im + ji / ImgVec<ImgT>::V * ImgVec<ImgT>::V);
             const float qj = jq % 4 == 0 ? q4.x : (jq % 4 == 1 ? q4.y : (jq % 4 == 2 ? q4.z : q4.w));
             const float v = fmaf(iv.get(ji % ImgVec<ImgT>::V), inv_s, nms);
-            const float h = h_of_q(qj);
+            const bool neg = EX ? __float_as_int(qj) < 0 : qj < 0.f;
+            const float h = neg ? -qj : 1.f - qj;
             float2 p[NP];
             p[0] = make_float2(__fmul_rn(h, v), h);
             if constexpr (NP == 2) {
-                const float hc = qj < 0.75f ? hc_of_q(qj) : 0.f;
+                const float hc = qj >= 0.75f ? 0.f : (neg ? 1.f + qj : qj);  // the mark of fix()
                 p[1] = make_float2(__fmul_rn(hc, v), hc);
             }
             f(j, p);
@@ -567,13 +569,13 @@ __device__ __forceinline__ XYTile xy_tile_of(int local, const BrickDev &B) {
 
 // Group A's x/y kernel: (H I~, H) into B.u2 (Li's form, NP = 1), or both sides of Eq. (10),
 // ((H I~, H), ((1-H) I~, 1-H)) interleaved per voxel (the Eq. (15) form, NP = 2).
-template <int R, class ImgT, int NP>
-__global__ void __launch_bounds__(kXYThreads, (SrcH<R, ImgT, NP>::CTAS)) k_ta_xy(GroupArgs G, TapPairs t) {
+template <int R, class ImgT, int NP, bool EX = false>
+__global__ void __launch_bounds__(kXYThreads, (SrcH<R, ImgT, NP, EX>::CTAS)) k_ta_xy(GroupArgs G, TapPairs t) {
     extern __shared__ __align__(128) unsigned char xsm[];
     const int b = find_brick(G.starts, G.nb, blockIdx.x);
     const BrickDev &B = G.bricks[b];
     const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
-    const SrcH<R, ImgT, NP> src{&B.tm_q, &B.tm_img, B.cs[1], -B.cs[0] * B.cs[1]};
+    const SrcH<R, ImgT, NP, EX> src{&B.tm_q, &B.tm_img, EX ? 1.f : B.cs[1], EX ? 0.f : -B.cs[0] * B.cs[1]};
     const OutXY out{B.u2, B.px, (long long)B.px * B.ny};
     xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
 }
@@ -810,7 +812,9 @@ constexpr int az4_stage() { return (kAZT + 2 * R) * 32; }  // float4 units per s
 template <int R>
 constexpr size_t az4_smem() { return 2 * sizeof(float4) * az4_stage<R>() + 2 * sizeof(uint64_t); }  // + barriers
 
-template <int R>
+// AB: the exact arithmetic of Li's form, IEEE divisions and a = l1 f1 - l2 f2,
+// b = l1 f1^2 - l2 f2^2 to B.ab instead of the fits.
+template <int R, bool AB = false>
 __global__ void __launch_bounds__(kAZThreads, 2) k_ta_z4(GroupArgs G, TapPairs t) {
     constexpr int T = 2 * R + 1;
     constexpr int WIN = kAZO + 2 * R;
@@ -850,15 +854,24 @@ __global__ void __launch_bounds__(kAZThreads, 2) k_ta_z4(GroupArgs G, TapPairs t
         }
         const long long pplane = (long long)B.px * B.ny;
         const long long off = (long long)(id.z0 + zb) * pplane + (long long)id.y * B.px + x;
-        float2 *fits = B.abxy + off;
+        float2 *fits = (AB ? reinterpret_cast<float2 *>(B.ab) : B.abxy) + off;
+        const float l1 = B.lambda1, l2 = B.lambda2;
         const int bnz = B.nz;
         float *const dump = B.dump;
 #pragma unroll
         for (int o = 0; o < kAZO; ++o) {
             const int zo = id.z0 + zb + o;
             if (zo < bnz) {
-                const float f1 = __fdividef(acc[0][o].x, acc[0][o].y), f2 = __fdividef(acc[1][o].x, acc[1][o].y);
-                *fits = make_float2(f1, f2);
+                float f1, f2;
+                if constexpr (AB) {
+                    f1 = acc[0][o].x / acc[0][o].y;
+                    f2 = acc[1][o].x / acc[1][o].y;
+                    *fits = make_float2(l1 * f1 - l2 * f2, l1 * (f1 * f1) - l2 * (f2 * f2));
+                } else {
+                    f1 = __fdividef(acc[0][o].x, acc[0][o].y);
+                    f2 = __fdividef(acc[1][o].x, acc[1][o].y);
+                    *fits = make_float2(f1, f2);
+                }
                 fits += pplane;
                 if (dump) {
                     const long long q = (long long)zo * B.nx * B.ny + (long long)id.y * B.nx + x;
@@ -993,7 +1006,9 @@ __device__ __forceinline__ float2 heaviside_q_fast2(float2 u, float eps) {
 // the rest of a step is one piece of code.
 //
 // Tile rows: two CTAs' rings fit an SM's shared memory; 14 rows make eight warps, two on
-// each of the SM's quarters, at 128 registers (nine warps are held to 96, and spilled).
+// each of the SM's quarters, at 128 registers (nine warps are held to 96, and spilled).  The
+// exact arithmetic takes 10 rows, six warps at up to 168 registers: nothing spills, so that
+// rsf_evolve_noalloc's launches need no local memory.
 //
 // Finite differences use reflect-101 for phi (the copies read the mirrored voxel) and
 // for the normal (the reads of n_x, n_y at the first and last column or row take the
@@ -1002,12 +1017,12 @@ __device__ __forceinline__ float2 heaviside_q_fast2(float2 u, float eps) {
 // 512^3, uint16, per launch: radius 6 1.034 -> 0.726 ms, 448 x 512 x 320 radius 10 0.663 -> 0.467 ms;
 // 500^3 uint8, Eq. (15) form 0.906 -> 0.575 ms; 64^3 uint8 21.7 -> 9.1 us (its chunks split).
 // At radius 6 it issues 117 thread instructions per voxel and reaches 0.60 of the HBM rate.
-template <int R>
-constexpr int tbz_rows() { return R <= 8 ? 14 : (R <= 10 ? 12 : 10); }
+template <int R, bool EX>
+constexpr int tbz_rows() { return R > 12 ? 8 : (R > 10 || EX ? 10 : (R > 8 ? 12 : 14)); }
 
-template <int R>
+template <int R, bool EX = false>
 struct TBZ {
-    static constexpr int TY = tbz_rows<R>();
+    static constexpr int TY = tbz_rows<R, EX>();
     static constexpr int NWC = TY / 2;                  // warps with outputs
     static constexpr int THREADS = (NWC + 1) * 32;
     static constexpr int M = (2 * R + 4 + 3) / 4 * 4;   // (a, b) planes in the ring
@@ -1097,13 +1112,51 @@ __device__ __forceinline__ void unit_normal2(float2 gx, float2 gy, float2 gz, bo
     nz = f2mul(gz, inv);
 }
 
+// The same by IEEE operations (the exact arithmetic).
+__device__ __forceinline__ float unit_normal_exact(float gx, float gy, float gz, float &hx, float &hy, float &hz) {
+    hx = gx * 0.5f;
+    hy = gy * 0.5f;
+    hz = gz * 0.5f;
+    return sqrtf(hx * hx + hy * hy + hz * hz) + 1e-10f;
+}
+template <bool EX>
+__device__ __forceinline__ void normal2(float2 gx, float2 gy, float2 gz, bool first_x, float2 &nx, float2 &ny,
+                                        float2 &nz) {
+    if constexpr (EX) {
+        float2 hx, hy, hz;
+        const float m0 = unit_normal_exact(gx.x, gy.x, gz.x, hx.x, hy.x, hz.x);
+        const float m1 = unit_normal_exact(gx.y, gy.y, gz.y, hx.y, hy.y, hz.y);
+        nx = make_float2(hx.x / m0, hx.y / m1);
+        ny = make_float2(hy.x / m0, hy.y / m1);
+        nz = make_float2(hz.x / m0, hz.y / m1);
+    } else {
+        unit_normal2(gx, gy, gz, first_x, nx, ny, nz);
+    }
+}
+// Data term and update of one column in the exact arithmetic, rounded as the compiler
+// contracts UpdateEpi of rsf_passes.cu.
+__device__ __forceinline__ float update_exact(float ph, float lap, float kap, float im, float K1, float Ka, float Kb,
+                                              float s2, const Coeffs &c, float &g) {
+    const float X = (c.lambda1 - c.lambda2) * K1, im2 = __fmul_rn(im, im);
+    g = s2 * (fmaf(X, im2, -__fmul_rn(2.f * im, Ka)) + Kb);
+    const float del = __fmul_rn(c.eps, INV_PI) / fmaf(ph, ph, __fmul_rn(c.eps, c.eps));
+    const float f = fmaf(c.nu, kap, -g);
+    return fmaf(c.dt, fmaf(c.mu, lap - kap, __fmul_rn(del, f)), ph);
+}
+// The small side of H with the sign of u (its zero too), by atanf and an IEEE division.
+__device__ __forceinline__ float heaviside_q_exact(float u, float eps) {
+    return copysignf(atanf(eps / fabsf(u)) * INV_PI, u);
+}
+
 // VEC: nx even and the image base aligned for two values, so that a thread's two
 // columns are both inside or both outside the brick and are read and written together.
 // DUMP: also write g, kappa and L of every output to B.dump (rsf_step_stages); a
 // separate instantiation keeps the iteration's kernel free of it.
-template <int R, class ImgT, bool VEC, bool DUMP>
+// EX: the exact arithmetic (IEEE divisions and square roots, atanf) on the centred FP32 image,
+// whose rows have q's pitch.
+template <int R, class ImgT, bool VEC, bool DUMP, bool EX>
 __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B, int bi, const TapPairs &t) {
-    using Z = TBZ<R>;
+    using Z = TBZ<R, EX>;
     constexpr int TY = Z::TY, M = Z::M, PW = Z::PW, PPL = Z::PPL, NXP = Z::NXP, NYP = Z::NYP, NPL = Z::NPL;
     constexpr int T = 2 * R + 1;
     using Img2 = ImgPair<ImgT>;
@@ -1227,6 +1280,7 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
     const float inv_s = B.cs[1], nms = -B.cs[0] * B.cs[1];
     const float eps = B.eps, eps2 = eps * eps;
     const float nu = B.nu, dt_mu = B.dt * B.mu, dt_eps_pi = B.dt * (eps * INV_PI);
+    const Coeffs co{eps, l1, l2, nu, B.mu, B.dt};
     float *const dump = DUMP ? B.dump : nullptr;
     const long long n = (long long)plane * nz;
     const ImgT *const img = reinterpret_cast<const ImgT *>(B.img);
@@ -1276,7 +1330,7 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
     float2 lxy0 = f2v(0.f), kxy0 = f2v(0.f), nzm = f2v(0.f), nz0 = f2v(0.f);
     float2 acc[4][2];         // (K*a, K*b) of four planes and both columns,
     Img2 raw[4];              // their image values
-    float pzq[4];             // and p_z
+    float pzq[4];             // and p_z (two planes at each step instead: 7 % slower)
     unsigned out = out0;      // offset of the step's first output plane at this thread's columns,
     unsigned qout = (unsigned)z0 * qplane + (unsigned)min(y, ny - 1) * (unsigned)B.qp + (unsigned)min(x, nx - 1);  // and in q
 
@@ -1317,7 +1371,7 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
         if constexpr (OUT == 0) {  // used after the barrier
 #pragma unroll
             for (int s = 0; s < 4; ++s) {
-                raw[s] = img_at(in_c, r0 + s, out + s * plane);
+                raw[s] = img_at(in_c, r0 + s, EX ? qout + s * qplane : out + s * plane);
                 pzq[s] = pz_at(in_c, r0 + s);
             }
         }
@@ -1326,14 +1380,14 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
         {
             const float2 xp = make_float2(ph1.y, pA[si + 2]), xm = make_float2(pA[si - 1], ph1.x);
             const float2 yp = ld2(pA + si + PW), ym = ld2(pA + si - PW);
-            unit_normal2(f2sub(xp, xm), f2sub(yp, ym), f2sub(ph2, ph0), !IN && first_x(r0 + 1), nx1, ny1, nz1);
+            normal2<EX>(f2sub(xp, xm), f2sub(yp, ym), f2sub(ph2, ph0), !IN && first_x(r0 + 1), nx1, ny1, nz1);
             const float2 m2 = f2mul(f2v(-2.f), ph1);
             lxy1 = f2add(f2add(f2add(xp, xm), m2), f2add(f2add(yp, ym), m2));
         }
         {
             const float2 xp = make_float2(ph2.y, pB[si + 2]), xm = make_float2(pB[si - 1], ph2.x);
             const float2 yp = ld2(pB + si + PW), ym = ld2(pB + si - PW);
-            unit_normal2(f2sub(xp, xm), f2sub(yp, ym), f2sub(ph3, ph1), !IN && first_x(r0 + 2), nx2, ny2, nz2);
+            normal2<EX>(f2sub(xp, xm), f2sub(yp, ym), f2sub(ph3, ph1), !IN && first_x(r0 + 2), nx2, ny2, nz2);
             const float2 m2 = f2mul(f2v(-2.f), ph2);
             lxy2 = f2add(f2add(f2add(xp, xm), m2), f2add(f2add(yp, ym), m2));
         }
@@ -1348,9 +1402,9 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
                 const float2 gy = f2sub(make_float2(pA[ss + PW], pB[ss + PW]), make_float2(pA[ss - PW], pB[ss - PW]));
                 const float2 gz = f2sub(make_float2(st2, st3), make_float2(st0, st1));
                 float2 a, b, d;
-                unit_normal2(gx, gy, gz, !IN && first_x(r0 + 1), a, b, d);
+                normal2<EX>(gx, gy, gz, !IN && first_x(r0 + 1), a, b, d);
                 nA[sni] = a.x;
-                if (!IN) unit_normal2(gx, gy, gz, first_x(r0 + 2), a, b, d);
+                if (!IN && !EX) unit_normal2(gx, gy, gz, first_x(r0 + 2), a, b, d);
                 nB[sni] = a.y;
             }
             st0 = st2;
@@ -1406,23 +1460,31 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
                 for (int s = 0; s < 2; ++s) {
                     if (!IN && s == 1 && r0 + 1 >= nout) break;
                     const float2 a0 = acc[2 * OUT + s][0], a1 = acc[2 * OUT + s][1];
-                    const float2 im = f2fma(raw[2 * OUT + s].template get<VEC>(), f2v(inv_s), f2v(nms));
-                    float2 g;
-                    if constexpr (R == 0) {  // Eq. (15), sigma_2 = 0: (a, b) are the fits (f1, f2)
-                        const float2 d1 = f2sub(im, make_float2(a0.x, a1.x)), d2 = f2sub(im, make_float2(a0.y, a1.y));
-                        g = f2fma(f2v(s2l1), f2mul(d1, d1), f2mul(f2v(-s2l2), f2mul(d2, d2)));
-                    } else {  // Li's data terms from K*a, K*b: s^2 [(l1 - l2) K1 I~^2 - 2 I~ K*a + K*b]
-                        const float2 t1 = f2mul(f2mul(cK, f2v(pzq[2 * OUT + s])), f2mul(im, im));
-                        const float2 t2 = f2fma(f2mul(f2v(m2s2), im), make_float2(a0.x, a1.x), t1);
-                        g = f2fma(f2v(s2), make_float2(a0.y, a1.y), t2);
+                    float2 g, pn, qn;
+                    if constexpr (EX) {
+                        const float2 im = raw[2 * OUT + s].template get<VEC>();
+                        const float pz = pzq[2 * OUT + s];
+                        pn.x = update_exact(ph[s].x, lap[s].x, kap[s].x, im.x, pxy.x * pz, a0.x, a0.y, s2, co, g.x);
+                        pn.y = update_exact(ph[s].y, lap[s].y, kap[s].y, im.y, pxy.y * pz, a1.x, a1.y, s2, co, g.y);
+                        qn = make_float2(heaviside_q_exact(pn.x, eps), heaviside_q_exact(pn.y, eps));
+                    } else {
+                        const float2 im = f2fma(raw[2 * OUT + s].template get<VEC>(), f2v(inv_s), f2v(nms));
+                        if constexpr (R == 0) {  // Eq. (15), sigma_2 = 0: (a, b) are the fits (f1, f2)
+                            const float2 d1 = f2sub(im, make_float2(a0.x, a1.x)), d2 = f2sub(im, make_float2(a0.y, a1.y));
+                            g = f2fma(f2v(s2l1), f2mul(d1, d1), f2mul(f2v(-s2l2), f2mul(d2, d2)));
+                        } else {  // Li's data terms from K*a, K*b: s^2 [(l1 - l2) K1 I~^2 - 2 I~ K*a + K*b]
+                            const float2 t1 = f2mul(f2mul(cK, f2v(pzq[2 * OUT + s])), f2mul(im, im));
+                            const float2 t2 = f2fma(f2mul(f2v(m2s2), im), make_float2(a0.x, a1.x), t1);
+                            g = f2fma(f2v(s2), make_float2(a0.y, a1.y), t2);
+                        }
+                        const float2 den = f2fma(ph[s], ph[s], f2v(eps2));
+                        // dt delta (Eq. 14), then phi + dt mu (L - kappa) + dt delta (nu kappa - g) (Eqs. 1, 13)
+                        const float2 dtdel = f2mul(f2v(dt_eps_pi), make_float2(rcp_approx(den.x), rcp_approx(den.y)));
+                        pn =
+                            f2fma(f2v(dt_mu), f2sub(lap[s], kap[s]),
+                                  f2fma(dtdel, f2fma(f2v(nu), kap[s], make_float2(-g.x, -g.y)), ph[s]));
+                        qn = heaviside_q_fast2(pn, eps);
                     }
-                    const float2 den = f2fma(ph[s], ph[s], f2v(eps2));
-                    // dt delta (Eq. 14), then phi + dt mu (L - kappa) + dt delta (nu kappa - g) (Eqs. 1, 13)
-                    const float2 dtdel = f2mul(f2v(dt_eps_pi), make_float2(rcp_approx(den.x), rcp_approx(den.y)));
-                    const float2 pn =
-                        f2fma(f2v(dt_mu), f2sub(lap[s], kap[s]),
-                              f2fma(dtdel, f2fma(f2v(nu), kap[s], make_float2(-g.x, -g.y)), ph[s]));
-                    const float2 qn = heaviside_q_fast2(pn, eps);
                     const unsigned o = s ? o1 : o0, oq = s ? q1 : q0;
                     if constexpr (VEC) {
                         if (act0) {
@@ -1483,14 +1545,15 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
     cp_async_wait0();  // no copy into this CTA's shared memory outlives it
 }
 
-template <int R, class ImgT, bool DUMP = false>
-__global__ void __launch_bounds__(TBZ<R>::THREADS, 2) k_tb_z(GroupArgs G, TapPairs t) {
+template <int R, class ImgT, bool DUMP = false, bool EX = false>
+__global__ void __launch_bounds__((TBZ<R, EX>::THREADS), 2) k_tb_z(GroupArgs G, TapPairs t) {
     const int bi = find_brick(G.starts, G.nb, blockIdx.x);
     const BrickDev &B = G.bricks[bi];
-    if (B.nx % 2 == 0 && reinterpret_cast<uintptr_t>(B.img) % (2 * sizeof(ImgT)) == 0)
-        tb_z_march<R, ImgT, true, DUMP>(G, B, bi, t);
+    const uintptr_t at = reinterpret_cast<uintptr_t>(B.phi[0]) | reinterpret_cast<uintptr_t>(B.phi[1]);
+    if (B.nx % 2 == 0 && at % 8 == 0 && reinterpret_cast<uintptr_t>(B.img) % (2 * sizeof(ImgT)) == 0)
+        tb_z_march<R, ImgT, true, DUMP, EX>(G, B, bi, t);
     else
-        tb_z_march<R, ImgT, false, DUMP>(G, B, bi, t);
+        tb_z_march<R, ImgT, false, DUMP, EX>(G, B, bi, t);
 }
 
 // ------------------------------------------------------------ launchers
@@ -1507,7 +1570,7 @@ int &az_persist() {
 }
 
 template <int R, class ImgT, int NP>
-constexpr size_t taxy_smem() { return XYSmem<R, SrcH<R, ImgT, NP>>::bytes; }
+constexpr size_t taxy_smem() { return XYSmem<R, SrcH<R, ImgT, NP, false>>::bytes; }
 template <int R, class S>
 constexpr size_t tbxy_smem() { return XYSmem<R, SrcAB<R, S>>::bytes; }
 

@@ -11,17 +11,29 @@ namespace tiled {
 
 namespace {
 // q of phi; rows of nx values at a pitch of qp (one row of n values when they are dense)
+template <bool EX>
 __global__ void k_q_init(const float *__restrict__ phi, float *__restrict__ q, long long rows, long long nx,
                          long long qp, float eps) {
+    const auto q_of = [&](float u) { return EX ? heaviside_q_exact(u, eps) : heaviside_q_fast(u, eps); };
     if (rows == 1) {
         for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nx; i += (long long)gridDim.x * blockDim.x)
-            q[i] = heaviside_q_fast(__ldg(phi + i), eps);
+            q[i] = q_of(__ldg(phi + i));
         return;
     }
     const int lane = threadIdx.x & 31;
     for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
          r += ((long long)gridDim.x * blockDim.x) >> 5)
-        for (int x = lane; x < nx; x += 32) q[r * qp + x] = heaviside_q_fast(__ldg(phi + r * nx + x), eps);
+        for (int x = lane; x < nx; x += 32) q[r * qp + x] = q_of(__ldg(phi + r * nx + x));
+}
+// the centred image (I - m) / s, rows of nx values at a pitch of ip
+template <class T>
+__global__ void k_center_rows(const T *__restrict__ vol, const float *__restrict__ cs, float *__restrict__ dst,
+                              long long rows, int nx, int ip) {
+    const float m = cs[0], inv_s = cs[1];
+    const int lane = threadIdx.x & 31;
+    for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
+         r += ((long long)gridDim.x * blockDim.x) >> 5)
+        for (int x = lane; x < nx; x += 32) dst[r * ip + x] = ((float)vol[r * nx + x] - m) * inv_s;
 }
 // rows of nx values copied to a pitch of ip
 template <class T>
@@ -125,19 +137,27 @@ struct XYBoxes { int rows, q, img, ab32, ab16; };
 template <int R>
 XYBoxes xy_boxes_r(int imgtype) {
     using namespace tiled;
-    const int img = imgtype == 0 ? SrcH<R, uint8_t, 1>::FI::W : (imgtype == 1 ? SrcH<R, uint16_t, 1>::FI::W : SrcH<R, float, 1>::FI::W);
-    return XYBoxes{XYG<R>::H, SrcH<R, float, 1>::FQ::W, img, SrcAB<R, float>::FA::W, SrcAB<R, __half>::FA::W};
+    const int img = imgtype == 0 ? SrcH<R, uint8_t, 1, false>::FI::W : (imgtype == 1 ? SrcH<R, uint16_t, 1, false>::FI::W : SrcH<R, float, 1, false>::FI::W);
+    return XYBoxes{XYG<R>::H, SrcH<R, float, 1, false>::FQ::W, img, SrcAB<R, float>::FA::W, SrcAB<R, __half>::FA::W};
 }
 XYBoxes xy_boxes(int R, int imgtype) {
     switch (R) {
+        case 1: return xy_boxes_r<1>(imgtype);
         case 2: return xy_boxes_r<2>(imgtype);
         case 3: return xy_boxes_r<3>(imgtype);
         case 4: return xy_boxes_r<4>(imgtype);
         case 5: return xy_boxes_r<5>(imgtype);
         case 6: return xy_boxes_r<6>(imgtype);
+        case 7: return xy_boxes_r<7>(imgtype);
         case 8: return xy_boxes_r<8>(imgtype);
+        case 9: return xy_boxes_r<9>(imgtype);
         case 10: return xy_boxes_r<10>(imgtype);
-        default: return xy_boxes_r<12>(imgtype);
+        case 11: return xy_boxes_r<11>(imgtype);
+        case 12: return xy_boxes_r<12>(imgtype);
+        case 13: return xy_boxes_r<13>(imgtype);
+        case 14: return xy_boxes_r<14>(imgtype);
+        case 15: return xy_boxes_r<15>(imgtype);
+        default: return xy_boxes_r<16>(imgtype);
     }
 }
 }  // namespace
@@ -154,8 +174,11 @@ cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, 
         default: e = encode_typed(&b.tm_img, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, b.img_t, 1, b.ip, b, box.img, box.rows, 1);
     }
     if (e != cudaSuccess) return e;
-    if (force == 1)  // the Eq. (15) form: four fields per voxel, no K*I~, no group B
-        return encode_map(&b.tm_u, b.u2, 4, b, 128, 1, zrows);
+    if (force != 0) {  // four fields per voxel, no K*I~; the Eq. (15) form: no group B
+        e = encode_map(&b.tm_u, b.u2, 4, b, 128, 1, zrows);
+        if (e != cudaSuccess || force == 1) return e;
+        return encode_map(&b.tm_ab, b.ab, 2, b, 2 * box.ab32, box.rows, 1);
+    }
     e = encode_map(&b.tm_u, b.u2, 2, b, 64, 1, zrows);
     if (e == cudaSuccess) e = encode_map(&b.tm_k, b.ki, 1, b, 32, 1, tiled::kAZT);
     if (e != cudaSuccess) return e;
@@ -175,7 +198,20 @@ cudaError_t tiled_start(const BrickDev &b, int imgtype, cudaStream_t s) {
         }
     }
     const bool dense = b.qp == b.nx;
-    tiled::k_q_init<<<1216, 256, 0, s>>>(b.phi[0], b.q, dense ? 1 : rows, dense ? rows * b.nx : b.nx, b.qp, b.eps);
+    tiled::k_q_init<false><<<1216, 256, 0, s>>>(b.phi[0], b.q, dense ? 1 : rows, dense ? rows * b.nx : b.nx, b.qp, b.eps);
+    return cudaGetLastError();
+}
+
+cudaError_t exact_start(const BrickDev &b, const void *vol, int vt, cudaStream_t s) {
+    const long long rows = (long long)b.ny * b.nz;
+    float *d = static_cast<float *>(const_cast<void *>(b.img));
+    const unsigned grid = (unsigned)(rows < 8 * 1216 ? (rows + 7) / 8 : 1216);
+    switch (vt) {
+        case 0: tiled::k_center_rows<<<grid, 256, 0, s>>>((const uint8_t *)vol, b.cs, d, rows, b.nx, b.ip); break;
+        case 1: tiled::k_center_rows<<<grid, 256, 0, s>>>((const uint16_t *)vol, b.cs, d, rows, b.nx, b.ip); break;
+        default: tiled::k_center_rows<<<grid, 256, 0, s>>>((const float *)vol, b.cs, d, rows, b.nx, b.ip);
+    }
+    tiled::k_q_init<true><<<grid, 256, 0, s>>>(b.phi[0], b.q, rows, b.nx, b.qp, b.eps);
     return cudaGetLastError();
 }
 
@@ -185,9 +221,21 @@ cudaError_t tiled_prepare_f16(int R);
 cudaError_t tiled_prepare_bf16(int R);
 
 cudaError_t tiled_prepare_eq15(int R);
+namespace tiled {  // the exact arithmetic, four radii per translation unit (rsf_exact_r*.cu)
+cudaError_t prepare_exact_r1(int R);
+cudaError_t prepare_exact_r5(int R);
+cudaError_t prepare_exact_r9(int R);
+cudaError_t prepare_exact_r13(int R);
+cudaError_t launch_exact_r1(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+cudaError_t launch_exact_r5(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+cudaError_t launch_exact_r9(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+cudaError_t launch_exact_r13(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+}  // namespace tiled
 cudaError_t tiled_launch_eq15(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
 
 cudaError_t tiled_prepare(int storage, int R, int force) {
+    if (force == kForceExact)
+        return R <= 4 ? tiled::prepare_exact_r1(R) : (R <= 8 ? tiled::prepare_exact_r5(R) : (R <= 12 ? tiled::prepare_exact_r9(R) : tiled::prepare_exact_r13(R)));
     const cudaError_t e = tiled::prepare_tb_z(force ? 0 : R);
     if (e != cudaSuccess) return e;
     if (force) return tiled_prepare_eq15(R);  // FP32 intermediates whatever the storage option
@@ -200,6 +248,9 @@ cudaError_t tiled_prepare(int storage, int R, int force) {
 }
 
 cudaError_t tiled_iterate(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s) {
+    const int R = g.taps.R;
+    if (g.force == kForceExact)
+        return R <= 4 ? tiled::launch_exact_r1(g, parity, prof, s) : (R <= 8 ? tiled::launch_exact_r5(g, parity, prof, s) : (R <= 12 ? tiled::launch_exact_r9(g, parity, prof, s) : tiled::launch_exact_r13(g, parity, prof, s)));
     if (g.force) return tiled_launch_eq15(g, parity, prof, s);
     switch (g.storage) {
         case 0: return tiled::launch_group_s<float>(g, parity, prof, s);
@@ -213,27 +264,40 @@ namespace {
 // Tile rows and (a, b) ring planes of the update kernel for radius R (0: the Eq. (15) form).
 struct UpdateTile { int rows, planes; };
 template <int R>
-UpdateTile update_tile_r() { return UpdateTile{tiled::TBZ<R>::TY, tiled::TBZ<R>::M}; }
-UpdateTile update_tile(int R) {
-    switch (R) {
-        case 0: return update_tile_r<0>();
-        case 2: return update_tile_r<2>();
-        case 3: return update_tile_r<3>();
-        case 4: return update_tile_r<4>();
-        case 5: return update_tile_r<5>();
-        case 6: return update_tile_r<6>();
-        case 8: return update_tile_r<8>();
-        case 10: return update_tile_r<10>();
-        default: return update_tile_r<12>();
+UpdateTile update_tile_r(bool exact) {
+    return exact ? UpdateTile{tiled::TBZ<R, true>::TY, tiled::TBZ<R, true>::M} : UpdateTile{tiled::TBZ<R>::TY, tiled::TBZ<R>::M};
+}
+UpdateTile update_tile(int force, int R) {
+    const bool exact = force == kForceExact;
+    switch (force == 1 ? 0 : R) {
+        case 0: return update_tile_r<0>(exact);
+        case 1: return update_tile_r<1>(exact);
+        case 2: return update_tile_r<2>(exact);
+        case 3: return update_tile_r<3>(exact);
+        case 4: return update_tile_r<4>(exact);
+        case 5: return update_tile_r<5>(exact);
+        case 6: return update_tile_r<6>(exact);
+        case 7: return update_tile_r<7>(exact);
+        case 8: return update_tile_r<8>(exact);
+        case 9: return update_tile_r<9>(exact);
+        case 10: return update_tile_r<10>(exact);
+        case 11: return update_tile_r<11>(exact);
+        case 12: return update_tile_r<12>(exact);
+        case 13: return update_tile_r<13>(exact);
+        case 14: return update_tile_r<14>(exact);
+        case 15: return update_tile_r<15>(exact);
+        default: return update_tile_r<16>(exact);
     }
 }
+// Output rows of the x/y kernels' tiles.
+int xy_rows(int R) { return R <= 8 ? tiled::XYG<8>::TH : (R <= 12 ? tiled::XYG<12>::TH : tiled::XYG<16>::TH); }
 }  // namespace
 
 void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]) {
-    const unsigned th = R <= 8 ? tiled::XYG<8>::TH : tiled::XYG<12>::TH;
+    const unsigned th = xy_rows(R);
     const unsigned ntx = (b.nx + tiled::kXYT - 1) / tiled::kXYT, nty = (b.ny + th - 1) / th;
     const unsigned nzp = (b.nz + b.xyp - 1) / b.xyp;
-    const int rows = update_tile(force ? 0 : R).rows;
+    const int rows = update_tile(force, R).rows;
     counts[0] = ntx * nty * nzp;
     counts[1] = (unsigned)((b.nz + tiled::kAZT - 1) / tiled::kAZT) * ((b.nx + 31) / 32) * b.ny;
     counts[2] = counts[0];
@@ -246,7 +310,7 @@ void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]) {
 // 0.480 ms, so 16 is the most); three or four share an SM.  Few CTAs run in whole waves; many even out but for
 // about half a CTA at the end.
 int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int sms) {
-    const int th = R <= 8 ? tiled::XYG<8>::TH : tiled::XYG<12>::TH;
+    const int th = xy_rows(R);
     const double slots = (force ? 3.0 : 4.0) * sms;
     int best = 1;
     double best_cost = 0.0;
@@ -269,7 +333,7 @@ int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int s
 // first copies).  Two CTAs share an SM.  Few CTAs run in whole waves; many even out but for
 // about half a CTA at the end.
 int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, int zc, int sms) {
-    const UpdateTile tile = update_tile(force ? 0 : R);
+    const UpdateTile tile = update_tile(force, R);
     const double fill = 4.0 + 0.4 * tile.planes, slots = 2.0 * sms;
     int best = zc, last = 0;
     double best_cost = 0.0;
@@ -324,6 +388,25 @@ size_t tiled_extra_bytes(const void *img, int nx, int ny, int nz, int imgtype, i
     if (field_bytes(storage, force, np) + need <= tiled_stage_bytes(storage, np)) return 0;
     return 4ull * q_pitch(nx) * rows + need <= 8ull * nx * rows ? 0 : need;
 }
+
+// Per pitched voxel: both x/y-convolved pairs 16 bytes (then, in the same memory, the
+// x/y-convolved (a, b)), (a, b) 8, the centred image at most 4.
+void exact_place_fields(BrickDev &b, void *stage, float *q) {
+    b.px = tiled_pitch(b.nx);
+    const long long np = (long long)b.px * b.ny * b.nz;
+    char *p = static_cast<char *>(stage);
+    b.u2 = b.abxy = reinterpret_cast<float2 *>(p);
+    b.ab = p + 16 * np;
+    b.ki = nullptr;
+    b.img = b.img_t = p + 24 * np;
+    b.q = q;
+    b.qp = b.ip = q_pitch(b.nx);
+}
+size_t exact_stage_bytes(int nx, int ny, int nz) {
+    return (24ull * tiled_pitch(nx) + 4ull * q_pitch(nx)) * ny * nz;
+}
+size_t exact_q_bytes(int nx, int ny, int nz) { return 4ull * q_pitch(nx) * ny * nz; }
+bool exact_supports(int R) { return R >= 1 && R <= RMAX; }
 
 void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q,
                         void *extra) {

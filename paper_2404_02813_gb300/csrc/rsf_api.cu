@@ -154,6 +154,8 @@ rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, cons
         buf.cap_bricks = cap;
         buf.cap_starts = capst;
     }
+    int sms = 0;
+    RSF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
     std::vector<rsf::BrickDev> all;
     std::vector<int> starts;
     all.reserve(total);
@@ -189,6 +191,7 @@ rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, cons
             g.starts[k] = buf.d_starts + s0 + (size_t)k * (nb + 1);
             g.ncta[k] = (unsigned)tot[k];
         }
+        g.overlap = rsf::tiled_overlap(g, sms);
         for (rsf::BrickDev b : gs.bricks) {
             const cudaError_t e = rsf::tiled_encode_maps(b, gs.force, gs.storage, gs.imgtype, gs.taps.R);
             if (e != cudaSuccess) return fail(RSF_E_CUDA, "TMA descriptor of a %dx%dx%d brick: %s", b.nx, b.ny, b.nz,

@@ -26,16 +26,11 @@ int &exact_persist() {
 template <int R>
 cudaError_t prepare_exact_r() {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_ta_xy<R, float, 2, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)exact_taxy_smem<R>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_ta_z4<R, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)az4_smem<R>())) !=
-        cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_tb_xy<R, float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)tbxy_smem<R, float>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_tb_z<R, float, false, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)TBZ<R, true>::bytes)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_tb_z<R, float, true, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)TBZ<R, true>::bytes)) != cudaSuccess) return e;
+    if ((e = prepare_kernel(k_ta_xy<R, float, 2, true>, exact_taxy_smem<R>())) != cudaSuccess) return e;
+    if ((e = prepare_kernel(k_ta_z4<R, true>, az4_smem<R>())) != cudaSuccess) return e;
+    if ((e = prepare_kernel(k_tb_xy<R, float>, tbxy_smem<R, float>())) != cudaSuccess) return e;
+    if ((e = prepare_kernel(k_tb_z<R, float, false, true>, TBZ<R, true>::bytes)) != cudaSuccess) return e;
+    if ((e = prepare_kernel(k_tb_z<R, float, true, true>, TBZ<R, true>::bytes)) != cudaSuccess) return e;
     int dev = 0, sms = 0, occ = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -52,26 +47,26 @@ cudaError_t launch_exact_r(const TiledGroup &g, int parity, Profiler *prof, cuda
     {
         ProfScope ps(prof, KID_TA_XY);
         G.starts = g.starts[0];
-        k_ta_xy<R, float, 2, true><<<g.ncta[0], kXYThreads, exact_taxy_smem<R>(), s>>>(G, tp);
+        launch_next(g.overlap, k_ta_xy<R, float, 2, true>, g.ncta[0], kXYThreads, exact_taxy_smem<R>(), s, G, tp);
     }
     {
         ProfScope ps(prof, KID_TA_Z);
         G.starts = g.starts[1];
         const unsigned grid = g.ncta[1] < (unsigned)exact_persist<R>() ? g.ncta[1] : (unsigned)exact_persist<R>();
-        k_ta_z4<R, true><<<grid, kAZThreads, az4_smem<R>(), s>>>(G, tp);
+        launch_next(g.overlap, k_ta_z4<R, true>, grid, kAZThreads, az4_smem<R>(), s, G, tp);
     }
     {
         ProfScope ps(prof, KID_TB_XY);
         G.starts = g.starts[2];
-        k_tb_xy<R, float><<<g.ncta[2], kXYThreads, tbxy_smem<R, float>(), s>>>(G, tp);
+        launch_next(g.overlap, k_tb_xy<R, float>, g.ncta[2], kXYThreads, tbxy_smem<R, float>(), s, G, tp);
     }
     {
         ProfScope ps(prof, KID_TB_Z);
         G.starts = g.starts[3];
         if (g.dump)
-            k_tb_z<R, float, true, true><<<g.ncta[3], TBZ<R, true>::THREADS, TBZ<R, true>::bytes, s>>>(G, tp);
+            launch_next(g.overlap, k_tb_z<R, float, true, true>, g.ncta[3], TBZ<R, true>::THREADS, TBZ<R, true>::bytes, s, G, tp);
         else
-            k_tb_z<R, float, false, true><<<g.ncta[3], TBZ<R, true>::THREADS, TBZ<R, true>::bytes, s>>>(G, tp);
+            launch_next(g.overlap, k_tb_z<R, float, false, true>, g.ncta[3], TBZ<R, true>::THREADS, TBZ<R, true>::bytes, s, G, tp);
     }
     return cudaGetLastError();
 }

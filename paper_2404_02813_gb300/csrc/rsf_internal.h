@@ -132,6 +132,7 @@ struct TiledGroup {
     const int *starts[4];   // device: per kernel, nb + 1 CTA offsets
     unsigned ncta[4];       // CTAs per kernel launch
     int dump;               // 1: some brick has a stage dump (its update kernel writes g, kappa, L)
+    bool overlap;           // its kernels may start before the one before has ended (tiled_overlap)
     int *err;               // device-visible error word of the kernels' bounded waits (nonzero: expired)
     unsigned fault_tx;      // bytes the TMA barriers expect beyond their copies (0; > 0 in a fault test)
 };
@@ -153,6 +154,8 @@ int tiled_pitch(int nx);
 cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, int R);
 cudaError_t tiled_prepare(int storage, int R, int force);
 cudaError_t tiled_iterate(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s);
+// Whether a group's consecutive kernels overlap at their boundary (programmatic dependent launch).
+bool tiled_overlap(const TiledGroup &g, int sms);
 // CTAs of the four kernels for one brick of a group of the given form and radius.
 void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]);
 // Planes per CTA of the x/y kernels for bricks launched together (results do not depend on it).

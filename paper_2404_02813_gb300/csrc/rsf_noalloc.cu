@@ -138,6 +138,7 @@ cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Ta
     g.taps = taps;
     g.nb = 1;
     rsf::tiled_cta_counts(b, g.force, taps.R, g.ncta);
+    g.overlap = rsf::tiled_overlap(g, sms);
     struct {
         rsf::BrickDev b;
         int starts[8];

@@ -204,6 +204,33 @@ __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, i
         "l"(reinterpret_cast<uint64_t>(map)), "r"(x), "r"(y), "r"(z), "r"(smem_addr(bar))
         : "memory");
 }
+// Programmatic dependent launch: every kernel of an iteration lets the next one start as
+// soon as all of its CTAs have (dependents_may_start, first thing), and waits for the
+// completion of the one before, its writes included, before it reads or writes a field
+// (wait_for_previous, every thread).  What comes before that -- finding the brick, offsets,
+// barriers -- overlaps the previous kernel's end; only descriptors and constants written
+// before the first iteration are read there.
+__device__ __forceinline__ void dependents_may_start() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void wait_for_previous() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+template <class K>
+cudaError_t prepare_kernel(K *kernel, size_t smem) {
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+}
+template <class... P, class... A>
+void launch_next(bool overlap, void (*kernel)(P...), unsigned grid, unsigned threads, size_t smem, cudaStream_t s,
+                 A... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = overlap ? 1 : 0;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, P(args)...);  // an error stays for cudaGetLastError
+}
 // records an error in the group's error word (mapped host memory), once per CTA
 __device__ __forceinline__ void report_error(int *err, int code) {
     if (err && threadIdx.x == 0) {
@@ -455,6 +482,7 @@ __device__ __forceinline__ void xy_tile(const GroupArgs &G, const Src &src, cons
         mbar_init_fence();
     }
     __syncthreads();
+    wait_for_previous();
     if (threadIdx.x == 0) {
         src.fence();
         for (int i = 0; i < NS && za + i < zb_end; ++i) src.issue(sm + i * Src::BYTES, x0, y0, za + i, bar + i, G.fault_tx);
@@ -572,6 +600,7 @@ __device__ __forceinline__ XYTile xy_tile_of(int local, const BrickDev &B) {
 template <int R, class ImgT, int NP, bool EX = false>
 __global__ void __launch_bounds__(kXYThreads, (SrcH<R, ImgT, NP, EX>::CTAS)) k_ta_xy(GroupArgs G, TapPairs t) {
     extern __shared__ __align__(128) unsigned char xsm[];
+    dependents_may_start();
     const int b = find_brick(G.starts, G.nb, blockIdx.x);
     const BrickDev &B = G.bricks[b];
     const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
@@ -584,6 +613,7 @@ __global__ void __launch_bounds__(kXYThreads, (SrcH<R, ImgT, NP, EX>::CTAS)) k_t
 template <int R, class S>
 __global__ void __launch_bounds__(kXYThreads, (SrcAB<R, S>::CTAS)) k_tb_xy(GroupArgs G, TapPairs t) {
     extern __shared__ __align__(128) unsigned char xsm[];
+    dependents_may_start();
     const int b = find_brick(G.starts, G.nb, blockIdx.x);
     const BrickDev &B = G.bricks[b];
     const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
@@ -667,6 +697,7 @@ __device__ __forceinline__ void az_walk(const GroupArgs &G, unsigned char *smem,
         report_error(G.err, kErrSmemAlign);
         return;
     }
+    dependents_may_start();
     const int total = __ldg(G.starts + G.nb);
     if (threadIdx.x == 0) {
         mbar_init(bars, 1);
@@ -674,6 +705,7 @@ __device__ __forceinline__ void az_walk(const GroupArgs &G, unsigned char *smem,
         mbar_init_fence();
     }
     __syncthreads();
+    wait_for_previous();
     unsigned phase = 0u, pending = 0u;  // bit s: parity of stage s's next phase; stage s awaits copies
     AZSlabId next{};
     int last_b = -1;  // thread 0: the brick whose maps it fenced last
@@ -1313,6 +1345,7 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
     const int nyu = y == 0 ? nyi + NYP : nyi - NYP, nyd = y == ny - 1 ? nyi - NYP : nyi + NYP;
     const int sni = (srow + 1) * NXP + (side ? kZX + 2 : 1);  // the column site's n_x
 
+    wait_for_previous();
     // prologue: phi planes -2 .. 5; (a, b) planes -R .. M - R - 1
     using Edge = std::integral_constant<bool, false>;
     using Inner = std::integral_constant<bool, true>;
@@ -1547,6 +1580,7 @@ __device__ __forceinline__ void tb_z_march(const GroupArgs &G, const BrickDev &B
 
 template <int R, class ImgT, bool DUMP = false, bool EX = false>
 __global__ void __launch_bounds__((TBZ<R, EX>::THREADS), 2) k_tb_z(GroupArgs G, TapPairs t) {
+    dependents_may_start();
     const int bi = find_brick(G.starts, G.nb, blockIdx.x);
     const BrickDev &B = G.bricks[bi];
     const uintptr_t at = reinterpret_cast<uintptr_t>(B.phi[0]) | reinterpret_cast<uintptr_t>(B.phi[1]);
@@ -1578,19 +1612,16 @@ constexpr size_t tbxy_smem() { return XYSmem<R, SrcAB<R, S>>::bytes; }
 template <int R, int NP>
 cudaError_t prepare_ta_xy() {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_ta_xy<R, uint8_t, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)taxy_smem<R, uint8_t, NP>())) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_ta_xy<R, uint16_t, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                  (int)taxy_smem<R, uint16_t, NP>())) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_ta_xy<R, float, NP>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                (int)taxy_smem<R, float, NP>());
+    if ((e = prepare_kernel(k_ta_xy<R, uint8_t, NP>, taxy_smem<R, uint8_t, NP>())) != cudaSuccess) return e;
+    if ((e = prepare_kernel(k_ta_xy<R, uint16_t, NP>, taxy_smem<R, uint16_t, NP>())) != cudaSuccess) return e;
+    return prepare_kernel(k_ta_xy<R, float, NP>, taxy_smem<R, float, NP>());
 }
 template <int R, int NP>
 void launch_ta_xy(const TiledGroup &g, const GroupArgs &G, const TapPairs &tp, cudaStream_t s) {
     switch (g.imgtype) {
-        case 0: k_ta_xy<R, uint8_t, NP><<<g.ncta[0], kXYThreads, taxy_smem<R, uint8_t, NP>(), s>>>(G, tp); break;
-        case 1: k_ta_xy<R, uint16_t, NP><<<g.ncta[0], kXYThreads, taxy_smem<R, uint16_t, NP>(), s>>>(G, tp); break;
-        default: k_ta_xy<R, float, NP><<<g.ncta[0], kXYThreads, taxy_smem<R, float, NP>(), s>>>(G, tp);
+        case 0: launch_next(g.overlap, k_ta_xy<R, uint8_t, NP>, g.ncta[0], kXYThreads, taxy_smem<R, uint8_t, NP>(), s, G, tp); break;
+        case 1: launch_next(g.overlap, k_ta_xy<R, uint16_t, NP>, g.ncta[0], kXYThreads, taxy_smem<R, uint16_t, NP>(), s, G, tp); break;
+        default: launch_next(g.overlap, k_ta_xy<R, float, NP>, g.ncta[0], kXYThreads, taxy_smem<R, float, NP>(), s, G, tp);
     }
 }
 
@@ -1598,8 +1629,7 @@ template <int R, class S>
 cudaError_t prepare_storage() {
     cudaError_t e;
     if ((e = prepare_ta_xy<R, 1>()) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_ta_z<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)az_smem<R>())) !=
-        cudaSuccess) return e;
+    if ((e = prepare_kernel(k_ta_z<R, S>, az_smem<R>())) != cudaSuccess) return e;
     {
         int dev = 0, sms = 0, occ = 0;
         if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
@@ -1608,7 +1638,7 @@ cudaError_t prepare_storage() {
             cudaSuccess) return e;
         az_persist<R, S>() = sms * (occ > 0 ? occ : 1);
     }
-    return cudaFuncSetAttribute(k_tb_xy<R, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tbxy_smem<R, S>());
+    return prepare_kernel(k_tb_xy<R, S>, tbxy_smem<R, S>());
 }
 
 // One iteration of Li's form (group A, group B, update) for radius R and storage S.
@@ -1625,12 +1655,12 @@ cudaError_t launch_storage(const TiledGroup &g, int parity, Profiler *prof, cuda
         ProfScope ps(prof, KID_TA_Z);
         G.starts = g.starts[1];
         const unsigned grid = g.ncta[1] < (unsigned)az_persist<R, S>() ? g.ncta[1] : (unsigned)az_persist<R, S>();
-        k_ta_z<R, S><<<grid, kAZThreads, az_smem<R>(), s>>>(G, tp);
+        launch_next(g.overlap, k_ta_z<R, S>, grid, kAZThreads, az_smem<R>(), s, G, tp);
     }
     {
         ProfScope ps(prof, KID_TB_XY);
         G.starts = g.starts[2];
-        k_tb_xy<R, S><<<g.ncta[2], kXYThreads, tbxy_smem<R, S>(), s>>>(G, tp);
+        launch_next(g.overlap, k_tb_xy<R, S>, g.ncta[2], kXYThreads, tbxy_smem<R, S>(), s, G, tp);
     }
     cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

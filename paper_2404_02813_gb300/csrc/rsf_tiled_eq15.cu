@@ -22,8 +22,7 @@ template <int R>
 cudaError_t prepare_eq15_r() {
     cudaError_t e;
     if ((e = prepare_ta_xy<R, 2>()) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_ta_z4<R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)az4_smem<R>())) !=
-        cudaSuccess) return e;
+    if ((e = prepare_kernel(k_ta_z4<R>, az4_smem<R>())) != cudaSuccess) return e;
     int dev = 0, sms = 0, occ = 0;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
@@ -46,7 +45,7 @@ cudaError_t launch_eq15_r(const TiledGroup &g, int parity, Profiler *prof, cudaS
         ProfScope ps(prof, KID_TA_Z);
         G.starts = g.starts[1];
         const unsigned grid = g.ncta[1] < (unsigned)az4_persist<R>() ? g.ncta[1] : (unsigned)az4_persist<R>();
-        k_ta_z4<R><<<grid, kAZThreads, az4_smem<R>(), s>>>(G, tp);
+        launch_next(g.overlap, k_ta_z4<R>, grid, kAZThreads, az4_smem<R>(), s, G, tp);
     }
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return e;

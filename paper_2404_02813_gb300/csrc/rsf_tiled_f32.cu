@@ -305,6 +305,15 @@ void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]) {
                 ((b.nz + b.zc - 1) / b.zc) * ((b.zc + b.zs - 1) / b.zs);
 }
 
+// Overlapping consecutive kernels hides a launch's latency and start-up, which counts where the
+// kernels are short (64^3: 1.74 -> 1.25 ms for 50 iterations; 253 x 189 x 147: 2.05 -> 1.90 ms
+// for 12), and costs long ones more than that: an SM whose shared-memory carve-out an earlier
+// kernel set lower keeps it until it drains, and with the largest carve-out everywhere the L1
+// is too small (five iterations of 512^3: 11.3 ms without overlap, 12.2 with it, 11.6 with the
+// carve-out too; 160^3 sub-volumes, 2400 CTAs, 9.65, 10.0, 9.80 ms).  The line: two waves of
+// the x/y kernels.
+bool tiled_overlap(const TiledGroup &g, int sms) { return g.ncta[0] <= 8u * (unsigned)sms; }
+
 // A CTA of the x/y kernels costs its planes plus about one plane time (set-up and the first
 // copies; 64^3: 1 plane per CTA 8.1 us, 16 planes 37 us; 512^3: 16 planes 0.463 ms, 32 planes
 // 0.480 ms, so 16 is the most); three or four share an SM.  Few CTAs run in whole waves; many even out but for

@@ -19,17 +19,16 @@ cudaError_t launch_update_r(const TiledGroup &g, int parity, Profiler *prof, cud
         t.g[0] = 1.f;
     }
     if (g.dump)
-        k_tb_z<R, ImgT, true><<<g.ncta[3], TBZ<R>::THREADS, TBZ<R>::bytes, s>>>(G, tap_pairs(t));
+        launch_next(g.overlap, k_tb_z<R, ImgT, true>, g.ncta[3], TBZ<R>::THREADS, TBZ<R>::bytes, s, G, tap_pairs(t));
     else
-        k_tb_z<R, ImgT><<<g.ncta[3], TBZ<R>::THREADS, TBZ<R>::bytes, s>>>(G, tap_pairs(t));
+        launch_next(g.overlap, k_tb_z<R, ImgT>, g.ncta[3], TBZ<R>::THREADS, TBZ<R>::bytes, s, G, tap_pairs(t));
     return cudaGetLastError();
 }
 template <int R, class ImgT>
 cudaError_t prepare_update_r() {
-    const cudaError_t e = cudaFuncSetAttribute(k_tb_z<R, ImgT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                               (int)TBZ<R>::bytes);
+    const cudaError_t e = prepare_kernel(k_tb_z<R, ImgT, false>, TBZ<R>::bytes);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_tb_z<R, ImgT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)TBZ<R>::bytes);
+    return prepare_kernel(k_tb_z<R, ImgT, true>, TBZ<R>::bytes);
 }
 
 template <class ImgT>

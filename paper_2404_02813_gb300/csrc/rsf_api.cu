@@ -337,6 +337,19 @@ cudaError_t xfer(void *dst, const void *src, size_t bytes, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+bool in_place(const void *p, int dev) {
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+        cudaGetLastError();
+        return false;
+    }
+    return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
+}
+static bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+    const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
+    return a && b && x < y + nb && y < x + na;
+}
+
 // Device-resident copy of the volume (the caller's own pointer when it already is one).
 static rsf_status device_volume(rsf_ctx *c, const void *volume, rsf_dtype vt, long long n, const void **out) {
     if (on_device(volume)) {
@@ -439,6 +452,7 @@ extern "C" void rsf_destroy(rsf_ctx *c) {
         dev_free(c, c->staging, c->staging_cap);
         dev_free(c, c->dump, c->dump_cap);
         free_desc(c, c->desc);
+        dev_free(c, c->d_setup, sizeof(rsf::SetupBrick) * (size_t)c->cap_setup);
         dev_free(c, c->pool, c->pool_cap);
         c->prof.release();
         cudaStreamDestroy(c->stream);
@@ -501,7 +515,18 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         RSF_CUDA(cudaMemsetAsync(f.phi[1], 0xFF, sizeof(float) * n, c->stream));
         RSF_CUDA(cudaMemsetAsync(f.q, 0xFF, 2 * sizeof(float) * n, c->stream));
     }
-    RSF_CUDA(xfer(f.phi[0], phi0, sizeof(float) * n, c->stream));
+    const size_t fb = sizeof(float) * (size_t)n;
+    // In the tiled schedule the first iteration reads phi0 and the last writes phi_out where they
+    // are (a copy each way is 16 of the 72 bytes a voxel-iteration moves), unless a kernel would
+    // still read the memory it writes.
+    bool phi0_here = false, out_here = false;
+    if ((tiled || exact) && iters > 0) {
+        const size_t sb = dump ? RSF_NSTAGES * fb : 0;
+        phi0_here = in_place(phi0, c->device) && !overlap(phi0, fb, dump, sb) && !(iters == 1 && overlap(phi0, fb, phi_out, fb));
+        out_here = in_place(phi_out, c->device) && !overlap(phi_out, fb, vol, dtype_size(vt) * (size_t)n) &&
+                   !overlap(phi_out, fb, dump, sb);
+    }
+    if (!phi0_here) RSF_CUDA(xfer(f.phi[0], phi0, fb, c->stream));
     int cur = 0;
     if (tiled || exact) {
         const int form = exact ? rsf::kForceExact : force;
@@ -537,24 +562,27 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
             b.zs = rsf::tiled_update_planes({b}, form, taps.R, b.zc, sms);
         }
         b.dump = dump;  // only rsf_step_stages asks for stages, and it runs one iteration
-        std::vector<GroupSpec> specs(1);
-        specs[0].storage = storage;
-        specs[0].force = form;
-        specs[0].imgtype = exact ? (int)RSF_F32 : (int)vt;
-        specs[0].taps = taps;
-        specs[0].bricks.push_back(b);
+        GroupSpec spec;
+        spec.storage = storage;
+        spec.force = form;
+        spec.imgtype = exact ? (int)RSF_F32 : (int)vt;
+        spec.taps = taps;
+        spec.bricks.push_back(b);
+        std::vector<GroupSpec> specs(3, spec);  // the first iteration, those between, the last
+        if (phi0_here) specs[0].bricks[0].phi[0] = const_cast<float *>(phi0);
+        if (out_here) (iters == 1 ? specs[0] : specs[2]).bricks[0].phi[iters & 1] = phi_out;
+        b = specs[0].bricks[0];
         std::vector<rsf::TiledGroup> groups;
         if ((st = upload_groups(c, c->desc, c->stream, specs, &groups))) return st;
-        const rsf::TiledGroup &g = groups[0];
         if (iters > 0) {
             if (exact)
                 RSF_CUDA(rsf::exact_start(b, vol, (int)vt, c->stream));
             else
-                RSF_CUDA(rsf::tiled_start(b, (int)vt, c->stream));
-            RSF_CUDA(rsf::tiled_ki_init(b, (int)vt, taps, c->d_err, c->stream));
+                RSF_CUDA(rsf::tiled_start(b, (int)vt, b.phi[0], c->stream));
+            RSF_CUDA(rsf::tiled_ki_init(groups[0], c->stream));
         }
         for (int it = 0; it < iters; ++it) {
-            cudaError_t e = rsf::tiled_iterate(g, it & 1, &c->prof, c->stream);
+            cudaError_t e = rsf::tiled_iterate(groups[it == 0 ? 0 : (it == iters - 1 ? 2 : 1)], it & 1, &c->prof, c->stream);
             if (e != cudaSuccess) return cuda_fail(e, "iteration launch");
         }
         cur = iters & 1;
@@ -566,7 +594,7 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
             cur ^= 1;
         }
     }
-    RSF_CUDA(xfer(phi_out, f.phi[cur], sizeof(float) * n, c->stream));
+    if (!out_here) RSF_CUDA(xfer(phi_out, f.phi[cur], fb, c->stream));
     if (stages && dump != stages)
         RSF_CUDA(xfer(stages, dump, sizeof(float) * n * RSF_NSTAGES, c->stream));
     RSF_CUDA(cudaStreamSynchronize(c->stream));

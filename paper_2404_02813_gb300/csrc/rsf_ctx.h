@@ -51,6 +51,8 @@ struct rsf_ctx {
     int opt_storage = RSF_STORE_F32;
     int opt_force = RSF_FORCE_LI;
     DescBuffers desc;                   // brick descriptors of rsf_evolve / rsf_evolve_batch launches
+    rsf::SetupBrick *d_setup = nullptr; // set-up descriptions of rsf_evolve_batch's bricks
+    int cap_setup = 0;
     int opt_autotune = 0;
     int opt_graph = 1;
     void *pool = nullptr;               // per-brick fields of rsf_evolve_batch
@@ -89,6 +91,8 @@ rsf_status device_error(const rsf_ctx *c);
 rsf_status dev_alloc(rsf_ctx *c, void **p, size_t bytes);
 void dev_free(rsf_ctx *c, void *p, size_t bytes);
 bool on_device(const void *p);
+// Device memory of device `dev` (or managed memory), which its kernels may use in place.
+bool in_place(const void *p, int dev);
 // Copy `bytes` on stream s between any two of device, pinned host and pageable
 // host memory; pinned host memory is read or written by a copy kernel.
 cudaError_t xfer(void *dst, const void *src, size_t bytes, cudaStream_t s);

@@ -65,14 +65,32 @@ bool axis_table(int n, int edge, int curtain, const std::vector<int> &starts, Ax
     return true;
 }
 
+// Every sub-volume's image and phi0 in one launch: blockIdx.y is the sub-volume, a warp copies
+// rows (one element per thread with 64-bit divisions: 22 us per array of 160^3; 12 images and level
+// sets here: 90 us, the copy rate).
+struct GatherArgs {
+    const int *start[3];      // per axis (x, y, z): first voxel of each sub-volume
+    int nb[3], ext[3], n[3];  // sub-volumes, their extents and the volume's, per axis
+    int first;                // blockIdx.y = 0's sub-volume (a launch takes at most 32768)
+    char *box0;               // sub-volume id's image and phi at box0 + id * stride
+    size_t stride, phi_at;
+};
 template <class T>
-__global__ void k_gather(const T *__restrict__ src, T *__restrict__ dst, int nx, int ny, int x0, int y0, int z0,
-                         int bx, int by, long long n) {
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n; i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % bx);
-        const long long r = i / bx;
+__global__ void __launch_bounds__(256) k_gather(const T *__restrict__ vol, const float *__restrict__ phi0, GatherArgs a) {
+    const int id = a.first + blockIdx.y, kx = id % a.nb[0], ky = id / a.nb[0] % a.nb[1], kz = id / a.nb[0] / a.nb[1];
+    const int bx = a.ext[0], by = a.ext[1];
+    const long long rows = (long long)by * a.ext[2];
+    T *const img = reinterpret_cast<T *>(a.box0 + id * a.stride);
+    float *const phi = reinterpret_cast<float *>(a.box0 + id * a.stride + a.phi_at);
+    const int lane = threadIdx.x & 31;
+    for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
+         r += ((long long)gridDim.x * blockDim.x) >> 5) {
         const int y = (int)(r % by), z = (int)(r / by);
-        dst[i] = src[((long long)(z0 + z) * ny + (y0 + y)) * nx + x0 + x];
+        const long long src = ((long long)(a.start[2][kz] + z) * a.n[1] + a.start[1][ky] + y) * a.n[0] + a.start[0][kx];
+        for (int x = lane; x < bx; x += 32) {
+            img[r * bx + x] = vol[src + x];
+            phi[r * bx + x] = phi0[src + x];
+        }
     }
 }
 
@@ -84,32 +102,35 @@ struct MergeArgs {
     int n[3], nb[3];
 };
 
-__global__ void k_merge(MergeArgs a, float *__restrict__ out) {
-    const long long total = (long long)a.n[0] * a.n[1] * a.n[2];
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int x = (int)(i % a.n[0]);
-        const long long r = i / a.n[0];
+// A warp per output row: the y and z tables are read once per row.
+__global__ void __launch_bounds__(256) k_merge(MergeArgs a, float *__restrict__ out) {
+    const int nx = a.n[0], lane = threadIdx.x & 31;
+    const long long rows = (long long)a.n[1] * a.n[2];
+    for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
+         r += ((long long)gridDim.x * blockDim.x) >> 5) {
         const int y = (int)(r % a.n[1]), z = (int)(r / a.n[1]);
-        float num = 0.f, den = 0.f;
-        const int cz = a.count[2][z], cy = a.count[1][y], cx = a.count[0][x];
-        for (int iz = 0; iz < cz; ++iz) {
-            const int kz = a.box[2][z * kMaxCover + iz], lz = a.local[2][z * kMaxCover + iz];
-            const float wz = a.weight[2][z * kMaxCover + iz];
-            for (int iy = 0; iy < cy; ++iy) {
-                const int ky = a.box[1][y * kMaxCover + iy], ly = a.local[1][y * kMaxCover + iy];
-                const float wzy = wz * a.weight[1][y * kMaxCover + iy];
-                const int ey = a.ext[1][ky];
-                for (int ix = 0; ix < cx; ++ix) {
-                    const int kx = a.box[0][x * kMaxCover + ix], lx = a.local[0][x * kMaxCover + ix];
-                    const float w = wzy * a.weight[0][x * kMaxCover + ix];
-                    const float *p = a.phi[((long long)kz * a.nb[1] + ky) * a.nb[0] + kx];
-                    num = fmaf(w, p[((long long)lz * ey + ly) * a.ext[0][kx] + lx], num);
-                    den += w;
+        const int cz = a.count[2][z], cy = a.count[1][y];
+        for (int x = lane; x < nx; x += 32) {
+            float num = 0.f, den = 0.f;
+            const int cx = a.count[0][x];
+            for (int iz = 0; iz < cz; ++iz) {
+                const int kz = a.box[2][z * kMaxCover + iz], lz = a.local[2][z * kMaxCover + iz];
+                const float wz = a.weight[2][z * kMaxCover + iz];
+                for (int iy = 0; iy < cy; ++iy) {
+                    const int ky = a.box[1][y * kMaxCover + iy], ly = a.local[1][y * kMaxCover + iy];
+                    const float wzy = wz * a.weight[1][y * kMaxCover + iy];
+                    const int ey = a.ext[1][ky];
+                    for (int ix = 0; ix < cx; ++ix) {
+                        const int kx = a.box[0][x * kMaxCover + ix], lx = a.local[0][x * kMaxCover + ix];
+                        const float w = wzy * a.weight[0][x * kMaxCover + ix];
+                        const float *p = a.phi[((long long)kz * a.nb[1] + ky) * a.nb[0] + kx];
+                        num = fmaf(w, p[((long long)lz * ey + ly) * a.ext[0][kx] + lx], num);
+                        den += w;
+                    }
                 }
             }
+            out[r * nx + x] = num / den;
         }
-        out[i] = num / den;
     }
 }
 
@@ -139,16 +160,12 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
     const long long nvox = (long long)nx * ny * nz;
 
     // device memory: sub-volume images and phi, staging of host inputs and output, tables
-    std::vector<long long> bvox(nbox);
     size_t bytes = 0;
     auto align = [](size_t b) { return (b + 255) & ~size_t(255); };
-    for (int kz = 0; kz < nb[2]; ++kz)
-        for (int ky = 0; ky < nb[1]; ++ky)
-            for (int kx = 0; kx < nb[0]; ++kx) {
-                const long long v = (long long)std::min(edge, n[0]) * std::min(edge, n[1]) * std::min(edge, n[2]);
-                bvox[((long long)kz * nb[1] + ky) * nb[0] + kx] = v;
-                bytes += align(es * v) + align(sizeof(float) * v);
-            }
+    const int ext[3] = {std::min(edge, n[0]), std::min(edge, n[1]), std::min(edge, n[2])};
+    const long long bvox = (long long)ext[0] * ext[1] * ext[2];  // every sub-volume has these extents
+    const size_t stride = align(es * bvox) + align(sizeof(float) * bvox);
+    bytes += stride * nbox;
     const bool host_vol = !on_device(volume), host_phi = !on_device(phi0), host_out = !on_device(phi_out);
     if (host_vol) bytes += align(es * nvox);
     if (host_phi) bytes += align(sizeof(float) * nvox);
@@ -156,7 +173,9 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
     size_t tab_bytes = sizeof(float *) * nbox;
     for (int a = 0; a < 3; ++a)
         tab_bytes += sizeof(int) * (nb[a] + n[a] * (1 + 2 * kMaxCover)) + sizeof(float) * n[a] * kMaxCover;
-    bytes += align(tab_bytes) + 1024;
+    const size_t with_starts = tab_bytes + sizeof(int) * (nb[0] + nb[1] + nb[2]);
+    bytes += std::max(align(tab_bytes) + 1024, align(with_starts));
+    tab_bytes = with_starts;
     void *mem = nullptr;
     if ((st = dev_alloc(c, &mem, bytes))) return st;
     struct Release {
@@ -174,6 +193,7 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
 
     std::vector<rsf_brick> bricks(nbox);
     std::vector<const float *> phis(nbox);
+    MergeArgs m{};
     {
         std::lock_guard<std::mutex> lk(c->mu);
         RSF_CUDA(cudaSetDevice(c->device));
@@ -189,37 +209,52 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
             RSF_CUDA(xfer(d, phi0, sizeof(float) * nvox, c->stream));
             ph0 = d;
         }
-        for (int kz = 0; kz < nb[2]; ++kz)
-            for (int ky = 0; ky < nb[1]; ++ky)
-                for (int kx = 0; kx < nb[0]; ++kx) {
-                    const long long id = ((long long)kz * nb[1] + ky) * nb[0] + kx;
-                    const int bx = std::min(edge, n[0]), by = std::min(edge, n[1]), bz = std::min(edge, n[2]);
-                    const int x0 = starts[0][kx], y0 = starts[1][ky], z0 = starts[2][kz];
-                    void *img = take(es * bvox[id]);
-                    float *ph = reinterpret_cast<float *>(take(sizeof(float) * bvox[id]));
-                    const int grid = (int)std::min<long long>(1216, (bvox[id] + 255) / 256);
-                    switch (vt) {
-                        case RSF_U8:
-                            k_gather<<<grid, 256, 0, c->stream>>>(static_cast<const uint8_t *>(vol),
-                                                                  static_cast<uint8_t *>(img), n[0], n[1], x0, y0,
-                                                                  z0, bx, by, bvox[id]);
-                            break;
-                        case RSF_U16:
-                            k_gather<<<grid, 256, 0, c->stream>>>(static_cast<const uint16_t *>(vol),
-                                                                  static_cast<uint16_t *>(img), n[0], n[1], x0, y0,
-                                                                  z0, bx, by, bvox[id]);
-                            break;
-                        default:
-                            k_gather<<<grid, 256, 0, c->stream>>>(static_cast<const float *>(vol),
-                                                                  static_cast<float *>(img), n[0], n[1], x0, y0, z0,
-                                                                  bx, by, bvox[id]);
-                    }
-                    k_gather<<<grid, 256, 0, c->stream>>>(ph0, ph, n[0], n[1], x0, y0, z0, bx, by, bvox[id]);
-                    RSF_CUDA(cudaGetLastError());
-                    bricks[id] = rsf_brick{img, vt, bx, by, bz, ph, ph, sigma, eps, lambda1, lambda2, nu, mu, dt,
-                                           iters};
-                    phis[id] = ph;
-                }
+        GatherArgs ga{};
+        ga.box0 = take(stride * nbox);
+        ga.stride = stride;
+        ga.phi_at = align(es * bvox);
+        for (long long id = 0; id < nbox; ++id) {
+            char *const box = ga.box0 + id * stride;
+            float *const ph = reinterpret_cast<float *>(box + ga.phi_at);
+            bricks[id] = rsf_brick{box, vt, ext[0], ext[1], ext[2], ph, ph, sigma, eps, lambda1, lambda2, nu, mu, dt, iters};
+            phis[id] = ph;
+        }
+        char *tb = take(tab_bytes);
+        std::vector<char> host_tab(tab_bytes);
+        size_t off = 0;
+        auto put = [&](const void *src, size_t b) {
+            memcpy(host_tab.data() + off, src, b);
+            const char *d = tb + off;
+            off += b;
+            return d;
+        };
+        m.phi = reinterpret_cast<const float *const *>(put(phis.data(), sizeof(float *) * nbox));
+        for (int a = 0; a < 3; ++a) {
+            std::vector<int> exts(nb[a], ext[a]);
+            m.ext[a] = reinterpret_cast<const int *>(put(exts.data(), sizeof(int) * nb[a]));
+            m.count[a] = reinterpret_cast<const int *>(put(tab[a].count.data(), sizeof(int) * n[a]));
+            m.box[a] = reinterpret_cast<const int *>(put(tab[a].box.data(), sizeof(int) * n[a] * kMaxCover));
+            m.local[a] = reinterpret_cast<const int *>(put(tab[a].local.data(), sizeof(int) * n[a] * kMaxCover));
+            m.weight[a] = reinterpret_cast<const float *>(put(tab[a].weight.data(), sizeof(float) * n[a] * kMaxCover));
+            ga.start[a] = reinterpret_cast<const int *>(put(starts[a].data(), sizeof(int) * nb[a]));
+            ga.nb[a] = nb[a];
+            ga.ext[a] = ext[a];
+            ga.n[a] = n[a];
+            m.n[a] = n[a];
+            m.nb[a] = nb[a];
+        }
+        RSF_CUDA(cudaMemcpyAsync(tb, host_tab.data(), off, cudaMemcpyHostToDevice, c->stream));
+        for (long long first = 0; first < nbox; first += 32768) {
+            ga.first = (int)first;
+            const dim3 grid((unsigned)std::min<long long>(((long long)ext[1] * ext[2] + 7) / 8, nbox >= 16 ? 152 : 1216),
+                            (unsigned)std::min<long long>(32768, nbox - first));
+            switch (vt) {
+                case RSF_U8: k_gather<<<grid, 256, 0, c->stream>>>(static_cast<const uint8_t *>(vol), ph0, ga); break;
+                case RSF_U16: k_gather<<<grid, 256, 0, c->stream>>>(static_cast<const uint16_t *>(vol), ph0, ga); break;
+                default: k_gather<<<grid, 256, 0, c->stream>>>(static_cast<const float *>(vol), ph0, ga);
+            }
+        }
+        RSF_CUDA(cudaGetLastError());
     }
     // every sub-volume evolved as its own volume, all together (same stream, so
     // the gathers above are ordered before the batch's first launch)
@@ -227,29 +262,7 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
 
     std::lock_guard<std::mutex> lk(c->mu);
     float *out = host_out ? reinterpret_cast<float *>(take(sizeof(float) * nvox)) : phi_out;
-    char *tb = take(tab_bytes);
-    std::vector<char> host_tab(tab_bytes);
-    size_t off = 0;
-    auto put = [&](const void *src, size_t b) {
-        memcpy(host_tab.data() + off, src, b);
-        const char *d = tb + off;
-        off += b;
-        return d;
-    };
-    MergeArgs m{};
-    m.phi = reinterpret_cast<const float *const *>(put(phis.data(), sizeof(float *) * nbox));
-    for (int a = 0; a < 3; ++a) {
-        std::vector<int> ext(nb[a], std::min(edge, n[a]));
-        m.ext[a] = reinterpret_cast<const int *>(put(ext.data(), sizeof(int) * nb[a]));
-        m.count[a] = reinterpret_cast<const int *>(put(tab[a].count.data(), sizeof(int) * n[a]));
-        m.box[a] = reinterpret_cast<const int *>(put(tab[a].box.data(), sizeof(int) * n[a] * kMaxCover));
-        m.local[a] = reinterpret_cast<const int *>(put(tab[a].local.data(), sizeof(int) * n[a] * kMaxCover));
-        m.weight[a] = reinterpret_cast<const float *>(put(tab[a].weight.data(), sizeof(float) * n[a] * kMaxCover));
-        m.n[a] = n[a];
-        m.nb[a] = nb[a];
-    }
-    RSF_CUDA(cudaMemcpyAsync(tb, host_tab.data(), off, cudaMemcpyHostToDevice, c->stream));
-    k_merge<<<(int)std::min<long long>(4864, (nvox + 255) / 256), 256, 0, c->stream>>>(m, out);
+    k_merge<<<(unsigned)std::min<long long>(4864, ((long long)ny * nz + 7) / 8), 256, 0, c->stream>>>(m, out);
     RSF_CUDA(cudaGetLastError());
     if (host_out) RSF_CUDA(xfer(phi_out, out, sizeof(float) * nvox, c->stream));
     RSF_CUDA(cudaStreamSynchronize(c->stream));

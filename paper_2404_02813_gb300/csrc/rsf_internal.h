@@ -74,7 +74,7 @@ constexpr int kStatBlocks = 1024;
 // centred image f.I.  `vol` is a device pointer of dtype vt (0 u8, 1 u16, 2 f32).
 cudaError_t setup_image(const void *vol, int vt, const Taps &taps, Fields &f, cudaStream_t s, bool centre = true);
 
-// Centring constants only (f.cs from the image statistics), no other field.
+// Centring constants only (f.cs from the image statistics), no other field; never synchronises.
 cudaError_t image_stats(const void *vol, int vt, Fields &f, cudaStream_t s);
 // Zero-padding profiles p_a(i) = sum of the in-volume taps (double sums rounded
 // once), nx + ny + nz floats: K*1 = p_x p_y p_z.
@@ -171,9 +171,30 @@ size_t tiled_extra_bytes(const void *img, int nx, int ny, int nz, int imgtype, i
 // those three blocks (256-byte aligned; stage may be larger than the minimum).
 void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q,
                         void *extra);
-// Before the first iteration: the image copied to b.img_t where its rows are not 16-byte
-// aligned, and q = +-atan(eps/|phi|)/pi (sign of phi) of b.phi[0].
-cudaError_t tiled_start(const BrickDev &b, int imgtype, cudaStream_t s);
+// One brick's work before the first iteration, for kernels that take many bricks at once
+// (blockIdx.y): image statistics, phi0 to phi (or nothing where they are the same), q of it,
+// the image copied to img_t where that differs.
+struct SetupBrick {
+    const void *img;
+    int imgtype;
+    int nx, qp, ip;
+    long long rows;         // ny * nz
+    const float *src;       // phi0
+    float *phi, *q;
+    void *img_t;
+    float *partials, *cs;   // 3 * kStatBlocks floats of scratch; the centring constants
+    float eps;
+};
+SetupBrick setup_of(const BrickDev &b, int imgtype, const float *phi0, float *partials, float *cs);
+// Statistics (partials, cs) and start (phi, q, img_t) of n bricks described in device memory.
+cudaError_t setup_stats(const SetupBrick *d, int n, cudaStream_t s);
+cudaError_t setup_start(const SetupBrick *d, int n, cudaStream_t s);
+// The start of one brick, described by value.
+cudaError_t tiled_start(const BrickDev &b, int imgtype, const float *phi0, cudaStream_t s);
+// K*I~ of a group's bricks (b.ki) before its first iteration (after the start; uses b.abxy as
+// scratch); nothing in the Eq. (15) form.
+cudaError_t tiled_ki_init(const TiledGroup &g, cudaStream_t s);
+
 // The exact arithmetic (rsf_exact.cuh): radii 1 to 16.  Fields in a stage block of
 // exact_stage_bytes and a q block of exact_q_bytes (at most the 8 nx ny nz above); before the
 // first iteration the centred image (b.img, FP32, pitched; from the caller's vol and b.cs)
@@ -183,10 +204,6 @@ size_t exact_stage_bytes(int nx, int ny, int nz);
 size_t exact_q_bytes(int nx, int ny, int nz);
 void exact_place_fields(BrickDev &b, void *stage, float *q);
 cudaError_t exact_start(const BrickDev &b, const void *vol, int vt, cudaStream_t s);
-// b.ki = K*I~ before the first tiled iteration (after tiled_start; b.cs set; uses b.abxy as
-// scratch); nothing when b.ki is null (the Eq. (15) form).  err: the error word of its waits.
-cudaError_t tiled_ki_init(const BrickDev &b, int imgtype, const Taps &taps, int *err, cudaStream_t s);
-
 // One iteration of the separable pass path: phi_in -> phi_out.
 // `stages`, when not null, receives RSF_NSTAGES fields (f1, f2, g, kappa, L).
 cudaError_t iterate_passes(const Taps &taps, const Coeffs &c, Fields &f, const float *phi_in, float *phi_out,

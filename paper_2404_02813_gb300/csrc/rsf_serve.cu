@@ -103,6 +103,12 @@ int lane_of(long long n) { return n < (1LL << 19) ? 0 : (n < (1LL << 21) ? 1 : (
 
 struct Server;
 
+// One brick's launch descriptor with the CTA offsets of its kernels.
+struct SetupDesc {
+    rsf::BrickDev b;
+    int starts[8];
+};
+
 struct DoneArg {
     Server *srv;
     std::shared_ptr<Request> r;
@@ -123,6 +129,7 @@ struct Server {
     Lane lanes[kLanes];
     cudaStream_t s_setup = nullptr;
     float *partials = nullptr;
+    SetupDesc *setup_desc = nullptr;  // of the admission being set up (device)
     int sms = 0;
     // statistics (mu)
     uint64_t submitted = 0, completed = 0, failed = 0, cancelled = 0, suspended = 0, admitted = 0;
@@ -287,12 +294,35 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
             cudaMemsetAsync(d.phi[1], 0xFF, sizeof(float) * n, s->s_setup) != cudaSuccess)
             return fail_admit(RSF_E_CUDA);
     }
-    if (xfer(d.phi[0], q.phi0, sizeof(float) * n, s->s_setup) != cudaSuccess)
+    const bool here = q.iters > 0 && in_place(q.phi0, c->device);  // then copied with q
+    if (!here && xfer(d.phi[0], q.phi0, sizeof(float) * n, s->s_setup) != cudaSuccess) return fail_admit(RSF_E_CUDA);
+    if (q.iters > 0 && rsf::tiled_start(d, (int)q.vt, here ? q.phi0 : d.phi[0], s->s_setup) != cudaSuccess)
         return fail_admit(RSF_E_CUDA);
-    if (q.iters > 0 && rsf::tiled_start(d, (int)q.vt, s->s_setup) != cudaSuccess)
-        return fail_admit(RSF_E_CUDA);
-    if (q.iters > 0 && rsf::tiled_ki_init(d, (int)q.vt, r->taps, s->ctx->d_err, s->s_setup) != cudaSuccess)
-        return fail_admit(RSF_E_CUDA);
+    if (q.iters > 0 && r->force == 0) {
+        // K*I~: a launch group of this brick alone, described in the server's scratch (the
+        // set-up stream takes one admission after the other)
+        SetupDesc sd{};
+        sd.b = d;
+        sd.b.xyp = rsf::tiled_xy_planes({d}, 0, r->taps.R, s->sms);
+        if (rsf::tiled_encode_maps(sd.b, 0, r->storage, (int)q.vt, r->taps.R) != cudaSuccess) return fail_admit(RSF_E_CUDA);
+        rsf::TiledGroup g{};
+        g.imgtype = (int)q.vt;
+        g.taps = r->taps;
+        g.nb = 1;
+        g.err = c->d_err;
+        rsf::tiled_cta_counts(sd.b, 0, r->taps.R, g.ncta);
+        g.bricks = &s->setup_desc->b;
+        for (int k = 0; k < 4; ++k) {
+            sd.starts[2 * k + 1] = (int)g.ncta[k];
+            g.starts[k] = s->setup_desc->starts + 2 * k;
+        }
+        ParamChunk ch;
+        ch.offset = 0;
+        ch.count = (int)(sizeof(sd) / sizeof(float));
+        memcpy(ch.v, &sd, sizeof(sd));
+        k_put<<<1, 256, 0, s->s_setup>>>(ch, reinterpret_cast<float *>(s->setup_desc));
+        if (rsf::tiled_ki_init(g, s->s_setup) != cudaSuccess) return fail_admit(RSF_E_CUDA);
+    }
     if (rsf::tiled_prepare(r->storage, r->taps.R, r->force) != cudaSuccess) return fail_admit(RSF_E_CUDA);
     if (cudaEventCreateWithFlags(&r->ready, cudaEventDisableTiming) != cudaSuccess) return fail_admit(RSF_E_CUDA);
     cudaEventRecord(r->ready, s->s_setup);
@@ -557,6 +587,11 @@ Server *server(rsf_ctx *c, rsf_status *st) {
         delete s;
         return nullptr;
     }
+    if ((*st = dev_alloc(c, (void **)&s->setup_desc, sizeof(SetupDesc)))) {
+        dev_free(c, s->partials, sizeof(float) * 3 * rsf::kStatBlocks);
+        delete s;
+        return nullptr;
+    }
     s->inject_admission = c->opt_inject_admission;
     s->inject_upload = c->opt_inject_upload;
     s->slots = c->opt_serve_slots;
@@ -578,6 +613,7 @@ void rsf_serve_shutdown(rsf_ctx *c) {
     s->cv.notify_all();
     if (s->th.joinable()) s->th.join();
     dev_free(c, s->partials, sizeof(float) * 3 * rsf::kStatBlocks);
+    dev_free(c, s->setup_desc, sizeof(SetupDesc));
     for (Lane &L : s->lanes) {
         free_desc(c, L.desc);
         cudaStreamDestroy(L.stream);

@@ -320,6 +320,7 @@ template <> struct ImgVec<float> {
 // EX: q from the exact arithmetic, whose zero keeps its sign (q = -0: H = 0)
 template <int R, class ImgT, int NP_, bool EX>
 struct SrcH {  // NP = 1: (H I~, H); NP = 2: also ((1-H) I~, 1-H), the other side of Eq. (10)
+    using V = float2;
     static constexpr int NP = NP_, CTAS = NP == 1 ? 4 : 3, NS = 1;
     static constexpr bool FIX = true;
     using G = XYG<R>;
@@ -376,7 +377,8 @@ struct SrcH {  // NP = 1: (H I~, H); NP = 2: also ((1-H) I~, 1-H), the other sid
 };
 
 template <int R, class ImgT>
-struct SrcI {  // (I~, 0): the centred image alone, for K*I~
+struct SrcI {  // the centred image alone, one float per voxel, for K*I~
+    using V = float;
     static constexpr int NP = 1, CTAS = 4, NS = 1;
     static constexpr bool FIX = false;
     using G = XYG<R>;
@@ -402,7 +404,7 @@ struct SrcI {  // (I~, 0): the centred image alone, for K*I~
             const int ji = j + FI::O;
             if (j == 0 || ji % ImgVec<ImgT>::V == 0) iv.load(im + ji / ImgVec<ImgT>::V * ImgVec<ImgT>::V);
             const bool in = in_y && (unsigned)(gx + j) < (unsigned)nx;
-            const float2 p[1] = {make_float2(in ? fmaf(iv.get(ji % ImgVec<ImgT>::V), inv_s, nms) : 0.f, 0.f)};
+            const float p[1] = {in ? fmaf(iv.get(ji % ImgVec<ImgT>::V), inv_s, nms) : 0.f};
             f(j, p);
         }
     }
@@ -411,6 +413,7 @@ struct SrcI {  // (I~, 0): the centred image alone, for K*I~
 // (a, b) as stored by rsf_ta_z: FP32 pairs, or 16-bit pairs widened as the window is read
 template <int R, class S>
 struct SrcAB {
+    using V = float2;
     static constexpr int NP = 1, CTAS = 3, NS = 2;
     static constexpr bool FIX = false;  // the zero fill is the convolution's padding
     using G = XYG<R>;
@@ -444,22 +447,26 @@ struct SrcAB {
     }
 };
 
-// Where the x/y-convolved pairs go: pitched, FP32, NP pairs interleaved per voxel.
+// Where the x/y-convolved fields go: pitched, FP32, a voxel's values side by side.
 struct OutXY {
-    float2 *u;
+    float *u;
     int px;
     long long pplane;
 };
 
 // Shared memory: NS staging buffers, the x-convolved rows, an mbarrier per buffer.  Row pitch
-// of the x-convolved rows: 34 float2 (17 units of 16 bytes) or 33 float4.
+// of the x-convolved rows: an odd number of 16-byte units (36 floats, 34 float2 or 33 float4).
 template <int R, class Src>
 struct XYSmem {
-    static constexpr int XS = Src::NP == 1 ? 34 : 33;
-    static constexpr int XC = Src::NP * (int)sizeof(float2) * XYG<R>::H * XS;
+    using V = typename Src::V;
+    static constexpr int XS = Src::NP == 2 ? 33 : (sizeof(V) == 8 ? 34 : 36);
+    static constexpr int XC = Src::NP * (int)sizeof(V) * XYG<R>::H * XS;
     static constexpr int NS = Src::NS;
     static constexpr size_t bytes = NS * Src::BYTES + XC + NS * sizeof(uint64_t);
 };
+
+__device__ __forceinline__ float2 tap_fma(float2 g, float2 v, float2 a) { return f2fma(g, v, a); }
+__device__ __forceinline__ float tap_fma(float2 g, float v, float a) { return fmaf(g.x, v, a); }
 
 // Planes [za, za + np) of tile (x0, y0).  Waits are bounded (expiry reported in the group's
 // error word).
@@ -469,7 +476,8 @@ __device__ __forceinline__ void xy_tile(const GroupArgs &G, const Src &src, cons
     using X = XYG<R>;
     constexpr int NP = Src::NP, T = X::T, YT = X::YT;
     constexpr int XS = XYSmem<R, Src>::XS, NS = XYSmem<R, Src>::NS;
-    float2 *xc = reinterpret_cast<float2 *>(sm + NS * Src::BYTES);
+    using V = typename Src::V;
+    V *xc = reinterpret_cast<V *>(sm + NS * Src::BYTES);
     uint64_t *bar = reinterpret_cast<uint64_t *>(sm + NS * Src::BYTES + XYSmem<R, Src>::XC);
     if (smem_addr(sm) % 128u != 0u) {
         report_error(G.err, kErrSmemAlign);
@@ -494,7 +502,7 @@ __device__ __forceinline__ void xy_tile(const GroupArgs &G, const Src &src, cons
     const bool fix = Src::FIX && (x0 < R || y0 < R || x0 + 32 + R > nx || y0 + X::TH + R > ny);
     const int yr = warp * YT;                                    // y phase: YT rows of one column
     const bool yrow = yr < rows, col = x0 + lane < nx;
-    float2 *o = out.u + ((long long)za * out.pplane + (long long)(y0 + yr) * out.px + x0 + lane) * NP;
+    V *o = reinterpret_cast<V *>(out.u) + ((long long)za * out.pplane + (long long)(y0 + yr) * out.px + x0 + lane) * NP;
     for (int z = za; z < zb_end; ++z) {
         const int i = (z - za) % NS;
         const unsigned phase = (unsigned)((z - za) / NS) & 1u;
@@ -511,20 +519,24 @@ __device__ __forceinline__ void xy_tile(const GroupArgs &G, const Src &src, cons
             __syncthreads();
         }
         if (xrow) {
-            float2 acc[NP][8];
+            V acc[NP][8];
 #pragma unroll
             for (int p = 0; p < NP; ++p)
 #pragma unroll
-                for (int i = 0; i < 8; ++i) acc[p][i] = make_float2(0.f, 0.f);
+                for (int i = 0; i < 8; ++i) acc[p][i] = V{};
             // each input feeds the outputs it contributes to: output i takes taps 0 .. T-1 in order
-            src.window(st, row, xo, [&](int j, const float2 *v) {
+            src.window(st, row, xo, [&](int j, const V *v) {
 #pragma unroll
                 for (int i = 0; i < 8; ++i)
                     if (j - i >= 0 && j - i < T)
 #pragma unroll
-                        for (int p = 0; p < NP; ++p) acc[p][i] = f2fma(t.g[j - i], v[p], acc[p][i]);
+                        for (int p = 0; p < NP; ++p) acc[p][i] = tap_fma(t.g[j - i], v[p], acc[p][i]);
             });
-            if constexpr (NP == 1) {
+            if constexpr (sizeof(V) == 4) {
+                float4 *dst = reinterpret_cast<float4 *>(xc + row * XS + xo);
+                dst[0] = make_float4(acc[0][0], acc[0][1], acc[0][2], acc[0][3]);
+                dst[1] = make_float4(acc[0][4], acc[0][5], acc[0][6], acc[0][7]);
+            } else if constexpr (NP == 1) {
                 float4 *dst = reinterpret_cast<float4 *>(xc + row * XS + xo);
 #pragma unroll
                 for (int i = 0; i < 4; ++i)
@@ -542,14 +554,14 @@ __device__ __forceinline__ void xy_tile(const GroupArgs &G, const Src &src, cons
             src.issue(st, x0, y0, z + NS, bar + i, G.fault_tx);
         }
         if (yrow) {
-            float2 res[YT][NP];
+            V res[YT][NP];
 #pragma unroll
             for (int i = 0; i < YT; ++i)
 #pragma unroll
-                for (int p = 0; p < NP; ++p) res[i][p] = make_float2(0.f, 0.f);
+                for (int p = 0; p < NP; ++p) res[i][p] = V{};
 #pragma unroll
             for (int j = 0; j < YT + 2 * R; ++j) {
-                float2 v[NP];
+                V v[NP];
                 if constexpr (NP == 1) {
                     v[0] = xc[(yr + j) * XS + lane];
                 } else {
@@ -561,13 +573,13 @@ __device__ __forceinline__ void xy_tile(const GroupArgs &G, const Src &src, cons
                 for (int i = 0; i < YT; ++i)
                     if (j - i >= 0 && j - i < T)
 #pragma unroll
-                        for (int p = 0; p < NP; ++p) res[i][p] = f2fma(t.g[j - i], v[p], res[i][p]);
+                        for (int p = 0; p < NP; ++p) res[i][p] = tap_fma(t.g[j - i], v[p], res[i][p]);
             }
             if (col) {
 #pragma unroll
                 for (int i = 0; i < YT; ++i) {
                     if (yr + i < rows) {
-                        float2 *d = o + (long long)(i * out.px) * NP;
+                        V *d = o + (long long)(i * out.px) * NP;
                         if constexpr (NP == 1)
                             *d = res[i][0];
                         else
@@ -605,7 +617,7 @@ __global__ void __launch_bounds__(kXYThreads, (SrcH<R, ImgT, NP, EX>::CTAS)) k_t
     const BrickDev &B = G.bricks[b];
     const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
     const SrcH<R, ImgT, NP, EX> src{&B.tm_q, &B.tm_img, EX ? 1.f : B.cs[1], EX ? 0.f : -B.cs[0] * B.cs[1]};
-    const OutXY out{B.u2, B.px, (long long)B.px * B.ny};
+    const OutXY out{reinterpret_cast<float *>(B.u2), B.px, (long long)B.px * B.ny};
     xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
 }
 
@@ -618,7 +630,7 @@ __global__ void __launch_bounds__(kXYThreads, (SrcAB<R, S>::CTAS)) k_tb_xy(Group
     const BrickDev &B = G.bricks[b];
     const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
     const SrcAB<R, S> src{&B.tm_ab};
-    const OutXY out{B.abxy, B.px, (long long)B.px * B.ny};
+    const OutXY out{reinterpret_cast<float *>(B.abxy), B.px, (long long)B.px * B.ny};
     xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
 }
 
@@ -919,44 +931,43 @@ __global__ void __launch_bounds__(kAZThreads, 2) k_ta_z4(GroupArgs G, TapPairs t
 
 // ------------------------------------------------------- set-up: K*I~
 
-// K*I~ of one brick, once per solve: the x/y kernel on (I~, 0) into b.abxy,
-// then a z convolution of its first component into b.ki.  Launched per brick
-// (the descriptor by value), on the x/y kernel's tiles and the slabs of group A.
+// K*I~ of a group's bricks, once per solve: the x/y kernel on I~ into b.abxy (read as one float
+// per voxel), then a z convolution into b.ki, on the x/y kernel's tiles and the slabs of group A.
 template <int R, class ImgT>
-__global__ void __launch_bounds__(kXYThreads, 4) k_ki_xy(const __grid_constant__ BrickDev B, int *err, TapPairs t) {
+__global__ void __launch_bounds__(kXYThreads, 4) k_ki_xy(GroupArgs G, TapPairs t) {
     extern __shared__ __align__(128) unsigned char xsm[];
-    const XYTile tl = xy_tile_of<R>(blockIdx.x, B);
+    const int b = find_brick(G.starts, G.nb, blockIdx.x);
+    const BrickDev &B = G.bricks[b];
+    const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
     const SrcI<R, ImgT> src{&B.tm_img, B.cs[1], -B.cs[0] * B.cs[1], tl.x0, tl.y0, B.nx, B.ny};
-    const OutXY out{B.abxy, B.px, (long long)B.px * B.ny};
-    GroupArgs G{};
-    G.err = err;
+    const OutXY out{reinterpret_cast<float *>(B.abxy), B.px, (long long)B.px * B.ny};
     xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
 }
 
 template <int R>
-__global__ void __launch_bounds__(kAZThreads) k_ki_z(BrickDev B, TapPairs t) {
+__global__ void __launch_bounds__(kAZThreads) k_ki_z(GroupArgs G, TapPairs t) {
     constexpr int T = 2 * R + 1;
     constexpr int WIN = kAZO + 2 * R;
-    const int nzt = (B.nz + kAZT - 1) / kAZT, nxt = (B.nx + 31) / 32;
-    const int zt = blockIdx.x % nzt, rest = blockIdx.x / nzt;
-    const int x = (rest % nxt) * 32 + (threadIdx.x & 31), y = rest / nxt;
-    const int z0 = zt * kAZT + (threadIdx.x >> 5) * kAZO;
+    const AZSlabId id = az_slab_of(G, blockIdx.x);
+    const BrickDev &B = G.bricks[id.b];
+    const int x = id.x0 + (threadIdx.x & 31), z0 = id.z0 + (threadIdx.x >> 5) * kAZO, nz = B.nz;
     if (x >= B.nx) return;
-    const long long pplane = (long long)B.px * B.ny;
-    const float2 *src = B.abxy + (long long)y * B.px + x;
+    const long long pplane = (long long)B.px * B.ny, col = (long long)id.y * B.px + x;
+    const float *src = reinterpret_cast<const float *>(B.abxy) + col;
+    float *const ki = B.ki + col;
     float w[WIN];
 #pragma unroll
     for (int j = 0; j < WIN; ++j) {
         const int zi = z0 - R + j;
-        w[j] = (unsigned)zi < (unsigned)B.nz ? __ldg(src + zi * pplane).x : 0.f;
+        w[j] = (unsigned)zi < (unsigned)nz ? __ldg(src + zi * pplane) : 0.f;
     }
 #pragma unroll
     for (int o = 0; o < kAZO; ++o) {
-        if (z0 + o < B.nz) {
+        if (z0 + o < nz) {
             float acc = 0.f;
 #pragma unroll
             for (int k = 0; k < T; ++k) acc = fmaf(t.g[k].x, w[o + k], acc);
-            B.ki[(long long)(z0 + o) * pplane + (long long)y * B.px + x] = acc;
+            ki[(z0 + o) * pplane] = acc;
         }
     }
 }

@@ -10,21 +10,49 @@ namespace rsf {
 namespace tiled {
 
 namespace {
-// q of phi; rows of nx values at a pitch of qp (one row of n values when they are dense)
-template <bool EX>
-__global__ void k_q_init(const float *__restrict__ phi, float *__restrict__ q, long long rows, long long nx,
-                         long long qp, float eps) {
-    const auto q_of = [&](float u) { return EX ? heaviside_q_exact(u, eps) : heaviside_q_fast(u, eps); };
-    if (rows == 1) {
-        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < nx; i += (long long)gridDim.x * blockDim.x)
-            q[i] = q_of(__ldg(phi + i));
-        return;
-    }
+// The start of one brick by gridDim.x blocks: phi0 to phi, q of it at a pitch of qp, the image
+// to img_t at a pitch of ip where that differs.  A warp per row, four values per lane and load
+// where rows are dense multiples of 4 (then the brick is one long row).
+template <class T>
+__device__ __forceinline__ void copy_rows(const T *__restrict__ src, T *__restrict__ dst, long long rows, int nx, int ip,
+                                          long long first, long long step) {
     const int lane = threadIdx.x & 31;
-    for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
-         r += ((long long)gridDim.x * blockDim.x) >> 5)
-        for (int x = lane; x < nx; x += 32) q[r * qp + x] = q_of(__ldg(phi + r * nx + x));
+    for (long long r = first; r < rows; r += step)
+        for (int x = lane; x < nx; x += 32) dst[r * ip + x] = src[r * nx + x];
 }
+template <bool EX>
+__device__ __forceinline__ void start_brick(const SetupBrick &b) {
+    const auto q_of = [&](float u) { return EX ? heaviside_q_exact(u, b.eps) : heaviside_q_fast(u, b.eps); };
+    const int lane = threadIdx.x & 31;
+    const long long first = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5, step = ((long long)gridDim.x * blockDim.x) >> 5;
+    const bool copy = b.src != b.phi;
+    const uintptr_t at = reinterpret_cast<uintptr_t>(b.src) | reinterpret_cast<uintptr_t>(b.phi);
+    if (b.qp == b.nx && at % 16 == 0) {
+        const long long n4 = b.rows * b.nx / 4;
+        for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < n4; i += (long long)gridDim.x * blockDim.x) {
+            const float4 u = __ldg(reinterpret_cast<const float4 *>(b.src) + i);
+            if (copy) reinterpret_cast<float4 *>(b.phi)[i] = u;
+            reinterpret_cast<float4 *>(b.q)[i] = make_float4(q_of(u.x), q_of(u.y), q_of(u.z), q_of(u.w));
+        }
+    } else {
+        for (long long r = first; r < b.rows; r += step)
+            for (int x = lane; x < b.nx; x += 32) {
+                const float u = __ldg(b.src + r * b.nx + x);
+                if (copy) b.phi[r * b.nx + x] = u;
+                b.q[r * b.qp + x] = q_of(u);
+            }
+    }
+    if (b.img_t != b.img) {
+        switch (b.imgtype) {
+            case 0: copy_rows(static_cast<const uint8_t *>(b.img), static_cast<uint8_t *>(b.img_t), b.rows, b.nx, b.ip, first, step); break;
+            case 1: copy_rows(static_cast<const uint16_t *>(b.img), static_cast<uint16_t *>(b.img_t), b.rows, b.nx, b.ip, first, step); break;
+            default: copy_rows(static_cast<const float *>(b.img), static_cast<float *>(b.img_t), b.rows, b.nx, b.ip, first, step);
+        }
+    }
+}
+template <bool EX>
+__global__ void __launch_bounds__(256) k_start(SetupBrick b) { start_brick<EX>(b); }
+__global__ void __launch_bounds__(256) k_start_many(const SetupBrick *__restrict__ d) { start_brick<false>(d[blockIdx.y]); }
 // the centred image (I - m) / s, rows of nx values at a pitch of ip
 template <class T>
 __global__ void k_center_rows(const T *__restrict__ vol, const float *__restrict__ cs, float *__restrict__ dst,
@@ -34,14 +62,6 @@ __global__ void k_center_rows(const T *__restrict__ vol, const float *__restrict
     for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
          r += ((long long)gridDim.x * blockDim.x) >> 5)
         for (int x = lane; x < nx; x += 32) dst[r * ip + x] = ((float)vol[r * nx + x] - m) * inv_s;
-}
-// rows of nx values copied to a pitch of ip
-template <class T>
-__global__ void k_pitch_rows(const T *__restrict__ src, T *__restrict__ dst, long long rows, int nx, int ip) {
-    const int lane = threadIdx.x & 31;
-    for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
-         r += ((long long)gridDim.x * blockDim.x) >> 5)
-        for (int x = lane; x < nx; x += 32) dst[r * ip + x] = src[r * nx + x];
 }
 }  // namespace
 
@@ -187,18 +207,24 @@ cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, 
     return encode_typed(&b.tm_ab, CU_TENSOR_MAP_DATA_TYPE_UINT32, 4, b.ab, 1, b.px, b, box.ab16, box.rows, 1);
 }
 
-cudaError_t tiled_start(const BrickDev &b, int imgtype, cudaStream_t s) {
-    const long long rows = (long long)b.ny * b.nz;
-    if (b.img_t != b.img) {
-        void *d = const_cast<void *>(b.img_t);
-        switch (imgtype) {
-            case 0: tiled::k_pitch_rows<<<1216, 256, 0, s>>>((const uint8_t *)b.img, (uint8_t *)d, rows, b.nx, b.ip); break;
-            case 1: tiled::k_pitch_rows<<<1216, 256, 0, s>>>((const uint16_t *)b.img, (uint16_t *)d, rows, b.nx, b.ip); break;
-            default: tiled::k_pitch_rows<<<1216, 256, 0, s>>>((const float *)b.img, (float *)d, rows, b.nx, b.ip);
-        }
-    }
-    const bool dense = b.qp == b.nx;
-    tiled::k_q_init<false><<<1216, 256, 0, s>>>(b.phi[0], b.q, dense ? 1 : rows, dense ? rows * b.nx : b.nx, b.qp, b.eps);
+SetupBrick setup_of(const BrickDev &b, int imgtype, const float *phi0, float *partials, float *cs) {
+    return SetupBrick{b.img, imgtype, b.nx, b.qp, b.ip, (long long)b.ny * b.nz, phi0, b.phi[0], b.q,
+                      const_cast<void *>(b.img_t), partials, cs, b.eps};
+}
+
+namespace {
+unsigned start_blocks(long long n) { return (unsigned)(n < 2048LL * 1216 ? (n + 2047) / 2048 : 1216); }
+}  // namespace
+
+cudaError_t setup_start(const SetupBrick *d, int n, cudaStream_t s) {
+    for (int o = 0; o < n; o += 32768)
+        tiled::k_start_many<<<dim3(n >= 8 ? 152 : 1216 / n, n - o < 32768 ? n - o : 32768), 256, 0, s>>>(d + o);
+    return cudaGetLastError();
+}
+
+cudaError_t tiled_start(const BrickDev &b, int imgtype, const float *phi0, cudaStream_t s) {
+    const SetupBrick d = setup_of(b, imgtype, phi0, nullptr, nullptr);
+    tiled::k_start<false><<<start_blocks(d.rows * d.nx), 256, 0, s>>>(d);
     return cudaGetLastError();
 }
 
@@ -211,7 +237,9 @@ cudaError_t exact_start(const BrickDev &b, const void *vol, int vt, cudaStream_t
         case 1: tiled::k_center_rows<<<grid, 256, 0, s>>>((const uint16_t *)vol, b.cs, d, rows, b.nx, b.ip); break;
         default: tiled::k_center_rows<<<grid, 256, 0, s>>>((const float *)vol, b.cs, d, rows, b.nx, b.ip);
     }
-    tiled::k_q_init<true><<<grid, 256, 0, s>>>(b.phi[0], b.q, rows, b.nx, b.qp, b.eps);
+    SetupBrick st = setup_of(b, 2, b.phi[0], nullptr, nullptr);
+    st.img_t = const_cast<void *>(st.img);
+    tiled::k_start<true><<<start_blocks(rows * b.nx), 256, 0, s>>>(st);
     return cudaGetLastError();
 }
 
@@ -449,40 +477,37 @@ void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *
 
 namespace {
 template <int R, class ImgT>
-cudaError_t ki_init_r(const BrickDev &b, const Taps &taps, int *err, cudaStream_t s) {
+cudaError_t ki_init_r(const TiledGroup &g, cudaStream_t s) {
     constexpr size_t sm = tiled::XYSmem<R, tiled::SrcI<R, ImgT>>::bytes;
     static_assert(sm <= 48 * 1024, "k_ki_xy needs no shared-memory opt-in");
-    const tiled::TapPairs tp = tiled::tap_pairs(taps);
-    unsigned counts[4];
-    tiled_cta_counts(b, 0, R, counts);
-    tiled::k_ki_xy<R, ImgT><<<counts[0], tiled::kXYThreads, sm, s>>>(b, err, tp);
-    tiled::k_ki_z<R><<<counts[1], tiled::kAZThreads, 0, s>>>(b, tp);
+    const tiled::TapPairs tp = tiled::tap_pairs(g.taps);
+    tiled::GroupArgs G{g.bricks, g.starts[0], g.nb, 0, g.err, 0u};
+    tiled::k_ki_xy<R, ImgT><<<g.ncta[0], tiled::kXYThreads, sm, s>>>(G, tp);
+    G.starts = g.starts[1];
+    tiled::k_ki_z<R><<<g.ncta[1], tiled::kAZThreads, 0, s>>>(G, tp);
     return cudaGetLastError();
 }
 template <int R>
-cudaError_t ki_init_i(const BrickDev &b, int imgtype, const Taps &taps, int *err, cudaStream_t s) {
-    switch (imgtype) {
-        case 0: return ki_init_r<R, uint8_t>(b, taps, err, s);
-        case 1: return ki_init_r<R, uint16_t>(b, taps, err, s);
-        default: return ki_init_r<R, float>(b, taps, err, s);
+cudaError_t ki_init_i(const TiledGroup &g, cudaStream_t s) {
+    switch (g.imgtype) {
+        case 0: return ki_init_r<R, uint8_t>(g, s);
+        case 1: return ki_init_r<R, uint16_t>(g, s);
+        default: return ki_init_r<R, float>(g, s);
     }
 }
 }  // namespace
 
-cudaError_t tiled_ki_init(const BrickDev &brick, int imgtype, const Taps &taps, int *err, cudaStream_t s) {
-    if (!brick.ki) return cudaSuccess;  // the Eq. (15) form convolves the complement directly
-    BrickDev b = brick;
-    const cudaError_t e = tiled_encode_maps(b, 0, 0, imgtype, taps.R);
-    if (e != cudaSuccess) return e;
-    switch (taps.R) {
-        case 2: return ki_init_i<2>(b, imgtype, taps, err, s);
-        case 3: return ki_init_i<3>(b, imgtype, taps, err, s);
-        case 4: return ki_init_i<4>(b, imgtype, taps, err, s);
-        case 5: return ki_init_i<5>(b, imgtype, taps, err, s);
-        case 6: return ki_init_i<6>(b, imgtype, taps, err, s);
-        case 8: return ki_init_i<8>(b, imgtype, taps, err, s);
-        case 10: return ki_init_i<10>(b, imgtype, taps, err, s);
-        case 12: return ki_init_i<12>(b, imgtype, taps, err, s);
+cudaError_t tiled_ki_init(const TiledGroup &g, cudaStream_t s) {
+    if (g.force != 0) return cudaSuccess;  // the other forms convolve the complement directly
+    switch (g.taps.R) {
+        case 2: return ki_init_i<2>(g, s);
+        case 3: return ki_init_i<3>(g, s);
+        case 4: return ki_init_i<4>(g, s);
+        case 5: return ki_init_i<5>(g, s);
+        case 6: return ki_init_i<6>(g, s);
+        case 8: return ki_init_i<8>(g, s);
+        case 10: return ki_init_i<10>(g, s);
+        case 12: return ki_init_i<12>(g, s);
         default: return cudaErrorInvalidValue;
     }
 }

@@ -375,8 +375,9 @@ rsf_status rsf_autotune_report(rsf_ctx *ctx, char *buf, int32_t cap);
  * first poll that returns a final status (later polls: RSF_E_NOTFOUND).
  * rsf_wait blocks up to timeout_ms (< 0: no limit) for a final status, then
  * behaves as rsf_poll; on expiry it returns RSF_E_TIMEOUT and keeps the ticket.
- * Active requests are advanced in four lanes by voxel count (below 2^19, 2^21,
- * 2^23 voxels, and larger), each on its own stream; within a lane every brick
+ * Active requests are advanced in lanes by voxel count (below 2^19, 2^21, 2^23
+ * voxels, and larger) and by what launches together (radius, image type, storage,
+ * form), up to 16, each on its own stream; within a lane every brick
  * advances one iteration per tick, in dispatches of one to eight ticks: while
  * no brick of the lane is due to finish and nothing waits in the queue, a
  * dispatch enqueues several ticks without a host round trip.

@@ -479,12 +479,17 @@ namespace {
 template <int R, class ImgT>
 cudaError_t ki_init_r(const TiledGroup &g, cudaStream_t s) {
     constexpr size_t sm = tiled::XYSmem<R, tiled::SrcI<R, ImgT>>::bytes;
-    static_assert(sm <= 48 * 1024, "k_ki_xy needs no shared-memory opt-in");
+    static_assert(sm <= 48 * 1024 && tiled::ki_smem<R>() <= 48 * 1024, "no shared-memory opt-in");
     const tiled::TapPairs tp = tiled::tap_pairs(g.taps);
     tiled::GroupArgs G{g.bricks, g.starts[0], g.nb, 0, g.err, 0u};
     tiled::k_ki_xy<R, ImgT><<<g.ncta[0], tiled::kXYThreads, sm, s>>>(G, tp);
     G.starts = g.starts[1];
-    tiled::k_ki_z<R><<<g.ncta[1], tiled::kAZThreads, 0, s>>>(G, tp);
+    int dev = 0, sms = 0;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (e != cudaSuccess) return e;
+    const unsigned most = (unsigned)(tiled::kAZCtas * sms);
+    tiled::k_ki_z<R><<<g.ncta[1] < most ? g.ncta[1] : most, tiled::kAZThreads, tiled::ki_smem<R>(), s>>>(G, tp);
     return cudaGetLastError();
 }
 template <int R>

@@ -11,9 +11,9 @@
 //              image by TMA; forms H I~ and H (Eqs. 6, 8-10; the image centred)
 //              as it reads them, convolves the pair along x then y (packed f32x2
 //              FMAs) and stores it (FP32).
-//   rsf_ta_z   x-z slabs (32 columns x 64 output planes) staged in shared
-//              memory by cp.async, two slabs in flight; z convolution over a
-//              register window; the local fits f1 = K*(H I~)/K*H and
+//   rsf_ta_z   x-z slabs (32 columns x 64 output planes) brought to shared
+//              memory by TMA, two slabs in flight; z convolution streamed into
+//              eight accumulators per column; the local fits f1 = K*(H I~)/K*H and
 //              f2 = K*((1-H) I~)/K*(1-H), the latter from the linearity of the
 //              convolution as (K*I~ - K*(H I~)) / (K*1 - K*H) with K*I~ fixed
 //              for the solve (rsf_ki_xy / rsf_ki_z, once) and K*1 the product of

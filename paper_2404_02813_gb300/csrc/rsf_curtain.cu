@@ -102,34 +102,71 @@ struct MergeArgs {
     int n[3], nb[3];
 };
 
-// A warp per output row: the y and z tables are read once per row.
+// A warp per output row: the y and z tables are read once per row.  A voxel's sum is a chain of
+// table, pointer and value loads (0.12 of the copy rate with one voxel at a time per lane), so a
+// lane sums four columns side by side, the x tables of their first sub-volume read up front (most
+// columns have no other).  320 x 288 x 256 from 12
+// sub-volumes of 160^3: 0.237 -> 0.175 ms, still the chain per row and sub-volume.
+constexpr int kMergeCols = 4;
 __global__ void __launch_bounds__(256) k_merge(MergeArgs a, float *__restrict__ out) {
     const int nx = a.n[0], lane = threadIdx.x & 31;
     const long long rows = (long long)a.n[1] * a.n[2];
     for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
          r += ((long long)gridDim.x * blockDim.x) >> 5) {
         const int y = (int)(r % a.n[1]), z = (int)(r / a.n[1]);
-        const int cz = a.count[2][z], cy = a.count[1][y];
-        for (int x = lane; x < nx; x += 32) {
-            float num = 0.f, den = 0.f;
-            const int cx = a.count[0][x];
+        const int cz = __ldg(a.count[2] + z), cy = __ldg(a.count[1] + y);
+        for (int x0 = lane; x0 < nx; x0 += 32 * kMergeCols) {
+            float num[kMergeCols], den[kMergeCols], w0[kMergeCols];
+            int cx[kMergeCols], k0[kMergeCols], l0[kMergeCols], e0[kMergeCols];
+            int most = 0;
+#pragma unroll
+            for (int c = 0; c < kMergeCols; ++c) {
+                const int x = min(x0 + 32 * c, nx - 1);  // a column past the row repeats the last one
+                cx[c] = __ldg(a.count[0] + x);
+                k0[c] = __ldg(a.box[0] + x * kMaxCover);
+                l0[c] = __ldg(a.local[0] + x * kMaxCover);
+                w0[c] = __ldg(a.weight[0] + x * kMaxCover);
+                num[c] = den[c] = 0.f;
+            }
+#pragma unroll
+            for (int c = 0; c < kMergeCols; ++c) {
+                e0[c] = __ldg(a.ext[0] + k0[c]);
+                most = max(most, cx[c]);
+            }
             for (int iz = 0; iz < cz; ++iz) {
-                const int kz = a.box[2][z * kMaxCover + iz], lz = a.local[2][z * kMaxCover + iz];
-                const float wz = a.weight[2][z * kMaxCover + iz];
+                const int kz = __ldg(a.box[2] + z * kMaxCover + iz), lz = __ldg(a.local[2] + z * kMaxCover + iz);
+                const float wz = __ldg(a.weight[2] + z * kMaxCover + iz);
                 for (int iy = 0; iy < cy; ++iy) {
-                    const int ky = a.box[1][y * kMaxCover + iy], ly = a.local[1][y * kMaxCover + iy];
-                    const float wzy = wz * a.weight[1][y * kMaxCover + iy];
-                    const int ey = a.ext[1][ky];
-                    for (int ix = 0; ix < cx; ++ix) {
-                        const int kx = a.box[0][x * kMaxCover + ix], lx = a.local[0][x * kMaxCover + ix];
-                        const float w = wzy * a.weight[0][x * kMaxCover + ix];
-                        const float *p = a.phi[((long long)kz * a.nb[1] + ky) * a.nb[0] + kx];
-                        num = fmaf(w, p[((long long)lz * ey + ly) * a.ext[0][kx] + lx], num);
-                        den += w;
+                    const int ky = __ldg(a.box[1] + y * kMaxCover + iy), ly = __ldg(a.local[1] + y * kMaxCover + iy);
+                    const float wzy = wz * __ldg(a.weight[1] + y * kMaxCover + iy);
+                    const long long row = (long long)lz * __ldg(a.ext[1] + ky) + ly;
+                    const float *const *const phi = a.phi + ((long long)kz * a.nb[1] + ky) * a.nb[0];
+                    const float *p[kMergeCols];
+                    float v[kMergeCols];
+#pragma unroll
+                    for (int c = 0; c < kMergeCols; ++c) p[c] = phi[k0[c]];
+#pragma unroll
+                    for (int c = 0; c < kMergeCols; ++c) v[c] = __ldg(p[c] + row * e0[c] + l0[c]);
+#pragma unroll
+                    for (int c = 0; c < kMergeCols; ++c) {
+                        const float w = wzy * w0[c];
+                        num[c] = fmaf(w, v[c], num[c]);
+                        den[c] += w;
                     }
+                    for (int ix = 1; ix < most; ++ix)
+#pragma unroll
+                        for (int c = 0; c < kMergeCols; ++c)
+                            if (ix < cx[c]) {
+                                const int i = min(x0 + 32 * c, nx - 1) * kMaxCover + ix, kx = __ldg(a.box[0] + i);
+                                const float w = wzy * __ldg(a.weight[0] + i);
+                                num[c] = fmaf(w, __ldg(phi[kx] + row * __ldg(a.ext[0] + kx) + __ldg(a.local[0] + i)), num[c]);
+                                den[c] += w;
+                            }
                 }
             }
-            out[r * nx + x] = num / den;
+#pragma unroll
+            for (int c = 0; c < kMergeCols; ++c)
+                if (x0 + 32 * c < nx) out[r * nx + x0 + 32 * c] = num[c] / den[c];
         }
     }
 }

@@ -543,7 +543,7 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         if (exact)
             rsf::exact_place_fields(b, f.t[0], f.q);
         else
-            rsf::tiled_place_fields(b, storage, force, (int)vt, f.t[0], sizeof(float) * 8 * (size_t)f.px * ny * nz, f.q, nullptr);
+            rsf::tiled_place_fields(b, storage, force, (int)vt, f.t[0], sizeof(float) * 8 * (size_t)f.px * ny * nz, f.q);
         b.eps = eps;
         b.lambda1 = lambda1;
         b.lambda2 = lambda2;

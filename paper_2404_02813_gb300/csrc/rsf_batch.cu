@@ -41,15 +41,13 @@ struct BrickState {
 size_t align256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 // Device bytes one brick needs in the pool.
-size_t brick_bytes(const rsf_brick &b, int storage, int force, bool stage_image) {
+size_t brick_bytes(const rsf_brick &b, int storage, bool stage_image) {
     const long long n = (long long)b.nx * b.ny * b.nz;
     const long long np = (long long)rsf::tiled_pitch((int)b.nx) * b.ny * b.nz;
     size_t s = 4 * align256(sizeof(float) * n);                          // phi[2], q block
     s += align256(sizeof(float) * (b.nx + b.ny + b.nz)) + align256(64);  // profiles, centring constants
     s += align256(rsf::tiled_stage_bytes(storage, np));
-    if (stage_image) s += align256(dtype_size(b.vt) * n);
-    return s + align256(rsf::tiled_extra_bytes(stage_image ? nullptr : b.volume, (int)b.nx, (int)b.ny, (int)b.nz,
-                                               (int)b.vt, storage, force));
+    return stage_image ? s + align256(dtype_size(b.vt) * n) : s;
 }
 
 int default_zc(const std::vector<rsf::BrickDev> &g, int sms) {
@@ -216,7 +214,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
     size_t total = 0;
     for (int i = 0; i < nb; ++i) {
         stage_img[i] = !on_device(bricks[i].volume);
-        total += brick_bytes(bricks[i], storage, force, stage_img[i]);
+        total += brick_bytes(bricks[i], storage, stage_img[i]);
     }
     if (total > c->pool_cap) {
         dev_free(c, c->pool, c->pool_cap);
@@ -264,9 +262,9 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         d.ny = (int)b.ny;
         d.nz = (int)b.nz;
         for (int k = 0; k < 2; ++k) d.phi[k] = reinterpret_cast<float *>(take(sizeof(float) * n));
-        void *q = take(2 * align256(sizeof(float) * n));
         rsf::zero_padding_profiles(make_taps(b.sigma), d.nx, d.ny, d.nz, reinterpret_cast<float *>(prof_host.data() + prof_at[i]));
         float *cs = reinterpret_cast<float *>(take(64));
+        void *q = take(rsf::tiled_q_bytes(d.nx, (long long)d.ny * d.nz));  // the stage block follows
         d.prof = reinterpret_cast<float *>(prof0 + prof_at[i]);
         d.cs = cs;
         const size_t stage_bytes = rsf::tiled_stage_bytes(storage, (long long)rsf::tiled_pitch(d.nx) * b.ny * b.nz);
@@ -278,8 +276,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         } else {
             d.img = b.volume;
         }
-        rsf::tiled_place_fields(d, storage, force, (int)b.vt, stage, stage_bytes, q,
-                                take(rsf::tiled_extra_bytes(d.img, d.nx, d.ny, d.nz, (int)b.vt, storage, force)));
+        rsf::tiled_place_fields(d, storage, force, (int)b.vt, stage, stage_bytes, q);
         d.eps = b.eps;
         d.lambda1 = b.lambda1;
         d.lambda2 = b.lambda2;

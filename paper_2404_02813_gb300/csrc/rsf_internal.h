@@ -91,6 +91,7 @@ void set_last_error(const char *msg);
 // scalars.  Device copies of these descriptors drive the batched launches.
 struct BrickDev {
     int nx, ny, nz, px;     // dimensions; x pitch of the intermediate fields
+    int up;                 // x pitch of u2: px, or nx where a copied image needs the room (tiled_place_fields)
     const void *img;        // image, nx*ny*nz values of the group's image type
     const void *img_t;      // the image as the TMA boxes read it: img, or a copy with 16-byte rows
     int ip;                 // row pitch of img_t (values)
@@ -163,14 +164,13 @@ int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int s
 // Planes per CTA of the update kernel (at most zc) for bricks launched together with z chunk zc.
 int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, int zc, int sms);
 // A brick's working memory beside its phi buffers: a stage block of
-// tiled_stage_bytes(storage, px ny nz) bytes, a q block of 8 nx ny nz bytes, and
-// tiled_extra_bytes (0 unless both are too small for a copied image).
+// tiled_stage_bytes(storage, px ny nz) bytes, and directly in front of it a q block of
+// tiled_q_bytes(nx, ny nz) bytes (anywhere for a stage block of 28 px ny nz bytes or more).
 size_t tiled_stage_bytes(int storage, long long np);
-size_t tiled_extra_bytes(const void *img, int nx, int ny, int nz, int imgtype, int storage, int force);
+size_t tiled_q_bytes(int nx, long long rows);
 // Sets b's pitches and field pointers from its dimensions and image (b.nx, ny, nz, img) in
-// those three blocks (256-byte aligned; stage may be larger than the minimum).
-void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q,
-                        void *extra);
+// those two blocks (256-byte aligned; stage may be larger than the minimum).
+void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q);
 // One brick's work before the first iteration, for kernels that take many bricks at once
 // (blockIdx.y): image statistics, phi0 to phi (or nothing where they are the same), q of it,
 // the image copied to img_t where that differs.

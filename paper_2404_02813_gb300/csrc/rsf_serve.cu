@@ -183,14 +183,12 @@ void CUDART_CB done_cb(void *p) {
 
 // Device bytes of one served brick: phi and q pairs, profiles, centring
 // constants, the pitched intermediate fields and (host images) a device copy.
-size_t footprint(const rsf_request &r, int force, bool stage_image) {
+size_t footprint(const rsf_request &r, bool stage_image) {
     const long long n = (long long)r.nx * r.ny * r.nz;
     const long long np = (long long)rsf::tiled_pitch((int)r.nx) * r.ny * r.nz;
     size_t b = 4 * align256(sizeof(float) * n) + align256(sizeof(float) * (r.nx + r.ny + r.nz)) + align256(64);
     b += align256(rsf::tiled_stage_bytes((int)r.storage, np));
-    if (stage_image) b += align256(dtype_size(r.vt) * n);
-    return b + align256(rsf::tiled_extra_bytes(stage_image ? nullptr : r.volume, (int)r.nx, (int)r.ny, (int)r.nz, (int)r.vt,
-                                               (int)r.storage, force));
+    return stage_image ? b + align256(dtype_size(r.vt) * n) : b;
 }
 
 // Finish a request that never became active (or failed in set-up).
@@ -232,7 +230,7 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
         return false;
     }
     const bool stage_img = !on_device(q.volume);
-    r->bytes = footprint(q, r->force, stage_img);
+    r->bytes = footprint(q, stage_img);
     {
         std::lock_guard<std::mutex> lk(c->alloc_mu);
         c->used += r->bytes;
@@ -274,11 +272,11 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
     d.ny = (int)q.ny;
     d.nz = (int)q.nz;
     for (int k = 0; k < 2; ++k) d.phi[k] = reinterpret_cast<float *>(take(sizeof(float) * n));
-    void *qb = take(2 * align256(sizeof(float) * n));
     float *prof = reinterpret_cast<float *>(take(sizeof(float) * (q.nx + q.ny + q.nz)));
     float *cs = reinterpret_cast<float *>(take(64));
     d.prof = prof;
     d.cs = cs;
+    void *qb = take(rsf::tiled_q_bytes(d.nx, (long long)d.ny * d.nz));  // the stage block follows
     const size_t stage_bytes = rsf::tiled_stage_bytes(r->storage, (long long)rsf::tiled_pitch(d.nx) * q.ny * q.nz);
     void *stage = take(stage_bytes);
     if (stage_img) {
@@ -289,8 +287,7 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
     } else {
         d.img = q.volume;
     }
-    rsf::tiled_place_fields(d, r->storage, r->force, (int)q.vt, stage, stage_bytes, qb,
-                            take(rsf::tiled_extra_bytes(d.img, d.nx, d.ny, d.nz, (int)q.vt, r->storage, r->force)));
+    rsf::tiled_place_fields(d, r->storage, r->force, (int)q.vt, stage, stage_bytes, qb);
     d.eps = q.eps;
     d.lambda1 = q.lambda1;
     d.lambda2 = q.lambda2;
@@ -519,7 +516,7 @@ void loop(Server *s) {
                     lk.lock();
                     continue;
                 }
-                const size_t need = footprint(r->req, r->force, !on_device(r->req.volume));
+                const size_t need = footprint(r->req, !on_device(r->req.volume));
                 uint64_t used, budget;
                 {
                     std::lock_guard<std::mutex> al(c->alloc_mu);
@@ -672,7 +669,7 @@ extern "C" rsf_status rsf_submit(rsf_ctx *c, const rsf_request *req, uint64_t *t
                            2 * (int64_t)req->halo >= req->nz))
         return fail(RSF_E_INVAL, "halo %d leaves no core in a %lld x %lld x %lld brick", (int)req->halo,
                     (long long)req->nx, (long long)req->ny, (long long)req->nz);
-    const size_t need = footprint(*req, c->opt_force, !on_device(req->volume));
+    const size_t need = footprint(*req, !on_device(req->volume));
     if (need > c->budget)
         return fail(RSF_E_NOMEM, "request needs %zu bytes of device memory; the budget is %llu", need,
                     (unsigned long long)c->budget);

@@ -618,7 +618,7 @@ __global__ void __launch_bounds__(kXYThreads, (SrcH<R, ImgT, NP, EX>::CTAS)) k_t
     const BrickDev &B = G.bricks[b];
     const XYTile tl = xy_tile_of<R>(blockIdx.x - __ldg(G.starts + b), B);
     const SrcH<R, ImgT, NP, EX> src{&B.tm_q, &B.tm_img, EX ? 1.f : B.cs[1], EX ? 0.f : -B.cs[0] * B.cs[1]};
-    const OutXY out{reinterpret_cast<float *>(B.u2), B.px, (long long)B.px * B.ny};
+    const OutXY out{reinterpret_cast<float *>(B.u2), B.up, (long long)B.up * B.ny};
     xy_tile<R>(G, src, out, B.nx, B.ny, B.nz, tl.x0, tl.y0, tl.za, B.xyp, t, xsm);
 }
 

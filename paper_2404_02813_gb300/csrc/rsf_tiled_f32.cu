@@ -230,7 +230,7 @@ cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, 
     }
     if (e != cudaSuccess) return e;
     if (force != 0) {  // four fields per voxel, no K*I~; the Eq. (15) form: no group B
-        e = encode_map(&b.tm_u, b.u2, 4, b, 128, 1, zrows);
+        e = encode_typed(&b.tm_u, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, b.u2, 4, b.up, b, 128, 1, zrows);
         if (e != cudaSuccess || force == 1) return e;
         return encode_map(&b.tm_ab, b.ab, 2, b, 2 * box.ab32, box.rows, 1);
     }
@@ -453,18 +453,12 @@ size_t field_bytes(int storage, int force, long long np) { return (size_t)(force
 int q_pitch(int nx) { return (nx + 3) / 4 * 4; }
 }  // namespace
 
-size_t tiled_extra_bytes(const void *img, int nx, int ny, int nz, int imgtype, int storage, int force) {
-    if (!copied_image(img, nx, imgtype)) return 0;
-    const long long rows = (long long)ny * nz, np = tiled_pitch(nx) * rows;
-    const size_t need = (size_t)image_size(imgtype) * image_pitch(nx, imgtype) * rows;
-    if (field_bytes(storage, force, np) + need <= tiled_stage_bytes(storage, np)) return 0;
-    return 4ull * q_pitch(nx) * rows + need <= 8ull * nx * rows ? 0 : need;
-}
+size_t tiled_q_bytes(int nx, long long rows) { return 2 * ((sizeof(float) * nx * rows + 255) / 256 * 256); }
 
 // Per pitched voxel: both x/y-convolved pairs 16 bytes (then, in the same memory, the
 // x/y-convolved (a, b)), (a, b) 8, the centred image at most 4.
 void exact_place_fields(BrickDev &b, void *stage, float *q) {
-    b.px = tiled_pitch(b.nx);
+    b.px = b.up = tiled_pitch(b.nx);
     const long long np = (long long)b.px * b.ny * b.nz;
     char *p = static_cast<char *>(stage);
     b.u2 = b.abxy = reinterpret_cast<float2 *>(p);
@@ -480,10 +474,9 @@ size_t exact_stage_bytes(int nx, int ny, int nz) {
 size_t exact_q_bytes(int nx, int ny, int nz) { return 4ull * q_pitch(nx) * ny * nz; }
 bool exact_supports(int R) { return R >= 1 && R <= RMAX; }
 
-void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q,
-                        void *extra) {
+void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *stage, size_t stage_bytes, void *q) {
     const long long rows = (long long)b.ny * b.nz;
-    b.px = tiled_pitch(b.nx);
+    b.px = b.up = tiled_pitch(b.nx);
     const long long np = b.px * rows;
     char *p = static_cast<char *>(stage);
     b.u2 = reinterpret_cast<float2 *>(p);
@@ -504,9 +497,21 @@ void tiled_place_fields(BrickDev &b, int storage, int force, int imgtype, void *
         b.ip = image_pitch(b.nx, imgtype);
         const size_t need = (size_t)image_size(imgtype) * b.ip * rows, used = field_bytes(storage, force, np);
         const size_t qb = 4ull * b.qp * rows;  // a multiple of 16
-        b.img_t = used + need <= stage_bytes ? p + used
-                                             : (qb + need <= 8ull * b.nx * rows ? static_cast<char *>(q) + qb
-                                                                                : static_cast<char *>(extra));
+        if (used + need <= stage_bytes) {
+            b.img_t = p + used;
+        } else {
+            b.img_t = static_cast<char *>(q) + qb;
+            if (qb + need > tiled_q_bytes(b.nx, rows)) {
+                // Eq. (15) form, 24 bytes per voxel of stage, FP32 rows of 4 k + 1 .. 3 values (or
+                // short rows): the image runs on into the stage block behind the q block, by at
+                // most 8 (qp - nx) bytes a row, and the pair field, without padded columns, ends
+                // 16 (px - nx) bytes a row earlier
+                const size_t spill = qb + need - tiled_q_bytes(b.nx, rows);
+                b.up = b.nx;
+                b.u2 = reinterpret_cast<float2 *>(p + spill);
+                b.abxy = reinterpret_cast<float2 *>(p + spill + 16ull * b.nx * rows);
+            }
+        }
     }
 }
 

@@ -52,7 +52,12 @@ def algo_bytes_per_voxel(img: int, st: int, force: str = "li") -> dict:
     }
 
 
-SETUP_LAUNCHES = 5  # statistics, their reduction, q of phi0, K*I~ (x/y pass, z pass)
+def setup_launches(force: str = "li") -> int:
+    """Of a call, for any number of bricks of one radius and image type: statistics, their
+    reduction, start (q of phi0, copied image); Li's form: K*I~ (x/y pass, z pass)."""
+    return 3 if force == "eq15" else 5
+
+
 NOMINAL_HBM_GBS = 7900.0
 # The paper's Table 1: one time step on a 500^3 volume takes 585 ms summed over
 # its kernels (Eq. (15) form, sigma_2 = 0), i.e. 1.25e8 / 0.585 s voxel-iterations/s.
@@ -61,21 +66,20 @@ PAPER_TABLE1_GVOX_IT_S = 1.25e8 / 0.585 / 1e9
 # DRAM traffic per voxel measured by ncu (dram__bytes_read.sum + dram__bytes_write.sum
 # per launch / voxels), keyed by kernel, with the SHA-256 of the kernel source file
 # it was captured from; reported only while that file is unchanged.
-NCU_SHA = "25911c66532ecdf4"
+NCU_SHA = "ca018349217ab567"
 NCU_TRAFFIC = {
     k: {"bytes_per_voxel": v, "source": "rsf_tiled.cuh", "source_sha": NCU_SHA,
         "capture": "384^3 uint16 light-sheet case, sigma 3, FP32 storage; scaled by voxels"}
-    for k, v in {"rsf_ta_xy": 13.20, "rsf_ta_z": 19.43, "rsf_tb_xy": 15.25, "rsf_tb_z": 21.98}.items()
+    for k, v in {"rsf_ta_xy": 13.39, "rsf_ta_z": 19.36, "rsf_tb_xy": 15.15, "rsf_tb_z": 21.62}.items()
 }
 
 # Warp instructions issued per voxel measured by ncu (smsp__inst_executed.sum / voxels),
-# same capture conditions and gating as NCU_TRAFFIC.  The kernels are issue-bound;
-# against one warp instruction per cycle per SM sub-partition (4 per SM) this gives
-# the issue roofline.
+# same capture conditions and gating as NCU_TRAFFIC; against one warp instruction per
+# cycle per SM sub-partition (4 per SM) this gives the issue roofline.
 NCU_INST = {
     k: {"warp_inst_per_voxel": v, "source": "rsf_tiled.cuh", "source_sha": NCU_SHA,
         "capture": "384^3 uint16 light-sheet case, sigma 3, FP32 storage"}
-    for k, v in {"rsf_ta_xy": 3.13, "rsf_ta_z": 2.78, "rsf_tb_xy": 2.21, "rsf_tb_z": 6.39}.items()
+    for k, v in {"rsf_ta_xy": 2.87, "rsf_ta_z": 2.42, "rsf_tb_xy": 1.68, "rsf_tb_z": 3.56}.items()
 }
 SM_SUBPARTITIONS = 4  # warp schedulers per SM, one warp instruction issued per cycle each
 
@@ -348,7 +352,7 @@ def run_batch(args, rank, world, local):
             "kernels": {k: {"launches": n, "ms": round(m, 3)} for k, (n, m) in prof.items() if n},
             "autotune": tuned,
             "clocks": clk,
-            "gpu_launches": (4 * iters + 5 * nb) * args.steps,  # per brick set-up: statistics (2), q, K*I~ (2)
+            "gpu_launches": (4 * iters + setup_launches()) * args.steps,
             "e2e": e2e,
         }
         if world == 1 and not args.no_cpu_baseline:
@@ -949,8 +953,8 @@ def main():
                      "note": "instruction issue roofline of the dominant kernel: ncu-counted warp instructions "
                              "per voxel x voxels / CUDA-event launch time, against one issue per cycle per SM "
                              "sub-partition at the sampled SM clock"}
-        launches = sum(n for n, _ in prof.values()) + (SETUP_LAUNCHES * args.steps if not args.curtain
-                                                       else (7 * nbox + 1) * args.steps)
+        launches = sum(n for n, _ in prof.values()) + (
+            setup_launches(force) + (2 if args.curtain else 0)) * args.steps  # the curtain's gather and merge
         line = {
             "metric": "GVoxel-iterations/s", "value": value, "unit": "GVoxel-iterations/s", "n_gpus": world,
             "steps": args.steps, "warmup": args.warmup, "ms_per_step": ms_max / args.steps,

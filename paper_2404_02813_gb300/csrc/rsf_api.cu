@@ -337,7 +337,8 @@ cudaError_t xfer(void *dst, const void *src, size_t bytes, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-bool in_place(const void *p, int dev) {
+bool in_place(const void *p, int dev, size_t size) {
+    if (reinterpret_cast<uintptr_t>(p) % size != 0) return false;
     cudaPointerAttributes a;
     if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
         cudaGetLastError();

@@ -91,8 +91,10 @@ rsf_status device_error(const rsf_ctx *c);
 rsf_status dev_alloc(rsf_ctx *c, void **p, size_t bytes);
 void dev_free(rsf_ctx *c, void *p, size_t bytes);
 bool on_device(const void *p);
-// Device memory of device `dev` (or managed memory), which its kernels may use in place.
-bool in_place(const void *p, int dev);
+// Memory that kernels of device `dev` may use in place as values of `size` bytes: device memory of
+// that device (another GPU's is only reached by copies) or managed memory, aligned to the value
+// (a copy takes any address, a kernel's load does not).
+bool in_place(const void *p, int dev, size_t size = sizeof(float));
 // Copy `bytes` on stream s between any two of device, pinned host and pageable
 // host memory; pinned host memory is read or written by a copy kernel.
 cudaError_t xfer(void *dst, const void *src, size_t bytes, cudaStream_t s);

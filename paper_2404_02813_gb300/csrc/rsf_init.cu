@@ -391,16 +391,17 @@ extern "C" rsf_status rsf_init_phi0(rsf_ctx *c, const void *volume, rsf_dtype vt
     const long long n = nx * ny * nz, plane = nx * ny;
     const size_t es = dtype_size(vt);
     auto align = [](size_t b) { return (b + 255) & ~size_t(255); };
-    const bool host_vol = !on_device(volume), host_phi = !on_device(phi0_out);
-    // device destinations are written in place, unless they share memory with something still read
+    const bool host_vol = !on_device(volume), host_phi = !in_place(phi0_out, c->device);
+    // destinations that this device's kernels may write are written in place, unless they share
+    // memory with something still read
     const auto overlap = [](const void *a, size_t na, const void *b, size_t nb) {
         const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
         return a && b && x < y + nb && y < x + na;
     };
     const size_t fb = sizeof(float) * (size_t)n;
     const bool shared = overlap(response_out, fb, seeds_out, n);
-    const bool own_D = !response_out || !on_device(response_out) || shared || overlap(response_out, fb, volume, es * n);
-    const bool own_mask = !seeds_out || !on_device(seeds_out) || shared || overlap(seeds_out, n, volume, es * n);
+    const bool own_D = !response_out || !in_place(response_out, c->device) || shared || overlap(response_out, fb, volume, es * n);
+    const bool own_mask = !seeds_out || !in_place(seeds_out, c->device, 1) || shared || overlap(seeds_out, n, volume, es * n);
     size_t bytes = align(sizeof(uint16_t) * n) + align(sizeof(float) * n) + align(sizeof(int) * nz) + 256;
     if (own_D) bytes += align(sizeof(float) * n);
     if (own_mask) bytes += align(n);

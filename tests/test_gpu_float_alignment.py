@@ -1,5 +1,6 @@
-"""phi0 and phi_out in device memory at addresses that no float may be read or written at: such
-buffers are copied, as host buffers are, and the results are the bits of aligned ones."""
+"""phi0, phi_out and the outputs of rsf_init_phi0 in device memory at addresses that no float may be
+read or written at: such buffers are copied, as host buffers are, and the results are the bits of
+aligned ones."""
 import ctypes
 
 import numpy as np
@@ -81,3 +82,24 @@ def test_batch_and_serving(ctx, off0, off1):
     assert L.rsf_wait(served.handle, t, 60000) == 0
     served.close()
     assert _floats(dst, off1) == ref
+
+
+@pytest.mark.parametrize("off", [1, 2, 3])
+@pytest.mark.parametrize("phi_off", [0, 1])
+def test_init_outputs(ctx, off, phi_off):
+    rng = np.random.default_rng(7)
+    vol = rng.normal(0.0, 1.0, size=SHAPE).astype(np.float32)
+    vol[5, 5:8, 20:23] += 60.0
+    vol = torch.from_numpy(vol).cuda()
+    seeds = torch.zeros(SHAPE, dtype=torch.uint8, device="cuda")
+    resp = torch.empty(SHAPE, dtype=torch.float32, device="cuda")
+    phi, n = ctx.init_phi0(vol, 1.5, 0.3, 2.0, seeds=seeds, response=resp)
+    dst, out, mask = _bytes_at(None, off), _bytes_at(None, phi_off), torch.zeros(N + 1, dtype=torch.uint8, device="cuda")
+    torch.cuda.synchronize()
+    nz, ny, nx = SHAPE
+    k = ctypes.c_int64()
+    st = rsf.load_library().rsf_init_phi0(ctx.handle, vol.data_ptr(), rsf.RSF_F32, nx, ny, nz, 1.5, 0.3, 2.0,
+                                          out.data_ptr() + phi_off, ctypes.byref(k), mask.data_ptr() + 1, dst.data_ptr() + off)
+    assert st == 0 and k.value == n > 0
+    assert _floats(dst, off) == resp.cpu().numpy().tobytes() and _floats(out, phi_off) == phi.cpu().numpy().tobytes()
+    assert mask[1:].cpu().numpy().tobytes() == seeds.cpu().numpy().tobytes()

@@ -346,7 +346,7 @@ bool in_place(const void *p, int dev, size_t size) {
     }
     return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
 }
-static bool overlap(const void *a, size_t na, const void *b, size_t nb) {
+bool share_bytes(const void *a, size_t na, const void *b, size_t nb) {
     const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
     return a && b && x < y + nb && y < x + na;
 }
@@ -523,9 +523,10 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     bool phi0_here = false, out_here = false;
     if ((tiled || exact) && iters > 0) {
         const size_t sb = dump ? RSF_NSTAGES * fb : 0;
-        phi0_here = in_place(phi0, c->device) && !overlap(phi0, fb, dump, sb) && !(iters == 1 && overlap(phi0, fb, phi_out, fb));
-        out_here = in_place(phi_out, c->device) && !overlap(phi_out, fb, vol, dtype_size(vt) * (size_t)n) &&
-                   !overlap(phi_out, fb, dump, sb);
+        phi0_here = in_place(phi0, c->device) && !share_bytes(phi0, fb, dump, sb) &&
+                    !(iters == 1 && share_bytes(phi0, fb, phi_out, fb));
+        out_here = in_place(phi_out, c->device) && !share_bytes(phi_out, fb, vol, dtype_size(vt) * (size_t)n) &&
+                   !share_bytes(phi_out, fb, dump, sb);
     }
     if (!phi0_here) RSF_CUDA(xfer(f.phi[0], phi0, fb, c->stream));
     int cur = 0;

@@ -95,6 +95,8 @@ bool on_device(const void *p);
 // that device (another GPU's is only reached by copies) or managed memory, aligned to the value
 // (a copy takes any address, a kernel's load does not).
 bool in_place(const void *p, int dev, size_t size = sizeof(float));
+// Whether [a, a + na) and [b, b + nb) have a byte in common (null shares nothing).
+bool share_bytes(const void *a, size_t na, const void *b, size_t nb);
 // Copy `bytes` on stream s between any two of device, pinned host and pageable
 // host memory; pinned host memory is read or written by a copy kernel.
 cudaError_t xfer(void *dst, const void *src, size_t bytes, cudaStream_t s);

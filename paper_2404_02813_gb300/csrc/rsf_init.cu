@@ -394,14 +394,10 @@ extern "C" rsf_status rsf_init_phi0(rsf_ctx *c, const void *volume, rsf_dtype vt
     const bool host_vol = !on_device(volume), host_phi = !in_place(phi0_out, c->device);
     // destinations that this device's kernels may write are written in place, unless they share
     // memory with something still read
-    const auto overlap = [](const void *a, size_t na, const void *b, size_t nb) {
-        const uintptr_t x = reinterpret_cast<uintptr_t>(a), y = reinterpret_cast<uintptr_t>(b);
-        return a && b && x < y + nb && y < x + na;
-    };
     const size_t fb = sizeof(float) * (size_t)n;
-    const bool shared = overlap(response_out, fb, seeds_out, n);
-    const bool own_D = !response_out || !in_place(response_out, c->device) || shared || overlap(response_out, fb, volume, es * n);
-    const bool own_mask = !seeds_out || !in_place(seeds_out, c->device, 1) || shared || overlap(seeds_out, n, volume, es * n);
+    const bool shared = share_bytes(response_out, fb, seeds_out, n);
+    const bool own_D = !response_out || !in_place(response_out, c->device) || shared || share_bytes(response_out, fb, volume, es * n);
+    const bool own_mask = !seeds_out || !in_place(seeds_out, c->device, 1) || shared || share_bytes(seeds_out, n, volume, es * n);
     size_t bytes = align(sizeof(uint16_t) * n) + align(sizeof(float) * n) + align(sizeof(int) * nz) + 256;
     if (own_D) bytes += align(sizeof(float) * n);
     if (own_mask) bytes += align(n);
@@ -451,14 +447,15 @@ extern "C" rsf_status rsf_init_phi0(rsf_ctx *c, const void *volume, rsf_dtype vt
     k_seeds<<<dim3((unsigned)((nx + 31) / 32), (unsigned)((ny + kSeedRows - 1) / kSeedRows), (unsigned)nz), 256, 0, s>>>(D, smax, mask, count, (int)nx, (int)ny, rel_threshold);
     k_dist_x<<<(unsigned)std::min<long long>(4864, (ny * nz + 7) / 8), 256, 0, s>>>(mask, dx, (int)nx, ny * nz);
     RSF_CUDA(cudaGetLastError());
+    // outputs that share memory are written in the order response, mask, phi0
+    if (response_out && own_D) RSF_CUDA(xfer(response_out, D, fb, s));
+    if (seeds_out && own_mask) RSF_CUDA(xfer(seeds_out, mask, n, s));
     RSF_CUDA((dist_line<true, false>(dx, dxy, (int)nx, (int)ny, nx, (int)nz, plane, r0, count, s)));
     RSF_CUDA((dist_line<false, true>(dxy, phi, (int)nx, (int)nz, plane, (int)ny, nx, r0, count, s)));
     unsigned long long found = 0;
     RSF_CUDA(cudaMemcpyAsync(&found, count, sizeof(found), cudaMemcpyDeviceToHost, s));
     RSF_CUDA(cudaStreamSynchronize(s));
     *nseeds = (int64_t)found;
-    if (response_out && own_D) RSF_CUDA(xfer(response_out, D, sizeof(float) * n, s));
-    if (seeds_out && own_mask) RSF_CUDA(xfer(seeds_out, mask, n, s));
     if (found && host_phi) RSF_CUDA(xfer(phi0_out, phi, sizeof(float) * n, s));
     RSF_CUDA(cudaStreamSynchronize(s));
     if (found == 0) return fail(RSF_E_INVAL, "no seed found (relative threshold %g)", (double)rel_threshold);

@@ -460,6 +460,9 @@ rsf_status rsf_prof_get(rsf_ctx *ctx, int32_t kernel, int64_t *launches, double 
  * All calls on a device share the array and it keeps the last call's
  * contents (nothing in it needs to start at zero); calls whose work overlaps
  * on the GPU race on it and must be serialised by the caller.
+ * The kernels wait for their own copies for a bounded time (1 s each).  Should
+ * such a wait run out, phi_out is NaN in every voxel: the call has returned by
+ * then and cannot say so.
  * Errors: RSF_E_INVAL (arguments, size limit), RSF_E_CUDA (launch failures).
  */
 rsf_status rsf_evolve_noalloc(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int64_t nz,

@@ -27,6 +27,7 @@
 #include "rsf.h"
 #include "rsf_ctx.h"
 #include "rsf_internal.h"
+#include "rsf_tiled.cuh"
 
 namespace {
 
@@ -41,7 +42,7 @@ constexpr long long kOffPart = kOffCs + 64;              // reduction partials
 constexpr long long kScratchFloats = kOffPart + 3 * rsf::kStatBlocks;
 constexpr int kMaxDevices = 64;
 // The tiled kernels' fields take the same memory from kOffI on: launch descriptor (with the
-// CTA offsets after it), q and stage blocks, where the x pitch (a multiple of 32) leaves room
+// CTA offsets and the error word after it), q and stage blocks, where the x pitch (a multiple of 32) leaves room
 // for them: always when nx is a multiple of 32, or below about 0.8 of the voxel limit at nx >= 33.
 constexpr size_t kDescBytes = (sizeof(rsf::BrickDev) + 64 + 255) / 256 * 256;
 constexpr size_t kFieldBytes = sizeof(float) * 9 * (size_t)kMaxVoxels;
@@ -108,6 +109,13 @@ __global__ void k_noalloc_put(ParamChunk c, float *__restrict__ dst) {
         dst[c.offset + i] = c.v[i];
 }
 
+// The result of a solve in which a kernel's bounded wait ran out (it then left tiles unwritten):
+// NaN throughout, as this entry has no other way to tell -- it returns before the kernels run.
+__global__ void __launch_bounds__(256) k_noalloc_check(const int *err, float *phi, int n) {
+    rsf::tiled::wait_for_previous();
+    if (*err == 0) return;
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) phi[i] = NAN;
+}
 
 void put_floats(const float *v, int n, float *dst, cudaStream_t s) {
     for (int o = 0; o < n; o += kParamChunk) {
@@ -120,8 +128,9 @@ void put_floats(const float *v, int n, float *dst, cudaStream_t s) {
 }
 
 // The iterations in the tiled schedule (rsf_exact.cuh), all fields in `mem`; phi[0] holds phi0.
+// fault_tx: as in TiledGroup.
 cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Taps &taps, int iters, char *mem, int dev,
-                         cudaStream_t s) {
+                         unsigned fault_tx, cudaStream_t s) {
     char *const q = mem + kDescBytes;
     rsf::exact_place_fields(b, q + (rsf::exact_q_bytes(b.nx, b.ny, b.nz) + 255) / 256 * 256, reinterpret_cast<float *>(q));
     int sms = 0;
@@ -142,6 +151,7 @@ cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Ta
     struct {
         rsf::BrickDev b;
         int starts[8];
+        int err;  // the bounded waits' error word, cleared with the descriptor's upload
     } d{};
     d.b = b;
     for (int k = 0; k < 4; ++k) d.starts[2 * k + 1] = (int)g.ncta[k];
@@ -149,18 +159,20 @@ cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Ta
     const rsf::BrickDev *db = reinterpret_cast<const rsf::BrickDev *>(mem);
     g.bricks = db;
     for (int k = 0; k < 4; ++k) g.starts[k] = reinterpret_cast<const int *>(mem + offsetof(decltype(d), starts)) + 2 * k;
+    g.err = reinterpret_cast<int *>(mem + offsetof(decltype(d), err));
+    g.fault_tx = fault_tx;
     put_floats(reinterpret_cast<const float *>(&d), (int)(sizeof(d) / sizeof(float)), reinterpret_cast<float *>(mem), s);
     if ((e = rsf::exact_start(b, vol, vt, s)) != cudaSuccess) return e;
     for (int it = 0; it < iters; ++it)
         if ((e = rsf::tiled_iterate(g, it & 1, nullptr, s)) != cudaSuccess) return e;
+    const int n = b.nx * b.ny * b.nz;
+    rsf::tiled::launch_next(g.overlap, k_noalloc_check, (n + 2047) / 2048, 256, 0, s, g.err, b.phi[iters & 1], n);
     return cudaGetLastError();
 }
 
-}  // namespace
-
-extern "C" rsf_status rsf_evolve_noalloc(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int64_t nz,
-                                         const float *phi0, float *phi_out, float sigma, float eps, float lambda1,
-                                         float lambda2, float nu, float mu, float dt, int32_t iters, void *stream) {
+rsf_status evolve(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int64_t nz, const float *phi0,
+                  float *phi_out, float sigma, float eps, float lambda1, float lambda2, float nu, float mu, float dt,
+                  int32_t iters, void *stream, unsigned fault_tx) {
     if (!volume || !phi0 || !phi_out) return err(RSF_E_INVAL, "null volume, phi0 or phi_out pointer");
     if (vt != RSF_U8 && vt != RSF_U16 && vt != RSF_F32) return err(RSF_E_INVAL, "unknown volume dtype");
     if (nx < 4 || ny < 4 || nz < 4) return err(RSF_E_INVAL, "each dimension must be >= 4");
@@ -235,7 +247,8 @@ extern "C" rsf_status rsf_evolve_noalloc(const void *volume, rsf_dtype vt, int64
         b.nu = nu;
         b.mu = mu;
         b.dt = dt;
-        if ((e = evolve_tiled(b, volume, (int)vt, taps, iters, reinterpret_cast<char *>(base + kOffI), dev, s)) != cudaSuccess)
+        if ((e = evolve_tiled(b, volume, (int)vt, taps, iters, reinterpret_cast<char *>(base + kOffI), dev, fault_tx,
+                              s)) != cudaSuccess)
             return err(RSF_E_CUDA, cudaGetErrorString(e));
         in = iters % 2 ? phi_out : scratch_phi;
     } else {
@@ -254,4 +267,21 @@ extern "C" rsf_status rsf_evolve_noalloc(const void *volume, rsf_dtype vt, int64
     }
     e = cudaGetLastError();
     return e == cudaSuccess ? RSF_OK : err(RSF_E_CUDA, cudaGetErrorString(e));
+}
+
+}  // namespace
+
+extern "C" rsf_status rsf_evolve_noalloc(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int64_t nz,
+                                         const float *phi0, float *phi_out, float sigma, float eps, float lambda1,
+                                         float lambda2, float nu, float mu, float dt, int32_t iters, void *stream) {
+    return evolve(volume, vt, nx, ny, nz, phi0, phi_out, sigma, eps, lambda1, lambda2, nu, mu, dt, iters, stream, 0u);
+}
+
+// Not part of the ABI, for tests: the same with copy barriers armed for 16 bytes more than the
+// copies bring (as RSF_OPT_FAULT_WAIT does on a context), so that every bounded wait runs out.
+extern "C" rsf_status rsf_test_noalloc_expired_waits(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int64_t nz,
+                                                     const float *phi0, float *phi_out, float sigma, float eps,
+                                                     float lambda1, float lambda2, float nu, float mu, float dt,
+                                                     int32_t iters, void *stream) {
+    return evolve(volume, vt, nx, ny, nz, phi0, phi_out, sigma, eps, lambda1, lambda2, nu, mu, dt, iters, stream, 16u);
 }

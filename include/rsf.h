@@ -455,7 +455,8 @@ rsf_status rsf_prof_get(rsf_ctx *ctx, int32_t kernel, int64_t *launches, double 
  * exits), which limits the volume to nx*ny*nz <= 262144 voxels (e.g. 64^3);
  * larger volumes are rejected with RSF_E_INVAL.  The first call on a device
  * looks up the array's device address (cudaGetSymbolAddress) with that device
- * current; make that first call before any stream capture.  Asynchronous:
+ * current and loads the code of every kernel width and image type; make that
+ * first call before any stream capture.  Asynchronous:
  * returns once the work is queued; phi_out is ready when `stream` reaches it.
  * All calls on a device share the array and it keeps the last call's
  * contents (nothing in it needs to start at zero); calls whose work overlaps

@@ -204,6 +204,19 @@ size_t exact_stage_bytes(int nx, int ny, int nz);
 size_t exact_q_bytes(int nx, int ny, int nz);
 void exact_place_fields(BrickDev &b, void *stage, float *q);
 cudaError_t exact_start(const BrickDev &b, const void *vol, int vt, cudaStream_t s);
+
+// Loads kernels on the current device (by default a kernel's code is loaded, and takes device
+// memory, at its first launch).
+template <class... K>
+cudaError_t load_kernels(K *...kernels) {
+    cudaError_t e = cudaSuccess;
+    cudaFuncAttributes a;
+    for (const void *k : {reinterpret_cast<const void *>(kernels)...})
+        if (e == cudaSuccess) e = cudaFuncGetAttributes(&a, k);
+    return e;
+}
+cudaError_t load_exact();   // the exact arithmetic at every radius, its set-up included
+cudaError_t load_passes();  // the six passes, statistics and centring
 // One iteration of the separable pass path: phi_in -> phi_out.
 // `stages`, when not null, receives RSF_NSTAGES fields (f1, f2, g, kappa, L).
 cudaError_t iterate_passes(const Taps &taps, const Coeffs &c, Fields &f, const float *phi_in, float *phi_out,

@@ -61,9 +61,22 @@ rsf_status err(rsf_status st, const char *msg) {
     return st;
 }
 
+// Values written into the static array through kernel parameters, so that no
+// host staging buffer and no allocation is involved (24 KB per launch).
+constexpr int kParamChunk = 6144;
+struct ParamChunk {
+    int offset, count;
+    float v[kParamChunk];
+};
+
+__global__ void k_noalloc_put(ParamChunk c, float *__restrict__ dst);
+__global__ void k_noalloc_check(const int *err, float *phi, int n);
+
 // Device address of the static array on the current device, looked up once per
 // device (with that device current).  The name g_noalloc_scratch is only a
-// host-side stand-in; kernels must be given this address.
+// host-side stand-in; kernels must be given this address.  The same first call
+// loads every kernel of this entry, so that no later one loads code (6 MB of
+// device memory over the kernel widths) in the middle of its caller's run.
 rsf_status scratch_on_current_device(float **out) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
@@ -78,6 +91,9 @@ rsf_status scratch_on_current_device(float **out) {
             snprintf(buf, sizeof buf, "cudaGetSymbolAddress of the static scratch failed: %s", cudaGetErrorString(e));
             return err(RSF_E_CUDA, buf);
         }
+        if ((e = rsf::load_kernels(k_noalloc_put, k_noalloc_check)) == cudaSuccess) e = rsf::load_passes();
+        if (e == cudaSuccess) e = rsf::load_exact();
+        if (e != cudaSuccess) return err(RSF_E_CUDA, cudaGetErrorString(e));
         g_scratch_dev[dev] = (float *)p;
     }
     *out = g_scratch_dev[dev];
@@ -95,14 +111,6 @@ bool is_device_ptr(const void *p, int dev) {
     }
     return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
 }
-
-// Values written into the static array through kernel parameters, so that no
-// host staging buffer and no allocation is involved (24 KB per launch).
-constexpr int kParamChunk = 6144;
-struct ParamChunk {
-    int offset, count;
-    float v[kParamChunk];
-};
 
 __global__ void k_noalloc_put(ParamChunk c, float *__restrict__ dst) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c.count; i += gridDim.x * blockDim.x)

@@ -387,6 +387,12 @@ cudaError_t centre_image(const void *vol, int vt, Fields &f, cudaStream_t s) {
     return cudaGetLastError();
 }
 
+cudaError_t load_passes() {
+    return load_kernels(k_stats<uint8_t>, k_stats<uint16_t>, k_stats<float>, k_stats_final, k_center<uint8_t>,
+                        k_center<uint16_t>, k_center<float>, k_xpass<4, LoadH4>, k_spass<4, StoreEpi<4>>,
+                        k_spass<4, FitsEpi>, k_xpass<2, LoadN<2>>, k_spass<2, StoreEpi<2>>, k_spass<2, UpdateEpi>);
+}
+
 cudaError_t iterate_passes(const Taps &t, const Coeffs &c, Fields &f, const float *phi_in, float *phi_out,
                            float *stages, Profiler *prof, cudaStream_t s) {
     const Dims &d = f.d;

@@ -310,6 +310,13 @@ cudaError_t tiled_prepare(int storage, int R, int force) {
     }
 }
 
+cudaError_t load_exact() {
+    cudaError_t e = load_kernels(tiled::k_start<true>, tiled::k_center_rows<uint8_t>, tiled::k_center_rows<uint16_t>,
+                                 tiled::k_center_rows<float>);
+    for (int R = 1; R <= RMAX && e == cudaSuccess; ++R) e = tiled_prepare(0, R, kForceExact);
+    return e;
+}
+
 cudaError_t tiled_iterate(const TiledGroup &g, int parity, Profiler *prof, cudaStream_t s) {
     const int R = g.taps.R;
     if (g.force == kForceExact)

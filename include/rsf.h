@@ -240,10 +240,13 @@ rsf_status rsf_step_stages(rsf_ctx *ctx, const void *volume, rsf_dtype vt, int64
 
 /*
  * rsf_set_option -- per-context settings of the iteration schedule.
- *   RSF_OPT_PATH    RSF_PATH_AUTO (default): the tiled four-kernel iteration
- *                   where it has kernels for the radius R (2-6, 8, 10, 12),
- *                   else the six-pass iteration; RSF_PATH_PASSES: always the
- *                   six-pass iteration; RSF_PATH_TILED: the tiled iteration
+ *   RSF_OPT_PATH    RSF_PATH_AUTO (default): the tiled four-kernel iteration,
+ *                   with fast arithmetic where that has kernels for the radius
+ *                   R (2-6, 8, 10, 12), else in the exact arithmetic of the
+ *                   six-pass iteration (the same bits); radius 0 and volumes of
+ *                   2^32 pitched voxels or more take the six-pass iteration.
+ *                   RSF_PATH_PASSES: always the six-pass iteration;
+ *                   RSF_PATH_TILED: the tiled iteration with fast arithmetic
  *                   (other radii then fail with RSF_E_INVAL).
  *   RSF_OPT_ZCHUNK  z chunk of the z-marching kernel: the planes of one CTA; 0
  *                   (default) picks it from the volume's size and may split

@@ -508,7 +508,8 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         return fail(RSF_E_INVAL, "the Eq. (15) force form needs the tiled path (radius %d, path option %d)", taps.R,
                     c->opt_path);
     // the exact arithmetic of the separable passes, in the tiled schedule where that takes the volume
-    const bool exact = !tiled && rsf::exact_supports(taps.R) && rsf::tiled_fits(nx, ny, nz);
+    // and the passes themselves are not asked for
+    const bool exact = c->opt_path != RSF_PATH_PASSES && !tiled && rsf::exact_supports(taps.R) && rsf::tiled_fits(nx, ny, nz);
     // the tiled schedule centres the image itself, on load or into its own field
     RSF_CUDA(rsf::setup_image(vol, (int)vt, taps, f, c->stream, !tiled && !exact));
     if (c->opt_poison) {  // NaN bytes in everything the iteration must write before it reads

@@ -3,7 +3,8 @@
 // FP32 image.  Every radius 1 to 16 (the fast arithmetic of rsf_tiled_*.cu has 2-6, 8, 10,
 // 12).  The same four kernels as the other forms (rsf_tiled.cuh) with EX / AB set; results
 // equal the six separable passes (rsf_passes.cu) bit for bit, which keep radius 0, volumes of
-// 2^32 pitched voxels or more and what does not fit rsf_evolve_noalloc's static memory.
+// 2^32 pitched voxels or more, what does not fit rsf_evolve_noalloc's static memory, and
+// RSF_PATH_PASSES.
 // 224 x 208 x 192 uint8, radius 7, per iteration: 1.53 ms in the passes (a normal's six
 // neighbours from global memory at each of seven places, 0.84 ms alone), 0.33 ms here: x/y
 // 0.087, z 0.043, x/y 0.038, update 0.158.

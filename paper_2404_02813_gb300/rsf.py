@@ -327,7 +327,8 @@ class Context:
         _check(load_library().rsf_set_option(self._h, int(key), int(value)))
 
     def set_path(self, name: str):
-        """'auto' (tiled where instantiated, else passes), 'passes' or 'tiled'."""
+        """'auto' (tiled; the six passes at radius 0 and from 2^32 pitched voxels on), 'passes' or 'tiled'
+        (its fast arithmetic only)."""
         self.set_option(OPT_PATH, PATHS[name])
 
     def evolve_batch(self, items):

@@ -140,7 +140,7 @@ void free_desc(rsf_ctx *c, DescBuffers &buf) {
 }
 
 rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, const std::vector<GroupSpec> &specs,
-                         std::vector<rsf::TiledGroup> *out) {
+                         HostCopies &copies, std::vector<rsf::TiledGroup> *out) {
     int total = 0;
     for (const GroupSpec &g : specs) total += (int)g.bricks.size();
     const int need_starts = 4 * (total + (int)specs.size());
@@ -200,10 +200,8 @@ rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, cons
         }
         out->push_back(g);
     }
-    RSF_CUDA(cudaMemcpyAsync(buf.d_bricks, all.data(), sizeof(rsf::BrickDev) * all.size(), cudaMemcpyHostToDevice,
-                             stream));
-    RSF_CUDA(cudaMemcpyAsync(buf.d_starts, starts.data(), sizeof(int) * starts.size(), cudaMemcpyHostToDevice,
-                             stream));
+    RSF_CUDA(copies.put(buf.d_bricks, std::move(all), stream));
+    RSF_CUDA(copies.put(buf.d_starts, std::move(starts), stream));
     return RSF_OK;
 }
 
@@ -511,7 +509,11 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     // and the passes themselves are not asked for
     const bool exact = c->opt_path != RSF_PATH_PASSES && !tiled && rsf::exact_supports(taps.R) && rsf::tiled_fits(nx, ny, nz);
     // the tiled schedule centres the image itself, on load or into its own field
-    RSF_CUDA(rsf::setup_image(vol, (int)vt, taps, f, c->stream, !tiled && !exact));
+    RSF_CUDA(tiled || exact ? rsf::image_stats(vol, (int)vt, f, c->stream) : rsf::centre_image(vol, (int)vt, f, c->stream));
+    HostCopies copies(c->stream);
+    std::vector<float> prof((size_t)(nx + ny + nz));
+    rsf::zero_padding_profiles(taps, (int)nx, (int)ny, (int)nz, prof.data());
+    RSF_CUDA(copies.put(f.prof, std::move(prof)));
     if (c->opt_poison) {  // NaN bytes in everything the iteration must write before it reads
         RSF_CUDA(cudaMemsetAsync(f.t[0], 0xFF, sizeof(float) * 8 * (size_t)c->cap_np, c->stream));
         RSF_CUDA(cudaMemsetAsync(f.phi[1], 0xFF, sizeof(float) * n, c->stream));
@@ -576,7 +578,7 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         if (out_here) (iters == 1 ? specs[0] : specs[2]).bricks[0].phi[iters & 1] = phi_out;
         b = specs[0].bricks[0];
         std::vector<rsf::TiledGroup> groups;
-        if ((st = upload_groups(c, c->desc, c->stream, specs, &groups))) return st;
+        if ((st = upload_groups(c, c->desc, c->stream, specs, copies, &groups))) return st;
         if (iters > 0) {
             if (exact)
                 RSF_CUDA(rsf::exact_start(b, vol, (int)vt, c->stream));
@@ -601,6 +603,7 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     if (stages && dump != stages)
         RSF_CUDA(xfer(stages, dump, sizeof(float) * n * RSF_NSTAGES, c->stream));
     RSF_CUDA(cudaStreamSynchronize(c->stream));
+    copies.done();
     return device_error(c);
 }
 

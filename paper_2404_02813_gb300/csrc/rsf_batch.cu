@@ -109,7 +109,8 @@ void apply_tuned(GroupSpec &g, const TunedGroup &t, int sms) {
 rsf_status time_iteration(rsf_ctx *c, const GroupSpec &g, cudaEvent_t e0, cudaEvent_t e1, float *ms) {
     std::vector<GroupSpec> one{g};
     std::vector<rsf::TiledGroup> up;
-    rsf_status st = upload_groups(c, c->desc, c->stream, one, &up);
+    HostCopies copies(c->stream);
+    rsf_status st = upload_groups(c, c->desc, c->stream, one, copies, &up);
     if (st) return st;
     for (int rep = 0; rep < 2; ++rep) {
         RSF_CUDA(cudaEventRecord(e0, c->stream));
@@ -117,6 +118,7 @@ rsf_status time_iteration(rsf_ctx *c, const GroupSpec &g, cudaEvent_t e0, cudaEv
         RSF_CUDA(cudaEventRecord(e1, c->stream));
     }
     RSF_CUDA(cudaEventSynchronize(e1));
+    copies.done();
     RSF_CUDA(cudaEventElapsedTime(ms, e0, e1));
     return device_error(c);
 }
@@ -298,9 +300,9 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
     // ---- centring constants, phi0, q, copied images: all bricks at once (per brick these are
     // short launches one after the other: 32 bricks of about 152^3 took 0.9 ms of them and a
     // synchronisation each, 0.54 ms together)
-    RSF_CUDA(cudaMemcpyAsync(prof0, prof_host.data(), prof_host.size(), cudaMemcpyHostToDevice, c->stream));
-    RSF_CUDA(cudaMemcpyAsync(c->d_setup, setup.data(), sizeof(rsf::SetupBrick) * setup.size(), cudaMemcpyHostToDevice,
-                             c->stream));
+    HostCopies copies(c->stream);
+    RSF_CUDA(copies.put(prof0, std::move(prof_host)));
+    RSF_CUDA(copies.put(c->d_setup, std::move(setup)));
     RSF_CUDA(rsf::setup_stats(c->d_setup, nb, c->stream));
     RSF_CUDA(rsf::setup_start(c->d_setup, nb, c->stream));
 
@@ -353,7 +355,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
             }
         }
         std::vector<rsf::TiledGroup> groups;
-        if ((st = upload_groups(c, c->desc, c->stream, specs, &groups))) return st;
+        if ((st = upload_groups(c, c->desc, c->stream, specs, copies, &groups))) return st;
         if (!tuned_once)
             for (const rsf::TiledGroup &g : groups) RSF_CUDA(rsf::tiled_ki_init(g, c->stream));
         tuned_once = true;
@@ -393,6 +395,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         if ((st = retire(t))) return st;
     }
     RSF_CUDA(cudaStreamSynchronize(c->stream));
+    copies.done();
     return device_error(c);
 }
 

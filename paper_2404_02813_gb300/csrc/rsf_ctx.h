@@ -7,6 +7,7 @@
 
 #include <cstdint>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <string>
 #include <vector>
@@ -104,7 +105,35 @@ size_t dtype_size(rsf_dtype vt);
 rsf_status check_args(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int64_t nz, const void *phi0,
                       const void *phi_out, float sigma, float eps, float dt, int32_t iters);
 rsf::Taps make_taps(float sigma);
+// Uploads of the host's own tables: a copy from pageable memory may still read its source after
+// the call that queues it, so the sources live here until the stream has passed them.  (Up to
+// 16 MB, behind a stream with 60 ms of work, the driver was seen to take the source first.)
+class HostCopies {
+    cudaStream_t s;
+    std::vector<std::shared_ptr<void>> kept;
+
+  public:
+    explicit HostCopies(cudaStream_t stream = nullptr) : s(stream) {}
+    HostCopies(const HostCopies &) = delete;
+    HostCopies &operator=(const HostCopies &) = delete;
+    ~HostCopies() {  // an early return
+        if (!kept.empty()) cudaStreamSynchronize(s);
+    }
+    template <class T>
+    cudaError_t put(void *dst, std::vector<T> &&src) { return put(dst, std::move(src), s); }
+    template <class T>
+    cudaError_t put(void *dst, std::vector<T> &&src, cudaStream_t stream) {
+        s = stream;
+        auto v = std::make_shared<std::vector<T>>(std::move(src));
+        kept.push_back(v);
+        return cudaMemcpyAsync(dst, v->data(), sizeof(T) * v->size(), cudaMemcpyHostToDevice, s);
+    }
+    // the stream has passed every copy but the last `last`
+    void done(size_t last = 0) {
+        if (kept.size() > last) kept.erase(kept.begin(), kept.end() - last);
+    }
+};
 rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t s, const std::vector<GroupSpec> &specs,
-                         std::vector<rsf::TiledGroup> *out);
+                         HostCopies &copies, std::vector<rsf::TiledGroup> *out);
 void free_desc(rsf_ctx *c, DescBuffers &buf);
 void rsf_serve_shutdown(rsf_ctx *c);

@@ -231,6 +231,7 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
     std::vector<rsf_brick> bricks(nbox);
     std::vector<const float *> phis(nbox);
     MergeArgs m{};
+    HostCopies copies(c->stream);
     {
         std::lock_guard<std::mutex> lk(c->mu);
         RSF_CUDA(cudaSetDevice(c->device));
@@ -280,7 +281,8 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
             m.n[a] = n[a];
             m.nb[a] = nb[a];
         }
-        RSF_CUDA(cudaMemcpyAsync(tb, host_tab.data(), off, cudaMemcpyHostToDevice, c->stream));
+        host_tab.resize(off);
+        RSF_CUDA(copies.put(tb, std::move(host_tab)));
         for (long long first = 0; first < nbox; first += 32768) {
             ga.first = (int)first;
             const dim3 grid((unsigned)std::min<long long>(((long long)ext[1] * ext[2] + 7) / 8, nbox >= 16 ? 152 : 1216),
@@ -303,5 +305,6 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
     RSF_CUDA(cudaGetLastError());
     if (host_out) RSF_CUDA(xfer(phi_out, out, sizeof(float) * nvox, c->stream));
     RSF_CUDA(cudaStreamSynchronize(c->stream));
+    copies.done();
     return RSF_OK;
 }

@@ -70,18 +70,14 @@ struct Fields {
 
 constexpr int kStatBlocks = 1024;
 
-// Set-up: centring constants, the K*1 profiles and (when `centre`) the
-// centred image f.I.  `vol` is a device pointer of dtype vt (0 u8, 1 u16, 2 f32).
-cudaError_t setup_image(const void *vol, int vt, const Taps &taps, Fields &f, cudaStream_t s, bool centre = true);
-
-// Centring constants only (f.cs from the image statistics), no other field; never synchronises.
+// Centring constants (f.cs) from the statistics of `vol`, a device pointer of dtype vt (0 u8,
+// 1 u16, 2 f32); enqueues on `s` and never synchronises.
 cudaError_t image_stats(const void *vol, int vt, Fields &f, cudaStream_t s);
 // Zero-padding profiles p_a(i) = sum of the in-volume taps (double sums rounded
 // once), nx + ny + nz floats: K*1 = p_x p_y p_z.
 void zero_padding_profiles(const Taps &taps, int nx, int ny, int nz, float *out);
 
-// The centring half of setup_image alone (statistics and centred image, no
-// profiles); enqueues on `s` and never synchronises.
+// The same and the centred image f.I.
 cudaError_t centre_image(const void *vol, int vt, Fields &f, cudaStream_t s);
 
 // Sets the calling thread's rsf_last_error() text.

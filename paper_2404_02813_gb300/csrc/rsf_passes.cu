@@ -342,43 +342,11 @@ cudaError_t image_stats(const void *vol, int vt, Fields &f, cudaStream_t s) {
     return cudaGetLastError();
 }
 
-cudaError_t setup_image(const void *vol, int vt, const Taps &taps, Fields &f, cudaStream_t s, bool centre) {
-    const Dims &d = f.d;
-    const int eb = 1184;  // elementwise grid: a multiple of the SM count, grid-stride beyond
-    switch (vt) {
-        case 0:
-            k_stats<uint8_t><<<kStatBlocks, 256, 0, s>>>((const uint8_t *)vol, d.n, f.partials);
-            break;
-        case 1:
-            k_stats<uint16_t><<<kStatBlocks, 256, 0, s>>>((const uint16_t *)vol, d.n, f.partials);
-            break;
-        default:
-            k_stats<float><<<kStatBlocks, 256, 0, s>>>((const float *)vol, d.n, f.partials);
-    }
-    k_stats_final<<<1, kStatBlocks, 0, s>>>(f.partials, d.n, f.cs);
-    if (centre) {
-        switch (vt) {
-            case 0: k_center<uint8_t><<<eb, 256, 0, s>>>((const uint8_t *)vol, d.n, f.cs, f.I); break;
-            case 1: k_center<uint16_t><<<eb, 256, 0, s>>>((const uint16_t *)vol, d.n, f.cs, f.I); break;
-            default: k_center<float><<<eb, 256, 0, s>>>((const float *)vol, d.n, f.cs, f.I);
-        }
-    }
-    std::vector<float> prof((size_t)d.nx + d.ny + d.nz);
-    zero_padding_profiles(taps, d.nx, d.ny, d.nz, prof.data());
-    // a copy from pageable memory has taken its source when the call returns
-    const cudaError_t e = cudaMemcpyAsync(f.prof, prof.data(), sizeof(float) * prof.size(), cudaMemcpyHostToDevice, s);
-    return e != cudaSuccess ? e : cudaGetLastError();
-}
-
 cudaError_t centre_image(const void *vol, int vt, Fields &f, cudaStream_t s) {
     const Dims &d = f.d;
-    const int eb = 1184;
-    switch (vt) {
-        case 0: k_stats<uint8_t><<<kStatBlocks, 256, 0, s>>>((const uint8_t *)vol, d.n, f.partials); break;
-        case 1: k_stats<uint16_t><<<kStatBlocks, 256, 0, s>>>((const uint16_t *)vol, d.n, f.partials); break;
-        default: k_stats<float><<<kStatBlocks, 256, 0, s>>>((const float *)vol, d.n, f.partials);
-    }
-    k_stats_final<<<1, kStatBlocks, 0, s>>>(f.partials, d.n, f.cs);
+    const int eb = 1184;  // elementwise grid: a multiple of the SM count, grid-stride beyond
+    const cudaError_t e = image_stats(vol, vt, f, s);
+    if (e != cudaSuccess) return e;
     switch (vt) {
         case 0: k_center<uint8_t><<<eb, 256, 0, s>>>((const uint8_t *)vol, d.n, f.cs, f.I); break;
         case 1: k_center<uint16_t><<<eb, 256, 0, s>>>((const uint16_t *)vol, d.n, f.cs, f.I); break;

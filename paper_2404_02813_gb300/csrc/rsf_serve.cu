@@ -101,6 +101,7 @@ struct Lane {
     bool groups_dirty = true;
     std::vector<rsf::TiledGroup> groups;
     DescBuffers desc;
+    HostCopies copies;                 // of its descriptors
     std::deque<cudaEvent_t> inflight;  // one event per dispatch not yet known complete
 };
 
@@ -418,7 +419,9 @@ bool rebuild_groups(Server *s, Lane &L) {
         rsf::set_last_error("injected descriptor upload failure");
         st = RSF_E_CUDA;
     } else {
-        st = upload_groups(s->ctx, L.desc, L.stream, specs, &L.groups);
+        // two tables an upload, a dispatch after each, fewer than kMaxAhead dispatches under way
+        L.copies.done(2 * kMaxAhead);
+        st = upload_groups(s->ctx, L.desc, L.stream, specs, L.copies, &L.groups);
     }
     if (st != RSF_OK) {
         L.groups.clear();
@@ -455,6 +458,8 @@ void dispatch(Server *s, Lane &L, bool queued) {
         L.active.clear();
         L.groups.clear();
         L.groups_dirty = true;
+        cudaStreamSynchronize(L.stream);  // no event follows this dispatch's uploads
+        L.copies.done();
         return;
     }
     // retire finished or cancelled bricks
@@ -646,6 +651,7 @@ void rsf_serve_shutdown(rsf_ctx *c) {
     dev_free(c, s->partials, sizeof(float) * 3 * rsf::kStatBlocks);
     dev_free(c, s->setup_desc, sizeof(SetupDesc));
     for (Lane &L : s->lanes) {
+        L.copies.done();
         free_desc(c, L.desc);
         cudaStreamDestroy(L.stream);
     }

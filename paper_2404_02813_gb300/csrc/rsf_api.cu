@@ -451,7 +451,6 @@ extern "C" void rsf_destroy(rsf_ctx *c) {
         dev_free(c, c->staging, c->staging_cap);
         dev_free(c, c->dump, c->dump_cap);
         free_desc(c, c->desc);
-        dev_free(c, c->d_setup, sizeof(rsf::SetupBrick) * (size_t)c->cap_setup);
         dev_free(c, c->pool, c->pool_cap);
         c->prof.release();
         cudaStreamDestroy(c->stream);

@@ -45,7 +45,7 @@ size_t brick_bytes(const rsf_brick &b, int storage, bool stage_image) {
     const long long n = (long long)b.nx * b.ny * b.nz;
     const long long np = (long long)rsf::tiled_pitch((int)b.nx) * b.ny * b.nz;
     size_t s = 4 * align256(sizeof(float) * n);                          // phi[2], q block
-    s += align256(sizeof(float) * (b.nx + b.ny + b.nz)) + align256(64);  // profiles, centring constants
+    s += align256(sizeof(float) * (b.nx + b.ny + b.nz)) + align256(64);  // profiles; constants, set-up entry
     s += align256(rsf::tiled_stage_bytes(storage, np));
     return stage_image ? s + align256(dtype_size(b.vt) * n) : s;
 }
@@ -226,14 +226,6 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         if (st) return st;
         c->pool_cap = total;
     }
-    if (nb > c->cap_setup) {
-        dev_free(c, c->d_setup, sizeof(rsf::SetupBrick) * (size_t)c->cap_setup);
-        c->d_setup = nullptr;
-        c->cap_setup = 0;
-        rsf_status st = dev_alloc(c, (void **)&c->d_setup, sizeof(rsf::SetupBrick) * (size_t)nb);
-        if (st) return st;
-        c->cap_setup = nb;
-    }
 
     // ---- per brick: placement; profiles of all bricks in one block, so that one copy brings them
     std::vector<BrickState> bs(nb);
@@ -248,6 +240,10 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         prof_at[i + 1] = prof_at[i] + align256(sizeof(float) * (bricks[i].nx + bricks[i].ny + bricks[i].nz));
     char *const prof0 = take(prof_at[nb]);
     std::vector<char> prof_host(prof_at[nb], 0);
+    // the 256 bytes of each brick's constants hold them (64) and its entry of the set-up table
+    constexpr size_t kEntry = 192;
+    static_assert(sizeof(rsf::SetupBrick) <= kEntry, "a brick's constants and its entry in 256 bytes");
+    char *const table = take(256 * (size_t)nb), *const cs0 = table + kEntry * nb;
     std::vector<rsf::SetupBrick> setup(nb);
     for (int i = 0; i < nb; ++i) {
         const rsf_brick &b = bricks[i];
@@ -265,7 +261,7 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
         d.nz = (int)b.nz;
         for (int k = 0; k < 2; ++k) d.phi[k] = reinterpret_cast<float *>(take(sizeof(float) * n));
         rsf::zero_padding_profiles(make_taps(b.sigma), d.nx, d.ny, d.nz, reinterpret_cast<float *>(prof_host.data() + prof_at[i]));
-        float *cs = reinterpret_cast<float *>(take(64));
+        float *cs = reinterpret_cast<float *>(cs0 + 64 * (size_t)i);
         void *q = take(rsf::tiled_q_bytes(d.nx, (long long)d.ny * d.nz));  // the stage block follows
         d.prof = reinterpret_cast<float *>(prof0 + prof_at[i]);
         d.cs = cs;
@@ -302,9 +298,10 @@ extern "C" rsf_status rsf_evolve_batch(rsf_ctx *c, const rsf_brick *bricks, int3
     // synchronisation each, 0.54 ms together)
     HostCopies copies(c->stream);
     RSF_CUDA(copies.put(prof0, std::move(prof_host)));
-    RSF_CUDA(copies.put(c->d_setup, std::move(setup)));
-    RSF_CUDA(rsf::setup_stats(c->d_setup, nb, c->stream));
-    RSF_CUDA(rsf::setup_start(c->d_setup, nb, c->stream));
+    const rsf::SetupBrick *const d_setup = reinterpret_cast<rsf::SetupBrick *>(table);
+    RSF_CUDA(copies.put(table, std::move(setup)));
+    RSF_CUDA(rsf::setup_stats(d_setup, nb, c->stream));
+    RSF_CUDA(rsf::setup_start(d_setup, nb, c->stream));
 
     // ---- iterate: fixed active sets between retirements
     std::vector<int> order(nb);

@@ -52,8 +52,6 @@ struct rsf_ctx {
     int opt_storage = RSF_STORE_F32;
     int opt_force = RSF_FORCE_LI;
     DescBuffers desc;                   // brick descriptors of rsf_evolve / rsf_evolve_batch launches
-    rsf::SetupBrick *d_setup = nullptr; // set-up descriptions of rsf_evolve_batch's bricks
-    int cap_setup = 0;
     int opt_autotune = 0;
     int opt_graph = 1;
     void *pool = nullptr;               // per-brick fields of rsf_evolve_batch

@@ -1,0 +1,47 @@
+"""Calls whose working memory fills the context's budget to the byte: each path takes no more than
+the fields it documents, so that descriptors and tables of its own never turn such a call away."""
+import numpy as np
+import pytest
+
+from paper_2404_02813_gb300 import rsf
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+STATS = 4 * 3 * 1024          # partial sums of the image statistics
+
+
+def _align(b):
+    return (b + 255) // 256 * 256
+
+
+def _params(sigma):
+    return dict(sigma=sigma, eps=1.0, lambda1=1.0, lambda2=2.0, nu=0.004 * 255.0 ** 2, mu=1.0, dt=0.1)
+
+
+def _case(shape, seed=4):
+    rng = np.random.default_rng(seed)
+    v = torch.from_numpy(np.rint(rng.uniform(0, 255, size=shape)).astype(np.uint8)).cuda()
+    return v, torch.from_numpy(rng.normal(0.0, 2.0, size=shape).astype(np.float32)).cuda()
+
+
+def _voxels(shape):
+    nz, ny, nx = shape
+    return nx * ny * nz, (nx + 31) // 32 * 32 * ny * nz
+
+
+def _brick(shape):
+    """phi, its copy and the q block; profiles; constants; the FP32 stage block."""
+    n, np_ = _voxels(shape)
+    return 4 * _align(4 * n) + _align(4 * sum(shape)) + 256 + _align(28 * np_)
+
+
+def test_many_bricks_without_iterations():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    shape, nb = (4, 4, 4), 200
+    v, ph = _case(shape)
+    ctx = rsf.Context(0, nb * _brick(shape) + STATS)
+    for out in ctx.evolve_batch([(v, ph, _params(3.0), 0)] * nb):
+        np.testing.assert_array_equal(out.cpu().numpy(), ph.cpu().numpy())
+    ctx.close()

@@ -69,8 +69,8 @@ bool axis_table(int n, int edge, int curtain, const std::vector<int> &starts, Ax
 // rows (one element per thread with 64-bit divisions: 22 us per array of 160^3; 12 images and level
 // sets here: 90 us, the copy rate).
 struct GatherArgs {
-    const int *start[3];      // per axis (x, y, z): first voxel of each sub-volume
-    int nb[3], ext[3], n[3];  // sub-volumes, their extents and the volume's, per axis
+    int step;                 // sub-volume k of an axis starts at min(k step, n - ext) (starts_of)
+    int nb[3], ext[3], n[3];  // sub-volumes, their extents and the volume's, per axis (x, y, z)
     int first;                // blockIdx.y = 0's sub-volume (a launch takes at most 32768)
     char *box0;               // sub-volume id's image and phi at box0 + id * stride
     size_t stride, phi_at;
@@ -79,6 +79,8 @@ template <class T>
 __global__ void __launch_bounds__(256) k_gather(const T *__restrict__ vol, const float *__restrict__ phi0, GatherArgs a) {
     const int id = a.first + blockIdx.y, kx = id % a.nb[0], ky = id / a.nb[0] % a.nb[1], kz = id / a.nb[0] / a.nb[1];
     const int bx = a.ext[0], by = a.ext[1];
+    const int x0 = min(kx * a.step, a.n[0] - bx), y0 = min(ky * a.step, a.n[1] - by);
+    const int z0 = min(kz * a.step, a.n[2] - a.ext[2]);
     const long long rows = (long long)by * a.ext[2];
     T *const img = reinterpret_cast<T *>(a.box0 + id * a.stride);
     float *const phi = reinterpret_cast<float *>(a.box0 + id * a.stride + a.phi_at);
@@ -86,7 +88,7 @@ __global__ void __launch_bounds__(256) k_gather(const T *__restrict__ vol, const
     for (long long r = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5; r < rows;
          r += ((long long)gridDim.x * blockDim.x) >> 5) {
         const int y = (int)(r % by), z = (int)(r / by);
-        const long long src = ((long long)(a.start[2][kz] + z) * a.n[1] + a.start[1][ky] + y) * a.n[0] + a.start[0][kx];
+        const long long src = ((long long)(z0 + z) * a.n[1] + y0 + y) * a.n[0] + x0;
         for (int x = lane; x < bx; x += 32) {
             img[r * bx + x] = vol[src + x];
             phi[r * bx + x] = phi0[src + x];
@@ -210,9 +212,7 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
     size_t tab_bytes = sizeof(float *) * nbox;
     for (int a = 0; a < 3; ++a)
         tab_bytes += sizeof(int) * (nb[a] + n[a] * (1 + 2 * kMaxCover)) + sizeof(float) * n[a] * kMaxCover;
-    const size_t with_starts = tab_bytes + sizeof(int) * (nb[0] + nb[1] + nb[2]);
-    bytes += std::max(align(tab_bytes) + 1024, align(with_starts));
-    tab_bytes = with_starts;
+    bytes += align(tab_bytes) + 1024;
     void *mem = nullptr;
     if ((st = dev_alloc(c, &mem, bytes))) return st;
     struct Release {
@@ -250,6 +250,7 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
         GatherArgs ga{};
         ga.box0 = take(stride * nbox);
         ga.stride = stride;
+        ga.step = edge - curtain;
         ga.phi_at = align(es * bvox);
         for (long long id = 0; id < nbox; ++id) {
             char *const box = ga.box0 + id * stride;
@@ -274,7 +275,6 @@ extern "C" rsf_status rsf_evolve_curtain(rsf_ctx *c, const void *volume, rsf_dty
             m.box[a] = reinterpret_cast<const int *>(put(tab[a].box.data(), sizeof(int) * n[a] * kMaxCover));
             m.local[a] = reinterpret_cast<const int *>(put(tab[a].local.data(), sizeof(int) * n[a] * kMaxCover));
             m.weight[a] = reinterpret_cast<const float *>(put(tab[a].weight.data(), sizeof(float) * n[a] * kMaxCover));
-            ga.start[a] = reinterpret_cast<const int *>(put(starts[a].data(), sizeof(int) * nb[a]));
             ga.nb[a] = nb[a];
             ga.ext[a] = ext[a];
             ga.n[a] = n[a];

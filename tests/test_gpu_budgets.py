@@ -45,3 +45,17 @@ def test_many_bricks_without_iterations():
     for out in ctx.evolve_batch([(v, ph, _params(3.0), 0)] * nb):
         np.testing.assert_array_equal(out.cpu().numpy(), ph.cpu().numpy())
     ctx.close()
+
+
+def test_curtain_of_many_subvolumes():
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    shape, edge, curtain = (4, 4, 20000), 4, 2
+    v, ph = _case(shape)
+    nb = (shape[2] - edge + 1) // 2 + 1
+    sub = _align(edge ** 3) + _align(4 * edge ** 3)
+    tables = 8 * nb + 4 * (nb + 2) + sum(4 * n * (1 + 2 * 4) + 4 * n * 4 for n in shape)
+    ctx = rsf.Context(0, nb * (sub + _brick((edge,) * 3)) + _align(tables) + 1024 + STATS)
+    out = ctx.evolve_curtain(v, ph, _params(3.0), 0, edge, curtain)
+    np.testing.assert_allclose(out.cpu().numpy(), ph.cpu().numpy(), rtol=2.0 ** -22, atol=0)
+    ctx.close()

@@ -131,35 +131,42 @@ void dev_free(rsf_ctx *c, void *p, size_t bytes) {
 }
 
 
-// Copy the brick descriptors of several launch groups and their per-kernel
-// CTA offsets to the device in one upload, and describe each group.
 void free_desc(rsf_ctx *c, DescBuffers &buf) {
     dev_free(c, buf.d_bricks, sizeof(rsf::BrickDev) * (size_t)buf.cap_bricks);
     dev_free(c, buf.d_starts, sizeof(int) * (size_t)buf.cap_starts);
     buf = DescBuffers{};
 }
 
+rsf_status reserve_desc(rsf_ctx *c, DescBuffers &buf, int bricks, int groups) {
+    const int need_starts = 4 * (bricks + groups);
+    if (bricks > buf.cap_bricks || need_starts > buf.cap_starts) {
+        free_desc(c, buf);
+        const int cap = std::max(bricks, 16), capst = std::max(need_starts, 4 * 32);
+        rsf_status st = dev_alloc(c, (void **)&buf.d_bricks, sizeof(rsf::BrickDev) * (size_t)cap);
+        if (st) return st;
+        buf.cap_bricks = cap;
+        st = dev_alloc(c, (void **)&buf.d_starts, sizeof(int) * (size_t)capst);
+        if (st) {
+            free_desc(c, buf);
+            return st;
+        }
+        buf.cap_starts = capst;
+    }
+    return RSF_OK;
+}
+
 rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t stream, const std::vector<GroupSpec> &specs,
                          HostCopies &copies, std::vector<rsf::TiledGroup> *out) {
     int total = 0;
     for (const GroupSpec &g : specs) total += (int)g.bricks.size();
-    const int need_starts = 4 * (total + (int)specs.size());
-    if (total > buf.cap_bricks || need_starts > buf.cap_starts) {
-        free_desc(c, buf);
-        const int cap = std::max(total, 16), capst = std::max(need_starts, 4 * 32);
-        rsf_status st = dev_alloc(c, (void **)&buf.d_bricks, sizeof(rsf::BrickDev) * (size_t)cap);
-        if (st) return st;
-        st = dev_alloc(c, (void **)&buf.d_starts, sizeof(int) * (size_t)capst);
-        if (st) return st;
-        buf.cap_bricks = cap;
-        buf.cap_starts = capst;
-    }
+    rsf_status st = reserve_desc(c, buf, total, (int)specs.size());
+    if (st) return st;
     int sms = 0;
     RSF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
     std::vector<rsf::BrickDev> all;
     std::vector<int> starts;
     all.reserve(total);
-    starts.reserve(need_starts);
+    starts.reserve(4 * ((size_t)total + specs.size()));
     out->clear();
     for (const GroupSpec &gs : specs) {
         const int nb = (int)gs.bricks.size();
@@ -504,9 +511,11 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
     if (force != RSF_FORCE_LI && !tiled)
         return fail(RSF_E_INVAL, "the Eq. (15) force form needs the tiled path (radius %d, path option %d)", taps.R,
                     c->opt_path);
-    // the exact arithmetic of the separable passes, in the tiled schedule where that takes the volume
-    // and the passes themselves are not asked for
-    const bool exact = c->opt_path != RSF_PATH_PASSES && !tiled && rsf::exact_supports(taps.R) && rsf::tiled_fits(nx, ny, nz);
+    // the exact arithmetic of the separable passes, in the tiled schedule where that takes the volume,
+    // the passes themselves are not asked for, and the budget holds the descriptors of its launches
+    // (the passes need none and give the same bits)
+    const bool exact = c->opt_path != RSF_PATH_PASSES && !tiled && rsf::exact_supports(taps.R) &&
+                       rsf::tiled_fits(nx, ny, nz) && reserve_desc(c, c->desc, 3, 3) == RSF_OK;
     // the tiled schedule centres the image itself, on load or into its own field
     RSF_CUDA(tiled || exact ? rsf::image_stats(vol, (int)vt, f, c->stream) : rsf::centre_image(vol, (int)vt, f, c->stream));
     HostCopies copies(c->stream);

@@ -131,6 +131,10 @@ class HostCopies {
         if (kept.size() > last) kept.erase(kept.begin(), kept.end() - last);
     }
 };
+// Device memory for the descriptors of `bricks` bricks in `groups` launch groups.
+rsf_status reserve_desc(rsf_ctx *c, DescBuffers &buf, int bricks, int groups);
+// Copies the brick descriptors of several launch groups and their per-kernel CTA offsets to the
+// device and describes each group.
 rsf_status upload_groups(rsf_ctx *c, DescBuffers &buf, cudaStream_t s, const std::vector<GroupSpec> &specs,
                          HostCopies &copies, std::vector<rsf::TiledGroup> *out);
 void free_desc(rsf_ctx *c, DescBuffers &buf);

@@ -36,6 +36,21 @@ def _brick(shape):
     return 4 * _align(4 * n) + _align(4 * sum(shape)) + 256 + _align(28 * np_)
 
 
+@pytest.mark.parametrize("sigma", [0.5, 3.5])
+@pytest.mark.parametrize("shape", [(4, 4, 4), (20, 18, 37)])
+def test_evolve_at_a_width_without_fast_kernels(sigma, shape):
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    v, ph = _case(shape)
+    n, np_ = _voxels(shape)
+    free = rsf.Context(0)
+    ref = free.evolve(v, ph, _params(sigma), 2).cpu().numpy()
+    free.close()
+    tight = rsf.Context(0, 5 * 4 * n + 8 * 4 * np_ + 4 * sum(shape) + 16 + STATS)
+    np.testing.assert_array_equal(tight.evolve(v, ph, _params(sigma), 2).cpu().numpy(), ref)
+    tight.close()
+
+
 def test_many_bricks_without_iterations():
     if not torch.cuda.is_available():
         pytest.skip("needs a CUDA GPU")

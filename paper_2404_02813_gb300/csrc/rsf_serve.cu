@@ -136,7 +136,6 @@ struct Server {
     Lane lanes[kLanes];
     cudaStream_t s_setup = nullptr;
     float *partials = nullptr;
-    SetupDesc *setup_desc = nullptr;  // of the admission being set up (device)
     int sms = 0;
     // statistics (mu)
     uint64_t submitted = 0, completed = 0, failed = 0, cancelled = 0, suspended = 0, admitted = 0;
@@ -198,25 +197,27 @@ void finish_now(Server *s, const std::shared_ptr<Request> &r, int status) {
     done_cb(a);
 }
 
-// The lane for a brick of this key: the one that has such bricks, else an idle one, else the
-// first of its cost class, else the one with the fewest bricks.  A launch group is never
-// split over lanes.
+// The lane for a brick of this key: the one that has such bricks, else an idle one (one that has
+// descriptors, or for which the budget holds some), else the first of its cost class, else the
+// one with the fewest bricks.  A launch group is never split over lanes.
 int lane_of(Server *s, const LaneKey &key) {
-    int idle = -1, kin = -1, least = 0;
+    int idle = -1, bare = -1, kin = -1, least = -1;
     for (int i = 0; i < kLanes; ++i) {
         const Lane &L = s->lanes[i];
         if (L.active.empty()) {
-            if (idle < 0) idle = i;
+            int &first = L.desc.cap_bricks > 0 ? idle : bare;
+            if (first < 0) first = i;
             continue;
         }
         for (const auto &r : L.active)
             if (LaneKey{class_of(r->n), r->taps.R, r->imgtype, r->storage, r->force} == key) return i;
         if (kin < 0 && std::get<0>(L.key) == std::get<0>(key)) kin = i;
-        if (L.active.size() < s->lanes[least].active.size()) least = i;
+        if (least < 0 || L.active.size() < s->lanes[least].active.size()) least = i;
     }
-    const int i = idle >= 0 ? idle : (kin >= 0 ? kin : least);
-    if (i == idle) s->lanes[i].key = key;
-    return i;
+    // (the only lane in use, should it get none: its dispatch then fails the request)
+    if (idle < 0 && bare >= 0 && (reserve_desc(s->ctx, s->lanes[bare].desc, 1, 1) == RSF_OK || least < 0)) idle = bare;
+    if (idle >= 0) s->lanes[idle].key = key;
+    return idle >= 0 ? idle : (kin >= 0 ? kin : least);
 }
 
 // Admission of one request on the set-up stream; returns false (and finishes
@@ -324,8 +325,10 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
     if (q.iters > 0 && rsf::tiled_start(d, (int)q.vt, here ? q.phi0 : d.phi[0], s->s_setup) != cudaSuccess)
         return fail_admit(RSF_E_CUDA);
     if (q.iters > 0 && r->force == 0) {
-        // K*I~: a launch group of this brick alone, described in the server's scratch (the
-        // set-up stream takes one admission after the other)
+        // K*I~: a launch group of this brick alone, described where its statistics' partial sums
+        // were (the set-up stream takes one admission after the other)
+        static_assert(sizeof(SetupDesc) <= sizeof(float) * 3 * rsf::kStatBlocks, "the descriptor in the partial sums' memory");
+        SetupDesc *const dev = reinterpret_cast<SetupDesc *>(s->partials);
         SetupDesc sd{};
         sd.b = d;
         sd.b.xyp = rsf::tiled_xy_planes({d}, 0, r->taps.R, s->sms);
@@ -336,16 +339,16 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
         g.nb = 1;
         g.err = c->d_err;
         rsf::tiled_cta_counts(sd.b, 0, r->taps.R, g.ncta);
-        g.bricks = &s->setup_desc->b;
+        g.bricks = &dev->b;
         for (int k = 0; k < 4; ++k) {
             sd.starts[2 * k + 1] = (int)g.ncta[k];
-            g.starts[k] = s->setup_desc->starts + 2 * k;
+            g.starts[k] = dev->starts + 2 * k;
         }
         ParamChunk ch;
         ch.offset = 0;
         ch.count = (int)(sizeof(sd) / sizeof(float));
         memcpy(ch.v, &sd, sizeof(sd));
-        k_put<<<1, 256, 0, s->s_setup>>>(ch, reinterpret_cast<float *>(s->setup_desc));
+        k_put<<<1, 256, 0, s->s_setup>>>(ch, s->partials);
         if (rsf::tiled_ki_init(g, s->s_setup) != cudaSuccess) return fail_admit(RSF_E_CUDA);
     }
     if (rsf::tiled_prepare(r->storage, r->taps.R, r->force) != cudaSuccess) return fail_admit(RSF_E_CUDA);
@@ -623,11 +626,6 @@ Server *server(rsf_ctx *c, rsf_status *st) {
         delete s;
         return nullptr;
     }
-    if ((*st = dev_alloc(c, (void **)&s->setup_desc, sizeof(SetupDesc)))) {
-        dev_free(c, s->partials, sizeof(float) * 3 * rsf::kStatBlocks);
-        delete s;
-        return nullptr;
-    }
     s->inject_admission = c->opt_inject_admission;
     s->inject_upload = c->opt_inject_upload;
     s->slots = c->opt_serve_slots;
@@ -649,7 +647,6 @@ void rsf_serve_shutdown(rsf_ctx *c) {
     s->cv.notify_all();
     if (s->th.joinable()) s->th.join();
     dev_free(c, s->partials, sizeof(float) * 3 * rsf::kStatBlocks);
-    dev_free(c, s->setup_desc, sizeof(SetupDesc));
     for (Lane &L : s->lanes) {
         L.copies.done();
         free_desc(c, L.desc);

@@ -8,7 +8,8 @@ from paper_2404_02813_gb300 import rsf
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-STATS = 4 * 3 * 1024          # partial sums of the image statistics
+STATS = 4 * 3 * 1024           # partial sums of the image statistics
+LANE = 16 * 1024 + 4 * 4 * 32  # launch descriptors of one serving lane (16 bricks)
 
 
 def _align(b):
@@ -74,3 +75,21 @@ def test_curtain_of_many_subvolumes():
     out = ctx.evolve_curtain(v, ph, _params(3.0), 0, edge, curtain)
     np.testing.assert_allclose(out.cpu().numpy(), ph.cpu().numpy(), rtol=2.0 ** -22, atol=0)
     ctx.close()
+
+
+def test_served_requests_of_two_groups():
+    """Two requests of one size class and different widths, budgeted with the descriptors of one lane."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    shape = (20, 24, 32)
+    v, ph = _case(shape)
+    ctx = rsf.Context(0, 2 * _brick(shape) + STATS + LANE)
+    ref = rsf.Context(0)
+    outs = [torch.full_like(ph, float("nan")) for _ in range(2)]
+    tickets = [ctx.submit(v, ph, _params(s), 40, o) for s, o in zip((2.0, 3.0), outs)]
+    for t in tickets:
+        assert ctx.wait(t, 60000) == 0
+    for s, o in zip((2.0, 3.0), outs):
+        np.testing.assert_array_equal(o.cpu().numpy(), ref.evolve(v, ph, _params(s), 40).cpu().numpy())
+    ctx.close()
+    ref.close()

@@ -25,6 +25,7 @@
 #include <cmath>
 #include <cstdint>
 #include <mutex>
+#include <utility>
 
 #include "rsf.h"
 #include "rsf_ctx.h"
@@ -65,23 +66,22 @@ __device__ __forceinline__ int max_key(float v) {
 __device__ __forceinline__ float key_value(int k) { return __int_as_float(k ^ ((k >> 31) & 0x7fffffff)); }
 
 // Determinant-of-Hessian response D of one 32 x 32 tile of a slice and the slice maximum.
-// RT > 0: the radius at compile time (round(3 s) of s = 1, 1.5, 2, 3), so that each lane
-// filters a register window -- four outputs of a row from aligned 16-byte reads, then four
-// outputs of a column -- with its taps as constant operands; RT = 0: any radius, a loop
-// over taps (384^3 uint16 at radius 5: 0.677 ms in that form, 0.368 ms with RT = 5; two passes
-// with the x-filtered fields in global memory took 1.53 ms).  Bound by instruction issue.
+// The radius R = round(3 s) is a template argument, each of 0 to 16 an instantiation, so that a
+// lane filters a register window -- four outputs of a row from aligned 16-byte reads, then four
+// outputs of a column -- with its taps as constant operands (384^3 uint16 at radius 5: 0.368 ms;
+// 0.677 ms with a loop over taps, 1.53 ms in two passes with the x-filtered fields in global
+// memory).  Bound by instruction issue.
 // Shared memory: image [H][P], x-filtered fields [3][H][36], H = 32 + 2R, P = H rounded up
 // to an odd number of 16-byte units.
 constexpr int kHX = 36;  // row pitch of the x-filtered fields: 9 units of 16 bytes
 __host__ __device__ constexpr int hessian_pitch(int R) { return ((kHT + 2 * R + 3) / 4 | 1) * 4; }
-template <class T, int RT>
+template <class T, int R>
 __global__ void __launch_bounds__(kHThreads) k_hessian(const T *__restrict__ img, float *__restrict__ D,
                                                        int *__restrict__ smax, int nx, int ny, DerivTaps tp, float s4) {
     extern __shared__ __align__(16) float hsm[];
     __shared__ float red[kHThreads / 32];
-    const int R = RT ? RT : tp.R, W = kHT + 2 * R, P = hessian_pitch(R);
+    constexpr int W = kHT + 2 * R, P = hessian_pitch(R), FS = W * kHX;  // FS: one x-filtered field
     float *const in = hsm, *const xf = hsm + W * P;
-    const int FS = W * kHX;  // one x-filtered field
     const int x0 = blockIdx.x * kHT, y0 = blockIdx.y * kHT;
     const long long plane = (long long)nx * ny, slice = blockIdx.z * plane;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -95,48 +95,32 @@ __global__ void __launch_bounds__(kHThreads) k_hessian(const T *__restrict__ img
         }
     }
     __syncthreads();
-    if constexpr (RT > 0) {
-        const int c4 = (lane & 7) * 4;  // four rows of eight groups of four columns
-        for (int r = warp * 4 + (lane >> 3); r < rows; r += kHThreads / 8) {
-            float v[(4 + 2 * RT + 3) / 4 * 4];
+    const int c4 = (lane & 7) * 4;  // four rows of eight groups of four columns
+    for (int r = warp * 4 + (lane >> 3); r < rows; r += kHThreads / 8) {
+        float v[(4 + 2 * R + 3) / 4 * 4];
 #pragma unroll
-            for (int j = 0; j < (4 + 2 * RT + 3) / 4; ++j) {
-                const float4 q = *reinterpret_cast<const float4 *>(in + r * P + c4 + 4 * j);
-                v[4 * j] = q.x;
-                v[4 * j + 1] = q.y;
-                v[4 * j + 2] = q.z;
-                v[4 * j + 3] = q.w;
-            }
-            float a[4], b[4], c[4];
-#pragma unroll
-            for (int o = 0; o < 4; ++o) {
-                a[o] = b[o] = c[o] = 0.f;
-#pragma unroll
-                for (int k = 0; k <= 2 * RT; ++k) {
-                    a[o] = fmaf(tp.g[k], v[o + k], a[o]);
-                    b[o] = fmaf(tp.g1[k], v[o + k], b[o]);
-                    c[o] = fmaf(tp.g2[k], v[o + k], c[o]);
-                }
-            }
-            float *const o = xf + r * kHX + c4;
-            *reinterpret_cast<float4 *>(o) = make_float4(a[0], a[1], a[2], a[3]);
-            *reinterpret_cast<float4 *>(o + FS) = make_float4(b[0], b[1], b[2], b[3]);
-            *reinterpret_cast<float4 *>(o + 2 * FS) = make_float4(c[0], c[1], c[2], c[3]);
+        for (int j = 0; j < (4 + 2 * R + 3) / 4; ++j) {
+            const float4 q = *reinterpret_cast<const float4 *>(in + r * P + c4 + 4 * j);
+            v[4 * j] = q.x;
+            v[4 * j + 1] = q.y;
+            v[4 * j + 2] = q.z;
+            v[4 * j + 3] = q.w;
         }
-    } else {
-        for (int r = warp; r < rows; r += kHThreads / 32) {
-            float a = 0.f, b = 0.f, c = 0.f;
+        float a[4], b[4], c[4];
+#pragma unroll
+        for (int o = 0; o < 4; ++o) {
+            a[o] = b[o] = c[o] = 0.f;
+#pragma unroll
             for (int k = 0; k <= 2 * R; ++k) {
-                const float v = in[r * P + lane + k];
-                a = fmaf(tp.g[k], v, a);
-                b = fmaf(tp.g1[k], v, b);
-                c = fmaf(tp.g2[k], v, c);
+                a[o] = fmaf(tp.g[k], v[o + k], a[o]);
+                b[o] = fmaf(tp.g1[k], v[o + k], b[o]);
+                c[o] = fmaf(tp.g2[k], v[o + k], c[o]);
             }
-            float *const o = xf + r * kHX + lane;
-            o[0] = a;
-            o[FS] = b;
-            o[2 * FS] = c;
         }
+        float *const o = xf + r * kHX + c4;
+        *reinterpret_cast<float4 *>(o) = make_float4(a[0], a[1], a[2], a[3]);
+        *reinterpret_cast<float4 *>(o + FS) = make_float4(b[0], b[1], b[2], b[3]);
+        *reinterpret_cast<float4 *>(o + 2 * FS) = make_float4(c[0], c[1], c[2], c[3]);
     }
     __syncthreads();
     float best = -INFINITY;
@@ -146,29 +130,16 @@ __global__ void __launch_bounds__(kHThreads) k_hessian(const T *__restrict__ img
 #pragma unroll
         for (int o = 0; o < 4; ++o) ixx[o] = iyy[o] = ixy[o] = 0.f;
         const float *const f = xf + r0 * kHX + lane;
-        if constexpr (RT > 0) {
 #pragma unroll
-            for (int j = 0; j < 4 + 2 * RT; ++j) {
-                const float v0 = f[j * kHX], v1 = f[FS + j * kHX], v2 = f[2 * FS + j * kHX];
+        for (int j = 0; j < 4 + 2 * R; ++j) {
+            const float v0 = f[j * kHX], v1 = f[FS + j * kHX], v2 = f[2 * FS + j * kHX];
 #pragma unroll
-                for (int o = 0; o < 4; ++o)
-                    if (j - o >= 0 && j - o <= 2 * RT) {
-                        ixx[o] = fmaf(tp.g[j - o], v2, ixx[o]);
-                        iyy[o] = fmaf(tp.g2[j - o], v0, iyy[o]);
-                        ixy[o] = fmaf(tp.g1[j - o], v1, ixy[o]);
-                    }
-            }
-        } else {
-            for (int k = 0; k <= 2 * R; ++k) {
-                const float g = tp.g[k], g1 = tp.g1[k], g2 = tp.g2[k];
-#pragma unroll
-                for (int o = 0; o < 4; ++o) {
-                    const float *const fo = f + (k + o) * kHX;
-                    ixx[o] = fmaf(g, fo[2 * FS], ixx[o]);
-                    iyy[o] = fmaf(g2, fo[0], iyy[o]);
-                    ixy[o] = fmaf(g1, fo[FS], ixy[o]);
+            for (int o = 0; o < 4; ++o)
+                if (j - o >= 0 && j - o <= 2 * R) {
+                    ixx[o] = fmaf(tp.g[j - o], v2, ixx[o]);
+                    iyy[o] = fmaf(tp.g2[j - o], v0, iyy[o]);
+                    ixy[o] = fmaf(tp.g1[j - o], v1, ixy[o]);
                 }
-            }
         }
         if (x0 + lane < nx) {
 #pragma unroll
@@ -190,20 +161,20 @@ __global__ void __launch_bounds__(kHThreads) k_hessian(const T *__restrict__ img
     }
 }
 
+template <class T, int... R>
+void launch_hessian_r(std::integer_sequence<int, R...>, dim3 grid, size_t sm, const T *img, float *D, int *smax, int nx,
+                      int ny, const DerivTaps &tp, float s4, cudaStream_t s) {
+    using Kernel = void (*)(const T *, float *, int *, int, int, DerivTaps, float);
+    constexpr Kernel kernels[] = {k_hessian<T, R>...};
+    kernels[tp.R]<<<grid, kHThreads, sm, s>>>(img, D, smax, nx, ny, tp, s4);
+}
 template <class T>
 void launch_hessian(const void *img, float *D, int *smax, int nx, int ny, int nz, const DerivTaps &tp, float s4,
                     cudaStream_t s) {
     const dim3 grid((unsigned)((nx + kHT - 1) / kHT), (unsigned)((ny + kHT - 1) / kHT), (unsigned)nz);
-    const int W = kHT + 2 * tp.R;
-    const size_t sm = sizeof(float) * (size_t)W * (hessian_pitch(tp.R) + 3 * kHX);  // at most 45 KB
-    const T *p = static_cast<const T *>(img);
-    switch (tp.R) {
-        case 3: k_hessian<T, 3><<<grid, kHThreads, sm, s>>>(p, D, smax, nx, ny, tp, s4); break;
-        case 5: k_hessian<T, 5><<<grid, kHThreads, sm, s>>>(p, D, smax, nx, ny, tp, s4); break;
-        case 6: k_hessian<T, 6><<<grid, kHThreads, sm, s>>>(p, D, smax, nx, ny, tp, s4); break;
-        case 9: k_hessian<T, 9><<<grid, kHThreads, sm, s>>>(p, D, smax, nx, ny, tp, s4); break;
-        default: k_hessian<T, 0><<<grid, kHThreads, sm, s>>>(p, D, smax, nx, ny, tp, s4);
-    }
+    const size_t sm = sizeof(float) * (size_t)(kHT + 2 * tp.R) * (hessian_pitch(tp.R) + 3 * kHX);  // at most 45 KB
+    launch_hessian_r(std::make_integer_sequence<int, kMaxR + 1>{}, grid, sm, static_cast<const T *>(img), D, smax, nx, ny,
+                     tp, s4, s);
 }
 
 // Seeds of 32 columns x kSeedRows rows of a slice: above t times the slice maximum and above

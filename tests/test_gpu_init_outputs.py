@@ -1,10 +1,11 @@
 """rsf_init_phi0 with outputs that share memory: the response is written first, then the seed mask,
-then phi0, wherever they lie."""
+then phi0, wherever they lie.  The response at every filter radius."""
 import ctypes
 
 import numpy as np
 import pytest
 
+import oracle
 from paper_2404_02813_gb300 import rsf
 
 torch = pytest.importorskip("torch")
@@ -54,3 +55,24 @@ def test_order_of_shared_outputs(at):
     assert _init(ctx, vol, base + at[0], base + at[1], base + at[2]) == n
     np.testing.assert_array_equal(buf.cpu().numpy(), want)
     ctx.close()
+
+
+@pytest.mark.parametrize("radius", range(17))
+@pytest.mark.parametrize("dtype", [np.uint8, np.float32])
+def test_response_at_every_radius(radius, dtype):
+    """Ragged tiles; the bound of test_gpu_init_lines (FP32 filters)."""
+    if not torch.cuda.is_available():
+        pytest.skip("needs a CUDA GPU")
+    rng = np.random.default_rng(radius)
+    vol = rng.uniform(0.0, 60.0, size=(2, 45, 71))
+    vol[1, 20:23, 30:33] += 150.0
+    vol = np.rint(vol).astype(dtype)
+    s = radius / 3 if radius else 0.1
+    resp = torch.empty(vol.shape, dtype=torch.float32, device="cuda")
+    ctx = rsf.Context(0)
+    ctx.init_phi0(torch.from_numpy(vol).cuda(), s, 0.3, 2.0, response=resp)
+    ctx.close()
+    resp, ref = resp.cpu().numpy(), oracle.doh_response(vol.astype(np.float64), s)
+    fin = np.isfinite(ref) & np.isfinite(resp)
+    assert fin.any()
+    np.testing.assert_allclose(resp[fin], ref[fin], rtol=0, atol=2e-5 * np.abs(ref[fin]).max())

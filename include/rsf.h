@@ -264,7 +264,8 @@ rsf_status rsf_step_stages(rsf_ctx *ctx, const void *volume, rsf_dtype vt, int64
  *                   shape by timing discarded first iterations, one knob after
  *                   the other: z planes per CTA of the x/y kernels (16, 8, 32,
  *                   fewer in groups too small to fill the GPU with that), the
- *                   update kernel's z chunk (a size heuristic, 32, 64, 128, 256) and the brick-to-CTA order (largest or smallest bricks
+ *                   update kernel's z chunk (a size heuristic, 32, 64, 128,
+ *                   256) and the brick-to-CTA order (largest or smallest bricks
  *                   first); the choice is remembered in the context per group
  *                   (radius, image type, storage, form, brick count, size
  *                   class) and listed by rsf_autotune_report.  0 (default):
@@ -281,14 +282,14 @@ rsf_status rsf_step_stages(rsf_ctx *ctx, const void *volume, rsf_dtype vt, int64
  *   RSF_OPT_FAULT_UPLOAD  k > 0: the serving loop's k-th upload of the active
  *                   bricks' launch descriptors fails on the host, without any
  *                   device work (for testing failure handling); the requests
- *                   active at that tick resolve RSF_E_CUDA with phi_out
+ *                   active in that lane resolve RSF_E_CUDA with phi_out
  *                   unwritten, queued ones are served afterwards; 0: off.
  *                   (A failed launch of a tick is handled the same way.)  Read
  *                   when the serving loop starts (the first rsf_submit).
- *   RSF_OPT_FAULT_WAIT  1: the z pass of group A arms each of its copy barriers
- *                   for 16 bytes more than its TMA copies deliver, so that its
- *                   bounded waits run out (1 s, then 1 s more for the copies in
- *                   flight) and the kernel records the expiry in the context's
+ *   RSF_OPT_FAULT_WAIT  1: the iteration's kernels arm each of their copy
+ *                   barriers for 16 bytes more than their TMA copies deliver,
+ *                   so that the bounded waits run out (1 s, then 1 s more for
+ *                   the copies in flight) and the kernels record the expiry in the context's
  *                   error word: the call returns RSF_E_CUDA, and so does every
  *                   later call on the context (for testing the device-side
  *                   failure path; no fault is raised); 0 (default): off.  Read
@@ -307,7 +308,7 @@ rsf_status rsf_step_stages(rsf_ctx *ctx, const void *volume, rsf_dtype vt, int64
  *                   brick of rsf_evolve_batch, each served request at
  *                   admission) fill the working fields the iteration writes
  *                   before it reads them -- the intermediate fields, the
- *                   second phi buffer and both Heaviside-argument buffers --
+ *                   second phi buffer and the Heaviside-argument block --
  *                   with all-ones bytes, a NaN in FP32, FP16 and BF16: a
  *                   result that depends on memory the iteration did not write
  *                   then carries NaN or differs from the unpoisoned one (a

@@ -1,6 +1,5 @@
 // rsf_ctx.h -- the context behind the C ABI's opaque rsf_ctx and the host
-// helpers shared by the translation units of the C ABI (rsf_api.cu,
-// rsf_batch.cu).  Not installed; not part of the ABI.
+// helpers shared by the translation units of the C ABI.  Not installed; not part of the ABI.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -64,7 +63,7 @@ struct rsf_ctx {
     int64_t opt_inject_upload = 0;      // and a descriptor upload of the active set
     int64_t opt_serve_slots = 64;       // bricks the serving loop advances together at most
     int opt_poison = 0;                 // fill working fields with NaN bytes before each solve (tests)
-    int opt_fault_wait = 0;             // z pass of group A expects bytes no copy delivers (tests)
+    int opt_fault_wait = 0;             // copy barriers expect bytes no copy delivers (tests)
     int *h_err = nullptr;               // error word of the kernels' bounded waits: mapped pinned host
     int *d_err = nullptr;               // memory and its device address; nonzero stays (the context is spent)
 };

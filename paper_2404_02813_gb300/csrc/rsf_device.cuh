@@ -44,20 +44,8 @@ __device__ __forceinline__ float heaviside_c(float u, float eps) {
     return u < 0.f ? 1.f - r : r;
 }
 
-// The tiled path stores the small side of Eq. (10), q = atan(eps/|u|)/pi in
-// (0, 1/2], carrying the sign of u (heaviside_q_fast in rsf_tiled.cuh); H is
-// -q for q < 0, else 1 - q.
-__device__ __forceinline__ float h_of_q(float q) { return q < 0.f ? -q : 1.f - q; }
-// 1 - H for the same q: 1 + q for q < 0, else q (its small side is q itself).
-__device__ __forceinline__ float hc_of_q(float q) { return q < 0.f ? 1.f + q : q; }
-
-// sqrt and reciprocal by the hardware approximations (PTX sqrt.approx.f32,
-// rcp.approx.ftz.f32, relative error of a few ulp); used for the unit normal only.
-__device__ __forceinline__ float sqrt_approx(float x) {
-    float y;
-    asm("sqrt.approx.f32 %0, %1;" : "=f"(y) : "f"(x));
-    return y;
-}
+// The hardware's reciprocal approximation (PTX rcp.approx.ftz.f32, relative error of a few ulp);
+// the tiled path's fast arithmetic only.
 __device__ __forceinline__ float rcp_approx(float x) {
     float y;
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));

@@ -43,7 +43,9 @@ constexpr long long kScratchFloats = kOffPart + 3 * rsf::kStatBlocks;
 constexpr int kMaxDevices = 64;
 // The tiled kernels' fields take the same memory from kOffI on: launch descriptor (with the
 // CTA offsets and the error word after it), q and stage blocks, where the x pitch (a multiple of 32) leaves room
-// for them: always when nx is a multiple of 32, or below about 0.8 of the voxel limit at nx >= 33.
+// for them: 24 bytes per voxel of a row rounded up to 32 and 8 of one rounded up to 4, where the
+// voxel limit has 36 per voxel -- always when nx is a multiple of 32, and up to 0.65 of the limit at
+// nx = 33, 0.78 at 40, 0.98 at 54, 0.82 at 65, 0.64 at 16, 0.18 at 4.
 constexpr size_t kDescBytes = (sizeof(rsf::BrickDev) + 64 + 255) / 256 * 256;
 constexpr size_t kFieldBytes = sizeof(float) * 9 * (size_t)kMaxVoxels;
 

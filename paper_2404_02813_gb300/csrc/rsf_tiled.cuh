@@ -47,7 +47,7 @@
 namespace rsf {
 namespace tiled {
 
-constexpr int kXYT = 32;          // x/y kernel: output tile edge (x and y)
+constexpr int kXYT = 32;          // x/y kernel: output columns of a tile (its rows: XYG)
 constexpr int kXYThreads = 256;   // 8 warps
 constexpr int kZX = 32;           // z march: columns (x) per CTA
 constexpr int kAZT = 64;          // x-z slab: output planes per CTA
@@ -74,31 +74,21 @@ __device__ __forceinline__ int clampi(int v, int lo, int hi) { return v < lo ? l
 
 template <class S> struct Store;
 template <> struct Store<float> {
-    using V4 = float4;
     using V2 = float2;
-    __device__ __forceinline__ static V4 pack4(float4 v) { return v; }
-    __device__ __forceinline__ static float4 unpack4(V4 v) { return v; }
     __device__ __forceinline__ static V2 pack2(float2 v) { return v; }
     __device__ __forceinline__ static float2 unpack2(V2 v) { return v; }
 };
 template <> struct Store<__half> {
-    using V4 = uint2;
     using V2 = uint32_t;
     __device__ __forceinline__ static uint32_t p(float a, float b) {
         __half2 h = __floats2half2_rn(a, b);
         return *reinterpret_cast<uint32_t *>(&h);
     }
     __device__ __forceinline__ static float2 u(uint32_t w) { return __half22float2(*reinterpret_cast<__half2 *>(&w)); }
-    __device__ __forceinline__ static V4 pack4(float4 v) { return make_uint2(p(v.x, v.y), p(v.z, v.w)); }
-    __device__ __forceinline__ static float4 unpack4(V4 v) {
-        const float2 a = u(v.x), b = u(v.y);
-        return make_float4(a.x, a.y, b.x, b.y);
-    }
     __device__ __forceinline__ static V2 pack2(float2 v) { return p(v.x, v.y); }
     __device__ __forceinline__ static float2 unpack2(V2 v) { return u(v); }
 };
 template <> struct Store<__nv_bfloat16> {
-    using V4 = uint2;
     using V2 = uint32_t;
     __device__ __forceinline__ static uint32_t p(float a, float b) {
         __nv_bfloat162 h = __floats2bfloat162_rn(a, b);
@@ -106,11 +96,6 @@ template <> struct Store<__nv_bfloat16> {
     }
     __device__ __forceinline__ static float2 u(uint32_t w) {
         return __bfloat1622float2(*reinterpret_cast<__nv_bfloat162 *>(&w));
-    }
-    __device__ __forceinline__ static V4 pack4(float4 v) { return make_uint2(p(v.x, v.y), p(v.z, v.w)); }
-    __device__ __forceinline__ static float4 unpack4(V4 v) {
-        const float2 a = u(v.x), b = u(v.y);
-        return make_float4(a.x, a.y, b.x, b.y);
     }
     __device__ __forceinline__ static V2 pack2(float2 v) { return p(v.x, v.y); }
     __device__ __forceinline__ static float2 unpack2(V2 v) { return u(v); }
@@ -131,7 +116,7 @@ struct GroupArgs {
     const BrickDev *bricks;
     const int *starts;  // nb + 1 CTA offsets of this kernel within the launch
     int nb;
-    int parity;         // launch parity: a brick reads phi[p], q[p] with p = parity ^ flip, writes the other
+    int parity;         // launch parity: a brick reads phi[p] with p = parity ^ flip, writes the other
     int *err;           // the group's error word (bounded waits), may be null
     unsigned fault_tx;  // extra bytes the TMA barriers expect (0; > 0 only in a fault test)
 };
@@ -340,8 +325,9 @@ struct SrcH {  // NP = 1: (H I~, H); NP = 2: also ((1-H) I~, 1-H), the other sid
         tma_load_3d(st, mq, x0 - FQ::RA, y0 - R, z, bar);
         tma_load_3d(st + IOFF, mi, x0 - FI::RA, y0 - R, z, bar);
     }
-    // q = 1 outside the brick: h_of_q(1) = 0, so both products vanish there (q itself is at
-    // most 1/2 in magnitude; zero-filled q would read as H = 1)
+    // q is the small side of Eq. (10), atan(eps/|phi|)/pi with the sign of phi: H = -q where it is
+    // negative, else 1 - q.  q = 1 outside the brick: H = 0, so both products vanish there (q
+    // itself is at most 1/2 in magnitude; zero-filled q would read as H = 1)
     __device__ __forceinline__ void fix(unsigned char *st, int x0, int y0, int nx, int ny) const {
         float *q = reinterpret_cast<float *>(st);
         const int lane = threadIdx.x & 31;
@@ -641,9 +627,9 @@ __global__ void __launch_bounds__(kXYThreads, (SrcAB<R, S>::CTAS)) k_tb_xy(Group
 // halos) of the x/y-convolved pair (H I~, H), and the kAZT planes of K*I~ the
 // slab's outputs use.  A persistent CTA walks the slabs of the launch
 // (consecutive slabs are consecutive z ranges of one row, so shared halos hit
-// L2) with a two-stage shared-memory buffer: the cp.async copies of the next
-// slab are in flight while the current one is convolved.  Rows outside the
-// brick are zero-filled by the copy (source size 0).
+// L2) with a two-stage shared-memory buffer: the TMA boxes of the next slab
+// are in flight while the current one is convolved.  Planes outside the brick
+// and columns past nx arrive as zeros.
 template <int R>
 constexpr int az_stage() { return (kAZT + 2 * R) * 32 + kAZT * 16; }  // float2 units per stage
 template <int R>

@@ -1,5 +1,5 @@
 // rsf_tiled_f32.cu -- instantiates the tiled iteration with FP32 storage (see
-// rsf_tiled.cuh), the q set-up kernel and the host-side launch dispatch.
+// rsf_tiled.cuh), the set-up kernels and the host-side launch dispatch.
 #include <cudaTypedefs.h>  // PFN_cuTensorMapEncodeTiled
 
 #include <cmath>
@@ -380,8 +380,8 @@ void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]) {
 // for 12), and costs long ones more than that: an SM whose shared-memory carve-out an earlier
 // kernel set lower keeps it until it drains, and with the largest carve-out everywhere the L1
 // is too small (five iterations of 512^3: 11.3 ms without overlap, 12.2 with it, 11.6 with the
-// carve-out too; 160^3 sub-volumes, 2400 CTAs, 9.65, 10.0, 9.80 ms).  The line: two waves of
-// the x/y kernels.
+// carve-out too; 160^3 sub-volumes, 2400 CTAs, 9.65, 10.0, 9.80 ms).  The line: eight CTAs per SM
+// in group A's x/y kernel, two waves of Li's form (four share an SM), 2.7 of the others (three).
 bool tiled_overlap(const TiledGroup &g, int sms) { return g.ncta[0] <= 8u * (unsigned)sms; }
 
 // A CTA of the x/y kernels costs its planes plus about one plane time (set-up and the first

@@ -567,12 +567,12 @@ static rsf_status run(rsf_ctx *c, const void *volume, rsf_dtype vt, int64_t nx, 
         b.zs = b.zc;
         int sms = 0;
         RSF_CUDA(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, c->device));
-        b.xyp = rsf::tiled_xy_planes({b}, form, taps.R, sms);
+        b.xyp = rsf::tiled_xy_planes(&b, 1, form, taps.R, sms);
         if (b.zc <= 0) {
             const long long nxy = (long long)((nx + 31) / 32) * ((ny + 7) / 8);
             const long long chunks = std::max<long long>(1, (16LL * sms + nxy - 1) / nxy);
             b.zc = (int)std::max<long long>(16, (nz + chunks - 1) / chunks);
-            b.zs = rsf::tiled_update_planes({b}, form, taps.R, b.zc, sms);
+            b.zs = rsf::tiled_update_planes(&b, 1, form, taps.R, b.zc, sms);
         }
         b.dump = dump;  // only rsf_step_stages asks for stages, and it runs one iteration
         GroupSpec spec;

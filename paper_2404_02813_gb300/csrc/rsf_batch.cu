@@ -72,7 +72,7 @@ std::string group_key(const GroupSpec &g) {
 
 // sms > 0: a chunk may be split over several CTAs; 0: one CTA per chunk.
 void set_zc(GroupSpec &g, int zc, int sms) {
-    const int zs = sms > 0 ? rsf::tiled_update_planes(g.bricks, g.force, g.taps.R, zc, sms) : zc;
+    const int zs = sms > 0 ? rsf::tiled_update_planes(g.bricks.data(), (int)g.bricks.size(), g.force, g.taps.R, zc, sms) : zc;
     for (rsf::BrickDev &b : g.bricks) {
         b.zc = zc;
         b.zs = zs;
@@ -92,7 +92,7 @@ rsf_status launch_all(rsf_ctx *c, const std::vector<rsf::TiledGroup> &groups, in
 // (16 is the most the size heuristic takes; 32 goes beyond it).
 constexpr int kXYPlanes = 16;
 void set_xyp(GroupSpec &g, int xyp, int sms) {
-    const int fit = rsf::tiled_xy_planes(g.bricks, g.force, g.taps.R, sms);
+    const int fit = rsf::tiled_xy_planes(g.bricks.data(), (int)g.bricks.size(), g.force, g.taps.R, sms);
     const int planes = fit == kXYPlanes ? xyp : std::min(xyp, fit);
     for (rsf::BrickDev &b : g.bricks) b.xyp = planes;
 }

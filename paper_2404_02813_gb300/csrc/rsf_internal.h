@@ -156,9 +156,9 @@ bool tiled_overlap(const TiledGroup &g, int sms);
 // CTAs of the four kernels for one brick of a group of the given form and radius.
 void tiled_cta_counts(const BrickDev &b, int force, int R, unsigned counts[4]);
 // Planes per CTA of the x/y kernels for bricks launched together (results do not depend on it).
-int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int sms);
+int tiled_xy_planes(const BrickDev *bricks, int nb, int force, int R, int sms);
 // Planes per CTA of the update kernel (at most zc) for bricks launched together with z chunk zc.
-int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, int zc, int sms);
+int tiled_update_planes(const BrickDev *bricks, int nb, int force, int R, int zc, int sms);
 // A brick's working memory beside its phi buffers: a stage block of
 // tiled_stage_bytes(storage, px ny nz) bytes, and directly in front of it a q block of
 // tiled_q_bytes(nx, ny nz) bytes (anywhere for a stage block of 28 px ny nz bytes or more).

@@ -147,9 +147,9 @@ cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Ta
     cudaError_t e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess) return e;
     if ((e = rsf::tiled_prepare(0, taps.R, rsf::kForceExact)) != cudaSuccess) return e;
-    b.xyp = rsf::tiled_xy_planes({b}, rsf::kForceExact, taps.R, sms);
+    b.xyp = rsf::tiled_xy_planes(&b, 1, rsf::kForceExact, taps.R, sms);
     b.zc = b.nz;
-    b.zs = rsf::tiled_update_planes({b}, rsf::kForceExact, taps.R, b.zc, sms);
+    b.zs = rsf::tiled_update_planes(&b, 1, rsf::kForceExact, taps.R, b.zc, sms);
     if ((e = rsf::tiled_encode_maps(b, rsf::kForceExact, 0, 2, taps.R)) != cudaSuccess) return e;
     rsf::TiledGroup g{};
     g.force = rsf::kForceExact;

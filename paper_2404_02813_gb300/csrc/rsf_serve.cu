@@ -331,7 +331,7 @@ bool admit(Server *s, const std::shared_ptr<Request> &r) {
         SetupDesc *const dev = reinterpret_cast<SetupDesc *>(s->partials);
         SetupDesc sd{};
         sd.b = d;
-        sd.b.xyp = rsf::tiled_xy_planes({d}, 0, r->taps.R, s->sms);
+        sd.b.xyp = rsf::tiled_xy_planes(&d, 1, 0, r->taps.R, s->sms);
         if (rsf::tiled_encode_maps(sd.b, 0, r->storage, (int)q.vt, r->taps.R) != cudaSuccess) return fail_admit(RSF_E_CUDA);
         rsf::TiledGroup g{};
         g.imgtype = (int)q.vt;
@@ -406,8 +406,9 @@ bool rebuild_groups(Server *s, Lane &L) {
             maxnz = std::max(maxnz, b.nz);
         }
         const int zc = (int)std::min<long long>(maxnz, std::max<long long>(16, work / std::max(1LL, 16LL * s->sms)));
-        const int xyp = rsf::tiled_xy_planes(g.bricks, g.force, g.taps.R, s->sms);
-        const int zs = rsf::tiled_update_planes(g.bricks, g.force, g.taps.R, zc, s->sms);
+        const int nb = (int)g.bricks.size();
+        const int xyp = rsf::tiled_xy_planes(g.bricks.data(), nb, g.force, g.taps.R, s->sms);
+        const int zs = rsf::tiled_update_planes(g.bricks.data(), nb, g.force, g.taps.R, zc, s->sms);
         for (rsf::BrickDev &b : g.bricks) {
             b.zc = zc;
             b.zs = zs;

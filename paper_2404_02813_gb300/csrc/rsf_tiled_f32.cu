@@ -388,15 +388,15 @@ bool tiled_overlap(const TiledGroup &g, int sms) { return g.ncta[0] <= 8u * (uns
 // copies; 64^3: 1 plane per CTA 8.1 us, 16 planes 37 us; 512^3: 16 planes 0.463 ms, 32 planes
 // 0.480 ms, so 16 is the most); three or four share an SM.  Few CTAs run in whole waves; many even out but for
 // about half a CTA at the end.
-int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int sms) {
+int tiled_xy_planes(const BrickDev *bricks, int nb, int force, int R, int sms) {
     const int th = xy_rows(R);
     const double slots = (force ? 3.0 : 4.0) * sms;
     int best = 1;
     double best_cost = 0.0;
     for (int p : {1, 2, 3, 4, 6, 8, 12, 16}) {
         double ctas = 0.0;
-        for (const BrickDev &b : bricks)
-            ctas += (double)((b.nx + tiled::kXYT - 1) / tiled::kXYT) * ((b.ny + th - 1) / th) * ((b.nz + p - 1) / p);
+        for (const BrickDev *b = bricks; b != bricks + nb; ++b)
+            ctas += (double)((b->nx + tiled::kXYT - 1) / tiled::kXYT) * ((b->ny + th - 1) / th) * ((b->nz + p - 1) / p);
         const double waves = ctas / slots;
         const double cost = (waves < 4.0 ? std::ceil(waves) : waves + 0.5) * (p + 1.0);
         if (p == 1 || cost < best_cost) {
@@ -411,7 +411,7 @@ int tiled_xy_planes(const std::vector<BrickDev> &bricks, int force, int R, int s
 // fill its rings (M (a, b) planes at 8 of the 22 bytes a voxel moves, and the latency of the
 // first copies).  Two CTAs share an SM.  Few CTAs run in whole waves; many even out but for
 // about half a CTA at the end.
-int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, int zc, int sms) {
+int tiled_update_planes(const BrickDev *bricks, int nb, int force, int R, int zc, int sms) {
     const UpdateTile tile = update_tile(force, R);
     const double fill = 4.0 + 0.4 * tile.planes, slots = 2.0 * sms;
     int best = zc, last = 0;
@@ -425,9 +425,9 @@ int tiled_update_planes(const std::vector<BrickDev> &bricks, int force, int R, i
         }
         last = zs;
         double ctas = 0.0;
-        for (const BrickDev &b : bricks) {
-            const int chunks = b.nz / zc, rest = b.nz % zc;
-            ctas += (double)((b.nx + tiled::kZX - 1) / tiled::kZX) * ((b.ny + tile.rows - 1) / tile.rows) *
+        for (const BrickDev *b = bricks; b != bricks + nb; ++b) {
+            const int chunks = b->nz / zc, rest = b->nz % zc;
+            ctas += (double)((b->nx + tiled::kZX - 1) / tiled::kZX) * ((b->ny + tile.rows - 1) / tile.rows) *
                     (chunks * ((zc + zs - 1) / zs) + (rest + zs - 1) / zs);
         }
         const double waves = ctas / slots;

@@ -102,18 +102,6 @@ rsf_status scratch_on_current_device(float **out) {
     return RSF_OK;
 }
 
-// Memory the kernels of device `dev` may read and write in place: device memory
-// of that device, or managed memory.  (Device memory of another GPU is refused:
-// without peer access a kernel here would fault on it.)
-bool is_device_ptr(const void *p, int dev) {
-    cudaPointerAttributes a;
-    if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
-        cudaGetLastError();
-        return false;
-    }
-    return (a.type == cudaMemoryTypeDevice && a.device == dev) || a.type == cudaMemoryTypeManaged;
-}
-
 __global__ void k_noalloc_put(ParamChunk c, float *__restrict__ dst) {
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < c.count; i += gridDim.x * blockDim.x)
         dst[c.offset + i] = c.v[i];
@@ -201,7 +189,8 @@ rsf_status evolve(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int6
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return err(RSF_E_CUDA, cudaGetErrorString(e));
-    if (!is_device_ptr(volume, dev) || !is_device_ptr(phi0, dev) || !is_device_ptr(phi_out, dev))
+    // (device memory of another GPU is refused too: without peer access a kernel here would fault on it)
+    if (!in_place(volume, dev, 1) || !in_place(phi0, dev, 1) || !in_place(phi_out, dev, 1))
         return err(RSF_E_INVAL, "rsf_evolve_noalloc takes device pointers of the current device only");
 
     float *base = nullptr;

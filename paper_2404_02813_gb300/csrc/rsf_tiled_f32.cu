@@ -190,36 +190,36 @@ cudaError_t encode_map(CUtensorMap *m, const void *base, int c, const BrickDev &
 // Box widths (values) and rows of the x/y kernels' staged planes.
 struct XYBoxes { int rows, q, img, ab32, ab16; };
 template <int R>
-XYBoxes xy_boxes_r(int imgtype) {
+XYBoxes xy_boxes_r(int imgtype, int ny) {
     using namespace tiled;
     const int img = imgtype == 0 ? SrcH<R, uint8_t, 1, false>::FI::W : (imgtype == 1 ? SrcH<R, uint16_t, 1, false>::FI::W : SrcH<R, float, 1, false>::FI::W);
-    return XYBoxes{XYG<R>::H, SrcH<R, float, 1, false>::FQ::W, img, SrcAB<R, float>::FA::W, SrcAB<R, __half>::FA::W};
+    return XYBoxes{xy_box_rows<R>(ny), SrcH<R, float, 1, false>::FQ::W, img, SrcAB<R, float>::FA::W, SrcAB<R, __half>::FA::W};
 }
-XYBoxes xy_boxes(int R, int imgtype) {
+XYBoxes xy_boxes(int R, int imgtype, int ny) {
     switch (R) {
-        case 1: return xy_boxes_r<1>(imgtype);
-        case 2: return xy_boxes_r<2>(imgtype);
-        case 3: return xy_boxes_r<3>(imgtype);
-        case 4: return xy_boxes_r<4>(imgtype);
-        case 5: return xy_boxes_r<5>(imgtype);
-        case 6: return xy_boxes_r<6>(imgtype);
-        case 7: return xy_boxes_r<7>(imgtype);
-        case 8: return xy_boxes_r<8>(imgtype);
-        case 9: return xy_boxes_r<9>(imgtype);
-        case 10: return xy_boxes_r<10>(imgtype);
-        case 11: return xy_boxes_r<11>(imgtype);
-        case 12: return xy_boxes_r<12>(imgtype);
-        case 13: return xy_boxes_r<13>(imgtype);
-        case 14: return xy_boxes_r<14>(imgtype);
-        case 15: return xy_boxes_r<15>(imgtype);
-        default: return xy_boxes_r<16>(imgtype);
+        case 1: return xy_boxes_r<1>(imgtype, ny);
+        case 2: return xy_boxes_r<2>(imgtype, ny);
+        case 3: return xy_boxes_r<3>(imgtype, ny);
+        case 4: return xy_boxes_r<4>(imgtype, ny);
+        case 5: return xy_boxes_r<5>(imgtype, ny);
+        case 6: return xy_boxes_r<6>(imgtype, ny);
+        case 7: return xy_boxes_r<7>(imgtype, ny);
+        case 8: return xy_boxes_r<8>(imgtype, ny);
+        case 9: return xy_boxes_r<9>(imgtype, ny);
+        case 10: return xy_boxes_r<10>(imgtype, ny);
+        case 11: return xy_boxes_r<11>(imgtype, ny);
+        case 12: return xy_boxes_r<12>(imgtype, ny);
+        case 13: return xy_boxes_r<13>(imgtype, ny);
+        case 14: return xy_boxes_r<14>(imgtype, ny);
+        case 15: return xy_boxes_r<15>(imgtype, ny);
+        default: return xy_boxes_r<16>(imgtype, ny);
     }
 }
 }  // namespace
 
 cudaError_t tiled_encode_maps(BrickDev &b, int force, int storage, int imgtype, int R) {
     const int zrows = tiled::kAZT + 2 * R;
-    const XYBoxes box = xy_boxes(R, imgtype);
+    const XYBoxes box = xy_boxes(R, imgtype, b.ny);
     b.tm_k = b.tm_ab = CUtensorMap{};
     cudaError_t e = encode_typed(&b.tm_q, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, 4, b.q, 1, b.qp, b, box.q, box.rows, 1);
     if (e != cudaSuccess) return e;

@@ -72,7 +72,7 @@ struct ParamChunk {
 };
 
 __global__ void k_noalloc_put(ParamChunk c, float *__restrict__ dst);
-__global__ void k_noalloc_check(const int *err, float *phi, int n);
+__global__ void k_noalloc_finish(const int *err, const float *phi, float *phi_out, int n);
 
 // Device address of the static array on the current device, looked up once per
 // device (with that device current).  The name g_noalloc_scratch is only a
@@ -93,7 +93,7 @@ rsf_status scratch_on_current_device(float **out) {
             snprintf(buf, sizeof buf, "cudaGetSymbolAddress of the static scratch failed: %s", cudaGetErrorString(e));
             return err(RSF_E_CUDA, buf);
         }
-        if ((e = rsf::load_kernels(k_noalloc_put, k_noalloc_check)) == cudaSuccess) e = rsf::load_passes();
+        if ((e = rsf::load_kernels(k_noalloc_put, k_noalloc_finish)) == cudaSuccess) e = rsf::load_passes();
         if (e == cudaSuccess) e = rsf::load_exact();
         if (e != cudaSuccess) return err(RSF_E_CUDA, cudaGetErrorString(e));
         g_scratch_dev[dev] = (float *)p;
@@ -107,12 +107,16 @@ __global__ void k_noalloc_put(ParamChunk c, float *__restrict__ dst) {
         dst[c.offset + i] = c.v[i];
 }
 
-// The result of a solve in which a kernel's bounded wait ran out (it then left tiles unwritten):
-// NaN throughout, as this entry has no other way to tell -- it returns before the kernels run.
-__global__ void __launch_bounds__(256) k_noalloc_check(const int *err, float *phi, int n) {
+// phi, where the last iteration left it, to phi_out.  After a solve in which a kernel's bounded wait
+// ran out (it then left tiles unwritten) phi_out is NaN throughout: this entry has no other way to
+// tell, as it returns before the kernels run.
+__global__ void __launch_bounds__(256) k_noalloc_finish(const int *err, const float *phi, float *phi_out, int n) {
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
     rsf::tiled::wait_for_previous();
-    if (*err == 0) return;
-    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) phi[i] = NAN;
+    const float v = phi[i];
+    const bool bad = *err != 0;
+    if (bad || phi != phi_out) phi_out[i] = bad ? NAN : v;
 }
 
 void put_floats(const float *v, int n, float *dst, cudaStream_t s) {
@@ -125,7 +129,8 @@ void put_floats(const float *v, int n, float *dst, cudaStream_t s) {
     }
 }
 
-// The iterations in the tiled schedule (rsf_exact.cuh), all fields in `mem`; phi[0] holds phi0.
+// The iterations in the tiled schedule (rsf_exact.cuh), all fields in `mem`; phi[0] holds phi0,
+// phi[1] is phi_out and gets the result.
 // fault_tx: as in TiledGroup.
 cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Taps &taps, int iters, char *mem, int dev,
                          unsigned fault_tx, cudaStream_t s) {
@@ -164,7 +169,7 @@ cudaError_t evolve_tiled(rsf::BrickDev b, const void *vol, int vt, const rsf::Ta
     for (int it = 0; it < iters; ++it)
         if ((e = rsf::tiled_iterate(g, it & 1, nullptr, s)) != cudaSuccess) return e;
     const int n = b.nx * b.ny * b.nz;
-    rsf::tiled::launch_next(g.overlap, k_noalloc_check, (n + 2047) / 2048, 256, 0, s, g.err, b.phi[iters & 1], n);
+    rsf::tiled::launch_next(g.overlap, k_noalloc_finish, (n + 255) / 256, 256, 0, s, g.err, b.phi[iters & 1], b.phi[1], n);
     return cudaGetLastError();
 }
 
@@ -249,7 +254,7 @@ rsf_status evolve(const void *volume, rsf_dtype vt, int64_t nx, int64_t ny, int6
         if ((e = evolve_tiled(b, volume, (int)vt, taps, iters, reinterpret_cast<char *>(base + kOffI), dev, fault_tx,
                               s)) != cudaSuccess)
             return err(RSF_E_CUDA, cudaGetErrorString(e));
-        in = iters % 2 ? phi_out : scratch_phi;
+        in = phi_out;
     } else {
         float *out = phi_out;
         for (int it = 0; it < iters; ++it) {

@@ -66,11 +66,11 @@ PAPER_TABLE1_GVOX_IT_S = 1.25e8 / 0.585 / 1e9
 # DRAM traffic per voxel measured by ncu (dram__bytes_read.sum + dram__bytes_write.sum
 # per launch / voxels), keyed by kernel, with the SHA-256 of the kernel source file
 # it was captured from; reported only while that file is unchanged.
-NCU_SHA = "ca018349217ab567"
+NCU_SHA = "b70feb34a7bf2a0a"
 NCU_TRAFFIC = {
     k: {"bytes_per_voxel": v, "source": "rsf_tiled.cuh", "source_sha": NCU_SHA,
         "capture": "384^3 uint16 light-sheet case, sigma 3, FP32 storage; scaled by voxels"}
-    for k, v in {"rsf_ta_xy": 13.39, "rsf_ta_z": 19.36, "rsf_tb_xy": 15.15, "rsf_tb_z": 21.62}.items()
+    for k, v in {"rsf_ta_xy": 13.44, "rsf_ta_z": 19.42, "rsf_tb_xy": 15.20, "rsf_tb_z": 21.69}.items()
 }
 
 # Warp instructions issued per voxel measured by ncu (smsp__inst_executed.sum / voxels),
@@ -79,7 +79,7 @@ NCU_TRAFFIC = {
 NCU_INST = {
     k: {"warp_inst_per_voxel": v, "source": "rsf_tiled.cuh", "source_sha": NCU_SHA,
         "capture": "384^3 uint16 light-sheet case, sigma 3, FP32 storage"}
-    for k, v in {"rsf_ta_xy": 2.87, "rsf_ta_z": 2.42, "rsf_tb_xy": 1.68, "rsf_tb_z": 3.56}.items()
+    for k, v in {"rsf_ta_xy": 2.86, "rsf_ta_z": 2.42, "rsf_tb_xy": 1.68, "rsf_tb_z": 3.56}.items()
 }
 SM_SUBPARTITIONS = 4  # warp schedulers per SM, one warp instruction issued per cycle each
 

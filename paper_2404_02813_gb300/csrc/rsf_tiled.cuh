@@ -246,7 +246,7 @@ __device__ __forceinline__ void report_error(int *err, int code) {
 // boxes are larger and whose phases shorter: two buffers, three CTAs per SM (0.342 against
 // 0.370 ms at 512^3 with one buffer and four CTAs).
 //
-// Per launch, before and now: 512^3 uint16 radius 6, (H I~, H) 0.541 -> 0.463 ms (issue and
+// Per launch, before and now: 512^3 uint16 radius 6, (H I~, H) 0.541 -> 0.459 ms (issue and
 // FMA pipe 60 and 50 % busy), (a, b) 0.393 -> 0.342 ms (0.92 of the HBM rate); 512 x 448 x
 // 320 radius 10 0.519 -> 0.400 and 0.327 -> 0.282 ms; both pairs, 500^3 uint8 radius 10,
 // 1.741 -> 1.12 ms (FMA pipe 65 %: 105 packed FMAs per voxel); (a, b) in BF16, 768^3, 1.764
